@@ -107,43 +107,244 @@ __global__ void __launch_bounds__(FSEL_THREADS) flat_select_kernel(const float* 
     if (tid == 0) slot_cnt[slot] = kept;
 }
 
-// slot (q, ch) holds slot_cnt keys at slot_keys[(q * nchunks + ch) * stride ...]; with `raw` they are the raw
-// candidate entries of the tensor-core kernel (cand_key turns them into keys).
-__global__ void __launch_bounds__(FSEL_THREADS) flat_merge_kernel(int nchunks, int k, int stride, int raw, uint32_t raw_sign,
-                                                                  const int32_t* __restrict__ slot_cnt,
-                                                                  const unsigned long long* __restrict__ slot_keys,
-                                                                  int64_t* __restrict__ out_ids,
-                                                                  float* __restrict__ out_scores) {
-    __shared__ unsigned long long keys[TOPK_CAP];
-    __shared__ int cnt;
-    const int tid = threadIdx.x, q = blockIdx.x;
-    auto sync = [] { __syncthreads(); };
-    if (tid == 0) cnt = 0;
-    __syncthreads();
-    unsigned long long tau = KEY_MAX;
-    for (int ch = 0; ch < nchunks; ++ch) {
-        const size_t slot = (size_t)q * nchunks + ch;
-        const int c = slot_cnt[slot];
-        if (cnt + c > TOPK_CAP) {
-            const int kept = block_select(keys, &cnt, k, tid, FSEL_THREADS, sync);
-            if (kept == k) tau = keys[k - 1];
+// Final selection of a query: the k best of its candidate lists, best first.
+//
+// List l of query q holds slot_cnt entries at slot_keys[(q * nlists + l) * stride ...]; with `raw` they are the raw
+// candidate entries of the tensor-core kernel (cand_key turns them into keys).  Latency is what counts here: a query
+// has a few hundred short lists (one per column range and half tile), and walking them one after the other cost
+// about a microsecond per list (290 us for one query over 100 000 rows, 264 us for 37 over a million, 308 us for 256
+// over ten million).  So the counts of up to FM_LISTS lists are fetched at once and summed, the entries are numbered
+// through, and every thread fetches FM_KPT of them side by side; a counting bisection on the keys (distinct, so it
+// always ends) finds a cut with between k and k + k/4 + 8 keys at or below it, and only those are ranked.  More
+// entries than one round holds go through further rounds against the cut of the rounds before.
+//
+// nq * parts CTAs.  Without starting thresholds a list keeps everything it saw, and one CTA would pull a hundred
+// thousand entries through one SM; a small batch then splits a query's lists into parts.  Each part leaves its keys in
+// the storage of its own first list (read by nobody else), and the part that finishes last (a ticket per query, zero
+// before the launch) selects among what the parts left.
+constexpr int FM_THREADS = 512, FM_KPT = 8, FM_LISTS = 512;
+constexpr int FM_ENTRIES = FM_THREADS * FM_KPT;  // entries of one round
+constexpr int FM_MAX_PARTS = 32;
+constexpr int FM_OLD = 4;                        // keys of earlier rounds a thread takes back: at most MAX_K * 5 / 4 + 8 in all
+static_assert(FM_OLD * FM_THREADS >= TOPK_CAP && MAX_K + MAX_K / 4 + 8 <= TOPK_CAP, "a round's survivors fit the buffer");
+constexpr int FM_TICKET_WORD = 32;               // tickets lie in the error block, one word per query
+constexpr int FM_TICKETS = 64 - FM_TICKET_WORD;
+
+struct FlatMergeState {
+    unsigned long long keys[TOPK_CAP];
+    int pre[FM_LISTS + 1];
+    int wsum[FM_THREADS / 32];
+    unsigned long long mn, mx;
+    uint32_t nv, round[3];
+    int cnt, last;
+};
+
+// Adds the entries of lists slot_of(l), l0 <= l < l1 (count cnts[slot], entries at entries[slot * stride ...]), to the
+// keys the buffer holds and leaves between min(k, all) and k + k/4 + 8 of the smallest there.
+template <class SlotOf>
+__device__ __forceinline__ void flat_merge_lists(FlatMergeState& S, const int32_t* cnts, const unsigned long long* entries,
+                                                 int l0, int l1, SlotOf slot_of, int stride, int raw, uint32_t raw_sign,
+                                                 int k) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t want_max = (uint32_t)(k + (k >> 2) + 8 > WARP_SORT_MAX ? k + (k >> 2) + 8 : WARP_SORT_MAX);
+    unsigned long long bound = KEY_MAX - 1;  // nothing above it can be a result
+    for (int g0 = l0; g0 < l1; g0 += FM_LISTS) {
+        const int ng = l1 - g0 < FM_LISTS ? l1 - g0 : FM_LISTS;
+        {   // exclusive prefix of the counts (FM_LISTS <= FM_THREADS: one list per thread)
+            const int c = tid < ng ? __ldcg(cnts + slot_of(g0 + tid)) : 0;
+            int incl = c;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            if (lane == 31) S.wsum[warp] = incl;
             __syncthreads();
-        }
-        for (int i0 = 0; i0 < c; i0 += FSEL_THREADS) {
-            const int i = i0 + tid;
-            unsigned long long key = KEY_MAX;
-            if (i < c) key = raw ? cand_key(slot_keys[slot * stride + i], raw_sign) : slot_keys[slot * stride + i];
-            warp_push(keys, &cnt, i < c && key < tau, key);
+            if (warp == 0) {
+                int w = lane < FM_THREADS / 32 ? S.wsum[lane] : 0;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, w, o);
+                    if (lane >= o) w += y;
+                }
+                if (lane < FM_THREADS / 32) S.wsum[lane] = w;
+            }
+            __syncthreads();
+            if (tid < ng) S.pre[tid + 1] = (warp ? S.wsum[warp - 1] : 0) + incl;
+            if (tid == 0) S.pre[0] = 0;
         }
         __syncthreads();
+        const int nitems = S.pre[ng];
+        // Many entries: the first round's bound leaves few of the rest, which are therefore streamed past it, a warp per
+        // list and with no numbering, at a tenth of the instructions of a round.  What passes joins the first round's
+        // keys in the buffer; if it does not fit, the pass counts for nothing and all rounds are taken.
+        bool streamed = false;
+        for (int r0 = 0; r0 < nitems; r0 += FM_ENTRIES) {  // uniform
+            if (r0 == FM_ENTRIES && nitems > 2 * FM_ENTRIES && bound != KEY_MAX - 1 && !streamed) {
+                const int before = S.cnt;
+                __syncthreads();
+                const uint32_t bound32 = (uint32_t)(bound >> 32);
+                for (int l = warp; l < ng; l += FM_THREADS / 32) {
+                    const int skip = r0 - S.pre[l], n = S.pre[l + 1] - S.pre[l];  // entries the first round has seen
+                    const unsigned long long* src = entries + (size_t)slot_of(g0 + l) * stride;
+                    for (int i0 = skip > 0 ? skip : 0; i0 < n; i0 += 32 * FM_KPT) {
+                        unsigned long long e[FM_KPT];
+                        bool any = false;
+#pragma unroll
+                        for (int j = 0; j < FM_KPT; ++j) {
+                            const int i = i0 + 32 * j + lane;
+                            e[j] = i < n ? __ldcg(src + i) : KEY_MAX;
+                        }
+#pragma unroll
+                        for (int j = 0; j < FM_KPT; ++j) {
+                            if (i0 + 32 * j + lane < n && raw) e[j] = cand_key(e[j], raw_sign);
+                            any = any || (uint32_t)(e[j] >> 32) <= bound32;
+                        }
+                        if (!__any_sync(0xffffffffu, any)) continue;
+#pragma unroll
+                        for (int j = 0; j < FM_KPT; ++j) warp_push(S.keys, &S.cnt, e[j] <= bound, e[j]);
+                    }
+                }
+                __syncthreads();
+                if (S.cnt <= TOPK_CAP) {  // uniform
+                    streamed = true;
+                    r0 = nitems;  // one last round with no new entries, which cuts the buffer
+                } else {
+                    __syncthreads();
+                    if (tid == 0) S.cnt = before;  // the first round's keys are intact; the pushes that fitted lie behind them
+                    __syncthreads();
+                }
+            }
+            unsigned long long mine[FM_KPT + FM_OLD];
+            unsigned long long mn = KEY_MAX, mx = 0ull;
+            uint32_t nv = 0;
+#pragma unroll
+            for (int j = 0; j < FM_KPT; ++j) {
+                const int e = r0 + j * FM_THREADS + tid;
+                mine[j] = KEY_MAX;
+                if (e < nitems) {
+                    int lo = 0, hi = ng;  // pre[lo] <= e < pre[hi]
+                    while (hi - lo > 1) {
+                        const int mid = (lo + hi) >> 1;
+                        if (S.pre[mid] <= e) lo = mid; else hi = mid;
+                    }
+                    mine[j] = __ldcg(entries + (size_t)slot_of(g0 + lo) * stride + (e - S.pre[lo]));
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < FM_KPT; ++j) {
+                if (r0 + j * FM_THREADS + tid >= nitems) continue;
+                if (raw) mine[j] = cand_key(mine[j], raw_sign);
+                if (mine[j] > bound) mine[j] = KEY_MAX;
+            }
+            const int old = S.cnt;
+#pragma unroll
+            for (int j = 0; j < FM_OLD; ++j) {
+                const int i = tid + j * FM_THREADS;
+                mine[FM_KPT + j] = i < old ? S.keys[i] : KEY_MAX;
+            }
+#pragma unroll
+            for (int j = 0; j < FM_KPT + FM_OLD; ++j) {
+                if (mine[j] == KEY_MAX) continue;
+                mn = mine[j] < mn ? mine[j] : mn;
+                mx = mine[j] > mx ? mine[j] : mx;
+                ++nv;
+            }
+            if (tid == 0) { S.mn = KEY_MAX; S.mx = 0ull; S.nv = 0u; S.round[0] = S.round[1] = S.round[2] = 0u; }
+            __syncthreads();  // the old keys and their count have been read, the shared words are initialised
+            if (tid == 0) S.cnt = 0;
+            nv = __reduce_add_sync(0xffffffffu, nv);
+            if (nv) {  // uniform within the warp
+                for (int o = 16; o; o >>= 1) {
+                    const unsigned long long a = shfl_xor_u64(mn, o), b = shfl_xor_u64(mx, o);
+                    mn = a < mn ? a : mn;
+                    mx = b > mx ? b : mx;
+                }
+                if (lane == 0) { atomicMin(&S.mn, mn); atomicMax(&S.mx, mx); atomicAdd(&S.nv, nv); }
+            }
+            __syncthreads();
+            uint32_t c_hi = S.nv;
+            // First on the score words alone (half the instructions of a 64-bit compare), then, if a group of equal
+            // scores is still too large, on whole keys: #(key <= lo) <= k and #(key <= hi) >= k throughout.
+            long long lo32 = (long long)(S.mn >> 32) - 1, hi32 = (long long)(S.mx >> 32);
+            int round = 0;
+            auto count = [&](auto below) {
+                uint32_t c = 0;
+#pragma unroll
+                for (int j = 0; j < FM_KPT + FM_OLD; ++j) c += below(mine[j]) ? 1u : 0u;  // never true of an empty slot
+                c = __reduce_add_sync(0xffffffffu, c);
+                const int slot = round % 3;
+                if (lane == 0 && c) atomicAdd(&S.round[slot], c);
+                if (tid == 0) S.round[(slot + 1) % 3] = 0u;  // next round's word; its last readers passed two barriers ago
+                __syncthreads();
+                ++round;
+                return S.round[slot];
+            };
+            // more entries follow and all survivors fit the buffer: no cut yet, the next rounds go by the old bound
+            const bool more = r0 + FM_ENTRIES < nitems || g0 + FM_LISTS < l1;
+            unsigned long long hi = KEY_MAX - 1;
+            if (c_hi > (more ? (uint32_t)TOPK_CAP : want_max)) {  // uniform
+                while (hi32 - lo32 > 1 && c_hi > want_max) {
+                    const uint32_t mid = bisect_mid(lo32, hi32, round);
+                    const uint32_t c = count([&](unsigned long long x) { return (uint32_t)(x >> 32) <= mid; });
+                    if (c < (uint32_t)k) lo32 = mid; else { hi32 = mid; c_hi = c; }
+                }
+                hi = ((unsigned long long)hi32 << 32) | 0xFFFFFFFFull;
+                unsigned long long lo = (unsigned long long)hi32 << 32;
+                while (hi - lo > 1 && c_hi > want_max) {  // only when the scores left are all equal
+                    const unsigned long long mid = lo + (hi - lo) / 2;
+                    const uint32_t c = count([&](unsigned long long x) { return x <= mid; });
+                    if (c < (uint32_t)k) lo = mid; else { hi = mid; c_hi = c; }
+                }
+                bound = hi;  // at least k keys lie at or below it
+            }
+#pragma unroll
+            for (int j = 0; j < FM_KPT + FM_OLD; ++j) warp_push(S.keys, &S.cnt, mine[j] <= hi && mine[j] != KEY_MAX, mine[j]);
+            __syncthreads();
+        }
     }
-    const int kept = block_select(keys, &cnt, k, tid, FSEL_THREADS, sync);
-    for (int i = tid; i < k; i += FSEL_THREADS) {
+}
+
+__global__ void __launch_bounds__(FM_THREADS, 2) flat_merge_kernel(int nlists, int parts, int k, int stride, int raw, uint32_t raw_sign,
+                                                                int32_t* __restrict__ slot_cnt,
+                                                                unsigned long long* __restrict__ slot_keys,
+                                                                uint32_t* __restrict__ tickets,
+                                                                int64_t* __restrict__ out_ids,
+                                                                float* __restrict__ out_scores) {
+    __shared__ FlatMergeState S;
+    const int tid = threadIdx.x, q = blockIdx.x / parts, part = blockIdx.x % parts;
+    auto sync = [] { __syncthreads(); };
+    if (tid == 0) S.cnt = 0;
+    __syncthreads();
+    int32_t* cnts = slot_cnt + (size_t)q * nlists;
+    unsigned long long* entries = slot_keys + (size_t)q * nlists * stride;
+    int l0 = (int)((long long)part * nlists / parts), l1 = (int)((long long)(part + 1) * nlists / parts);
+    const int first = l0;
+    for (int pass = 0;; ++pass) {
+        // second pass: the first lists of all parts
+        auto slot_of = [&](int l) { return pass ? (int)((long long)l * nlists / parts) : l; };
+        flat_merge_lists(S, cnts, entries, l0, l1, slot_of, stride, pass ? 0 : raw, raw_sign, k);
+        if (pass || parts == 1) break;  // uniform
+        const int n = S.cnt;  // at most k + k/4 + 8 <= stride: the launcher checked
+        for (int i = tid; i < n; i += FM_THREADS) entries[(size_t)first * stride + i] = S.keys[i];
+        if (tid == 0) cnts[first] = n;
+        __syncthreads();  // the part's keys and count are written ...
+        if (tid == 0) {
+            __threadfence();  // ... and ordered before the ticket
+            S.last = atomicAdd(tickets + q, 1u) == (uint32_t)(parts - 1) ? 1 : 0;
+            __threadfence();
+            S.cnt = 0;
+        }
+        __syncthreads();
+        if (!S.last) return;  // uniform
+        l0 = 0;
+        l1 = parts;
+    }
+    const int kept = block_select_short(S.keys, &S.cnt, k, tid, FM_THREADS, sync);
+    for (int i = tid; i < k; i += FM_THREADS) {
         int64_t id = -1;
         float sc = __int_as_float(0xff800000);
         if (i < kept) {
-            id = (int64_t)(uint32_t)(keys[i] & 0xFFFFFFFFull);
-            sc = -orderable_f32((uint32_t)(keys[i] >> 32));
+            id = (int64_t)(uint32_t)(S.keys[i] & 0xFFFFFFFFull);
+            sc = -orderable_f32((uint32_t)(S.keys[i] >> 32));
         }
         out_ids[(size_t)q * k + i] = id;
         out_scores[(size_t)q * k + i] = sc;
@@ -167,10 +368,12 @@ static int sm_count() {
 
 static bool flat_on_tensor_cores(int d, int k) { return gemm_cand_cap(k) != 0 && d % 8 == 0; }
 
-// Pilot pass of the flat search: worth it for large databases; the sample must hold 4 k rows.
+// Pilot pass of the flat search: worth it for large databases; the sample must hold 4 k rows.  Whole column tiles: the
+// score matrix then has 16-byte aligned rows and takes 16-byte stores (with 32 679 columns, stored one float at a
+// time, the pilot of 256 queries took 88 us).
 static int flat_pilot_cols(int64_t N, int k) {
     if (N < (1 << 18)) return 0;
-    const int64_t np = N / gemm_pilot_stride(N);
+    const int64_t np = N / gemm_pilot_stride(N) / 256 * 256;
     return np >= 4LL * k ? (int)np : 0;
 }
 
@@ -249,8 +452,21 @@ cudaError_t launch_flat_search(const void* db, int64_t N, int d, const void* que
         }
         e = launch_gemm_select(G, s);
         if (e != cudaSuccess) return e;
-        flat_merge_kernel<<<nq, FSEL_THREADS, 0, s>>>(nlists, k, cap, 1, gemm_cand_sign(G.alpha, G.colterm), cand_cnt, cand,
-                                                      out_ids, out_scores);
+        // Parts per query: a starting threshold leaves a few thousand entries per query, one round of one CTA; without
+        // one, parts of half a round each while the batch alone does not fill the GPU.
+        int parts = 1;
+        if (!np && nq <= FM_TICKETS && k + (k >> 2) + 8 <= cap && WARP_SORT_MAX <= cap) {
+            const int64_t tiles = (N + 255) / 256, cols = (tiles + nsplit - 1) / nsplit * (256 / GEMM_COL_HALVES);
+            const int64_t most = (int64_t)nlists * (cols < cap ? cols : cap);
+            parts = (int)((most + FM_ENTRIES / 2 - 1) / (FM_ENTRIES / 2));
+            const int room = sm_count() / nq;
+            if (parts > room) parts = room;
+            if (parts > FM_MAX_PARTS) parts = FM_MAX_PARTS;
+            if (parts > nlists) parts = nlists;
+            if (parts < 1) parts = 1;
+        }
+        flat_merge_kernel<<<nq * parts, FM_THREADS, 0, s>>>(nlists, parts, k, cap, 1, gemm_cand_sign(G.alpha, G.colterm), cand_cnt,
+                                                            cand, G.err + FM_TICKET_WORD, out_ids, out_scores);
         count_launch();
         return cudaGetLastError();
     }
@@ -273,7 +489,7 @@ cudaError_t launch_flat_search(const void* db, int64_t N, int d, const void* que
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    flat_merge_kernel<<<nq, FSEL_THREADS, 0, s>>>(nchunks, k, k, 0, 0u, slot_cnt, slot_keys, out_ids, out_scores);
+    flat_merge_kernel<<<nq, FM_THREADS, 0, s>>>(nchunks, 1, k, k, 0, 0u, slot_cnt, slot_keys, nullptr, out_ids, out_scores);
     count_launch();
     return cudaGetLastError();
 }

@@ -708,43 +708,35 @@ cudaError_t launch_gemm_select(const GemmLaunch& L, cudaStream_t s) {
 }
 
 // ---- pilot thresholds: per row, a value with at least nsel of the row's n sample scores at or below it --------
-// One CTA per row: the row is read once (as ordered score bits), then bisected between its minimum and maximum
-// with CTA-wide counts; the search stops as soon as the count lies in [nsel, nsel + nsel/4] and returns the next
+// One CTA per row: the row is read once (as ordered score bits, REG per thread in registers), then bisected between
+// its minimum and maximum; the search stops as soon as the count lies in [nsel, nsel + nsel/4] and returns the next
 // representable value above the cut, so that "score < tau" keeps ties of the cut itself.
-// A row that fits the registers and gives every warp enough values is not bisected CTA-wide: each of the W warps
+// A short row (WARP_CUT) that gives every warp enough values is not bisected CTA-wide: each of the W warps
 // bisects its own share for a value with at least ceil(nsel / W) of its values at or below it (warp-wide counts,
 // no barrier), and the row's threshold is the largest of the W values: at least nsel sample scores lie at or below
-// it, which is all a threshold has to guarantee; it is a little looser than the sample's exact nsel-th smallest.
-constexpr int RT_THREADS = 256;
-constexpr int RT_REG = 16;  // values a thread keeps in registers (rows of up to RT_REG * RT_THREADS scores)
-template <bool IN_REGS>
+// it, which is all a threshold has to guarantee; it is a little looser than the sample's exact nsel-th smallest, and
+// over 32 warps it would be more than twice as loose.
+// Rows of up to 32 768 scores (gemm_pilot_stride) fit 1024 threads' registers; held in shared memory by 256 threads
+// instead, the 37 rows of a flat search over a million rows took 30 us.
+template <int RT_THREADS, int RT_REG, bool WARP_CUT>
 __global__ void __launch_bounds__(RT_THREADS) row_tau_kernel(const float* __restrict__ scores, int n, int nsel,
                                                              float* __restrict__ row_tau) {
-    extern __shared__ uint32_t rt_vals[];  // [n] when the row does not fit the registers
-    __shared__ uint32_t red[2][RT_THREADS / 32];
+    constexpr int W = RT_THREADS / 32;
+    __shared__ uint32_t red[2][W];
+    __shared__ uint32_t s_round[3];
     const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const float* r = scores + (size_t)row * n;
     uint32_t mine[RT_REG];
     uint32_t mn = 0xFFFFFFFFu, mx = 0u;
-    if (IN_REGS) {
 #pragma unroll
-        for (int j = 0; j < RT_REG; ++j) {
-            const int i = tid + j * RT_THREADS;
-            mine[j] = i < n ? f32_orderable(__ldg(r + i)) : 0xFFFFFFFFu;
-            if (i < n) { mn = mine[j] < mn ? mine[j] : mn; mx = mine[j] > mx ? mine[j] : mx; }
-        }
-    } else {
-        for (int i = tid; i < n; i += RT_THREADS) {
-            const uint32_t o = f32_orderable(__ldg(r + i));
-            rt_vals[i] = o;
-            mn = o < mn ? o : mn;
-            mx = o > mx ? o : mx;
-        }
+    for (int j = 0; j < RT_REG; ++j) {
+        const int i = tid + j * RT_THREADS;
+        mine[j] = i < n ? f32_orderable(__ldg(r + i)) : 0xFFFFFFFFu;
+        if (i < n) { mn = mine[j] < mn ? mine[j] : mn; mx = mine[j] > mx ? mine[j] : mx; }
     }
     mn = __reduce_min_sync(0xffffffffu, mn);
     mx = __reduce_max_sync(0xffffffffu, mx);
-    if (IN_REGS) {
-        constexpr int W = RT_THREADS / 32;
+    if (WARP_CUT) {
         const int m = (nsel + W - 1) / W;
         // values are dealt out round-robin by thread: the last warp holds the fewest
         const int fewest = (n / RT_THREADS) * 32 + (n % RT_THREADS > RT_THREADS - 32 ? n % RT_THREADS - (RT_THREADS - 32) : 0);
@@ -774,33 +766,29 @@ __global__ void __launch_bounds__(RT_THREADS) row_tau_kernel(const float* __rest
         }
     }
     if (lane == 0) { red[0][warp] = mn; red[1][warp] = mx; }
+    if (tid == 0) s_round[0] = s_round[1] = s_round[2] = 0u;
     __syncthreads();
-    mn = red[0][0]; mx = red[1][0];
-    for (int w = 1; w < RT_THREADS / 32; ++w) {
+    for (int w = 0; w < W; ++w) {
         mn = red[0][w] < mn ? red[0][w] : mn;
         mx = red[1][w] > mx ? red[1][w] : mx;
     }
-    __syncthreads();
     long long lo = (long long)mn - 1, hi = mx;  // #(<= lo) < nsel <= #(<= hi)
     uint32_t c_hi = (uint32_t)n;
     const uint32_t want_max = (uint32_t)(nsel + nsel / 4);
-    int round = 0;
+    int slot = 0, round = 0;
     while (hi - lo > 1 && c_hi > want_max) {  // uniform: every thread holds the same lo, hi, c_hi
-        const uint32_t mid = (uint32_t)(lo + (hi - lo) / 2);
+        const uint32_t mid = bisect_mid(lo, hi, round++);
+        const int next = slot == 2 ? 0 : slot + 1;
         uint32_t c = 0;
-        if (IN_REGS) {
 #pragma unroll
-            for (int j = 0; j < RT_REG; ++j) c += mine[j] <= mid ? 1u : 0u;  // padding holds the largest pattern
-        } else {
-            for (int i = tid; i < n; i += RT_THREADS) c += rt_vals[i] <= mid ? 1u : 0u;
-        }
+        for (int j = 0; j < RT_REG; ++j) c += mine[j] <= mid ? 1u : 0u;  // padding holds the largest pattern
         c = __reduce_add_sync(0xffffffffu, c);
-        if (lane == 0) red[round & 1][warp] = c;  // the other buffer may still be read by slower warps
+        if (lane == 0 && c) atomicAdd(&s_round[slot], c);
+        if (tid == 0) s_round[next] = 0u;  // its last readers passed two barriers ago
         __syncthreads();
-        c = 0;
-        for (int w = 0; w < RT_THREADS / 32; ++w) c += red[round & 1][w];
+        c = s_round[slot];
         if (c < (uint32_t)nsel) lo = mid; else { hi = mid; c_hi = c; }
-        ++round;
+        slot = next;
     }
     if (tid == 0) {
         const uint32_t T = (uint32_t)hi;
@@ -808,12 +796,10 @@ __global__ void __launch_bounds__(RT_THREADS) row_tau_kernel(const float* __rest
     }
 }
 cudaError_t launch_row_tau(const float* scores, int nrows, int n, int nsel, float* row_tau, cudaStream_t s) {
-    if (n <= RT_REG * RT_THREADS) {
-        row_tau_kernel<true><<<nrows, RT_THREADS, 0, s>>>(scores, n, nsel, row_tau);
-    } else {
-        if ((size_t)n * 4 > 200 * 1024) return cudaErrorInvalidValue;
-        row_tau_kernel<false><<<nrows, RT_THREADS, (size_t)n * 4, s>>>(scores, n, nsel, row_tau);
-    }
+    if (n <= 16 * 256) row_tau_kernel<256, 16, true><<<nrows, 256, 0, s>>>(scores, n, nsel, row_tau);
+    else if (n <= 16 * 1024) row_tau_kernel<1024, 16, false><<<nrows, 1024, 0, s>>>(scores, n, nsel, row_tau);
+    else if (n <= 32 * 1024) row_tau_kernel<1024, 32, false><<<nrows, 1024, 0, s>>>(scores, n, nsel, row_tau);
+    else return cudaErrorInvalidValue;
     count_launch();
     return cudaGetLastError();
 }
@@ -830,8 +816,6 @@ cudaError_t gemm_select_init() {
     if (e == cudaSuccess) e = gemm_attr<GEMM_CAP_LARGE / 32, LOOP_SINGLE>();
     if (e == cudaSuccess) e = gemm_attr<GEMM_CAP_LARGE / 32, LOOP_PAIR>();
     if (e == cudaSuccess) e = gemm_attr<GEMM_CAP_LARGE / 32, LOOP_TWO_CTA>();
-    if (e == cudaSuccess)  // rows of up to 51 200 pilot scores in shared memory
-        e = cudaFuncSetAttribute(row_tau_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     return e;
 }
 

@@ -10,6 +10,19 @@
 
 namespace rago {
 
+// Next value to try in a bisection over ordered score bits, strictly between lo and hi (hi - lo > 1; lo may be one below
+// the smallest pattern).  The first rounds halve the range of the VALUES: scores that lie on both sides of zero put
+// half of all bit patterns between them next to zero, and halving the patterns spends seven rounds on leaving those.
+// An outlier would cost the values a round per binary order of magnitude, so later rounds halve the patterns.
+constexpr int BISECT_VALUE_ROUNDS = 10;
+__device__ __forceinline__ uint32_t bisect_mid(long long lo, long long hi, int round) {
+    if (round < BISECT_VALUE_ROUNDS) {
+        const uint32_t m = f32_orderable(0.5f * orderable_f32(lo < 0 ? 0u : (uint32_t)lo) + 0.5f * orderable_f32((uint32_t)hi));
+        if ((long long)m > lo && (long long)m < hi) return m;  // not so for neighbours, infinities and NaN
+    }
+    return (uint32_t)(lo + (hi - lo) / 2);
+}
+
 // Ascending bitonic sort of n keys (n a power of two) by `nthreads` threads; sync() is the barrier
 // those threads share.  Ends with a barrier.
 template <class Sync>

@@ -452,3 +452,28 @@ def test_thousands_of_identical_vectors_still_give_k_distinct_results(k):
     for i in range(3):
         assert not match_results(ids[i], dists[i], oi[i], od[i], rel=REL, rescore=rs.for_query(data.queries[i].numpy())), i
     ix.close()
+
+
+@pytest.mark.parametrize("N,nq,k", [(100_003, 1, 300),      # the final selection split into parts, ragged last tile
+                                    (262_143, 33, 7),       # one row short of the pilot pass, more queries than tickets
+                                    (262_144, 5, 128),      # the first size with pilot thresholds
+                                    (2_500_000, 2, 400),    # entries streamed past the first round's bound
+                                    (60_000, 2, 1)])
+def test_flat_final_selection_matches_fp64(N, nq, k):
+    db, q = synth.make_flat(N, 64, nq, seed=N, device="cuda")
+    ids, scores = binding.rago_flat_search(db, q, k)
+    exact = q.double() @ db.double().T
+    want, _ = exact.topk(k, 1)
+    assert torch.allclose(scores.double(), want, rtol=0, atol=64 * 2.0 ** -24)  # 64 products of unit-norm rows in fp32
+    assert torch.allclose(exact.gather(1, ids), want, rtol=0, atol=64 * 2.0 ** -24)
+    assert all(len(set(row)) == k for row in ids.tolist())
+
+
+def test_flat_final_selection_orders_equal_scores_by_row():
+    """All scores equal: the cut has to be found on the row numbers."""
+    db = torch.zeros((70_000, 64), dtype=torch.bfloat16, device="cuda")
+    db[:, 0] = 1.0
+    q = db[:3].clone()
+    for k in (1, 100, 300):
+        ids, scores = binding.rago_flat_search(db, q, k)
+        assert torch.equal(ids.cpu(), torch.arange(k).expand(3, k)) and bool((scores == 1.0).all())
