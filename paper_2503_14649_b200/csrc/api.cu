@@ -433,12 +433,13 @@ rago_status rago_search(const rago_index* index, const float* queries, int32_t n
     // Batches of at most 64 queries: the selection launch also builds the tables and plans the scan (its last CTA
     // to finish), one launch less on the latency-bound path.  The ticket word lies in the block cleared above.
     FusedPlan fp;
+    const int lead = scan_query_lead(ix, nq, nprobe, k);
     const bool fused = fused_plan_args(ix, nq, npairs, queries, lut_img, lut_inv, work_prefix, qthresh, slot_cnt,
-                                       (int)L.nslots, reinterpret_cast<uint32_t*>(ws + L.err) + ERR_TICKET_WORD, &fp);
+                                       (int)L.nslots, lead, reinterpret_cast<uint32_t*>(ws + L.err) + ERR_TICKET_WORD, &fp);
     st = run_coarse(ix, queries, nq, nprobe, ws, L, fused ? &fp : nullptr, kernel_clears, s);
     if (st != RAGO_OK) return st;
     if (!fused) {
-        e = launch_plan_work(ix, probe_list, npairs, ix->plan.tile_vecs, reinterpret_cast<int32_t*>(ws + L.pair_tiles),
+        e = launch_plan_work(ix, probe_list, npairs, ix->plan.tile_vecs, lead, reinterpret_cast<int32_t*>(ws + L.pair_tiles),
                              work_prefix, qthresh, nq, slot_cnt, (int)L.nslots, queries, lut_img, lut_inv,
                              L.prebuilt ? reinterpret_cast<float*>(ws + L.lut_scale) : nullptr, s);
         if (e != cudaSuccess) return cuda_fail(e, "work planning");

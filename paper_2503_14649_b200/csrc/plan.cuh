@@ -24,7 +24,7 @@ struct FusedPlan {
     int nq;                      // queries of the batch = selection CTAs of the launch
     uint32_t* ticket;            // zero before the launch; the planning CTA leaves it zero again
     const int64_t* offsets;      // [nlist + 1]
-    int tile_vecs;
+    int tile_vecs, lead;
     int64_t* prefix;             // [npairs + 1]
     unsigned long long* qthresh; // [nq]
     int32_t* slot_cnt;
@@ -43,10 +43,14 @@ cudaError_t launch_select_probes_cand(const IndexImpl* ix, const float* queries,
                                       cudaStream_t s);
 // scan.cu
 bool fused_plan_args(const IndexImpl* ix, int nq, int npairs, const float* queries, uint8_t* lut_img, float* lut_inv,
-                     int64_t* work_prefix, unsigned long long* qthresh, int32_t* slot_cnt, int nslots, uint32_t* ticket,
+                     int64_t* work_prefix, unsigned long long* qthresh, int32_t* slot_cnt, int nslots, int lead, uint32_t* ticket,
                      FusedPlan* fp);
 
 #ifdef __CUDACC__
+// Units in front of pair p's first tile on the line of work units (see scan_query_lead): those of a query's start, except
+// for the first query, whose start costs no CTA more than any other's first one.
+__device__ __forceinline__ int pair_lead(int p, int nprobe, int lead) { return lead != 0 && p > 0 && p % nprobe == 0 ? lead : 0; }
+
 // Part `part` of `parts` of query q's table, by all threads of the CTA.  sm: d + M floats of shared memory.
 __device__ __forceinline__ void build_table_part(const TableArgs& t, int q, int part, int parts, float* sm) {
     const int d = t.d, dsub = t.dsub, M = t.M, tid = threadIdx.x, nthreads = blockDim.x;
@@ -97,7 +101,7 @@ __device__ __forceinline__ void build_table_part(const TableArgs& t, int q, int 
 // of shared memory.  The probe lists may have been written by other CTAs of the same launch (the caller has ordered
 // those writes before this call): they are read past the L1 cache.
 __device__ __forceinline__ void plan_pairs_cta(const int32_t* probe_list, const int64_t* __restrict__ offsets, int npairs,
-                                               int tile_vecs, int64_t* __restrict__ prefix,
+                                               int nprobe, int tile_vecs, int lead, int64_t* __restrict__ prefix,
                                                unsigned long long* __restrict__ qthresh, int nq,
                                                int32_t* __restrict__ slot_cnt, int nslots, long long* warp_sums) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -110,7 +114,7 @@ __device__ __forceinline__ void plan_pairs_cta(const int32_t* probe_list, const 
         mine[j] = 0;
         if (p < npairs) {
             const int l = __ldcg(probe_list + p);
-            mine[j] = (offsets[l + 1] - offsets[l] + tile_vecs - 1) / tile_vecs;
+            mine[j] = (offsets[l + 1] - offsets[l] + tile_vecs - 1) / tile_vecs + pair_lead(p, nprobe, lead);
         }
         v += mine[j];
     }

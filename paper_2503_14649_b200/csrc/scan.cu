@@ -65,11 +65,11 @@ constexpr uint32_t SMEM_BASE_EXPECTED = 1024;   // shared-window address of dyna
 constexpr int CTRL_BYTES = 1024;
 
 struct TileDesc {
-    int32_t pair;      // index into probe_list (query * nprobe + rank)
+    int32_t pair;      // index into probe_list (query * nprobe + rank), -1: the CTA has no tile
     float term;        // the pair's (query, list) term of the score
     uint32_t pos0;     // storage position of the tile's first vector
     int32_t nvec;      // vectors in this tile
-    int32_t newpair;   // bit 0: first tile of this pair inside this CTA; bit 1: cut the candidate buffer before this tile
+    int32_t newpair;   // bit 0: first tile of this pair inside this CTA; bit 1: cut the candidate buffer before this tile; bit 2: last tile of the CTA
     int32_t vrem;      // index of the first vector's term inside the staged term block (0..3)
     uint32_t tile_addr;  // shared address of the stage's code tile
     uint32_t vt_addr;    // shared address of the stage's per-vector terms
@@ -91,8 +91,10 @@ struct ScanArgs {
     const uint8_t* lut_img;  // [nq][LUT_BYTES] tables built ahead of the scan (small batches), or null
     const float* lut_inv;    // [nq] fp32 value of one integer unit of each such table
     int32_t npairs, nprobe, d, dsub, metric, k, stages;
+    int32_t lead;            // work units in front of a query's first tile (scan_query_lead)
     int32_t stream_once;     // the batch is small: code tiles are fetched with an evict-first hint, so that the centroid
                              // table the next search's coarse step reads stays in L2
+    int32_t prefetch;        // pull tiles into L2 ahead of their copies
     uint32_t dyn_bytes;
 };
 
@@ -384,7 +386,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
     // round trip (the offsets in a second one), and the consumers know their first query without the producer.
     const bool few_pairs = a.npairs <= 32;
     const long long pw = few_pairs ? a.work_prefix[lane < a.npairs ? lane : a.npairs] : 0;  // >= npairs: the total
-    int c_list = 0; long long c_off = 0, c_len = 0, c_ws = 0, c_we = 0; float c_term = 0.f;  // producer: lane i's cached pair
+    int c_list = 0; long long c_off = 0, c_len = 0, c_ws = 0, c_we = 0; float c_term = 0.f; int c_tv = C::TV;  // producer: lane i's cached pair
     if (few_pairs && warp == NCW && lane < a.npairs) {
         c_list = a.probe_list[lane];
         c_term = a.probe_term[lane];
@@ -392,12 +394,11 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
         c_off = a.list_offsets[c_list];
         c_len = a.list_offsets[c_list + 1] - c_off;
     }
-    // This CTA's share of the work units (tiles).
+    // This CTA's share of the work units: the tiles whose place on the line of units lies in [u_begin, u_end).
     const long long W = a.work_prefix[a.npairs];
     const long long u_begin = (long long)blockIdx.x * W / gridDim.x;
     const long long u_end = (long long)(blockIdx.x + 1) * W / gridDim.x;
-    const int T = (int)(u_end - u_begin);
-    if (T <= 0) return;
+    if (u_end <= u_begin) return;
     // few pairs: the pair whose range contains u_begin = the largest p with work_prefix[p] <= u_begin
     const int first_pair = few_pairs ? __popc(__ballot_sync(0xffffffffu, pw <= u_begin)) - 1 : -1;
 
@@ -416,21 +417,34 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
         }
         int cache_base = few_pairs ? 0 : lo;  // lane i caches pair cache_base + i
         if (few_pairs) {
-            c_ws = pw;
+            c_ws = pw + pair_lead(lane, a.nprobe, a.lead);
             if (lane >= a.npairs) { c_ws = c_we = W; }
         }
+        // A list of several tiles is cut into tiles of one size (whole groups of 32 vectors) instead of full tiles and a
+        // remainder: with two or three tiles in flight, a short tile leaves too little time for the copy behind it.
+        // (Not for a few pairs, where a CTA has a tile or two and the division would stand before its first copy.)
+        auto tile_size = [&]() {
+            const uint32_t nt = (uint32_t)(c_we - c_ws), n = (uint32_t)c_len;  // positions are 32-bit
+            c_tv = C::TV;
+            if (nt > 1u) {
+                const uint32_t share = n / nt;
+                c_tv = (int)((share + (share * nt != n ? 32u : 31u)) & ~31u);
+            }
+        };
+        static_assert(C::TV % 32 == 0, "a rounded-up tile must not exceed the tile it was cut from");
         auto fill = [&]() {
             const int p = cache_base + lane;
             if (p < a.npairs) {
                 c_list = a.probe_list[p];
                 c_off = a.list_offsets[c_list];
                 c_len = a.list_offsets[c_list + 1] - c_off;
-                c_ws = a.work_prefix[p];
+                c_ws = a.work_prefix[p] + pair_lead(p, a.nprobe, a.lead);  // place of its first tile
                 c_we = a.work_prefix[p + 1];
                 c_term = a.probe_term[p];
             } else {
                 c_list = 0; c_off = 0; c_len = 0; c_ws = c_we = W; c_term = 0.f;
             }
+            tile_size();
         };
         if (!few_pairs) fill();
         int cur = few_pairs ? first_pair : 0;
@@ -440,45 +454,58 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
         int issued = 0;
         int pst = 0;          // n % S, kept by counting (S is a run-time value: no division per tile)
         uint32_t pround = 0;  // n / S
-        for (int n = 0; n < T && !dead; ++n, ++u) {
+        // Moves to the first tile at or after unit u (skips empty pairs and leads); false: there is none in the share.
+        auto advance = [&]() -> bool {
+            for (;;) {
+                const long long first = __shfl_sync(0xffffffffu, c_ws, cur), we = __shfl_sync(0xffffffffu, c_we, cur);
+                if (u < first) u = first;
+                if (u >= u_end) return false;
+                if (u < we) return true;
+                if (++cur == 32) { cache_base += 32; fill(); cur = 0; }
+            }
+        };
+        bool more = advance();
+        if (!more && lane == 0) {  // a share without a tile: a descriptor with no copy says so
+            ctrl->desc[0].pair = -1;
+            mbar_arrive(smem_u32(&ctrl->full[0]));
+        }
+        for (int n = 0; more; ++n) {
             const int st = pst;
             const uint32_t round = pround;
             if (++pst == S) { pst = 0; ++pround; }
-            // advance to the pair that owns unit u (skips empty pairs); all of this before the wait for the
-            // stage, so that as little as possible stands between a stage coming free and its refill
-            for (;;) {
-                const long long we = __shfl_sync(0xffffffffu, c_we, cur);
-                if (u < we) break;
-                if (++cur == 32) { cache_base += 32; fill(); cur = 0; }
-            }
             const long long ws = __shfl_sync(0xffffffffu, c_ws, cur);
             const long long off = __shfl_sync(0xffffffffu, c_off, cur);
             const long long len = __shfl_sync(0xffffffffu, c_len, cur);
             const float term = __shfl_sync(0xffffffffu, c_term, cur);
+            const int tv = __shfl_sync(0xffffffffu, c_tv, cur);
+            const int pair = cache_base + cur;
+            const long long t_in_pair = u - ws;
+            const long long v0 = t_in_pair * tv;
+            const int nvec = (int)(len - v0 < tv ? len - v0 : tv);
+            const uint32_t pos0 = (uint32_t)(off + v0);
+            const uint32_t bytes = (uint32_t)nvec * C::M;
+            // per-vector terms: start rounded down to a 16-byte boundary, length rounded up
+            const uint32_t vbytes = a.vterm ? (((pos0 & 3u) + (uint32_t)nvec) * 4u + 15u) & ~15u : 0u;
+            const uint32_t bar = smem_u32(&ctrl->full[st]);
+            const long long u_this = u++;
+            more = advance();
+            // All of the above stands before the wait for the stage, so that as little as possible lies between its coming
+            // free and its refill (looking for the next tile after the wait: 48-byte codes, 300 queries 1 588 us, before it 1 500).
             if (round > 0) dead = !mbar_wait(smem_u32(&ctrl->empty[st]), (round - 1) & 1, abort_flag, a.err);
             if (dead) break;
             if (lane == 0) {
-                const long long t_in_pair = u - ws;
-                const long long v0 = t_in_pair * C::TV;
-                long long nvec = len - v0;
-                if (nvec > C::TV) nvec = C::TV;
-                const uint32_t pos0 = (uint32_t)(off + v0);
                 TileDesc& D = ctrl->desc[st];
-                D.pair = cache_base + cur;
+                D.pair = pair;
                 D.term = term;
                 D.pos0 = pos0;
-                D.nvec = (int32_t)nvec;
+                D.nvec = nvec;
                 // everything tiles n-S+1 .. n can still push must fit behind what is in the buffer now
                 const int cnt_seen = *reinterpret_cast<volatile int*>(&ctrl->cnt);
                 const int cut = cnt_seen + (S + 1) * C::TV > C::KCAP ? 2 : 0;
-                D.newpair = ((n == 0 || t_in_pair == 0) ? 1 : 0) | cut;
+                D.newpair = ((n == 0 || t_in_pair == 0) ? 1 : 0) | cut | (more ? 0 : 4);
                 D.vrem = (int32_t)(pos0 & 3u);
                 D.tile_addr = P.tile[st];
                 D.vt_addr = P.vt[st];
-                const uint32_t bytes = (uint32_t)nvec * C::M;
-                // per-vector terms: start rounded down to a 16-byte boundary, length rounded up
-                const uint32_t vbytes = a.vterm ? (((pos0 & 3u) + (uint32_t)nvec) * 4u + 15u) & ~15u : 0u;
-                const uint32_t bar = smem_u32(&ctrl->full[st]);
                 mbar_arrive_expect_tx(bar, bytes + vbytes);
                 if (a.stream_once) {  // small batch: the codes are read once and should leave L2 first
                     bulk_g2s_hint(P.tile[st], a.codes + (size_t)pos0 * C::M, bytes, bar, once_policy);
@@ -487,13 +514,17 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
                     bulk_g2s(P.tile[st], a.codes + (size_t)pos0 * C::M, bytes, bar);
                     if (vbytes) bulk_g2s(P.vt[st], a.vterm + (pos0 & ~3u), vbytes, bar);
                 }
-                // pull the tiles a few steps ahead in this list into L2, so that their copies find them there
-                for (int ahead = (t_in_pair == 0 ? 1 : SCAN_PF); ahead <= SCAN_PF; ++ahead) {
-                    const long long vp = v0 + (long long)ahead * C::TV;
-                    if (vp >= len) break;
-                    long long np = len - vp;
-                    if (np > C::TV) np = C::TV;
-                    l2_prefetch(a.codes + (size_t)(off + vp) * C::M, (uint32_t)np * C::M);
+                // pull the tiles a few steps ahead in this list into L2, with their terms, so that their copies find them there
+                if (a.prefetch) {
+                    for (int ahead = (t_in_pair == 0 ? 1 : SCAN_PF); ahead <= SCAN_PF && u_this + ahead < u_end; ++ahead) {
+                        const long long vp = v0 + (long long)ahead * tv;
+                        if (vp >= len) break;
+                        long long np = len - vp;
+                        if (np > tv) np = tv;
+                        const long long first = off + vp;
+                        l2_prefetch(a.codes + (size_t)first * C::M, (uint32_t)np * C::M);
+                        if (a.vterm) l2_prefetch(a.vterm + (first & ~3ll), (uint32_t)(((first & 3) + np) * 4 + 15) & ~15u);
+                    }
                 }
             }
             issued = n + 1;
@@ -776,13 +807,15 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
     if (few_pairs) begin_query(first_pair / a.nprobe);
     int cst = 0;            // n % S and the parity of n / S, kept by counting
     uint32_t cparity = 0;
-    for (int n = 0; n < T && !dead; ++n) {
+    for (bool last = false; !last && !dead;) {
         const int st = cst;
         const uint32_t parity = cparity;
         if (++cst == S) { cst = 0; cparity ^= 1u; }
         dead = dead || !mbar_wait(smem_u32(&ctrl->full[st]), parity, abort_flag, a.err);
         if (dead) break;
         const TileDesc D = ctrl->desc[st];
+        if (D.pair < 0) break;
+        last = (D.newpair & 4) != 0;
         if (D.newpair & 1) {
             const int q = D.pair / a.nprobe;
             if (q != cur_q) {
@@ -934,6 +967,23 @@ cudaError_t scan_plan(const IndexImpl* ix, ScanPlan* plan) {
     return cudaFuncSetAttribute(v->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_OPTIN);
 }
 
+// Work units (tiles) that stand for the start of a query on the line that is cut into one share per CTA.  Every CTA opens
+// the query its share begins with; one that meets the start of another query closes the first (cut, rank), fetches
+// the second's table and fills its candidate buffer without a threshold, which takes as long as scanning several tiles: in
+// shares of equal tile counts the CTAs with the most query starts finished last (48-byte codes, 300 queries: 17 us per
+// start, last CTA at 1 595 us against a mean of 1 457; 32 bytes, 16 queries: 5.5 us, 36 against 26).  Per start: k <= 32
+// about 5.5 us; more with a 4 096-key buffer 7 us, with a 2 048-key buffer (more cuts) 17; per tile 1 us for 36 KB, no
+// less than 0.8 us.  Where a share is shorter than the start of a query the tiles are short or few, no CTA waits long
+// for another, and leads only leave CTAs without work (64 queries over 100 000 vectors 64.8 -> 67.1 us per call): none.
+int scan_query_lead(const IndexImpl* ix, int nq, int nprobe, int k) {
+    if (nq < 2 || ix->nlist < 1) return 0;
+    const float start_us = k <= 32 ? 5.5f : (ix->plan.lut_bytes <= 65536 ? 7.f : 17.f);
+    const float tile_us = (float)(ix->plan.tile_vecs * ix->M) / 36000.f;
+    const int lead = (int)(start_us / (tile_us > 0.8f ? tile_us : 0.8f) + 0.5f);
+    const int64_t tiles_per_list = (ix->N / ix->nlist + ix->plan.tile_vecs) / ix->plan.tile_vecs;  // of a list of average length
+    return (int64_t)nq * nprobe * tiles_per_list >= (int64_t)lead * ix->plan.ctas ? lead : 0;
+}
+
 cudaError_t launch_scan(const IndexImpl* ix, const ScanPlan& plan, const float* queries, const int32_t* probe_list,
                         const float* probe_term, const int64_t* work_prefix, int nq, int nprobe, int k,
                         unsigned long long* qthresh, int32_t* slot_cnt, unsigned long long* slot_keys,
@@ -947,8 +997,15 @@ cudaError_t launch_scan(const IndexImpl* ix, const ScanPlan& plan, const float* 
     a.qthresh = qthresh; a.slot_cnt = slot_cnt; a.slot_keys = slot_keys; a.err = err_word;
     a.lut_img = lut_img; a.lut_inv = lut_inv;
     a.npairs = nq * nprobe; a.nprobe = nprobe; a.d = ix->d; a.dsub = ix->dsub;
+    a.lead = scan_query_lead(ix, nq, nprobe, k);
     a.metric = ix->metric; a.k = k; a.stages = plan.stages; a.dyn_bytes = (uint32_t)plan.smem_bytes;
     a.stream_once = nq <= 64 ? 1 : 0;
+    // Prefetching into L2 pays where the tiles in flight are small (a copy from DRAM takes longer than the tile in front
+    // of it is scanned) and the batch does not meet each list several times, which brings most tiles from L2 anyway and
+    // makes the prefetches only extra traffic.  Without / with, us per call: 48-byte codes, 2.3 probes per list
+    // 1672 / 1618; 96 bytes, 0.6 probes 753 / 741; 96 bytes, 8 probes 8890 / 9100 (with terms 9190); 64 bytes (60 KB
+    // tiles), 4 096 queries 14 560 / 14 730, 33 queries 226.9 / 233.8.
+    a.prefetch = plan.tile_vecs * ix->M <= 40 * 1024 && (long long)a.npairs <= 4ll * ix->nlist ? 1 : 0;
     const cudaError_t e = launch_overlapped(v->kernel, dim3(plan.ctas), dim3(v->threads), plan.smem_bytes, s, a);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
@@ -1191,15 +1248,15 @@ cudaError_t launch_vector_terms(const IndexImpl* ix, float* vterm, cudaStream_t 
 // (2) one CTA scans the totals, (3) every CTA adds its offset.
 constexpr int PT_THREADS = 256;
 __global__ void __launch_bounds__(PT_THREADS) pair_tiles_kernel(const int32_t* __restrict__ probe_list,
-                                                                const int64_t* __restrict__ offsets, int npairs,
-                                                                int tile_vecs, int64_t* __restrict__ prefix,
+                                                                const int64_t* __restrict__ offsets, int npairs, int nprobe,
+                                                                int tile_vecs, int lead, int64_t* __restrict__ prefix,
                                                                 long long* __restrict__ block_sums) {
     __shared__ long long warp_sums[PT_THREADS / 32];
     const int p = blockIdx.x * PT_THREADS + threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     long long v = 0;
     if (p < npairs) {
         const int l = probe_list[p];
-        v = (offsets[l + 1] - offsets[l] + tile_vecs - 1) / tile_vecs;
+        v = (offsets[l + 1] - offsets[l] + tile_vecs - 1) / tile_vecs + pair_lead(p, nprobe, lead);
     }
     long long incl = v;
     for (int o = 1; o < 32; o <<= 1) {
@@ -1261,8 +1318,8 @@ __global__ void __launch_bounds__(PT_THREADS) add_offsets_kernel(int64_t* __rest
 // With table_parts > 0 the CTAs after the first build the batch's lookup tables meanwhile (the tables depend on the
 // queries only, so nothing orders them against the planning).
 __global__ void __launch_bounds__(PFX_THREADS) plan_small_kernel(const int32_t* __restrict__ probe_list,
-                                                                 const int64_t* __restrict__ offsets, int npairs,
-                                                                 int tile_vecs, int64_t* __restrict__ prefix,
+                                                                 const int64_t* __restrict__ offsets, int npairs, int nprobe,
+                                                                 int tile_vecs, int lead, int64_t* __restrict__ prefix,
                                                                  unsigned long long* __restrict__ qthresh, int nq,
                                                                  int32_t* __restrict__ slot_cnt, int nslots,
                                                                  const TableArgs tables, int table_parts) {
@@ -1275,13 +1332,13 @@ __global__ void __launch_bounds__(PFX_THREADS) plan_small_kernel(const int32_t* 
         return;
     }
     __shared__ long long warp_sums[32];
-    plan_pairs_cta(probe_list, offsets, npairs, tile_vecs, prefix, qthresh, nq, slot_cnt, nslots, warp_sums);
+    plan_pairs_cta(probe_list, offsets, npairs, nprobe, tile_vecs, lead, prefix, qthresh, nq, slot_cnt, nslots, warp_sums);
 }
 
 // Small batches whose probe selection plans the scan itself (see FusedPlan): what that kernel needs, or false when
 // the batch does not qualify (tables not prebuilt, too many pairs for one CTA, more than 64 queries).
 bool fused_plan_args(const IndexImpl* ix, int nq, int npairs, const float* queries, uint8_t* lut_img, float* lut_inv,
-                     int64_t* work_prefix, unsigned long long* qthresh, int32_t* slot_cnt, int nslots, uint32_t* ticket,
+                     int64_t* work_prefix, unsigned long long* qthresh, int32_t* slot_cnt, int nslots, int lead, uint32_t* ticket,
                      FusedPlan* fp) {
     fp->enabled = 0;
     if (!lut_img || npairs > PLAN_SMALL_MAX || nq > 64) return false;
@@ -1290,6 +1347,7 @@ bool fused_plan_args(const IndexImpl* ix, int nq, int npairs, const float* queri
     fp->ticket = ticket;
     fp->offsets = ix->list_offsets;
     fp->tile_vecs = ix->plan.tile_vecs;
+    fp->lead = lead;
     fp->prefix = work_prefix;
     fp->qthresh = qthresh;
     fp->slot_cnt = slot_cnt;
@@ -1299,7 +1357,7 @@ bool fused_plan_args(const IndexImpl* ix, int nq, int npairs, const float* queri
     return true;
 }
 
-cudaError_t launch_plan_work(const IndexImpl* ix, const int32_t* probe_list, int npairs, int tile_vecs,
+cudaError_t launch_plan_work(const IndexImpl* ix, const int32_t* probe_list, int npairs, int tile_vecs, int lead,
                              int32_t* pair_tiles, int64_t* work_prefix, unsigned long long* qthresh, int nq,
                              int32_t* slot_cnt, int nslots, const float* queries, uint8_t* lut_img, float* lut_inv,
                              float* lut_scale, cudaStream_t s) {
@@ -1312,7 +1370,7 @@ cudaError_t launch_plan_work(const IndexImpl* ix, const int32_t* probe_list, int
         const int parts = fused_tables ? table_parts(ix, nq) : 0;
         launch_overlapped(plan_small_kernel, dim3(1 + parts * nq), dim3(PFX_THREADS),
                           parts ? (size_t)(ix->d + ix->M) * 4 : 0, s,
-            probe_list, ix->list_offsets, npairs, tile_vecs, work_prefix, qthresh, nq, slot_cnt, nslots,
+            probe_list, ix->list_offsets, npairs, npairs / nq, tile_vecs, lead, work_prefix, qthresh, nq, slot_cnt, nslots,
             table_args(ix, queries, lut_img, lut_inv), parts);
         count_launch();
         return cudaGetLastError();
@@ -1320,8 +1378,8 @@ cudaError_t launch_plan_work(const IndexImpl* ix, const int32_t* probe_list, int
     // pair_tiles (npairs int32 of scratch) holds the per-CTA totals: one 64-bit word per 256 pairs
     const int nblocks = (npairs + PT_THREADS - 1) / PT_THREADS;
     long long* block_sums = reinterpret_cast<long long*>(pair_tiles);
-    pair_tiles_kernel<<<nblocks, PT_THREADS, 0, s>>>(probe_list, ix->list_offsets, npairs, tile_vecs, work_prefix,
-                                                    block_sums);
+    pair_tiles_kernel<<<nblocks, PT_THREADS, 0, s>>>(probe_list, ix->list_offsets, npairs, npairs / nq, tile_vecs, lead,
+                                                    work_prefix, block_sums);
     scan_totals_kernel<<<1, PFX_THREADS, 0, s>>>(block_sums, nblocks, work_prefix + npairs);
     add_offsets_kernel<<<nblocks, PT_THREADS, 0, s>>>(work_prefix, npairs, block_sums);
     count_launch(3);
