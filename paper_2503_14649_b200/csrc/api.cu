@@ -174,7 +174,8 @@ static rago_status run_coarse(const IndexImpl* ix, const float* queries, int nq,
     } else if (L.tc) {
         // queries -> stacked bf16 parts, then the tensor-core kernel with the selection fused in
         const int parts = ix->cparts_n;
-        e = launch_split_bf16(queries, (size_t)nq * ix->d, parts, ws + L.qparts, s);
+        e = launch_split_bf16(queries, (size_t)nq * ix->d, parts, ws + L.qparts,
+                              kernel_clears ? reinterpret_cast<uint32_t*>(ws + L.err) : nullptr, s);
         if (e != cudaSuccess) return cuda_fail(e, "query split kernel");
         alignas(64) unsigned char tmap_a[128];
         e = make_tmap_bf16(tmap_a, ws + L.qparts, (uint64_t)parts * nq, (uint64_t)ix->d, 128);
@@ -202,6 +203,7 @@ static rago_status run_coarse(const IndexImpl* ix, const float* queries, int nq,
         G.cand_cnt = reinterpret_cast<int32_t*>(ws + L.cand_cnt);
         G.scores = scores;
         G.err = reinterpret_cast<uint32_t*>(ws + L.err);
+        G.clear_block = nullptr;
         if (L.pilot_cols) {
             // pilot pass: score every pilot_stride-th list, take each query's nsel-th smallest as its starting threshold
             GemmLaunch P = G;
@@ -310,7 +312,7 @@ rago_status rago_index_load(rago_index** out, const void* coarse_centroids, rago
         if (!ix->coarse_bf16) {
             ix->cparts_n = 3;
             e = cudaMalloc(&ix->cparts, (size_t)3 * nlist * d * 2);
-            if (e == cudaSuccess) e = launch_split_bf16(static_cast<const float*>(coarse_centroids), (size_t)nlist * d, 3, ix->cparts, s);
+            if (e == cudaSuccess) e = launch_split_bf16(static_cast<const float*>(coarse_centroids), (size_t)nlist * d, 3, ix->cparts, nullptr, s);
             bsrc = ix->cparts;
         }
         if (e == cudaSuccess && gemm_select_init() == cudaSuccess &&
@@ -415,9 +417,10 @@ rago_status rago_search(const rago_index* index, const float* queries, int32_t n
     IndexImpl* mix = const_cast<IndexImpl*>(ix);
     const int npairs = nq * nprobe;
 
-    // The error block is cleared first: by the tiny-batch coarse kernel or the two-level kernel itself when that is the first kernel
-    // of the search (a memset between two searches would keep their launches from overlapping), else by a memset.
-    const bool kernel_clears = L.tree_S ? true : (!L.tc && coarse_small_applies(ix, nq));
+    // The error block is cleared first: by the first kernel of the search where that is the two-level kernel, the query
+    // split or the tiny-batch coarse kernel (a memset between two searches would keep their launches from overlapping),
+    // else by a memset.
+    const bool kernel_clears = L.tree_S || L.tc || coarse_small_applies(ix, nq);
     cudaError_t e = kernel_clears ? cudaSuccess : cudaMemsetAsync(ws + L.err, 0, 256, s);
     if (e != cudaSuccess) return cuda_fail(e, "clearing the error word");
     int32_t* probe_list = reinterpret_cast<int32_t*>(ws + L.probe_list);
@@ -512,8 +515,7 @@ rago_status rago_flat_search(const void* db, int64_t N, int32_t d, const void* q
     const size_t need = flat_workspace_bytes(N, d, nq, k);
     if (workspace_bytes < need) return fail(RAGO_ENOMEM, "workspace holds %zu bytes, %zu needed", workspace_bytes, need);
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    cudaError_t e = cudaMemsetAsync(workspace, 0, 256, s);
-    if (e == cudaSuccess) e = launch_flat_search(db, N, d, queries, nq, k, out_ids, out_scores, workspace, s);
+    cudaError_t e = launch_flat_search(db, N, d, queries, nq, k, out_ids, out_scores, workspace, s);
     if (e != cudaSuccess) return cuda_fail(e, "flat search");
     return RAGO_OK;
 }

@@ -243,6 +243,7 @@ struct GemmLaunch {
     int mode, nsel, cap;
     unsigned long long* cand; int32_t* cand_cnt;  // [nrows][nsplit * GEMM_COL_HALVES][cap] keys and their counts
     float* scores; uint32_t* err;
+    uint32_t* clear_block;       // error block this launch zeroes (it is the first of its search), or null
 };
 // Candidate lists leave the tensor-core kernel as RAW entries: low word = column, high word = fp32 bits of the
 // score xor a sign word (0x80000000 when the kernel stores the accumulator value of a score = -value).  Readers
@@ -261,7 +262,7 @@ int gemm_cand_cap(int nsel);  // 0: nsel too large for the fused selection
 void gemm_grid(int nrows, int64_t ncols, int d, int num_sms, int* mg, int* nsplit, int* mgroups);
 void gemm_set_pairing(int mode);
 cudaError_t launch_gemm_select(const GemmLaunch& L, cudaStream_t s);
-cudaError_t launch_split_bf16(const float* x, size_t n, int parts, void* out, cudaStream_t s);
+cudaError_t launch_split_bf16(const float* x, size_t n, int parts, void* out, uint32_t* clear_block, cudaStream_t s);
 cudaError_t launch_selftest_wait(uint32_t* err_word, uint32_t max_polls, int with_tmem, uint32_t* observed, cudaStream_t s);
 // scan.cu
 bool scan_supported(int M);
@@ -287,7 +288,6 @@ cudaError_t launch_merge(const IndexImpl* ix, const int64_t* work_prefix, int nq
                          const int32_t* slot_cnt, const unsigned long long* slot_keys, const unsigned long long* qthresh,
                          const float* queries, const int32_t* probe_list, const float* probe_bias, int64_t* out_ids,
                          float* out_dists, cudaStream_t s);
-cudaError_t launch_fill_u64(unsigned long long* p, size_t n, unsigned long long v, cudaStream_t s);
 // flat.cu
 size_t flat_workspace_bytes(int64_t N, int d, int nq, int k);
 cudaError_t launch_flat_search(const void* db, int64_t N, int d, const void* queries, int nq, int k, int64_t* out_ids,

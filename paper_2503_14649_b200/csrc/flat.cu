@@ -310,6 +310,8 @@ __global__ void __launch_bounds__(FM_THREADS, 2) flat_merge_kernel(int nlists, i
                                                                 int64_t* __restrict__ out_ids,
                                                                 float* __restrict__ out_scores) {
     __shared__ FlatMergeState S;
+    grid_dependency_wait();
+    grid_dependents_may_launch();
     const int tid = threadIdx.x, q = blockIdx.x / parts, part = blockIdx.x % parts;
     auto sync = [] { __syncthreads(); };
     if (tid == 0) S.cnt = 0;
@@ -432,6 +434,7 @@ cudaError_t launch_flat_search(const void* db, int64_t N, int d, const void* que
         G.mode = 0; G.nsel = k < N ? k : (int)N; G.cap = cap;
         G.cand = cand; G.cand_cnt = cand_cnt; G.scores = nullptr;
         G.err = static_cast<uint32_t*>(workspace);
+        G.clear_block = np ? nullptr : G.err;  // the first launch clears the error block and the tickets in it
         if (np) {
             // pilot pass over every stride-th row: each query starts from the k-th best score of that sample
             alignas(64) unsigned char tmap_p[128], tmap_ph[128];
@@ -445,6 +448,7 @@ cudaError_t launch_flat_search(const void* db, int64_t N, int d, const void* que
             P.ncols = np; P.b_part_rows = np;
             gemm_grid(nq, np, d, sm_count(), &P.mg, &P.nsplit, &pg);
             P.mode = 1; P.scores = pilot_scores;
+            P.clear_block = G.err;
             e = launch_gemm_select(P, s);
             if (e == cudaSuccess) e = launch_row_tau(pilot_scores, nq, np, G.nsel, row_tau, s);
             if (e != cudaSuccess) return e;
@@ -465,11 +469,13 @@ cudaError_t launch_flat_search(const void* db, int64_t N, int d, const void* que
             if (parts > nlists) parts = nlists;
             if (parts < 1) parts = 1;
         }
-        flat_merge_kernel<<<nq * parts, FM_THREADS, 0, s>>>(nlists, parts, k, cap, 1, gemm_cand_sign(G.alpha, G.colterm), cand_cnt,
-                                                            cand, G.err + FM_TICKET_WORD, out_ids, out_scores);
+        e = launch_overlapped(flat_merge_kernel, dim3(nq * parts), dim3(FM_THREADS), 0, s, nlists, parts, k, cap, 1,
+                              gemm_cand_sign(G.alpha, G.colterm), cand_cnt, cand, G.err + FM_TICKET_WORD, out_ids, out_scores);
         count_launch();
-        return cudaGetLastError();
+        return e != cudaSuccess ? e : cudaGetLastError();
     }
+    const cudaError_t ec = cudaMemsetAsync(workspace, 0, 256, s);
+    if (ec != cudaSuccess) return ec;
     const int nchunks = (int)((N + FLAT_CHUNK - 1) / FLAT_CHUNK);
     uint8_t* w = static_cast<uint8_t*>(workspace) + 256;
     float* scores = reinterpret_cast<float*>(w);

@@ -217,6 +217,7 @@ struct GemmArgs {
     int32_t* cand_cnt;           // [nrows][nsplit][GEMM_COL_HALVES]
     float* scores;               // [nrows][ncols] (mode 1)
     uint32_t* err;
+    uint32_t* clear_block;       // 64 words this launch zeroes (the first kernel of a search), or null
 };
 
 // Cut one list of n (> nsel) keys down to between nsel and nkeep keys and return the new threshold.
@@ -414,6 +415,11 @@ gemm_select_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     if (TWO) cluster_sync_all();  // the peer's barriers exist before anything of ours is aimed at them
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    // Everything above touched shared and tensor memory only and overlaps the kernel before this one.
+    grid_dependency_wait();
+    grid_dependents_may_launch();
+    // error block of the search: nothing reports to it for the first second (the limit of a wait)
+    if (a.clear_block != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && tid < 64) a.clear_block[tid] = 0u;
 
     // PAIR / TWO: blockIdx.y counts pairs of row tiles (the last pair may hold one tile); else row tiles.
     // TWO: the two CTAs of a cluster are neighbours in x and share a column range.
@@ -675,7 +681,7 @@ cudaError_t launch_gemm_select(const GemmLaunch& L, cudaStream_t s) {
     a.alpha = L.alpha; a.colterm = L.colterm; a.colterm_stride = L.colterm_stride > 0 ? L.colterm_stride : 1;
     a.row_tau = L.row_tau;
     a.mode = L.mode; a.nsel = L.nsel;
-    a.cand = L.cand; a.cand_cnt = L.cand_cnt; a.scores = L.scores; a.err = L.err;
+    a.cand = L.cand; a.cand_cnt = L.cand_cnt; a.scores = L.scores; a.err = L.err; a.clear_block = L.clear_block;
     const CUtensorMap* ma = reinterpret_cast<const CUtensorMap*>(L.tmap_a);
     const CUtensorMap* mb = reinterpret_cast<const CUtensorMap*>(L.mg == 3 ? L.tmap_b_half : L.tmap_b);
     const bool large = L.mode == 0 && L.cap == GEMM_CAP_LARGE;
@@ -685,11 +691,14 @@ cudaError_t launch_gemm_select(const GemmLaunch& L, cudaStream_t s) {
     cfg.blockDim = dim3(G_THREADS);
     cfg.dynamicSmemBytes = G_SMEM_BYTES;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
     if (L.mg == 3) {  // the two CTAs of a pair are neighbours in x
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr; cfg.numAttrs = 1;
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = 2; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+        cfg.numAttrs = 2;
     }
     cudaError_t e;
 #define RAGO_GEMM_LAUNCH(NKV, LOOPV) e = cudaLaunchKernelEx(&cfg, gemm_select_kernel<NKV, LOOPV>, *ma, *mb, a)
@@ -726,6 +735,8 @@ __global__ void __launch_bounds__(RT_THREADS) row_tau_kernel(const float* __rest
     __shared__ uint32_t s_round[3];
     const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const float* r = scores + (size_t)row * n;
+    grid_dependency_wait();
+    grid_dependents_may_launch();
     uint32_t mine[RT_REG];
     uint32_t mn = 0xFFFFFFFFu, mx = 0u;
 #pragma unroll
@@ -796,10 +807,11 @@ __global__ void __launch_bounds__(RT_THREADS) row_tau_kernel(const float* __rest
     }
 }
 cudaError_t launch_row_tau(const float* scores, int nrows, int n, int nsel, float* row_tau, cudaStream_t s) {
-    if (n <= 16 * 256) row_tau_kernel<256, 16, true><<<nrows, 256, 0, s>>>(scores, n, nsel, row_tau);
-    else if (n <= 16 * 1024) row_tau_kernel<1024, 16, false><<<nrows, 1024, 0, s>>>(scores, n, nsel, row_tau);
-    else if (n <= 32 * 1024) row_tau_kernel<1024, 32, false><<<nrows, 1024, 0, s>>>(scores, n, nsel, row_tau);
-    else return cudaErrorInvalidValue;
+    cudaError_t e = cudaErrorInvalidValue;
+    if (n <= 16 * 256) e = launch_overlapped(row_tau_kernel<256, 16, true>, dim3(nrows), dim3(256), 0, s, scores, n, nsel, row_tau);
+    else if (n <= 16 * 1024) e = launch_overlapped(row_tau_kernel<1024, 16, false>, dim3(nrows), dim3(1024), 0, s, scores, n, nsel, row_tau);
+    else if (n <= 32 * 1024) e = launch_overlapped(row_tau_kernel<1024, 32, false>, dim3(nrows), dim3(1024), 0, s, scores, n, nsel, row_tau);
+    if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
 }
@@ -869,7 +881,12 @@ cudaError_t launch_selftest_wait(uint32_t* err_word, uint32_t max_polls, int wit
 }
 
 // ---- fp32 -> stacked bf16 parts: out[p][i] = bf16 part p of x[i] ---------------------------------
-__global__ void split_bf16_kernel(const float* __restrict__ x, size_t n, int parts, __nv_bfloat16* __restrict__ out) {
+// clear_block: 64 words zeroed (the error block, when this is the first kernel of a search), or null.
+__global__ void split_bf16_kernel(const float* __restrict__ x, size_t n, int parts, __nv_bfloat16* __restrict__ out,
+                                  uint32_t* __restrict__ clear_block) {
+    grid_dependency_wait();
+    grid_dependents_may_launch();
+    if (clear_block != nullptr && blockIdx.x == 0 && threadIdx.x < 64) clear_block[threadIdx.x] = 0u;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         float r = x[i];
         for (int p = 0; p < parts; ++p) {
@@ -879,13 +896,13 @@ __global__ void split_bf16_kernel(const float* __restrict__ x, size_t n, int par
         }
     }
 }
-cudaError_t launch_split_bf16(const float* x, size_t n, int parts, void* out, cudaStream_t s) {
+cudaError_t launch_split_bf16(const float* x, size_t n, int parts, void* out, uint32_t* clear_block, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
     const size_t want = (n + 255) / 256;
     const int blocks = (int)(want < 148 * 8 ? want : 148 * 8);
-    split_bf16_kernel<<<blocks, 256, 0, s>>>(x, n, parts, static_cast<__nv_bfloat16*>(out));
+    const cudaError_t e = launch_overlapped(split_bf16_kernel, dim3(blocks), dim3(256), 0, s, x, n, parts, static_cast<__nv_bfloat16*>(out), clear_block);
     count_launch();
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace rago

@@ -418,16 +418,4 @@ cudaError_t launch_merge(const IndexImpl* ix, const int64_t* work_prefix, int nq
     return cudaGetLastError();
 }
 
-__global__ void fill_u64_kernel(unsigned long long* p, size_t n, unsigned long long v) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        p[i] = v;
-}
-cudaError_t launch_fill_u64(unsigned long long* p, size_t n, unsigned long long v, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    const int blocks = (int)((n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024);
-    fill_u64_kernel<<<blocks, 256, 0, s>>>(p, n, v);
-    count_launch();
-    return cudaGetLastError();
-}
-
 }  // namespace rago

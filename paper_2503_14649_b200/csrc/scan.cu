@@ -1042,6 +1042,8 @@ cudaError_t launch_codeword_norms(const float* codebooks, int M, int dsub, float
 constexpr int BT_THREADS = 256;
 __global__ void __launch_bounds__(BT_THREADS) build_tables_kernel(const TableArgs t) {
     extern __shared__ float bt_smem[];
+    grid_dependency_wait();
+    grid_dependents_may_launch();
     build_table_part(t, blockIdx.y, blockIdx.x, gridDim.x, bt_smem);
 }
 static TableArgs table_args(const IndexImpl* ix, const float* queries, uint8_t* lut_img, float* lut_inv) {
@@ -1065,6 +1067,8 @@ __global__ void __launch_bounds__(128) table_scales_kernel(const float* __restri
                                                             const float* __restrict__ cwmax, int d, int dsub, int M,
                                                             float* __restrict__ lut_scale, float* __restrict__ lut_inv) {
     __shared__ float red[4];
+    grid_dependency_wait();
+    grid_dependents_may_launch();
     const int q = blockIdx.x, tid = threadIdx.x;
     const float* qrow = queries + (size_t)q * d;
     float mx = 0.f;
@@ -1095,6 +1099,8 @@ template <int DSUB>
 __global__ void __launch_bounds__(256) build_tables_batch_kernel(const TableArgs t, const float* __restrict__ lut_scale,
                                                                   int nq, int qchunk) {
     constexpr int EPT = BTB_CW_FLOATS / DSUB;  // entries per thread
+    grid_dependency_wait();
+    grid_dependents_may_launch();
     const int d = t.d, M = t.M, tid = threadIdx.x;
     const int G = blockDim.x / M;
     const int m = tid % M, g = tid / M;
@@ -1160,7 +1166,7 @@ cudaError_t launch_build_tables(const IndexImpl* ix, const float* queries, int n
     const int dsub = ix->dsub;
     const TableArgs t = table_args(ix, queries, lut_img, lut_inv);
     if (nq > 64 && lut_scale && (dsub == 4 || dsub == 8 || dsub == 12 || dsub == 16)) {
-        table_scales_kernel<<<nq, 128, 0, s>>>(queries, ix->cwmax, ix->d, dsub, ix->M, lut_scale, lut_inv);
+        launch_overlapped(table_scales_kernel, dim3(nq), dim3(128), 0, s, queries, ix->cwmax, ix->d, dsub, ix->M, lut_scale, lut_inv);
         const int ept = BTB_CW_FLOATS / dsub;
         const int G = 256 / ix->M;  // >= 2: the scan supports M <= 128
         const int threads = ix->M * G;
@@ -1169,15 +1175,15 @@ cudaError_t launch_build_tables(const IndexImpl* ix, const float* queries, int n
         if (qchunk < 1) qchunk = 1;
         const dim3 grid(parts, (nq + qchunk - 1) / qchunk);
         switch (dsub) {
-            case 4: build_tables_batch_kernel<4><<<grid, threads, 0, s>>>(t, lut_scale, nq, qchunk); break;
-            case 8: build_tables_batch_kernel<8><<<grid, threads, 0, s>>>(t, lut_scale, nq, qchunk); break;
-            case 12: build_tables_batch_kernel<12><<<grid, threads, 0, s>>>(t, lut_scale, nq, qchunk); break;
-            default: build_tables_batch_kernel<16><<<grid, threads, 0, s>>>(t, lut_scale, nq, qchunk); break;
+            case 4: launch_overlapped(build_tables_batch_kernel<4>, grid, dim3(threads), 0, s, t, lut_scale, nq, qchunk); break;
+            case 8: launch_overlapped(build_tables_batch_kernel<8>, grid, dim3(threads), 0, s, t, lut_scale, nq, qchunk); break;
+            case 12: launch_overlapped(build_tables_batch_kernel<12>, grid, dim3(threads), 0, s, t, lut_scale, nq, qchunk); break;
+            default: launch_overlapped(build_tables_batch_kernel<16>, grid, dim3(threads), 0, s, t, lut_scale, nq, qchunk); break;
         }
         count_launch(2);
         return cudaGetLastError();
     }
-    build_tables_kernel<<<dim3(table_parts(ix, nq), nq), BT_THREADS, (size_t)(ix->d + ix->M) * 4, s>>>(t);
+    launch_overlapped(build_tables_kernel, dim3(table_parts(ix, nq), nq), dim3(BT_THREADS), (size_t)(ix->d + ix->M) * 4, s, t);
     count_launch();
     return cudaGetLastError();
 }
@@ -1245,13 +1251,15 @@ cudaError_t launch_vector_terms(const IndexImpl* ix, float* vterm, cudaStream_t 
 
 // ---- work planning: tiles per pair and their exclusive prefix sum ------------------------------
 // Three small launches: (1) tiles per pair with a CTA-local exclusive scan and one total per CTA,
-// (2) one CTA scans the totals, (3) every CTA adds its offset.
+// (2) one CTA scans the totals, (3) every CTA adds its offset; thresholds and slot counters are reset on the way.
 constexpr int PT_THREADS = 256;
 __global__ void __launch_bounds__(PT_THREADS) pair_tiles_kernel(const int32_t* __restrict__ probe_list,
                                                                 const int64_t* __restrict__ offsets, int npairs, int nprobe,
                                                                 int tile_vecs, int lead, int64_t* __restrict__ prefix,
                                                                 long long* __restrict__ block_sums) {
     __shared__ long long warp_sums[PT_THREADS / 32];
+    grid_dependency_wait();
+    grid_dependents_may_launch();
     const int p = blockIdx.x * PT_THREADS + threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     long long v = 0;
     if (p < npairs) {
@@ -1276,6 +1284,8 @@ __global__ void __launch_bounds__(PFX_THREADS) scan_totals_kernel(long long* __r
                                                                   int64_t* __restrict__ total_out) {
     __shared__ long long warp_sums[32];
     __shared__ long long carry_s;
+    grid_dependency_wait();
+    grid_dependents_may_launch();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) carry_s = 0;
     __syncthreads();
@@ -1308,9 +1318,15 @@ __global__ void __launch_bounds__(PFX_THREADS) scan_totals_kernel(long long* __r
 }
 
 __global__ void __launch_bounds__(PT_THREADS) add_offsets_kernel(int64_t* __restrict__ prefix, int npairs,
-                                                                 const long long* __restrict__ block_sums) {
+                                                                 const long long* __restrict__ block_sums,
+                                                                 unsigned long long* __restrict__ qthresh, int nq,
+                                                                 int32_t* __restrict__ slot_cnt, int nslots) {
+    grid_dependency_wait();
+    grid_dependents_may_launch();
     const int p = blockIdx.x * PT_THREADS + threadIdx.x;
     if (p < npairs) prefix[p] += block_sums[blockIdx.x];
+    for (int i = p; i < nq; i += gridDim.x * PT_THREADS) qthresh[i] = KEY_MAX;
+    for (int i = p; i < nslots; i += gridDim.x * PT_THREADS) slot_cnt[i] = 0;
 }
 
 // Small batches: one CTA does the whole preparation of a search (tiles per pair, their prefix sum,
@@ -1378,15 +1394,13 @@ cudaError_t launch_plan_work(const IndexImpl* ix, const int32_t* probe_list, int
     // pair_tiles (npairs int32 of scratch) holds the per-CTA totals: one 64-bit word per 256 pairs
     const int nblocks = (npairs + PT_THREADS - 1) / PT_THREADS;
     long long* block_sums = reinterpret_cast<long long*>(pair_tiles);
-    pair_tiles_kernel<<<nblocks, PT_THREADS, 0, s>>>(probe_list, ix->list_offsets, npairs, npairs / nq, tile_vecs, lead,
-                                                    work_prefix, block_sums);
-    scan_totals_kernel<<<1, PFX_THREADS, 0, s>>>(block_sums, nblocks, work_prefix + npairs);
-    add_offsets_kernel<<<nblocks, PT_THREADS, 0, s>>>(work_prefix, npairs, block_sums);
+    launch_overlapped(pair_tiles_kernel, dim3(nblocks), dim3(PT_THREADS), 0, s, probe_list, ix->list_offsets, npairs, npairs / nq,
+                      tile_vecs, lead, work_prefix, block_sums);
+    launch_overlapped(scan_totals_kernel, dim3(1), dim3(PFX_THREADS), 0, s, block_sums, nblocks, work_prefix + npairs);
+    launch_overlapped(add_offsets_kernel, dim3(nblocks), dim3(PT_THREADS), 0, s, work_prefix, npairs, block_sums, qthresh, nq,
+                      slot_cnt, nslots);
     count_launch(3);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = launch_fill_u64(qthresh, (size_t)nq, KEY_MAX, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(slot_cnt, 0, (size_t)nslots * 4, s);
-    return e;
+    return cudaGetLastError();
 }
 
 }  // namespace rago
