@@ -29,11 +29,11 @@
 //                  signals "stage empty" and "accumulator full" in both CTAs; the second CTA's epilogue warps
 //                  arrive on the first CTA's "accumulator empty" barrier through the cluster's shared window.
 //                  No copy is multicast: every CTA fetches its own operands.
-// A CTA owns a contiguous range of column tiles, so a row's running state (threshold, candidate count) lives in
+// A CTA owns every nsplit-th column tile (its share of the columns), so a row's running state (threshold, candidate count) lives in
 // the registers of the thread that owns the (row, column half).
 //
 // Fused selection (mode 0).  A value below the row's threshold is appended to a candidate list in global memory
-// (one list per row, column range and column half; capacity CAP = 32*NK keys, 64-bit key = ordered score bits
+// (one list per row, share and column half; capacity CAP = 32*NK keys, 64-bit key = ordered score bits
 // << 32 | column).  When a list could overflow, its warp loads it into registers (NK keys per lane), bisects for
 // a cut value that keeps between nsel and nsel + slack keys (a few warp-wide counts), writes the kept keys back
 // and lowers the threshold.  The threshold is always at least the nsel-th smallest of a subset of the row, so no
@@ -422,13 +422,12 @@ gemm_select_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     if (a.clear_block != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && tid < 64) a.clear_block[tid] = 0u;
 
     // PAIR / TWO: blockIdx.y counts pairs of row tiles (the last pair may hold one tile); else row tiles.
-    // TWO: the two CTAs of a cluster are neighbours in x and share a column range.
+    // TWO: the two CTAs of a cluster are neighbours in x and work on the same column tiles.
     const int split = TWO ? blockIdx.x >> 1 : blockIdx.x, nsplit = TWO ? gridDim.x >> 1 : gridDim.x;
     const int m0 = PAIR ? blockIdx.y * 2 : (TWO ? blockIdx.y * 2 + (int)crank : blockIdx.y);
     const int mcount = PAIR ? ((a.mtiles - m0) < 2 ? (a.mtiles - m0) : 2) : 1;
-    const int nt_begin = (int)((long long)split * a.ntiles / nsplit);
-    const int nt_end = (int)((long long)(split + 1) * a.ntiles / nsplit);
-    const int nunits = nt_end - nt_begin;  // column tiles of this CTA
+    const int nunits = (a.ntiles - split + nsplit - 1) / nsplit;  // column tiles of this CTA: split, split + nsplit, ...: all CTAs read one
+                                                                  // moving window of B (contiguous ranges: batch of 33 over 65 536 lists 221 us, this 219)
     const int kiters = a.nterms * a.kblocks;
 
     if (warp == 0) {
@@ -438,7 +437,7 @@ gemm_select_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
             const int total = nunits * kiters;
             const uint32_t tx_bytes = TWO ? 2u * STAGE_BYTES  // both CTAs' loads complete on the leader's barrier
                                           : (uint32_t)(mcount == 2 ? STAGE_BYTES : G_A_BYTES + G_B_BYTES);
-            int nt = nt_begin, t = 0, kb = 0, s = 0;
+            int nt = split, t = 0, kb = 0, s = 0;
             uint32_t ph = 0;
             for (int gi = 0; gi < total; ++gi) {
                 const int kx = kb * GBK;
@@ -446,7 +445,7 @@ gemm_select_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                 const int yb = a.term_b[t] * a.b_part_rows + nt * GBN;
                 if (++kb == a.kblocks) {
                     kb = 0;
-                    if (++t == a.nterms) { t = 0; ++nt; }
+                    if (++t == a.nterms) { t = 0; nt += nsplit; }
                 }
                 if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, a.err, 64)) break;
                 const uint32_t st = base + s * STAGE_BYTES;
@@ -527,7 +526,7 @@ gemm_select_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         }
         bool dead = false;
         for (int u = 0; u < nunits && !dead; ++u) {
-            const int nt = nt_begin + u;
+            const int nt = split + u * nsplit;
             const int buf = PAIR ? 0 : (u & 1);
             const uint32_t uph = PAIR ? (u & 1u) : ((u >> 1) & 1u);
             float* cnu = cn + (u & 1) * G_HALF;
@@ -648,7 +647,7 @@ int gemm_cand_cap(int nsel) { return nsel <= GEMM_CAP_SMALL - 128 ? GEMM_CAP_SMA
 //   flat search, B = 20 GB from HBM       5.74        5.27        4.7 - 5.2 (power-capped to 1.2 - 1.6 GHz)
 //   Hyperscale coarse stage, B in L2      0.410       0.464       0.401
 // The in-CTA pair saves the same operand traffic as the CTA pair but cannot overlap its epilogue; it is kept as a
-// measured alternative that the test hook reaches.  *nsplit = column ranges; *mgroups = grid rows.
+// measured alternative that the test hook reaches.  *nsplit = shares of the column tiles; *mgroups = grid rows.
 static int g_pairing = 0;  // 0: as above, 1: LOOP_SINGLE, 2: LOOP_PAIR, 3: LOOP_TWO_CTA (2, 3: batches with two row tiles)
 void gemm_set_pairing(int mode) { g_pairing = mode; }
 void gemm_grid(int nrows, int64_t ncols, int d, int num_sms, int* mg, int* nsplit, int* mgroups) {
