@@ -5,6 +5,7 @@
 // before the final cut, so the probe order follows the plain definition up to fp32 rounding.
 // With a bf16 coarse quantiser the query is rounded to bf16 first (coarse step only).
 #include <cstring>
+#include <type_traits>
 
 #include "plan.cuh"
 #include "topk.cuh"
@@ -103,6 +104,18 @@ __global__ void __launch_bounds__(256) coarse_scores_kernel(const float* __restr
     }
 }
 
+// Loads of index data that are issued where they stand (not moved past the wait for the kernel in front).
+__device__ __forceinline__ float4 ldg_const_f4(const float* p) {
+    float4 v;
+    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint2 ldg_const_u2(const void* p) {
+    uint2 v;
+    asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
+
 // ---- score matrix for tiny batches (the latency-bound iterative-retrieval shape) -------------------
 // For up to CS_MAXQ queries: a warp takes CS_CPW centroid rows at a time and keeps one partial sum per (row, query),
 // so the centroid table is read exactly once per batch however few queries there are.  The launch is bound by the
@@ -119,6 +132,39 @@ __global__ void __launch_bounds__(256) coarse_small_kernel(const float* __restri
                                                            const float* __restrict__ cnorm, int nq, int nlist, int d,
                                                            int metric, float* __restrict__ scores, uint32_t* __restrict__ clear_block) {
     extern __shared__ __align__(16) float qs[];  // [nq][d], rounded to bf16 values for a bf16 index
+    const int lane = threadIdx.x & 31;
+    const int warps = (gridDim.x * blockDim.x) >> 5;
+    constexpr int QG = NQ <= 4 ? NQ : 8;   // queries multiplied against the rows held in registers at a time
+    constexpr int NGROUPS = NQ / QG;
+    constexpr int CHUNK = 4;               // 16-byte (fp32) / 8-byte (bf16) loads per lane and row in one round: 512 values
+    int c0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * CS_CPW;
+    float4 cv[CS_CPW][CHUNK];
+    auto load_rows = [&](int jb) {
+#pragma unroll
+        for (int u = 0; u < CS_CPW; ++u) {
+            const int c = c0 + u < nlist ? c0 + u : nlist - 1;  // rows past the end repeat the last one, unused
+#pragma unroll
+            for (int h = 0; h < CHUNK; ++h) {
+                const int j0 = jb + h * 128 + lane * 4;
+                if (j0 < d) {
+                    if (BF16) {
+                        const uint2 raw = ldg_const_u2(static_cast<const __nv_bfloat16*>(C) + (size_t)c * d + j0);
+                        cv[u][h].x = __uint_as_float(raw.x << 16); cv[u][h].y = __uint_as_float(raw.x & 0xFFFF0000u);
+                        cv[u][h].z = __uint_as_float(raw.y << 16); cv[u][h].w = __uint_as_float(raw.y & 0xFFFF0000u);
+                    } else {
+                        cv[u][h] = ldg_const_f4(static_cast<const float*>(C) + (size_t)c * d + j0);
+                    }
+                } else {
+                    cv[u][h] = make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+            }
+        }
+    };
+    // The centroids belong to the index and no kernel on the stream writes them: a warp asks for its first rows before
+    // it waits for the kernel in front, so in a stream of searches the table is on its way while the previous search
+    // is still merging, and the queries are staged meanwhile.
+    if (c0 < nlist) load_rows(0);
+    bool loaded = true;
     grid_dependency_wait();
     grid_dependents_may_launch();
     // first kernel of a search: the workspace's 256-byte error block (error word, ticket) starts at zero; doing it
@@ -140,37 +186,10 @@ __global__ void __launch_bounds__(256) coarse_small_kernel(const float* __restri
         }
     }
     __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const int warps = (gridDim.x * blockDim.x) >> 5;
-    constexpr int QG = NQ <= 4 ? NQ : 8;   // queries multiplied against the rows held in registers at a time
-    constexpr int NGROUPS = NQ / QG;
-    constexpr int CHUNK = 4;               // 16-byte (fp32) / 8-byte (bf16) loads per lane and row in one round: 512 values
-    for (int c0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * CS_CPW; c0 < nlist; c0 += warps * CS_CPW) {
+    for (; c0 < nlist; c0 += warps * CS_CPW) {
         float cn[CS_CPW];
 #pragma unroll
         for (int u = 0; u < CS_CPW; ++u) cn[u] = metric == RAGO_L2 ? __ldg(cnorm + (c0 + u < nlist ? c0 + u : nlist - 1)) : 0.f;
-        float4 cv[CS_CPW][CHUNK];
-        auto load_rows = [&](int jb) {
-#pragma unroll
-            for (int u = 0; u < CS_CPW; ++u) {
-                const int c = c0 + u < nlist ? c0 + u : nlist - 1;  // rows past the end repeat the last one, unused
-#pragma unroll
-                for (int h = 0; h < CHUNK; ++h) {
-                    const int j0 = jb + h * 128 + lane * 4;
-                    if (j0 < d) {
-                        if (BF16) {
-                            const uint2 raw = *reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(C) + (size_t)c * d + j0);
-                            cv[u][h].x = __uint_as_float(raw.x << 16); cv[u][h].y = __uint_as_float(raw.x & 0xFFFF0000u);
-                            cv[u][h].z = __uint_as_float(raw.y << 16); cv[u][h].w = __uint_as_float(raw.y & 0xFFFF0000u);
-                        } else {
-                            cv[u][h] = *reinterpret_cast<const float4*>(static_cast<const float*>(C) + (size_t)c * d + j0);
-                        }
-                    } else {
-                        cv[u][h] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    }
-                }
-            }
-        };
 #pragma unroll
         for (int g = 0; g < NGROUPS; ++g) {
             if (g * QG >= nq) break;  // uniform
@@ -182,7 +201,8 @@ __global__ void __launch_bounds__(256) coarse_small_kernel(const float* __restri
             for (int jb = 0; jb < d; jb += 128 * CHUNK) {
                 // the rows of a block of 512 values stay in registers for every group of queries; a longer row is
                 // read again for the second group (from the caches)
-                if (g == 0 || d > 128 * CHUNK) load_rows(jb);
+                if ((g == 0 || d > 128 * CHUNK) && !loaded) load_rows(jb);
+                loaded = false;
 #pragma unroll
                 for (int h = 0; h < CHUNK; ++h) {
                     const int j0 = jb + h * 128 + lane * 4;
@@ -439,7 +459,46 @@ cudaError_t launch_tree_candidates(const IndexImpl* ix, const float* queries, in
 }
 
 // ---- per-query selection of the nprobe best lists ----------------------------------------------
-constexpr int SEL_MAX_SPLIT = 512;  // candidate lists per query the kernel can index (one per column range of the GEMM)
+// sum (q-c)^2 (L2) or <q,c> of one query and centroid `row`, by one warp (d a multiple of 4), valid in every lane;
+// round_q: the query is rounded to bf16 first.  The row's loads of STEPS steps are in flight together (fp32: 512 values,
+// bf16: 1024): fetched one step at a time, a 768-dimensional row cost six memory round trips.  The order of the sum is
+// the plain loop's.
+template <bool BF16>
+__device__ __forceinline__ float warp_exact_score(const float* qrow, const void* C, uint32_t row, int d, int metric, bool round_q,
+                                                  int lane) {
+    constexpr int STEPS = BF16 ? 8 : 4;
+    using Raw = typename std::conditional<BF16, uint2, float4>::type;  // four values as they lie in memory
+    const Raw* src = reinterpret_cast<const Raw*>(static_cast<const uint8_t*>(C) + (size_t)row * d * (BF16 ? 2 : 4));
+    float acc = 0.f;
+    for (int jb = lane * 4; jb < d; jb += 128 * STEPS) {
+        Raw raw[STEPS];
+#pragma unroll
+        for (int u = 0; u < STEPS; ++u)
+            if (jb + u * 128 < d) raw[u] = __ldg(src + ((jb + u * 128) >> 2));
+#pragma unroll
+        for (int u = 0; u < STEPS; ++u) {
+            if (jb + u * 128 >= d) continue;
+            float4 q = *reinterpret_cast<const float4*>(qrow + jb + u * 128), c;
+            if constexpr (BF16) {
+                c.x = __uint_as_float(raw[u].x << 16); c.y = __uint_as_float(raw[u].x & 0xFFFF0000u);
+                c.z = __uint_as_float(raw[u].y << 16); c.w = __uint_as_float(raw[u].y & 0xFFFF0000u);
+            } else {
+                c = raw[u];
+            }
+            if (BF16 && round_q) { q.x = round_bf16(q.x); q.y = round_bf16(q.y); q.z = round_bf16(q.z); q.w = round_bf16(q.w); }
+            if (metric == RAGO_L2) {
+                const float t0 = q.x - c.x, t1 = q.y - c.y, t2 = q.z - c.z, t3 = q.w - c.w;
+                acc = fmaf(t0, t0, fmaf(t1, t1, fmaf(t2, t2, fmaf(t3, t3, acc))));
+            } else {
+                acc = fmaf(q.x, c.x, fmaf(q.y, c.y, fmaf(q.z, c.z, fmaf(q.w, c.w, acc))));
+            }
+        }
+    }
+    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    return acc;
+}
+
+constexpr int SEL_MAX_SPLIT = 512;  // candidate lists per query the kernel can index (one per share of the GEMM's column tiles)
 
 // Candidates come either from a score row (scores != null: all nlist lists) or from the candidate
 // lists the tensor-core kernel left behind (cand[q][split][cap] raw entries, see cand_key, with counts cand_cnt[q][split]).
@@ -492,10 +551,19 @@ __global__ void __launch_bounds__(SEL_THREADS) select_probes_kernel(
         // the counts are fetched side by side (one thread reading them in turn paid a global round trip per list)
         for (int sp = tid; sp < nsplit; sp += SEL_THREADS) pre[sp + 1] = cand_cnt[(size_t)q * nsplit + sp];
         __syncthreads();
-        if (tid == 0) {
-            int acc = 0;
-            for (int sp = 0; sp < nsplit; ++sp) { const int c = pre[sp + 1]; pre[sp] = acc; acc += c; }
-            pre[nsplit] = acc;
+        if (warp == 0) {  // running sum of the counts, in place: 32 of them at a time (one thread took 10 ns for each)
+            int carry = 0;
+            for (int b = 0; b < nsplit; b += 32) {
+                const int sp = b + lane;
+                int incl = sp < nsplit ? pre[sp + 1] : 0;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += y;
+                }
+                if (sp < nsplit) pre[sp + 1] = carry + incl;
+                carry += __shfl_sync(0xffffffffu, incl, 31);
+            }
+            if (lane == 0) pre[0] = 0;
         }
     }
     __syncthreads();
@@ -679,19 +747,17 @@ __global__ void __launch_bounds__(SEL_THREADS) select_probes_kernel(
     }
     // collect the items below the cut, and those at the cut up to payload P
     if (in_regs) {
-        bool any = false;  // most warps hold nothing at or below the cut: one vote instead of SEL_REG
+        // Few items are taken and this code runs once, so its size is what it costs: a bit per register slot, then a loop
+        // that reads the taken items again, instead of SEL_REG copies of the look-up (batch of 33, candidate lists: 10 us).
+        uint32_t taken = 0u;
 #pragma unroll
-        for (int j = 0; j < SEL_REG; ++j) any = any || (mine[j] != 0xFFFFFFFFu && mine[j] <= T);
-        if (__any_sync(0xffffffffu, any)) {
-#pragma unroll
-        for (int j = 0; j < SEL_REG; ++j) {
-            bool take = mine[j] != 0xFFFFFFFFu && mine[j] <= T;
-            unsigned long long key = KEY_MAX;
-            if (FROM_SCORES) key = ((unsigned long long)mine[j] << 32) | (uint32_t)(tid + j * SEL_THREADS);
-            else if (take) key = item(tid + j * SEL_THREADS);
-            if (take && mine[j] == T && (uint32_t)key > P) take = false;
+        for (int j = 0; j < SEL_REG; ++j) taken |= (mine[j] != 0xFFFFFFFFu && mine[j] <= T) ? 1u << j : 0u;
+        while (__any_sync(0xffffffffu, taken != 0u)) {
+            bool take = taken != 0u;
+            const unsigned long long key = take ? item(tid + (__ffs(taken) - 1) * SEL_THREADS) : KEY_MAX;
+            taken &= taken - 1u;
+            if ((uint32_t)(key >> 32) == T && (uint32_t)key > P) take = false;
             warp_push(keys, &cnt, take, key);
-        }
         }
     } else {
         for (int l0 = 0; l0 < nitems; l0 += SEL_THREADS) {
@@ -707,26 +773,7 @@ __global__ void __launch_bounds__(SEL_THREADS) select_probes_kernel(
     const float* qrow = Q + (size_t)q * d;
     for (int i = warp; i < kept; i += SEL_THREADS / 32) {
         const uint32_t l = (uint32_t)(keys[i] & 0xFFFFFFFFull);
-        float acc = 0.f;
-        for (int j = lane * 4; j < d; j += 128) {  // d is a multiple of 4: 16-byte (fp32) / 8-byte (bf16) loads
-            float4 qv = *reinterpret_cast<const float4*>(qrow + j);
-            float4 cv;
-            if (BF16) {
-                qv.x = round_bf16(qv.x); qv.y = round_bf16(qv.y); qv.z = round_bf16(qv.z); qv.w = round_bf16(qv.w);
-                const uint2 raw = *reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(C) + (size_t)l * d + j);
-                cv.x = __uint_as_float(raw.x << 16); cv.y = __uint_as_float(raw.x & 0xFFFF0000u);
-                cv.z = __uint_as_float(raw.y << 16); cv.w = __uint_as_float(raw.y & 0xFFFF0000u);
-            } else {
-                cv = *reinterpret_cast<const float4*>(static_cast<const float*>(C) + (size_t)l * d + j);
-            }
-            if (metric == RAGO_L2) {
-                const float t0 = qv.x - cv.x, t1 = qv.y - cv.y, t2 = qv.z - cv.z, t3 = qv.w - cv.w;
-                acc = fmaf(t0, t0, fmaf(t1, t1, fmaf(t2, t2, fmaf(t3, t3, acc))));
-            } else {
-                acc = fmaf(qv.x, cv.x, fmaf(qv.y, cv.y, fmaf(qv.z, cv.z, fmaf(qv.w, cv.w, acc))));
-            }
-        }
-        for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        const float acc = warp_exact_score<BF16>(qrow, C, l, d, metric, BF16, lane);
         if (lane == 0) keys2[i] = make_key(metric == RAGO_L2 ? acc : -acc, l);
     }
     __syncthreads();
@@ -746,12 +793,7 @@ __global__ void __launch_bounds__(SEL_THREADS) select_probes_kernel(
     if (BF16 && metric == RAGO_L2) {
         for (int i = warp; i < nprobe; i += SEL_THREADS / 32) {
             const uint32_t l = (uint32_t)(keys[i] & 0xFFFFFFFFull);
-            float acc = 0.f;
-            for (int j = lane; j < d; j += 32) {
-                const float t = qrow[j] - load_c<BF16>(C, (size_t)l * d + j);
-                acc = fmaf(t, t, acc);
-            }
-            for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            const float acc = warp_exact_score<BF16>(qrow, C, l, d, RAGO_L2, false, lane);
             if (lane == 0) probe_bias[(size_t)q * nprobe + i] = acc;
         }
     }
@@ -765,7 +807,7 @@ __global__ void __launch_bounds__(SEL_THREADS) select_probes_kernel(
                 long long v = 0;  // tiles of pair tid (nprobe <= MAX_K = SEL_THREADS)
                 if (tid < nprobe) {
                     const uint32_t l = (uint32_t)(keys[tid] & 0xFFFFFFFFull);
-                    v = (fp.offsets[l + 1] - fp.offsets[l] + fp.tile_vecs - 1) / fp.tile_vecs;
+                    v = tiles_of(fp.offsets[l + 1] - fp.offsets[l], fp.tile_vecs);
                 }
                 fp.qthresh[0] = KEY_MAX;  // every thread the same value; the stores leave with the loads above
                 for (int i = tid; i < fp.nslots; i += SEL_THREADS) fp.slot_cnt[i] = 0;
@@ -798,12 +840,18 @@ __global__ void __launch_bounds__(SEL_THREADS) select_probes_kernel(
     }
 }
 
-template <bool BF16, int THREADS, int REG>
+// Registers per thread for the items of candidate lists: every slot is a copy of the look-up that the CTA has to fetch, so
+// only large selections (behind pilot thresholds the lists hold some 16 to 20 times the wanted items) take as many as a score
+// row does.
+template <bool BF16, int THREADS, int REG, int REG_LISTS>
 static void launch_select_source(const IndexImpl* ix, const float* queries, const float* scores,
                                  const unsigned long long* cand, const int32_t* cand_cnt, uint32_t cand_sign, int nsplit, int cap, int nq,
                                  int nprobe, int32_t* probe_list, float* probe_term, float* probe_bias, const FusedPlan& fp, cudaStream_t s) {
     const dim3 grid(fp.enabled ? nq * (1 + fp.table_parts) : nq);
     const size_t smem = fp.enabled ? (size_t)(ix->d + ix->M) * 4 : 0;
+    const bool pilot = ix->pilot_stride && ix->nlist >= 8192 && ix->nlist / ix->pilot_stride >= 4 * (nprobe + PROBE_GUARD);
+    const int most = ix->tree_n1 ? ix->tree_max_cand : (pilot ? 20 * (nprobe + PROBE_GUARD) : ix->nlist);  // items of a query, usually
+    const bool few = most <= THREADS * REG_LISTS;
     if (scores && ix->nlist <= THREADS * REG)
         launch_overlapped(select_probes_kernel<BF16, THREADS, REG, true, true>, grid, dim3(THREADS), smem, s,
             queries, ix->centroids, scores, cand, cand_cnt, cand_sign, nsplit, cap, ix->nlist, ix->d, ix->metric, nprobe, probe_list,
@@ -813,20 +861,21 @@ static void launch_select_source(const IndexImpl* ix, const float* queries, cons
             queries, ix->centroids, scores, cand, cand_cnt, cand_sign, nsplit, cap, ix->nlist, ix->d, ix->metric, nprobe, probe_list,
             probe_term, probe_bias, fp);
     else
-        launch_overlapped(select_probes_kernel<BF16, THREADS, REG, false, false>, grid, dim3(THREADS), smem, s,
+        launch_overlapped(few ? select_probes_kernel<BF16, THREADS, REG_LISTS, false, false> : select_probes_kernel<BF16, THREADS, REG, false, false>,
+            grid, dim3(THREADS), smem, s,
             queries, ix->centroids, scores, cand, cand_cnt, cand_sign, nsplit, cap, ix->nlist, ix->d, ix->metric, nprobe, probe_list,
             probe_term, probe_bias, fp);
 }
-template <int THREADS, int REG>
+template <int THREADS, int REG, int REG_LISTS>
 static void launch_select_shape(const IndexImpl* ix, const float* queries, const float* scores,
                                 const unsigned long long* cand, const int32_t* cand_cnt, uint32_t cand_sign, int nsplit, int cap, int nq,
                                 int nprobe, int32_t* probe_list, float* probe_term, float* probe_bias, const FusedPlan& fp,
                                 cudaStream_t s) {
     if (ix->coarse_bf16)
-        launch_select_source<true, THREADS, REG>(ix, queries, scores, cand, cand_cnt, cand_sign, nsplit, cap, nq, nprobe, probe_list,
+        launch_select_source<true, THREADS, REG, REG_LISTS>(ix, queries, scores, cand, cand_cnt, cand_sign, nsplit, cap, nq, nprobe, probe_list,
                                                  probe_term, probe_bias, fp, s);
     else
-        launch_select_source<false, THREADS, REG>(ix, queries, scores, cand, cand_cnt, cand_sign, nsplit, cap, nq, nprobe, probe_list,
+        launch_select_source<false, THREADS, REG, REG_LISTS>(ix, queries, scores, cand, cand_cnt, cand_sign, nsplit, cap, nq, nprobe, probe_list,
                                                   probe_term, probe_bias, fp, s);
 }
 // fp (may be null): the kernel also plans the scan of the batch and builds its lookup tables (batches of at most 64
@@ -840,10 +889,10 @@ static cudaError_t launch_select_any(const IndexImpl* ix, const float* queries, 
     std::memset(&off, 0, sizeof(off));
     if (fp && fp->enabled && nq > 64) return cudaErrorInvalidValue;
     if (nq <= 64)
-        launch_select_shape<1024, 16>(ix, queries, scores, cand, cand_cnt, cand_sign, nsplit, cap, nq, nprobe, probe_list, probe_term,
+        launch_select_shape<1024, 16, 4>(ix, queries, scores, cand, cand_cnt, cand_sign, nsplit, cap, nq, nprobe, probe_list, probe_term,
                                       probe_bias, fp ? *fp : off, s);
     else
-        launch_select_shape<256, 20>(ix, queries, scores, cand, cand_cnt, cand_sign, nsplit, cap, nq, nprobe, probe_list, probe_term,
+        launch_select_shape<256, 20, 12>(ix, queries, scores, cand, cand_cnt, cand_sign, nsplit, cap, nq, nprobe, probe_list, probe_term,
                                      probe_bias, off, s);
     count_launch();
     return cudaGetLastError();

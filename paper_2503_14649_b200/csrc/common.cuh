@@ -229,7 +229,7 @@ cudaError_t launch_tree_candidates(const IndexImpl* ix, const float* queries, in
 constexpr int TREE_LIMIT_B1 = 64, TREE_LIMIT_N1 = 4096;
 // gemm_select.cu
 constexpr int GEMM_CAP_SMALL = 512, GEMM_CAP_LARGE = 1024;  // candidate-list capacities (keys per list)
-constexpr int GEMM_COL_HALVES = 2;  // a row has one candidate list per column range of the grid AND per half of a 256-column tile
+constexpr int GEMM_COL_HALVES = 2;  // a row has one candidate list per share of the grid AND per half of a 256-column tile
 struct GemmLaunch {
     const void* tmap_a;          // CUtensorMap of A: bf16 [a parts * a_part_rows][d]
     const void* tmap_b;          // CUtensorMap of B: bf16 [b parts * b_part_rows][d], boxes of 256 rows
@@ -237,7 +237,7 @@ struct GemmLaunch {
     int nrows; int64_t ncols; int d;
     int a_part_rows; int64_t b_part_rows;
     int nterms; int term_a[6], term_b[6];
-    int mg, nsplit;              // from gemm_grid: main loop (1 single, 2 pair in a CTA, 3 CTA pair) and column ranges
+    int mg, nsplit;              // from gemm_grid: main loop (1 single, 2 pair in a CTA, 3 CTA pair) and shares of the column tiles
     float alpha; const float* colterm; int colterm_stride;
     const float* row_tau;        // initial per-row thresholds (mode 0) or null
     int mode, nsel, cap;

@@ -1,7 +1,7 @@
 // Exact flat search: score = <q, y_i> over bf16 inputs, fp32 accumulation, k largest per query.
 //
 // Main path (k <= 960): the tensor-core kernel of gemm_select.cu with rows = queries and columns =
-// database rows; every CTA streams its own range of the database once (both 128-query row tiles are
+// database rows; every CTA streams its own share of the database once (both 128-query row tiles are
 // multiplied against a database tile while it is hot) and keeps each query's k best of that range;
 // flat_merge_kernel merges the ranges.  No score is ever written to memory.
 // Fallback (larger k): the database is processed in panels of PANEL rows on the fp32 pipes: scores of
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(FSEL_THREADS) flat_select_kernel(const float* 
 //
 // List l of query q holds slot_cnt entries at slot_keys[(q * nlists + l) * stride ...]; with `raw` they are the raw
 // candidate entries of the tensor-core kernel (cand_key turns them into keys).  Latency is what counts here: a query
-// has a few hundred short lists (one per column range and half tile), and walking them one after the other cost
+// has a few hundred short lists (one per share of the columns and half tile), and walking them one after the other cost
 // about a microsecond per list (290 us for one query over 100 000 rows, 264 us for 37 over a million, 308 us for 256
 // over ten million).  So the counts of up to FM_LISTS lists are fetched at once and summed, the entries are numbered
 // through, and every thread fetches FM_KPT of them side by side; a counting bisection on the keys (distinct, so it
@@ -380,7 +380,7 @@ static int flat_pilot_cols(int64_t N, int k) {
 }
 
 // Workspace, tensor-core path: [err 256 B][cand nq*nlists*cap u64][cand_cnt nq*nlists i32][pilot scores nq*np f32][row_tau nq f32]
-//            (nlists = column ranges of the grid x GEMM_COL_HALVES candidate lists per query)
+//            (nlists = shares of the grid x GEMM_COL_HALVES candidate lists per query)
 //            fallback:         [err 256 B][scores nq*PANEL f32][slot_cnt nq*nchunks i32][slot_keys nq*nchunks*k u64]
 size_t flat_workspace_bytes(int64_t N, int d, int nq, int k) {
     if (flat_on_tensor_cores(d, k)) {

@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(THREADS) merge_kernel(
 // Small batches (latency): the same result by a shorter chain of dependent memory accesses.  A query's slots are
 // consecutive in memory, so the CTA's 1024 threads fetch ALL of their keys (at most KPT each) and the slot counts in
 // one round trip, keep them in registers, find a cut with between k and k + k/4 + 8 keys at or below it by a counting
-// bisection on the 64-bit keys (distinct, so it always ends), and only the keys up to the cut go to shared memory to
+// bisection on the score words, then on whole keys if scores are equal (keys are distinct, so it always ends), and only the keys up to the cut go to shared memory to
 // be sorted.  The ids of the winners are fetched together with the values the cancellation check needs.
 template <int KPT>
 __global__ void __launch_bounds__(1024) merge_small_kernel(
@@ -246,8 +246,7 @@ __global__ void __launch_bounds__(1024) merge_small_kernel(
     constexpr int THREADS = 1024, BUF = 2 * MAX_K;
     __shared__ unsigned long long keys[BUF];
     __shared__ int cnt;
-    __shared__ unsigned long long s_mn, s_mx;
-    __shared__ uint32_t s_nv, s_round[3];
+    __shared__ uint32_t s_mn, s_mx, s_nv, s_round[3];
     __shared__ int p_list[MAX_K];
     __shared__ uint32_t p_lo[MAX_K], p_hi[MAX_K];
     __shared__ int redo[MAX_K], redo_list[MAX_K];
@@ -256,7 +255,7 @@ __global__ void __launch_bounds__(1024) merge_small_kernel(
     auto sync = [] { __syncthreads(); };
     grid_dependency_wait();
     grid_dependents_may_launch();
-    if (tid == 0) { cnt = 0; nredo = 0; s_mn = KEY_MAX; s_mx = 0ull; s_nv = 0u; s_round[0] = s_round[1] = s_round[2] = 0u; }
+    if (tid == 0) { cnt = 0; nredo = 0; s_mn = 0xFFFFFFFFu; s_mx = 0u; s_nv = 0u; s_round[0] = s_round[1] = s_round[2] = 0u; }
     const long long W = work_prefix[npairs];
     const long long u0 = work_prefix[(size_t)q * nprobe], u1 = work_prefix[(size_t)(q + 1) * nprobe];
     unsigned long long tau = qthresh[q];
@@ -289,48 +288,52 @@ __global__ void __launch_bounds__(1024) merge_small_kernel(
             }
         }
     }
-    unsigned long long mn = KEY_MAX, mx = 0ull;
-    uint32_t nv = 0;
+    uint32_t mn = 0xFFFFFFFFu, mx = 0u, nv = 0u;  // score words
 #pragma unroll
-    for (int j = 0; j < KPT; ++j)
-        if (mine[j] != KEY_MAX) { mn = mine[j] < mn ? mine[j] : mn; mx = mine[j] > mx ? mine[j] : mx; ++nv; }
+    for (int j = 0; j < KPT; ++j) {
+        const uint32_t o = (uint32_t)(mine[j] >> 32);
+        if (mine[j] != KEY_MAX) { mn = o < mn ? o : mn; mx = o > mx ? o : mx; ++nv; }
+    }
     __syncthreads();  // the shared words are initialised
     nv = __reduce_add_sync(0xffffffffu, nv);
     if (nv) {  // uniform within the warp
-        for (int o = 16; o; o >>= 1) {
-            const unsigned long long a = shfl_xor_u64(mn, o), b = shfl_xor_u64(mx, o);
-            mn = a < mn ? a : mn; mx = b > mx ? b : mx;
-        }
+        mn = __reduce_min_sync(0xffffffffu, mn);
+        mx = __reduce_max_sync(0xffffffffu, mx);
         if (lane == 0) { atomicMin(&s_mn, mn); atomicMax(&s_mx, mx); atomicAdd(&s_nv, nv); }
     }
     __syncthreads();
-    mn = s_mn; mx = s_mx;
-    const uint32_t nvalid = s_nv;
+    uint32_t c_hi = s_nv;
     uint32_t want_max = (uint32_t)(k + (k >> 2) + 8);  // <= BUF
     if (want_max < (uint32_t)WARP_SORT_MAX) want_max = WARP_SORT_MAX;  // as many as the short selection ranks in one go
-    unsigned long long T = mx;  // keys up to T are collected
-    if (nvalid > want_max) {    // uniform.  k >= 2 here would not be needed: count(<= mn) = 1 <= k always
-        unsigned long long lo = mn, hi = mx;  // #(key <= lo) <= k  and  #(key <= hi) >= k; lo itself is always kept
-        uint32_t c_hi = nvalid;
+    unsigned long long T = KEY_MAX - 1;  // keys up to T are collected
+    if (c_hi > want_max) {    // uniform
+        // bisected on the score words (half the instructions of a 64-bit compare); if a group of equal scores is still too
+        // large, on whole keys: #(key <= lo) <= k and #(key <= T) >= k throughout
         int round = 0;
-        if (k > 1) {
-            while (hi - lo > 1 && c_hi > want_max) {  // uniform
-                const unsigned long long mid = lo + (hi - lo) / 2;
-                uint32_t c = 0;
+        auto count = [&](auto below) {
+            uint32_t c = 0;
 #pragma unroll
-                for (int j = 0; j < KPT; ++j) c += mine[j] <= mid ? 1u : 0u;  // mid < mx < the empty-slot pattern
-                c = __reduce_add_sync(0xffffffffu, c);
-                const int slot = round % 3;
-                if (lane == 0 && c) atomicAdd(&s_round[slot], c);
-                if (tid == 0) s_round[(slot + 1) % 3] = 0u;  // next round's word; its last readers passed two barriers ago
-                __syncthreads();
-                c = s_round[slot];
-                if (c < (uint32_t)k) lo = mid; else { hi = mid; c_hi = c; }
-                ++round;
-            }
-            T = hi;
-        } else {
-            T = mn;
+            for (int j = 0; j < KPT; ++j) c += below(mine[j]) ? 1u : 0u;  // never true of an empty slot
+            c = __reduce_add_sync(0xffffffffu, c);
+            const int slot = round % 3;
+            if (lane == 0 && c) atomicAdd(&s_round[slot], c);
+            if (tid == 0) s_round[(slot + 1) % 3] = 0u;  // next round's word; its last readers passed two barriers ago
+            __syncthreads();
+            ++round;
+            return s_round[slot];
+        };
+        long long lo32 = (long long)s_mn - 1, hi32 = s_mx;
+        while (hi32 - lo32 > 1 && c_hi > want_max) {
+            const uint32_t mid = bisect_mid(lo32, hi32, round);
+            const uint32_t c = count([&](unsigned long long x) { return (uint32_t)(x >> 32) <= mid; });
+            if (c < (uint32_t)k) lo32 = mid; else { hi32 = mid; c_hi = c; }
+        }
+        T = ((unsigned long long)hi32 << 32) | 0xFFFFFFFFull;
+        unsigned long long lo = (unsigned long long)hi32 << 32;
+        while (T - lo > 1 && c_hi > want_max) {
+            const unsigned long long mid = lo + (T - lo) / 2;
+            const uint32_t c = count([&](unsigned long long x) { return x <= mid; });
+            if (c < (uint32_t)k) lo = mid; else { T = mid; c_hi = c; }
         }
     }
 #pragma unroll

@@ -1,9 +1,10 @@
 // Lookup-table construction + asymmetric-distance scan of the probed inverted lists.
 //
-// One persistent CTA per SM walks a contiguous, equally sized share of the batch's code tiles
-// (pairs (query, probed list) in probe order, each list cut into tiles of TV vectors).  A producer
+// One persistent CTA per SM walks a contiguous share of the batch's code tiles (pairs (query, probed list) in probe
+// order, each list cut into equal tiles of at most TV vectors); shares hold the same number of tiles, the start of a
+// query counting as several (scan_query_lead).  A producer
 // warp streams code tiles global -> shared with 1-D bulk copies (cp.async.bulk + mbarrier, a ring of
-// S tiles in flight, the tiles two steps further down the list prefetched into L2); consumer warps
+// S tiles in flight, where it pays the tiles two steps further down the list prefetched into L2); consumer warps
 // build the lookup table of the current QUERY in shared memory (or, for small batches, fetch the
 // image a kernel before the scan has built), then every lane owns one (virtual) code row of the tile
 // and sums table entries.
@@ -1130,8 +1131,11 @@ __global__ void __launch_bounds__(256) build_tables_batch_kernel(const TableArgs
     const float lut_s = t.metric == RAGO_IP ? -1.f : -2.f;
     const int q0 = blockIdx.y * qchunk;
     const int q1 = q0 + qchunk < nq ? q0 + qchunk : nq;
-    float qn[DSUB];
+    // the next query's values and scale, fetched while the current one is multiplied (a scale fetched in the step that
+    // uses it put a memory round trip into every step: 4 096 queries, 64 sub-spaces 239 us)
+    float qn[DSUB], scale_n = 0.f;
     auto fetch = [&](int q) {
+        scale_n = __ldg(lut_scale + q);
         const float* src = t.queries + (size_t)q * d + m * DSUB;
 #pragma unroll
         for (int u = 0; u < DSUB; u += 4) {
@@ -1144,8 +1148,8 @@ __global__ void __launch_bounds__(256) build_tables_batch_kernel(const TableArgs
         float qv[DSUB];
 #pragma unroll
         for (int u = 0; u < DSUB; ++u) qv[u] = lut_s * qn[u];
+        const float scale = scale_n;
         if (q + 1 < q1) fetch(q + 1);
-        const float scale = __ldg(lut_scale + q);
         uint8_t* img = t.lut_img + (size_t)q * t.lut_bytes;
 #pragma unroll
         for (int i = 0; i < EPT; ++i) {
@@ -1264,7 +1268,7 @@ __global__ void __launch_bounds__(PT_THREADS) pair_tiles_kernel(const int32_t* _
     long long v = 0;
     if (p < npairs) {
         const int l = probe_list[p];
-        v = (offsets[l + 1] - offsets[l] + tile_vecs - 1) / tile_vecs + pair_lead(p, nprobe, lead);
+        v = tiles_of(offsets[l + 1] - offsets[l], tile_vecs) + pair_lead(p, nprobe, lead);
     }
     long long incl = v;
     for (int o = 1; o < 32; o <<= 1) {
