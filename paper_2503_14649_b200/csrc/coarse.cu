@@ -459,13 +459,12 @@ cudaError_t launch_tree_candidates(const IndexImpl* ix, const float* queries, in
 }
 
 // ---- per-query selection of the nprobe best lists ----------------------------------------------
-// sum (q-c)^2 (L2) or <q,c> of one query and centroid `row`, by one warp (d a multiple of 4), valid in every lane;
-// round_q: the query is rounded to bf16 first.  The row's loads of STEPS steps are in flight together (fp32: 512 values,
+// sum (q-c)^2 (L2) or <q,c> of one query (rounded to bf16 for bf16 centroids) and centroid `row`, by one warp (d a multiple
+// of 4), valid in every lane.  The row's loads of STEPS steps are in flight together (fp32: 512 values,
 // bf16: 1024): fetched one step at a time, a 768-dimensional row cost six memory round trips.  The order of the sum is
 // the plain loop's.
 template <bool BF16>
-__device__ __forceinline__ float warp_exact_score(const float* qrow, const void* C, uint32_t row, int d, int metric, bool round_q,
-                                                  int lane) {
+__device__ __forceinline__ float warp_exact_score(const float* qrow, const void* C, uint32_t row, int d, int metric, int lane) {
     constexpr int STEPS = BF16 ? 8 : 4;
     using Raw = typename std::conditional<BF16, uint2, float4>::type;  // four values as they lie in memory
     const Raw* src = reinterpret_cast<const Raw*>(static_cast<const uint8_t*>(C) + (size_t)row * d * (BF16 ? 2 : 4));
@@ -485,7 +484,7 @@ __device__ __forceinline__ float warp_exact_score(const float* qrow, const void*
             } else {
                 c = raw[u];
             }
-            if (BF16 && round_q) { q.x = round_bf16(q.x); q.y = round_bf16(q.y); q.z = round_bf16(q.z); q.w = round_bf16(q.w); }
+            if (BF16) { q.x = round_bf16(q.x); q.y = round_bf16(q.y); q.z = round_bf16(q.z); q.w = round_bf16(q.w); }
             if (metric == RAGO_L2) {
                 const float t0 = q.x - c.x, t1 = q.y - c.y, t2 = q.z - c.z, t3 = q.w - c.w;
                 acc = fmaf(t0, t0, fmaf(t1, t1, fmaf(t2, t2, fmaf(t3, t3, acc))));
@@ -773,7 +772,7 @@ __global__ void __launch_bounds__(SEL_THREADS) select_probes_kernel(
     const float* qrow = Q + (size_t)q * d;
     for (int i = warp; i < kept; i += SEL_THREADS / 32) {
         const uint32_t l = (uint32_t)(keys[i] & 0xFFFFFFFFull);
-        const float acc = warp_exact_score<BF16>(qrow, C, l, d, metric, BF16, lane);
+        const float acc = warp_exact_score<BF16>(qrow, C, l, d, metric, lane);
         if (lane == 0) keys2[i] = make_key(metric == RAGO_L2 ? acc : -acc, l);
     }
     __syncthreads();
@@ -793,7 +792,19 @@ __global__ void __launch_bounds__(SEL_THREADS) select_probes_kernel(
     if (BF16 && metric == RAGO_L2) {
         for (int i = warp; i < nprobe; i += SEL_THREADS / 32) {
             const uint32_t l = (uint32_t)(keys[i] & 0xFFFFFFFFull);
-            const float acc = warp_exact_score<BF16>(qrow, C, l, d, RAGO_L2, false, lane);
+            float acc = 0.f;
+            for (int jb = lane; jb < d; jb += 32 * 8) {  // eight loads of the row in flight
+                float c[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) c[u] = jb + 32 * u < d ? load_c<BF16>(C, (size_t)l * d + jb + 32 * u) : 0.f;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    if (jb + 32 * u >= d) continue;
+                    const float t = qrow[jb + 32 * u] - c[u];
+                    acc = fmaf(t, t, acc);
+                }
+            }
+            for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
             if (lane == 0) probe_bias[(size_t)q * nprobe + i] = acc;
         }
     }

@@ -235,8 +235,8 @@ __global__ void __launch_bounds__(THREADS) merge_kernel(
 // Small batches (latency): the same result by a shorter chain of dependent memory accesses.  A query's slots are
 // consecutive in memory, so the CTA's 1024 threads fetch ALL of their keys (at most KPT each) and the slot counts in
 // one round trip, keep them in registers, find a cut with between k and k + k/4 + 8 keys at or below it by a counting
-// bisection on the score words, then on whole keys if scores are equal (keys are distinct, so it always ends), and only the keys up to the cut go to shared memory to
-// be sorted.  The ids of the winners are fetched together with the values the cancellation check needs.
+// bisection on the score words, then on whole keys if scores are equal (keys are distinct, so it always ends), and only
+// the keys up to the cut go to shared memory to be sorted.  The ids of the winners are fetched together with the values the cancellation check needs.
 template <int KPT>
 __global__ void __launch_bounds__(1024) merge_small_kernel(
     const int64_t* __restrict__ work_prefix, const int64_t* __restrict__ ids, int npairs, int nprobe, int k, int ctas,
