@@ -278,6 +278,19 @@ rago_status rago_debug_set_gemm_pairing(int32_t mode);
 rago_status rago_selftest_wait_timeout(void* workspace, uint32_t max_polls, int32_t with_tmem, void* cuda_stream);
 
 /*
+ * Test hook (no counterpart in the paper): the final selection of rago_flat_search alone, over the caller's
+ * candidate lists.  A search never leaves lists like those a test wants to see: count words that no kernel wrote,
+ * or an order of scores that defeats the kernel's shortcuts.
+ *
+ *   counts    dev [nq][nlists] int32; a count outside [0, stride] is taken as the nearer of the two
+ *   entries   dev [nq][nlists][stride] uint64: low word the row number, high word the score's fp32 bits; row numbers
+ *             of one query are distinct
+ *   1 <= nlists <= 4096, 1 <= stride <= 4096, nq >= 1, 1 <= k <= 1024; outputs as rago_flat_search's
+ */
+rago_status rago_selftest_final_selection(int32_t* counts, uint64_t* entries, int32_t nlists, int32_t stride, int32_t nq, int32_t k,
+                                          int64_t* out_ids, float* out_scores, void* cuda_stream);
+
+/*
  * Which kernel computes the coarse scores: 0 = automatic (tensor cores for batches of more than 16
  * queries, the fp32 kernel for smaller ones), 1 = always the fp32 kernel, 2 = always tensor cores.
  * The tensor-core kernel multiplies bf16 operands; fp32 queries and centroids are split into three

@@ -27,7 +27,7 @@ STAGE_NAMES = ("coarse_scores", "probe_select", "plan", "table_scan", "merge")
 EXPORTS = ("rago_index_load", "rago_index_load_pq4", "rago_index_set_coarse_tree", "rago_index_free", "rago_search_workspace_bytes", "rago_search",
            "rago_search_probes", "rago_search_probes_noalloc", "rago_search_host", "rago_host_staging_bytes", "rago_flat_search",
            "rago_flat_workspace_bytes", "rago_check", "rago_set_coarse_mode", "rago_profile_enable", "rago_profile_read",
-           "rago_merge_results", "rago_selftest_wait_timeout", "rago_debug_set_gemm_pairing", "rago_kernel_launches", "rago_last_error")
+           "rago_merge_results", "rago_selftest_wait_timeout", "rago_selftest_final_selection", "rago_debug_set_gemm_pairing", "rago_kernel_launches", "rago_last_error")
 
 
 class RagoError(RuntimeError):
@@ -61,6 +61,7 @@ def lib() -> ctypes.CDLL:
         L.rago_merge_results.argtypes = [vp, vp, i32, i64, i32, i32, i32, i32, vp, vp, vp]
         L.rago_check.argtypes = [vp, vp]
         L.rago_selftest_wait_timeout.argtypes = [vp, ctypes.c_uint32, i32, vp]
+        L.rago_selftest_final_selection.argtypes = [vp, vp, i32, i32, i32, i32, vp, vp, vp]
         L.rago_debug_set_gemm_pairing.argtypes = [i32]
         L.rago_set_coarse_mode.argtypes = [vp, i32]
         L.rago_profile_enable.argtypes = [vp, i32]
@@ -231,6 +232,16 @@ def rago_debug_set_gemm_pairing(mode: int):
 def rago_selftest_wait_timeout(workspace: torch.Tensor, max_polls: int, with_tmem: bool):
     """Launch the bounded-wait self-test on `workspace` (see rago.h); follow with rago_check(workspace)."""
     _check(lib().rago_selftest_wait_timeout(_ptr(workspace), int(max_polls), int(bool(with_tmem)), _stream()))
+
+
+def rago_selftest_final_selection(counts: torch.Tensor, entries: torch.Tensor, k: int):
+    """Flat search's final selection over counts int32 [nq, nlists] and entries int64 [nq, nlists, stride] (see rago.h)."""
+    nq, nlists, stride = entries.shape
+    out_ids = torch.empty((nq, k), dtype=torch.int64, device=entries.device)
+    out_scores = torch.empty((nq, k), dtype=torch.float32, device=entries.device)
+    _check(lib().rago_selftest_final_selection(_ptr(counts), _ptr(entries), nlists, stride, nq, k, _ptr(out_ids),
+                                               _ptr(out_scores), _stream()))
+    return out_ids, out_scores
 
 
 def rago_check(workspace: torch.Tensor):

@@ -596,6 +596,15 @@ rago_status rago_selftest_wait_timeout(void* workspace, uint32_t max_polls, int3
     return RAGO_OK;
 }
 
+rago_status rago_selftest_final_selection(int32_t* counts, uint64_t* entries, int32_t nlists, int32_t stride, int32_t nq, int32_t k,
+                                          int64_t* out_ids, float* out_scores, void* cuda_stream) {
+    if (!counts || !entries || !out_ids || !out_scores) return fail(RAGO_EINVAL, "null pointer");
+    if (nlists < 1 || nlists > 4096 || stride < 1 || stride > 4096 || nq < 1 || k < 1 || k > MAX_K) return fail(RAGO_EINVAL, "bad sizes");
+    const cudaError_t e = launch_selftest_final_selection(counts, reinterpret_cast<unsigned long long*>(entries), nlists, stride, nq, k,
+                                                          out_ids, out_scores, static_cast<cudaStream_t>(cuda_stream));
+    return e != cudaSuccess ? cuda_fail(e, "final selection") : RAGO_OK;
+}
+
 rago_status rago_set_coarse_mode(rago_index* index, int32_t mode) {
     if (!index) return fail(RAGO_EINVAL, "index is null");
     if (mode < 0 || mode > 2) return fail(RAGO_EINVAL, "mode = %d: 0 auto, 1 fp32 pipes, 2 tensor cores", mode);

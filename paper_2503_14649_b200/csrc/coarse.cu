@@ -548,7 +548,7 @@ __global__ void __launch_bounds__(SEL_THREADS) select_probes_kernel(
     const float* srow = FROM_SCORES ? scores + (size_t)q * nlist : nullptr;
     if (!FROM_SCORES) {  // the valid entries of the query's lists, numbered consecutively
         // the counts are fetched side by side (one thread reading them in turn paid a global round trip per list)
-        for (int sp = tid; sp < nsplit; sp += SEL_THREADS) pre[sp + 1] = cand_cnt[(size_t)q * nsplit + sp];
+        for (int sp = tid; sp < nsplit; sp += SEL_THREADS) pre[sp + 1] = list_count(cand_cnt[(size_t)q * nsplit + sp], cap);
         __syncthreads();
         if (warp == 0) {  // running sum of the counts, in place: 32 of them at a time (one thread took 10 ns for each)
             int carry = 0;

@@ -252,6 +252,8 @@ __host__ __device__ inline uint32_t gemm_cand_sign(float alpha, const float* col
 __host__ __device__ inline unsigned long long cand_key(unsigned long long entry, uint32_t sign) {
     return ((unsigned long long)ord_bits((uint32_t)(entry >> 32) ^ sign) << 32) | (uint32_t)entry;
 }
+// Entries a reader takes from a candidate list, whatever its count word holds.
+__host__ __device__ inline int list_count(int32_t written, int cap) { return written < 0 ? 0 : (written < cap ? written : cap); }
 cudaError_t gemm_select_init();
 cudaError_t make_tmap_bf16(void* out_map, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows,
                            uint64_t row_stride = 0);
@@ -290,6 +292,8 @@ cudaError_t launch_merge(const IndexImpl* ix, const int64_t* work_prefix, int nq
                          float* out_dists, cudaStream_t s);
 // flat.cu
 size_t flat_workspace_bytes(int64_t N, int d, int nq, int k);
+cudaError_t launch_selftest_final_selection(int32_t* counts, unsigned long long* entries, int nlists, int stride, int nq, int k,
+                                            int64_t* out_ids, float* out_scores, cudaStream_t s);
 cudaError_t launch_flat_search(const void* db, int64_t N, int d, const void* queries, int nq, int k, int64_t* out_ids,
                                float* out_scores, void* workspace, cudaStream_t s);
 

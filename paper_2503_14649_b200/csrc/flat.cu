@@ -151,7 +151,7 @@ __device__ __forceinline__ void flat_merge_lists(FlatMergeState& S, const int32_
     for (int g0 = l0; g0 < l1; g0 += FM_LISTS) {
         const int ng = l1 - g0 < FM_LISTS ? l1 - g0 : FM_LISTS;
         {   // exclusive prefix of the counts (FM_LISTS <= FM_THREADS: one list per thread)
-            const int c = tid < ng ? __ldcg(cnts + slot_of(g0 + tid)) : 0;
+            const int c = tid < ng ? list_count(__ldcg(cnts + slot_of(g0 + tid)), stride) : 0;
             int incl = c;
             for (int o = 1; o < 32; o <<= 1) {
                 const int y = __shfl_up_sync(0xffffffffu, incl, o);
@@ -496,6 +496,15 @@ cudaError_t launch_flat_search(const void* db, int64_t N, int d, const void* que
         if (e != cudaSuccess) return e;
     }
     flat_merge_kernel<<<nq, FM_THREADS, 0, s>>>(nchunks, 1, k, k, 0, 0u, slot_cnt, slot_keys, nullptr, out_ids, out_scores);
+    count_launch();
+    return cudaGetLastError();
+}
+
+// The final selection alone, over the caller's raw lists (test hook).
+cudaError_t launch_selftest_final_selection(int32_t* counts, unsigned long long* entries, int nlists, int stride, int nq, int k,
+                                            int64_t* out_ids, float* out_scores, cudaStream_t s) {
+    flat_merge_kernel<<<nq, FM_THREADS, 0, s>>>(nlists, 1, k, stride, 1, gemm_cand_sign(-1.f, nullptr), counts, entries, nullptr,
+                                                out_ids, out_scores);
     count_launch();
     return cudaGetLastError();
 }

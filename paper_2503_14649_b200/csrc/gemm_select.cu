@@ -562,7 +562,8 @@ gemm_select_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                 else mbar_arrive(tempty_bar(buf));
             }
         }
-        if (a.mode == 0 && !dead) {
+        // also after an expired wait: the readers of the lists must not find an earlier call's counts
+        if (a.mode == 0) {
 #pragma unroll
             for (int g = 0; g < 2; ++g) {
                 const int r = (m0 + g) * GBM + q4 * 32 + lane;

@@ -1,0 +1,48 @@
+"""Flat search's final selection alone, over lists that a search does not leave in a test."""
+
+import pytest
+import torch
+
+from paper_2503_14649_b200 import binding
+
+pytestmark = pytest.mark.gpu
+
+
+def _lists(scores):
+    """Raw entries [nq, nlists, stride] over scores of that shape; row numbers follow the storage order."""
+    nq, nlists, stride = scores.shape
+    rows = torch.arange(nlists * stride, dtype=torch.int64, device=scores.device).view(1, nlists, stride).expand(nq, -1, -1)
+    return (scores.contiguous().view(torch.int32).long() << 32) | rows
+
+
+def _check(scores, counts, k):
+    """The k best of the entries below each list's count, equal scores by row number."""
+    nq, nlists, stride = scores.shape
+    ids, got = binding.rago_selftest_final_selection(counts, _lists(scores).contiguous(), k)
+    torch.cuda.synchronize()
+    taken = torch.arange(stride, device=scores.device).view(1, 1, -1) < counts.clamp(0, stride).unsqueeze(2)
+    flat = torch.where(taken, scores, torch.full_like(scores, -float("inf"))).view(nq, -1)
+    want, rows = flat.sort(dim=1, descending=True, stable=True)
+    m = min(k, flat.shape[1])
+    valid = torch.arange(m, device=scores.device).view(1, -1) < taken.view(nq, -1).sum(1, keepdim=True)
+    assert torch.equal(got[:, :m], want[:, :m])
+    assert torch.equal(ids[:, :m], torch.where(valid, rows[:, :m], torch.full_like(rows[:, :m], -1)))
+    assert bool((ids[:, m:] == -1).all()) and bool(torch.isneginf(got[:, m:]).all())
+
+
+def _normal(*shape, seed):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    return torch.randn(*shape, generator=g, device="cuda")
+
+
+# An expired wait ends a search with an error word, and the readers of its lists must stay inside them whatever the
+# count words hold (a search that reads past its lists would take the GPU's context down instead).
+@pytest.mark.parametrize("nlists,stride,k", [(1, 512, 10), (296, 512, 100), (600, 40, 300), (3, 1024, 1024)])
+def test_count_words_that_no_kernel_wrote_stay_inside_the_lists(nlists, stride, k):
+    scores = _normal(4, nlists, stride, seed=nlists)
+    counts = torch.randint(0, stride + 1, (4, nlists), dtype=torch.int32, device="cuda")
+    for i, v in enumerate((-1, -(2 ** 31), 2 ** 31 - 1, stride + 1, 0x7F7F7F7F, 0)):
+        counts.view(-1)[i::7] = v
+    counts[3] = -5
+    _check(scores, counts, k)
