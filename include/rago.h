@@ -155,6 +155,8 @@ rago_status rago_search_workspace_bytes(const rago_index* index, int32_t nq, int
  *
  * With a RAGO_BF16 coarse quantiser the query is rounded to bf16 (nearest-even) for the coarse
  * step only; tables are built from the fp32 query.  Ties are broken by storage position.
+ * A query with NaN or infinite values (or values whose products overflow) is answered with lists and results that
+ * mean nothing; the other queries of the batch are not affected.
  * nq == 0 is a no-op.
  *
  * Accuracy of out_dists (fp32).  Candidates are RANKED by an expanded form of the score,

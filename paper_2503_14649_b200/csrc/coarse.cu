@@ -767,7 +767,24 @@ __global__ void __launch_bounds__(SEL_THREADS) select_probes_kernel(
         }
     }
     __syncthreads();
-    const int kept = block_select_short(keys, &cnt, nsel, tid, SEL_THREADS, sync);
+    int kept = block_select_short(keys, &cnt, nsel, tid, SEL_THREADS, sync);
+    // A NaN score is not selected, and candidate lists hold nothing that does not lie below +inf: a query with such
+    // scores has fewer lists than it probes.  The smallest list numbers it does not hold yet stand in, which is what a
+    // row of equal scores gives, so that every list number handed on is one of the index.
+    if (kept < nprobe) {  // uniform
+        for (int l = tid; l < nprobe; l += SEL_THREADS) {
+            int below_l = 0;
+            bool held = false;
+            for (int i = 0; i < kept; ++i) {
+                const int o = (int)(uint32_t)keys[i];
+                below_l += o < l ? 1 : 0;
+                held = held || o == l;
+            }
+            if (!held && l - below_l < nprobe - kept) keys[kept + l - below_l] = (unsigned long long)l;
+        }
+        __syncthreads();
+        kept = nprobe;
+    }
     // exact re-score of the survivors, one warp per candidate
     const float* qrow = Q + (size_t)q * d;
     for (int i = warp; i < kept; i += SEL_THREADS / 32) {
