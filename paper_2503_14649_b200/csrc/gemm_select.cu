@@ -407,17 +407,20 @@ gemm_select_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         fence_barrier_init();
         fence_proxy_async();
     }
+    // Everything above touched shared memory only and overlaps the kernel before this one.
+    grid_dependency_wait();
+    grid_dependents_may_launch();  // none of this library's kernels that follow takes tensor memory
+    // Tensor memory is taken after the wait.  The kernel in front may be a caller's that lets its successor start and only
+    // then allocates, with so little shared memory that a CTA of both fits an SM: holding all columns while waiting for it to
+    // end, when it waits for columns, would stop both for good.
     if (warp == 0) {
         if (TWO) tmem_alloc_pair(smem_u32(tmem_slot), G_TMEM_COLS); else tmem_alloc(smem_u32(tmem_slot), G_TMEM_COLS);
     }
     tc_fence_before();
     __syncthreads();
-    if (TWO) cluster_sync_all();  // the peer's barriers exist before anything of ours is aimed at them
+    if (TWO) cluster_sync_all();  // the peer's barriers and tensor memory exist before anything of ours is aimed at them
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    // Everything above touched shared and tensor memory only and overlaps the kernel before this one.
-    grid_dependency_wait();
-    grid_dependents_may_launch();
     // error block of the search: nothing reports to it for the first second (the limit of a wait)
     if (a.clear_block != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && tid < 64) a.clear_block[tid] = 0u;
 
