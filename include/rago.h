@@ -264,6 +264,17 @@ rago_status rago_check(void* workspace, void* cuda_stream);
 rago_status rago_debug_set_gemm_pairing(int32_t mode);
 
 /*
+ * Test hook (no counterpart in the paper): which way a search of these sizes goes, so that a test or a measurement
+ * that means a certain path can say so.  Launches nothing.  out receives RAGO_PLAN_WORDS words:
+ *   0  coarse step: fp32 kernel, tensor-core score matrix, tensor-core candidate lists, or two-level lists
+ *   1  candidate lists per query, 2 their capacity, 3 lists sampled by the pilot pass (0: none)
+ *   4  1 if the kernel behind the tensor-core launch is scheduled while that runs
+ */
+#define RAGO_PLAN_WORDS 5
+enum { RAGO_PLAN_FP32 = 0, RAGO_PLAN_MATRIX = 1, RAGO_PLAN_LISTS = 2, RAGO_PLAN_TREE = 3 };
+rago_status rago_debug_search_plan(const rago_index* index, int32_t nq, int32_t nprobe, int32_t k, int32_t* out);
+
+/*
  * Test hook for the failure path of rago_check (no counterpart in the paper: the library's kernels wait on
  * copies and on the tensor pipe, every such wait is bounded, and this call lets a test see a bound expire
  * without anything being wrong).  Launches one small kernel in which a wait on a barrier that nothing signals

@@ -22,12 +22,14 @@ STATUS_NAMES = {0: "RAGO_OK", 1: "RAGO_EINVAL", 2: "RAGO_EALIGN", 3: "RAGO_EUNSU
 RAGO_L2, RAGO_IP = 0, 1
 RAGO_F32, RAGO_BF16 = 0, 1
 NUM_STAGES = 5
+PLAN_NAMES = ("route", "lists", "cap", "pilot_cols", "early_successor")
+PLAN_ROUTES = ("fp32", "matrix", "lists", "tree")
 STAGE_NAMES = ("coarse_scores", "probe_select", "plan", "table_scan", "merge")
 
 EXPORTS = ("rago_index_load", "rago_index_load_pq4", "rago_index_set_coarse_tree", "rago_index_free", "rago_search_workspace_bytes", "rago_search",
            "rago_search_probes", "rago_search_probes_noalloc", "rago_search_host", "rago_host_staging_bytes", "rago_flat_search",
            "rago_flat_workspace_bytes", "rago_check", "rago_set_coarse_mode", "rago_profile_enable", "rago_profile_read",
-           "rago_merge_results", "rago_selftest_wait_timeout", "rago_selftest_final_selection", "rago_debug_set_gemm_pairing", "rago_kernel_launches", "rago_last_error")
+           "rago_merge_results", "rago_selftest_wait_timeout", "rago_selftest_final_selection", "rago_debug_set_gemm_pairing", "rago_debug_search_plan", "rago_kernel_launches", "rago_last_error")
 
 
 class RagoError(RuntimeError):
@@ -63,6 +65,7 @@ def lib() -> ctypes.CDLL:
         L.rago_selftest_wait_timeout.argtypes = [vp, ctypes.c_uint32, i32, vp]
         L.rago_selftest_final_selection.argtypes = [vp, vp, i32, i32, i32, i32, vp, vp, vp]
         L.rago_debug_set_gemm_pairing.argtypes = [i32]
+        L.rago_debug_search_plan.argtypes = [vp, i32, i32, i32, vp]
         L.rago_set_coarse_mode.argtypes = [vp, i32]
         L.rago_profile_enable.argtypes = [vp, i32]
         L.rago_profile_read.argtypes = [vp, ctypes.POINTER(ctypes.c_float)]
@@ -202,6 +205,13 @@ class Index:
                                                     _stream()))
             self._tree = (level1, child_offsets)
         self._ws = None  # workspace sizes depend on it
+
+    def rago_debug_search_plan(self, nq: int, nprobe: int, k: int) -> dict:
+        """Which way a search of these sizes goes (see rago.h); "route" is one of PLAN_ROUTES."""
+        out = (ctypes.c_int32 * len(PLAN_NAMES))()
+        _check(lib().rago_debug_search_plan(self._h, nq, nprobe, k, out))
+        plan = dict(zip(PLAN_NAMES, out))
+        return dict(plan, route=PLAN_ROUTES[plan["route"]])
 
     def rago_profile_enable(self, enable: bool = True):
         _check(lib().rago_profile_enable(self._h, int(enable)))

@@ -584,6 +584,21 @@ rago_status rago_debug_set_gemm_pairing(int32_t mode) {
     return RAGO_OK;
 }
 
+rago_status rago_debug_search_plan(const rago_index* index, int32_t nq, int32_t nprobe, int32_t k, int32_t* out) {
+    const IndexImpl* ix = reinterpret_cast<const IndexImpl*>(index);
+    const rago_status st = check_search_args(ix, nq, nprobe, k);
+    if (st != RAGO_OK) return st;
+    if (!out) return fail(RAGO_EINVAL, "out is null");
+    const Layout L = make_layout(ix, nq, nprobe, k);
+    const bool lists = L.tree_S || (L.tc && L.tc_mode == 0);
+    out[0] = L.tree_S ? RAGO_PLAN_TREE : (!L.tc ? RAGO_PLAN_FP32 : (lists ? RAGO_PLAN_LISTS : RAGO_PLAN_MATRIX));
+    out[1] = L.tree_S ? L.tree_S : (lists ? L.tc_nsplit * GEMM_COL_HALVES : 0);
+    out[2] = L.tree_S ? L.tree_cap : (lists ? L.tc_cap : 0);
+    out[3] = L.pilot_cols;
+    out[4] = L.tc && gemm_early_successor(nq, L.tc_mg, L.tc_nsplit) ? 1 : 0;
+    return RAGO_OK;
+}
+
 rago_status rago_selftest_wait_timeout(void* workspace, uint32_t max_polls, int32_t with_tmem, void* cuda_stream) {
     if (!workspace) return fail(RAGO_EINVAL, "workspace is null");
     if (!aligned(workspace, 256)) return fail(RAGO_EALIGN, "workspace needs 256-byte alignment");

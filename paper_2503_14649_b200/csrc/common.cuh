@@ -263,6 +263,7 @@ cudaError_t launch_row_tau(const float* scores, int nrows, int n, int nsel, floa
 int gemm_cand_cap(int nsel);  // 0: nsel too large for the fused selection
 void gemm_grid(int nrows, int64_t ncols, int d, int num_sms, int* mg, int* nsplit, int* mgroups);
 void gemm_set_pairing(int mode);
+bool gemm_early_successor(int nrows, int mg, int nsplit);  // the kernel behind is scheduled while the launch runs
 cudaError_t launch_gemm_select(const GemmLaunch& L, cudaStream_t s);
 cudaError_t launch_split_bf16(const float* x, size_t n, int parts, void* out, uint32_t* clear_block, cudaStream_t s);
 cudaError_t launch_selftest_wait(uint32_t* err_word, uint32_t max_polls, int with_tmem, uint32_t* observed, cudaStream_t s);

@@ -218,6 +218,7 @@ struct GemmArgs {
     float* scores;               // [nrows][ncols] (mode 1)
     uint32_t* err;
     uint32_t* clear_block;       // 64 words this launch zeroes (the first kernel of a search), or null
+    int early_successor;         // the kernel behind may be scheduled while this one runs
 };
 
 // Cut one list of n (> nsel) keys down to between nsel and nkeep keys and return the new threshold.
@@ -409,7 +410,7 @@ gemm_select_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     }
     // Everything above touched shared memory only and overlaps the kernel before this one.
     grid_dependency_wait();
-    grid_dependents_may_launch();  // none of this library's kernels that follow takes tensor memory
+    if (a.early_successor) grid_dependents_may_launch();  // none of this library's kernels that follow takes tensor memory
     // Tensor memory is taken after the wait.  The kernel in front may be a caller's that lets its successor start and only
     // then allocates, with so little shared memory that a CTA of both fits an SM: holding all columns while waiting for it to
     // end, when it waits for columns, would stop both for good.
@@ -672,6 +673,16 @@ void gemm_grid(int nrows, int64_t ncols, int d, int num_sms, int* mg, int* nspli
 }
 
 
+// A launch of at most half as many CTAs as there are SMs lets the kernel behind start early: its CTAs wait on idle SMs.  Behind
+// a launch that fills the GPU they would be packed onto the SMs whose CTA ends first, and a selection of about one CTA per
+// SM then runs two or three to an SM.  us per call, early / not: 100 queries, 200 of 65 536 lists (bf16, d = 256)
+// 124 / 105, flat 33 queries over 100 000 rows, k = 100 331 / 249, 1 query 35 / 31; for 17 queries over 300 to 18 000 lists (2 to
+// 71 CTAs), where it stays, 38 / 42 to 37.4 / 38.7.
+bool gemm_early_successor(int nrows, int mg, int nsplit) {
+    const int mtiles = (nrows + GBM - 1) / GBM;
+    return (mg == 1 ? mtiles * nsplit : (mtiles + 1) / 2 * nsplit * (mg == 3 ? 2 : 1)) <= 74;
+}
+
 cudaError_t launch_gemm_select(const GemmLaunch& L, cudaStream_t s) {
     GemmArgs a;
     a.nrows = L.nrows; a.ncols = (int)L.ncols;
@@ -694,6 +705,7 @@ cudaError_t launch_gemm_select(const GemmLaunch& L, cudaStream_t s) {
     cfg.blockDim = dim3(G_THREADS);
     cfg.dynamicSmemBytes = G_SMEM_BYTES;
     cfg.stream = s;
+    a.early_successor = gemm_early_successor(L.nrows, L.mg, L.nsplit) ? 1 : 0;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
