@@ -5,7 +5,6 @@
 // before the final cut, so the probe order follows the plain definition up to fp32 rounding.
 // With a bf16 coarse quantiser the query is rounded to bf16 first (coarse step only).
 #include <cstring>
-#include <type_traits>
 
 #include "plan.cuh"
 #include "topk.cuh"
@@ -460,37 +459,41 @@ cudaError_t launch_tree_candidates(const IndexImpl* ix, const float* queries, in
 
 // ---- per-query selection of the nprobe best lists ----------------------------------------------
 // sum (q-c)^2 (L2) or <q,c> of one query (rounded to bf16 for bf16 centroids) and centroid `row`, by one warp (d a multiple
-// of 4), valid in every lane.  The row's loads of STEPS steps are in flight together (fp32: 512 values,
-// bf16: 1024): fetched one step at a time, a 768-dimensional row cost six memory round trips.  The order of the sum is
-// the plain loop's.
+// of 4), valid in every lane; the order of the sum is the same in both forms.  fp32: the row's loads of four steps (512
+// values) are in flight together; fetched one step at a time, a 768-dimensional row cost six memory round trips.  bf16: the
+// plain loop, which the compiler unrolls by four; with eight guarded steps in flight the code around the few bytes of a
+// short row, or of many rows, cost more than the round trips (300 queries, 200 of 16 384 lists, d = 1024: 229 us against 182).
 template <bool BF16>
 __device__ __forceinline__ float warp_exact_score(const float* qrow, const void* C, uint32_t row, int d, int metric, int lane) {
-    constexpr int STEPS = BF16 ? 8 : 4;
-    using Raw = typename std::conditional<BF16, uint2, float4>::type;  // four values as they lie in memory
-    const Raw* src = reinterpret_cast<const Raw*>(static_cast<const uint8_t*>(C) + (size_t)row * d * (BF16 ? 2 : 4));
     float acc = 0.f;
-    for (int jb = lane * 4; jb < d; jb += 128 * STEPS) {
-        Raw raw[STEPS];
+    auto add = [&](float4 q, float4 c) {
+        if (metric == RAGO_L2) {
+            const float t0 = q.x - c.x, t1 = q.y - c.y, t2 = q.z - c.z, t3 = q.w - c.w;
+            acc = fmaf(t0, t0, fmaf(t1, t1, fmaf(t2, t2, fmaf(t3, t3, acc))));
+        } else {
+            acc = fmaf(q.x, c.x, fmaf(q.y, c.y, fmaf(q.z, c.z, fmaf(q.w, c.w, acc))));
+        }
+    };
+    if constexpr (BF16) {
+        for (int j = lane * 4; j < d; j += 128) {  // 8-byte loads
+            float4 q = *reinterpret_cast<const float4*>(qrow + j), c;
+            q.x = round_bf16(q.x); q.y = round_bf16(q.y); q.z = round_bf16(q.z); q.w = round_bf16(q.w);
+            const uint2 raw = *reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(C) + (size_t)row * d + j);
+            c.x = __uint_as_float(raw.x << 16); c.y = __uint_as_float(raw.x & 0xFFFF0000u);
+            c.z = __uint_as_float(raw.y << 16); c.w = __uint_as_float(raw.y & 0xFFFF0000u);
+            add(q, c);
+        }
+    } else {
+        constexpr int STEPS = 4;
+        const float4* src = reinterpret_cast<const float4*>(static_cast<const float*>(C) + (size_t)row * d);
+        for (int jb = lane * 4; jb < d; jb += 128 * STEPS) {
+            float4 c[STEPS];
 #pragma unroll
-        for (int u = 0; u < STEPS; ++u)
-            if (jb + u * 128 < d) raw[u] = __ldg(src + ((jb + u * 128) >> 2));
+            for (int u = 0; u < STEPS; ++u)
+                if (jb + u * 128 < d) c[u] = __ldg(src + ((jb + u * 128) >> 2));
 #pragma unroll
-        for (int u = 0; u < STEPS; ++u) {
-            if (jb + u * 128 >= d) continue;
-            float4 q = *reinterpret_cast<const float4*>(qrow + jb + u * 128), c;
-            if constexpr (BF16) {
-                c.x = __uint_as_float(raw[u].x << 16); c.y = __uint_as_float(raw[u].x & 0xFFFF0000u);
-                c.z = __uint_as_float(raw[u].y << 16); c.w = __uint_as_float(raw[u].y & 0xFFFF0000u);
-            } else {
-                c = raw[u];
-            }
-            if (BF16) { q.x = round_bf16(q.x); q.y = round_bf16(q.y); q.z = round_bf16(q.z); q.w = round_bf16(q.w); }
-            if (metric == RAGO_L2) {
-                const float t0 = q.x - c.x, t1 = q.y - c.y, t2 = q.z - c.z, t3 = q.w - c.w;
-                acc = fmaf(t0, t0, fmaf(t1, t1, fmaf(t2, t2, fmaf(t3, t3, acc))));
-            } else {
-                acc = fmaf(q.x, c.x, fmaf(q.y, c.y, fmaf(q.z, c.z, fmaf(q.w, c.w, acc))));
-            }
+            for (int u = 0; u < STEPS; ++u)
+                if (jb + u * 128 < d) add(*reinterpret_cast<const float4*>(qrow + jb + u * 128), c[u]);
         }
     }
     for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -810,16 +813,9 @@ __global__ void __launch_bounds__(SEL_THREADS) select_probes_kernel(
         for (int i = warp; i < nprobe; i += SEL_THREADS / 32) {
             const uint32_t l = (uint32_t)(keys[i] & 0xFFFFFFFFull);
             float acc = 0.f;
-            for (int jb = lane; jb < d; jb += 32 * 8) {  // eight loads of the row in flight
-                float c[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) c[u] = jb + 32 * u < d ? load_c<BF16>(C, (size_t)l * d + jb + 32 * u) : 0.f;
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    if (jb + 32 * u >= d) continue;
-                    const float t = qrow[jb + 32 * u] - c[u];
-                    acc = fmaf(t, t, acc);
-                }
+            for (int j = lane; j < d; j += 32) {
+                const float t = qrow[j] - load_c<BF16>(C, (size_t)l * d + j);
+                acc = fmaf(t, t, acc);
             }
             for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
             if (lane == 0) probe_bias[(size_t)q * nprobe + i] = acc;
