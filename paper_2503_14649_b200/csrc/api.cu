@@ -91,9 +91,7 @@ static Layout make_layout(const IndexImpl* ix, int nq, int nprobe, int k) {
         gemm_grid(nq, ix->nlist, ix->d * ix->cparts_n, ix->num_sms, &L.tc_mg, &L.tc_nsplit, &mgroups);
         L.tc_cap = gemm_cand_cap(nsel);
         L.qparts = take((size_t)ix->cparts_n * nq * ix->d * 2);
-        // a pilot pass pays off when a CTA sees many column tiles per row and the sample can hold nsel values
-        const int np = ix->pilot_stride ? ix->nlist / ix->pilot_stride : 0;
-        const bool pilot = np >= 4 * nsel && ix->nlist >= 8192;
+        const int pilot = coarse_pilot_cols(ix, nprobe);
         // Lists that would keep every score (no starting thresholds, no more columns per list than it holds) only spread
         // them: the score matrix is half the bytes in 16-byte stores, and the selection reads it in order.
         const int tiles = (ix->nlist + 255) / 256, per_list = (tiles + L.tc_nsplit - 1) / L.tc_nsplit * (256 / GEMM_COL_HALVES);
@@ -102,8 +100,8 @@ static Layout make_layout(const IndexImpl* ix, int nq, int nprobe, int k) {
             L.cand = take((size_t)nq * L.tc_nsplit * GEMM_COL_HALVES * L.tc_cap * 8);
             L.cand_cnt = take((size_t)nq * L.tc_nsplit * GEMM_COL_HALVES * 4);
             if (pilot) {
-                L.pilot_cols = np;
-                L.pilot_scores = take((size_t)nq * np * 4);
+                L.pilot_cols = pilot;
+                L.pilot_scores = take((size_t)nq * pilot * 4);
                 L.row_tau = take((size_t)nq * 4);
             }
         }

@@ -873,8 +873,7 @@ static void launch_select_source(const IndexImpl* ix, const float* queries, cons
                                  int nprobe, int32_t* probe_list, float* probe_term, float* probe_bias, const FusedPlan& fp, cudaStream_t s) {
     const dim3 grid(fp.enabled ? nq * (1 + fp.table_parts) : nq);
     const size_t smem = fp.enabled ? (size_t)(ix->d + ix->M) * 4 : 0;
-    const bool pilot = ix->pilot_stride && ix->nlist >= 8192 && ix->nlist / ix->pilot_stride >= 4 * (nprobe + PROBE_GUARD);
-    const int most = ix->tree_n1 ? ix->tree_max_cand : (pilot ? 20 * (nprobe + PROBE_GUARD) : ix->nlist);  // items of a query, usually
+    const int most = ix->tree_n1 ? ix->tree_max_cand : (coarse_pilot_cols(ix, nprobe) ? 20 * (nprobe + PROBE_GUARD) : ix->nlist);  // items of a query, usually
     const bool few = most <= THREADS * REG_LISTS;
     if (scores && ix->nlist <= THREADS * REG)
         launch_overlapped(select_probes_kernel<BF16, THREADS, REG, true, true>, grid, dim3(THREADS), smem, s,

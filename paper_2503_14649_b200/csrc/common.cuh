@@ -227,6 +227,14 @@ cudaError_t launch_coarse_scores(const IndexImpl* ix, const float* queries, int 
 cudaError_t launch_tree_candidates(const IndexImpl* ix, const float* queries, int nq, int S, int cap,
                                    unsigned long long* cand, int32_t* cand_cnt, uint32_t* clear_block, cudaStream_t s);
 constexpr int TREE_LIMIT_B1 = 64, TREE_LIMIT_N1 = 4096;
+// Lists the pilot pass of the tensor-core coarse step samples, 0: no pass.  It pays off when a CTA sees many column tiles
+// per row and the sample can hold the wanted values.
+inline int coarse_pilot_cols(const IndexImpl* ix, int nprobe) {
+    int nsel = nprobe + PROBE_GUARD;
+    if (nsel > ix->nlist) nsel = ix->nlist;
+    const int np = ix->pilot_stride ? ix->nlist / ix->pilot_stride : 0;
+    return np >= 4 * nsel && ix->nlist >= 8192 ? np : 0;
+}
 // gemm_select.cu
 constexpr int GEMM_CAP_SMALL = 512, GEMM_CAP_LARGE = 1024;  // candidate-list capacities (keys per list)
 constexpr int GEMM_COL_HALVES = 2;  // a row has one candidate list per share of the grid AND per half of a 256-column tile

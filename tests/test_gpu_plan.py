@@ -25,3 +25,11 @@ def test_only_a_launch_that_leaves_sms_idle_lets_its_successor_start(nlist, nq, 
     ix = _index(nlist)
     assert ix.rago_debug_search_plan(nq, 32, 10)["early_successor"] == early
     ix.close()
+
+
+# The sample is every 16th list of at least 8192 and holds four times the wanted lists; lists hold at most 960 wanted ones.
+@pytest.mark.parametrize("nlist,nprobe,cols", [(8192, 120, 512), (8192, 121, 0), (8176, 8, 0), (8193, 8, 0), (65_536, 952, 4096), (65_536, 953, 0)])
+def test_pilot_pass(nlist, nprobe, cols):
+    ix = _index(nlist)
+    assert ix.rago_debug_search_plan(100, nprobe, 10)["pilot_cols"] == cols
+    ix.close()
