@@ -269,8 +269,10 @@ rago_status rago_debug_set_gemm_pairing(int32_t mode);
  *   0  coarse step: fp32 kernel, tensor-core score matrix, tensor-core candidate lists, or two-level lists
  *   1  candidate lists per query, 2 their capacity, 3 lists sampled by the pilot pass (0: none)
  *   4  1 if the kernel behind the tensor-core launch is scheduled while that runs
+ *   5  entries of a query's candidate lists that its selection holds in registers; 6 where the lists' counts
+ *      (int32 [nq][lists]) lie in the workspace of the call, in units of 256 bytes
  */
-#define RAGO_PLAN_WORDS 5
+#define RAGO_PLAN_WORDS 7
 enum { RAGO_PLAN_FP32 = 0, RAGO_PLAN_MATRIX = 1, RAGO_PLAN_LISTS = 2, RAGO_PLAN_TREE = 3 };
 rago_status rago_debug_search_plan(const rago_index* index, int32_t nq, int32_t nprobe, int32_t k, int32_t* out);
 

@@ -593,6 +593,8 @@ rago_status rago_debug_search_plan(const rago_index* index, int32_t nq, int32_t 
     out[1] = L.tree_S ? L.tree_S : (lists ? L.tc_nsplit * GEMM_COL_HALVES : 0);
     out[2] = L.tree_S ? L.tree_cap : (lists ? L.tc_cap : 0);
     out[3] = L.pilot_cols;
+    out[5] = lists ? select_list_slots(ix, nq, nprobe) : 0;
+    out[6] = lists ? (int32_t)(L.cand_cnt / 256) : 0;
     out[4] = L.tc && gemm_early_successor(nq, L.tc_mg, L.tc_nsplit) ? 1 : 0;
     return RAGO_OK;
 }

@@ -865,16 +865,33 @@ __global__ void __launch_bounds__(SEL_THREADS) select_probes_kernel(
 }
 
 // Registers per thread for the items of candidate lists: every slot is a copy of the look-up that the CTA has to fetch, so
-// only large selections (behind pilot thresholds the lists hold some 16 to 20 times the wanted items) take as many as a score
-// row does.
+// a selection takes few of them where its items fit (12 instead of 20: 3000 queries, 64 of 8192 lists 218 us against
+// 232; 4 instead of 16: 64 queries, 96 of 65 536 lists 70 against 73), and as many as a score row does where they do not (the
+// re-reading path; 100 queries, 120 of 65 536 lists: 105 us against 78).  Items of a query, measured over 8192 to 262 144 lists
+// and 8 to 200 probes: behind a pilot row of at most 4096 samples, whose threshold is the largest of its warps', 24 to 40
+// times the wanted ones in the mean and at most about 1200 + 30 times; behind a longer one 18 times, at most 300 + 24 times.
+// Batches that fit the GPU at once end with their largest query; larger ones go by the mean, 600 + 28 times, and wide CTAs,
+// which re-read four times as fast, by 600 + 27 times (120 probes: 54 us with 4 slots, 56 with 16).
+constexpr int SEL_WIDE = 1024, SEL_WIDE_REG = 16, SEL_WIDE_REG_LISTS = 4;      // batches of up to 64 queries: threads, slots
+constexpr int SEL_NARROW = 256, SEL_NARROW_REG = 20, SEL_NARROW_REG_LISTS = 12;
+static int select_list_items(const IndexImpl* ix, int nq, int nprobe) {
+    if (ix->tree_n1) return ix->tree_max_cand;
+    const int np = coarse_pilot_cols(ix, nprobe), nsel = nprobe + PROBE_GUARD;
+    if (!np) return ix->nlist;
+    if (np > 4096) return (int)((300 + 24ll * nsel) * ix->pilot_stride / 16);
+    return nq <= 64 ? 600 + 27 * nsel : (nq <= 6 * ix->num_sms ? 1200 + 30 * nsel : 600 + 28 * nsel);
+}
+int select_list_slots(const IndexImpl* ix, int nq, int nprobe) {
+    const int few = nq <= 64 ? SEL_WIDE * SEL_WIDE_REG_LISTS : SEL_NARROW * SEL_NARROW_REG_LISTS;
+    return select_list_items(ix, nq, nprobe) <= few ? few : (nq <= 64 ? SEL_WIDE * SEL_WIDE_REG : SEL_NARROW * SEL_NARROW_REG);
+}
 template <bool BF16, int THREADS, int REG, int REG_LISTS>
 static void launch_select_source(const IndexImpl* ix, const float* queries, const float* scores,
                                  const unsigned long long* cand, const int32_t* cand_cnt, uint32_t cand_sign, int nsplit, int cap, int nq,
                                  int nprobe, int32_t* probe_list, float* probe_term, float* probe_bias, const FusedPlan& fp, cudaStream_t s) {
     const dim3 grid(fp.enabled ? nq * (1 + fp.table_parts) : nq);
     const size_t smem = fp.enabled ? (size_t)(ix->d + ix->M) * 4 : 0;
-    const int most = ix->tree_n1 ? ix->tree_max_cand : (coarse_pilot_cols(ix, nprobe) ? 20 * (nprobe + PROBE_GUARD) : ix->nlist);  // items of a query, usually
-    const bool few = most <= THREADS * REG_LISTS;
+    const bool few = select_list_slots(ix, nq, nprobe) == THREADS * REG_LISTS;
     if (scores && ix->nlist <= THREADS * REG)
         launch_overlapped(select_probes_kernel<BF16, THREADS, REG, true, true>, grid, dim3(THREADS), smem, s,
             queries, ix->centroids, scores, cand, cand_cnt, cand_sign, nsplit, cap, ix->nlist, ix->d, ix->metric, nprobe, probe_list,
@@ -912,10 +929,10 @@ static cudaError_t launch_select_any(const IndexImpl* ix, const float* queries, 
     std::memset(&off, 0, sizeof(off));
     if (fp && fp->enabled && nq > 64) return cudaErrorInvalidValue;
     if (nq <= 64)
-        launch_select_shape<1024, 16, 4>(ix, queries, scores, cand, cand_cnt, cand_sign, nsplit, cap, nq, nprobe, probe_list, probe_term,
+        launch_select_shape<SEL_WIDE, SEL_WIDE_REG, SEL_WIDE_REG_LISTS>(ix, queries, scores, cand, cand_cnt, cand_sign, nsplit, cap, nq, nprobe, probe_list, probe_term,
                                       probe_bias, fp ? *fp : off, s);
     else
-        launch_select_shape<256, 20, 12>(ix, queries, scores, cand, cand_cnt, cand_sign, nsplit, cap, nq, nprobe, probe_list, probe_term,
+        launch_select_shape<SEL_NARROW, SEL_NARROW_REG, SEL_NARROW_REG_LISTS>(ix, queries, scores, cand, cand_cnt, cand_sign, nsplit, cap, nq, nprobe, probe_list, probe_term,
                                      probe_bias, off, s);
     count_launch();
     return cudaGetLastError();

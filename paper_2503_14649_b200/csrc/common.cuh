@@ -226,6 +226,7 @@ cudaError_t launch_coarse_scores(const IndexImpl* ix, const float* queries, int 
                                  cudaStream_t s);
 cudaError_t launch_tree_candidates(const IndexImpl* ix, const float* queries, int nq, int S, int cap,
                                    unsigned long long* cand, int32_t* cand_cnt, uint32_t* clear_block, cudaStream_t s);
+int select_list_slots(const IndexImpl* ix, int nq, int nprobe);  // items of candidate lists a selection holds in registers
 constexpr int TREE_LIMIT_B1 = 64, TREE_LIMIT_N1 = 4096;
 // Lists the pilot pass of the tensor-core coarse step samples, 0: no pass.  It pays off when a CTA sees many column tiles
 // per row and the sample can hold the wanted values.

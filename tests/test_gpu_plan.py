@@ -33,3 +33,27 @@ def test_pilot_pass(nlist, nprobe, cols):
     ix = _index(nlist)
     assert ix.rago_debug_search_plan(100, nprobe, 10)["pilot_cols"] == cols
     ix.close()
+
+
+# Queries whose entries exceed the registers go through a path that reads them again in every pass.
+@pytest.mark.parametrize("nlist,nq,nprobe,bf16", [
+    (8192, 200, 96, True), (16_384, 300, 40, False), (16_384, 300, 64, False), (65_536, 100, 64, True), (65_536, 100, 96, True),
+    (65_536, 100, 120, False), (16_384, 1000, 80, True), (8192, 40, 96, False), (65_536, 64, 100, True), (65_536, 64, 120, False),
+    (131_072, 100, 104, True)])
+def test_a_selections_registers_hold_the_entries_that_the_lists_leave(nlist, nq, nprobe, bf16):
+    ix = _index(nlist, bf16=bf16)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(nq)
+    q = torch.randn(nq, 64, generator=g, device="cuda")
+    plan = ix.rago_debug_search_plan(nq, nprobe, 1)
+    assert plan["route"] == "lists" and plan["pilot_cols"] > 0
+    ws = torch.zeros(ix.search_workspace_bytes(nq, nprobe, 1), dtype=torch.uint8, device="cuda")
+    ix.rago_search_probes(q, nprobe, workspace=ws)
+    torch.cuda.synchronize()
+    ix.rago_check(ws)
+    at = 256 * plan["counts_at"]
+    items = ws[at:at + 4 * nq * plan["lists"]].view(torch.int32).view(nq, -1).sum(1)
+    assert int(items.min()) >= nprobe + 8
+    allowed = 0.02 if nq <= 888 else 0.25  # of the queries: the largest ones end a batch that fits the GPU at once
+    assert float((items > plan["slots"]).float().mean()) <= allowed, (int(items.max()), plan["slots"])
+    ix.close()
