@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(FSEL_THREADS) flat_select_kernel(const float* 
 // always ends) finds a cut with between k and k + k/4 + 8 keys at or below it, and only those are ranked.  More
 // entries than one round holds go through further rounds against the cut of the rounds before.
 //
-// nq * parts CTAs.  Without starting thresholds a list keeps everything it saw, and one CTA would pull a hundred
+// nq * parts CTAs.  Without starting thresholds a list keeps what it saw up to its capacity, and one CTA would pull a hundred
 // thousand entries through one SM; a small batch then splits a query's lists into parts.  Each part leaves its keys in
 // the storage of its own first list (read by nobody else), and the part that finishes last (a ticket per query, zero
 // before the launch) selects among what the parts left.
@@ -139,14 +139,27 @@ struct FlatMergeState {
     int cnt, last;
 };
 
+// Most keys a part leaves; the short selection ranks WARP_SORT_MAX as fast as fewer.
+__host__ __device__ inline int flat_merge_most(int k) { return k + (k >> 2) + 8 > WARP_SORT_MAX ? k + (k >> 2) + 8 : WARP_SORT_MAX; }
+
 // Adds the entries of lists slot_of(l), l0 <= l < l1 (count cnts[slot], entries at entries[slot * stride ...]), to the
-// keys the buffer holds and leaves between min(k, all) and k + k/4 + 8 of the smallest there.
+// keys the buffer holds and leaves there the min(k, all) smallest and a few more: at most flat_merge_most(k), in the last pass
+// (`last`) what sorts as fast, or up to TOPK_CAP where the last FM_LISTS lists turn out to be empty.
 template <class SlotOf>
 __device__ __forceinline__ void flat_merge_lists(FlatMergeState& S, const int32_t* cnts, const unsigned long long* entries,
                                                  int l0, int l1, SlotOf slot_of, int stride, int raw, uint32_t raw_sign,
-                                                 int k) {
+                                                 int k, bool last) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t want_max = (uint32_t)(k + (k >> 2) + 8 > WARP_SORT_MAX ? k + (k >> 2) + 8 : WARP_SORT_MAX);
+    uint32_t want_max = (uint32_t)flat_merge_most(k);
+    if (last && k > RANK_MAX) {  // sorted, not ranked: up to the next power of two costs the same, beyond it twice as much
+        const uint32_t pow2 = 1u << (32 - __clz(k - 1));
+        if (pow2 >= (uint32_t)(k + (k >> 6) + 4)) want_max = pow2;
+    }
+    // Of n_all entries, n_seen seen and n_held of those at or below the bound: would the rest pass into the buffer?
+    auto rest_fits = [](int n_held, int n_seen, int n_all) {
+        const float rest = (float)n_held * (float)(n_all - n_seen) / (float)n_seen;
+        return rest + 4.f * sqrtf(rest) + (float)n_held <= (float)TOPK_CAP;
+    };
     unsigned long long bound = KEY_MAX - 1;  // nothing above it can be a result
     for (int g0 = l0; g0 < l1; g0 += FM_LISTS) {
         const int ng = l1 - g0 < FM_LISTS ? l1 - g0 : FM_LISTS;
@@ -173,17 +186,20 @@ __device__ __forceinline__ void flat_merge_lists(FlatMergeState& S, const int32_
         }
         __syncthreads();
         const int nitems = S.pre[ng];
-        // Many entries: the first round's bound leaves few of the rest, which are therefore streamed past it, a warp per
-        // list and with no numbering, at a tenth of the instructions of a round.  What passes joins the first round's
-        // keys in the buffer; if it does not fit, the pass counts for nothing and all rounds are taken.
-        bool streamed = false;
+        // Many entries: once the bound of the rounds taken leaves so few of the rest that they fit the buffer (after one
+        // round for k = 10; 17 of 65 for k = 400), the rest is streamed past it, a warp per list and with no numbering, at a
+        // tenth of the instructions of a round.  If it does not fit after all (rows in an order of their own), the
+        // pass counts for nothing and the other rounds are taken.  Streaming after the first round whatever k threw the
+        // pass away for large k: 33 queries over 250 001 rows, k = 400, 644 us, this 272.
+        bool tried = false;
         for (int r0 = 0; r0 < nitems; r0 += FM_ENTRIES) {  // uniform
-            if (r0 == FM_ENTRIES && nitems > 2 * FM_ENTRIES && bound != KEY_MAX - 1 && !streamed) {
+            if (!tried && nitems - r0 > FM_ENTRIES && bound != KEY_MAX - 1 && r0 > 0 && rest_fits(S.cnt, r0, nitems)) {
+                tried = true;
                 const int before = S.cnt;
                 __syncthreads();
                 const uint32_t bound32 = (uint32_t)(bound >> 32);
                 for (int l = warp; l < ng; l += FM_THREADS / 32) {
-                    const int skip = r0 - S.pre[l], n = S.pre[l + 1] - S.pre[l];  // entries the first round has seen
+                    const int skip = r0 - S.pre[l], n = S.pre[l + 1] - S.pre[l];  // entries the rounds have seen
                     const unsigned long long* src = entries + (size_t)slot_of(g0 + l) * stride;
                     for (int i0 = skip > 0 ? skip : 0; i0 < n; i0 += 32 * FM_KPT) {
                         unsigned long long e[FM_KPT];
@@ -205,11 +221,10 @@ __device__ __forceinline__ void flat_merge_lists(FlatMergeState& S, const int32_
                 }
                 __syncthreads();
                 if (S.cnt <= TOPK_CAP) {  // uniform
-                    streamed = true;
                     r0 = nitems;  // one last round with no new entries, which cuts the buffer
                 } else {
                     __syncthreads();
-                    if (tid == 0) S.cnt = before;  // the first round's keys are intact; the pushes that fitted lie behind them
+                    if (tid == 0) S.cnt = before;  // the rounds' keys are intact; the pushes that fitted lie behind them
                     __syncthreads();
                 }
             }
@@ -278,10 +293,12 @@ __device__ __forceinline__ void flat_merge_lists(FlatMergeState& S, const int32_
                 ++round;
                 return S.round[slot];
             };
-            // more entries follow and all survivors fit the buffer: no cut yet, the next rounds go by the old bound
+            // more entries follow and all survivors fit the buffer: no cut yet, the next rounds go by the old bound, unless
+            // a cut now lets the rest be streamed
             const bool more = r0 + FM_ENTRIES < nitems || g0 + FM_LISTS < l1;
+            const bool cut_to_stream = !tried && nitems - r0 > 2 * FM_ENTRIES && rest_fits((int)want_max, r0 + FM_ENTRIES, nitems);
             unsigned long long hi = KEY_MAX - 1;
-            if (c_hi > (more ? (uint32_t)TOPK_CAP : want_max)) {  // uniform
+            if (c_hi > (more && !cut_to_stream ? (uint32_t)TOPK_CAP : want_max)) {  // uniform
                 while (hi32 - lo32 > 1 && c_hi > want_max) {
                     const uint32_t mid = bisect_mid(lo32, hi32, round);
                     const uint32_t c = count([&](unsigned long long x) { return (uint32_t)(x >> 32) <= mid; });
@@ -323,9 +340,9 @@ __global__ void __launch_bounds__(FM_THREADS, 2) flat_merge_kernel(int nlists, i
     for (int pass = 0;; ++pass) {
         // second pass: the first lists of all parts
         auto slot_of = [&](int l) { return pass ? (int)((long long)l * nlists / parts) : l; };
-        flat_merge_lists(S, cnts, entries, l0, l1, slot_of, stride, pass ? 0 : raw, raw_sign, k);
+        flat_merge_lists(S, cnts, entries, l0, l1, slot_of, stride, pass ? 0 : raw, raw_sign, k, pass || parts == 1);
         if (pass || parts == 1) break;  // uniform
-        const int n = S.cnt;  // at most k + k/4 + 8 <= stride: the launcher checked
+        const int n = S.cnt;  // at most flat_merge_most(k) <= stride: the launcher checked (a part has at most FM_LISTS lists)
         for (int i = tid; i < n; i += FM_THREADS) entries[(size_t)first * stride + i] = S.keys[i];
         if (tid == 0) cnts[first] = n;
         __syncthreads();  // the part's keys and count are written ...
@@ -459,7 +476,7 @@ cudaError_t launch_flat_search(const void* db, int64_t N, int d, const void* que
         // Parts per query: a starting threshold leaves a few thousand entries per query, one round of one CTA; without
         // one, parts of half a round each while the batch alone does not fill the GPU.
         int parts = 1;
-        if (!np && nq <= FM_TICKETS && k + (k >> 2) + 8 <= cap && WARP_SORT_MAX <= cap) {
+        if (!np && nq <= FM_TICKETS && flat_merge_most(k) <= cap && nlists <= FM_LISTS) {
             const int64_t tiles = (N + 255) / 256, cols = (tiles + nsplit - 1) / nsplit * (256 / GEMM_COL_HALVES);
             const int64_t most = (int64_t)nlists * (cols < cap ? cols : cap);
             parts = (int)((most + FM_ENTRIES / 2 - 1) / (FM_ENTRIES / 2));

@@ -46,3 +46,19 @@ def test_count_words_that_no_kernel_wrote_stay_inside_the_lists(nlists, stride, 
         counts.view(-1)[i::7] = v
     counts[3] = -5
     _check(scores, counts, k)
+
+
+# A list's entries ascend, descend or stand in any order, so that what the first entries say about the rest holds or does
+# not: the rest is streamed past their bound, streamed in vain, or taken in rounds; a last group of lists may be empty.
+@pytest.mark.parametrize("nlists,stride,k", [(296, 512, 1), (296, 512, 10), (296, 896, 400), (100, 1024, 960), (40, 256, 300), (520, 64, 100)])
+@pytest.mark.parametrize("order", ["random", "ascending", "descending", "equal"])
+def test_final_selection_over_many_entries_in_any_order(nlists, stride, k, order):
+    scores = _normal(3, nlists, stride, seed=k)
+    if order in ("ascending", "descending"):
+        scores = scores.view(3, -1).sort(dim=1, descending=order == "descending")[0].view(3, nlists, stride)
+    elif order == "equal":
+        scores = (scores * 2).round()  # a few values, thousands of rows each
+    counts = torch.full((3, nlists), stride, dtype=torch.int32, device="cuda")
+    counts[1, ::3] = 0
+    counts[2, 512:] = 0
+    _check(scores.contiguous(), counts, k)
