@@ -330,6 +330,15 @@ __global__ void __launch_bounds__(FM_THREADS, 2) flat_merge_kernel(int nlists, i
     grid_dependency_wait();
     grid_dependents_may_launch();
     const int tid = threadIdx.x, q = blockIdx.x / parts, part = blockIdx.x % parts;
+    if (!raw && nlists == 1) {  // uniform: one chunk of at most k keys, which flat_select_kernel left in order
+        const int n = list_count(slot_cnt[q], k);
+        for (int i = tid; i < k; i += FM_THREADS) {
+            const unsigned long long key = i < n ? slot_keys[(size_t)q * stride + i] : KEY_MAX;
+            out_ids[(size_t)q * k + i] = i < n ? (int64_t)(uint32_t)(key & 0xFFFFFFFFull) : -1;
+            out_scores[(size_t)q * k + i] = i < n ? -orderable_f32((uint32_t)(key >> 32)) : __int_as_float(0xff800000);
+        }
+        return;
+    }
     auto sync = [] { __syncthreads(); };
     if (tid == 0) S.cnt = 0;
     __syncthreads();

@@ -3,7 +3,7 @@
 import pytest
 import torch
 
-from paper_2503_14649_b200 import binding
+from paper_2503_14649_b200 import binding, synth
 
 pytestmark = pytest.mark.gpu
 
@@ -62,3 +62,17 @@ def test_final_selection_over_many_entries_in_any_order(nlists, stride, k, order
     counts[1, ::3] = 0
     counts[2, 512:] = 0
     _check(scores.contiguous(), counts, k)
+
+
+# k beyond the fused selection: panels on the fp32 pipes, one chunk of rows (its keys are the answer) or two; k above N.
+@pytest.mark.parametrize("N,k", [(900, 1024), (1, 961), (3000, 1000), (65_536, 1024), (65_537, 961)])
+def test_flat_search_beyond_the_fused_selection(N, k):
+    db, q = synth.make_flat(N, 64, 20, seed=N, device="cuda")
+    ids, scores = binding.rago_flat_search(db, q, k)
+    exact = q.double() @ db.double().T
+    m = min(k, N)
+    want, _ = exact.topk(m, 1)
+    assert torch.allclose(scores[:, :m].double(), want, rtol=0, atol=64 * 2.0 ** -24)  # 64 products of unit-norm rows in fp32
+    assert torch.allclose(exact.gather(1, ids[:, :m]), want, rtol=0, atol=64 * 2.0 ** -24)
+    assert all(len(set(row)) == m for row in ids[:, :m].tolist())
+    assert bool((ids[:, m:] == -1).all()) and bool(torch.isneginf(scores[:, m:]).all())
