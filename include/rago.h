@@ -271,8 +271,9 @@ rago_status rago_debug_set_gemm_pairing(int32_t mode);
  *   4  1 if the kernel behind the tensor-core launch is scheduled while that runs
  *   5  entries of a query's candidate lists that its selection holds in registers; 6 where the lists' counts
  *      (int32 [nq][lists]) lie in the workspace of the call, in units of 256 bytes
+ *   7  work units that stand for the start of a query when the scan's tiles are dealt out; 8 whether it prefetches tiles
  */
-#define RAGO_PLAN_WORDS 7
+#define RAGO_PLAN_WORDS 9
 enum { RAGO_PLAN_FP32 = 0, RAGO_PLAN_MATRIX = 1, RAGO_PLAN_LISTS = 2, RAGO_PLAN_TREE = 3 };
 rago_status rago_debug_search_plan(const rago_index* index, int32_t nq, int32_t nprobe, int32_t k, int32_t* out);
 

@@ -22,7 +22,8 @@ STATUS_NAMES = {0: "RAGO_OK", 1: "RAGO_EINVAL", 2: "RAGO_EALIGN", 3: "RAGO_EUNSU
 RAGO_L2, RAGO_IP = 0, 1
 RAGO_F32, RAGO_BF16 = 0, 1
 NUM_STAGES = 5
-PLAN_NAMES = ("route", "lists", "cap", "pilot_cols", "early_successor", "slots", "counts_at")
+PLAN_NAMES = ("route", "lists", "cap", "pilot_cols", "early_successor", "slots", "counts_at", "lead",
+              "prefetch")
 PLAN_ROUTES = ("fp32", "matrix", "lists", "tree")
 STAGE_NAMES = ("coarse_scores", "probe_select", "plan", "table_scan", "merge")
 

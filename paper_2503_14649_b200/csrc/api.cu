@@ -586,16 +586,18 @@ rago_status rago_debug_search_plan(const rago_index* index, int32_t nq, int32_t 
     const IndexImpl* ix = reinterpret_cast<const IndexImpl*>(index);
     const rago_status st = check_search_args(ix, nq, nprobe, k);
     if (st != RAGO_OK) return st;
-    if (!out) return fail(RAGO_EINVAL, "out is null");
+    if (!out || nq < 1) return fail(RAGO_EINVAL, "out is null or nq is 0");
     const Layout L = make_layout(ix, nq, nprobe, k);
     const bool lists = L.tree_S || (L.tc && L.tc_mode == 0);
     out[0] = L.tree_S ? RAGO_PLAN_TREE : (!L.tc ? RAGO_PLAN_FP32 : (lists ? RAGO_PLAN_LISTS : RAGO_PLAN_MATRIX));
     out[1] = L.tree_S ? L.tree_S : (lists ? L.tc_nsplit * GEMM_COL_HALVES : 0);
     out[2] = L.tree_S ? L.tree_cap : (lists ? L.tc_cap : 0);
     out[3] = L.pilot_cols;
+    out[4] = L.tc && gemm_early_successor(nq, L.tc_mg, L.tc_nsplit) ? 1 : 0;
     out[5] = lists ? select_list_slots(ix, nq, nprobe) : 0;
     out[6] = lists ? (int32_t)(L.cand_cnt / 256) : 0;
-    out[4] = L.tc && gemm_early_successor(nq, L.tc_mg, L.tc_nsplit) ? 1 : 0;
+    out[7] = scan_query_lead(ix, nq, nprobe, k);
+    out[8] = scan_prefetches(ix, (int64_t)nq * nprobe) ? 1 : 0;
     return RAGO_OK;
 }
 

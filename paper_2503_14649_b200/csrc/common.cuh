@@ -282,6 +282,7 @@ cudaError_t scan_plan(const IndexImpl* ix, ScanPlan* plan);
 cudaError_t launch_vector_terms(const IndexImpl* ix, float* vterm, cudaStream_t s);
 cudaError_t launch_transpose_codebook(const float* cb, int M, int dsub, float* cbT, cudaStream_t s);
 int scan_query_lead(const IndexImpl* ix, int nq, int nprobe, int k);  // work units that stand for the start of a query
+bool scan_prefetches(const IndexImpl* ix, int64_t npairs);  // tiles are pulled into L2 ahead of their copies
 cudaError_t launch_plan_work(const IndexImpl* ix, const int32_t* probe_list, int npairs, int tile_vecs, int lead,
                              int32_t* pair_tiles, int64_t* work_prefix, unsigned long long* qthresh, int nq,
                              int32_t* slot_cnt, int nslots, const float* queries, uint8_t* lut_img, float* lut_inv,

@@ -985,6 +985,21 @@ int scan_query_lead(const IndexImpl* ix, int nq, int nprobe, int k) {
     return (int64_t)nq * nprobe * tiles_per_list >= (int64_t)lead * ix->plan.ctas ? lead : 0;
 }
 
+// Prefetching into L2 pays where the tiles in flight are small (a copy from DRAM takes longer than the tile in front
+// of it is scanned) and the batch does not meet each list several times, which brings most tiles from L2 anyway and
+// makes the prefetches only extra traffic.  Without / with, us per call: 48-byte codes, 2.3 probes per list
+// 1672 / 1618; 96 bytes, 0.6 probes 753 / 741; 96 bytes, 8 probes 8890 / 9100 (with terms 9190); 64 bytes (60 KB
+// tiles), 4 096 queries 14 560 / 14 730, 33 queries 226.9 / 233.8.
+// Long lists of a database beyond L2 come from DRAM however often they are met, which shows where a tile is scanned in a
+// short time (48 and 80 bytes: 23 and 20 KB).  64 lists of 47 000 vectors, 600 queries with 32 probes, without / with: 48 bytes
+// 9 520 / 8 940, 80 bytes 19 490 / 18 950.  With lists below 32 tiles, inside L2, and for the other sizes (6 M vectors in 64
+// lists, 16 bytes 3%, 64 bytes 3%, 96 bytes 1% more) it is the other way round or equal.
+bool scan_prefetches(const IndexImpl* ix, int64_t npairs) {
+    const int tile_bytes = ix->plan.tile_vecs * ix->M;
+    const bool long_lists = ix->N / ix->nlist >= 32ll * ix->plan.tile_vecs && ix->N * ix->M > (128ll << 20);
+    return (tile_bytes <= 40 * 1024 && npairs <= 4ll * ix->nlist) || (ix->M >= 48 && tile_bytes <= 24 * 1024 && long_lists);
+}
+
 cudaError_t launch_scan(const IndexImpl* ix, const ScanPlan& plan, const float* queries, const int32_t* probe_list,
                         const float* probe_term, const int64_t* work_prefix, int nq, int nprobe, int k,
                         unsigned long long* qthresh, int32_t* slot_cnt, unsigned long long* slot_keys,
@@ -1001,12 +1016,7 @@ cudaError_t launch_scan(const IndexImpl* ix, const ScanPlan& plan, const float* 
     a.lead = scan_query_lead(ix, nq, nprobe, k);
     a.metric = ix->metric; a.k = k; a.stages = plan.stages; a.dyn_bytes = (uint32_t)plan.smem_bytes;
     a.stream_once = nq <= 64 ? 1 : 0;
-    // Prefetching into L2 pays where the tiles in flight are small (a copy from DRAM takes longer than the tile in front
-    // of it is scanned) and the batch does not meet each list several times, which brings most tiles from L2 anyway and
-    // makes the prefetches only extra traffic.  Without / with, us per call: 48-byte codes, 2.3 probes per list
-    // 1672 / 1618; 96 bytes, 0.6 probes 753 / 741; 96 bytes, 8 probes 8890 / 9100 (with terms 9190); 64 bytes (60 KB
-    // tiles), 4 096 queries 14 560 / 14 730, 33 queries 226.9 / 233.8.
-    a.prefetch = plan.tile_vecs * ix->M <= 40 * 1024 && (long long)a.npairs <= 4ll * ix->nlist ? 1 : 0;
+    a.prefetch = scan_prefetches(ix, a.npairs) ? 1 : 0;
     const cudaError_t e = launch_overlapped(v->kernel, dim3(plan.ctas), dim3(v->threads), plan.smem_bytes, s, a);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();

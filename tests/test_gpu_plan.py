@@ -57,3 +57,13 @@ def test_a_selections_registers_hold_the_entries_that_the_lists_leave(nlist, nq,
     allowed = 0.02 if nq <= 888 else 0.25  # of the queries: the largest ones end a batch that fits the GPU at once
     assert float((items > plan["slots"]).float().mean()) <= allowed, (int(items.max()), plan["slots"])
     ix.close()
+
+
+# Tiles of 480 (48 bytes), 256 (80) and 384 (96) vectors.  Few probes per list, many; lists of 47 000 vectors beyond L2, in it.
+@pytest.mark.parametrize("N,nlist,M,nq,nprobe,prefetch", [
+    (3_000_000, 64, 48, 600, 32, 1), (400_000, 64, 48, 600, 32, 0), (3_000_000, 512, 48, 600, 32, 0), (3_000_000, 512, 48, 60, 32, 1),
+    (3_000_000, 64, 80, 40, 64, 1), (3_000_000, 64, 96, 40, 64, 0), (3_000_000, 64, 96, 4, 64, 1), (3_000_000, 64, 64, 1, 64, 0)])
+def test_scan_prefetches_what_comes_from_dram(N, nlist, M, nq, nprobe, prefetch):
+    ix = _index(nlist, d=2 * M, M=M, N=N, metric="ip")
+    assert ix.rago_debug_search_plan(nq, nprobe, 10)["prefetch"] == prefetch
+    ix.close()
