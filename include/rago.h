@@ -139,7 +139,9 @@ rago_status rago_index_free(rago_index* index);
 /* Bytes of device scratch rago_search / rago_search_probes / rago_search_host need for a batch
  * of nq queries with these nprobe and k (1 <= nprobe <= nlist, 1 <= k <= 1024).  Its largest parts are
  * the per-query lookup tables (64 to 160 KB each, for at most 4096 queries of a batch: 128 KB per
- * query at M = 96) and, for batches the tensor-core coarse step does not take, nq * nlist scores. */
+ * query at M = 96) and what the coarse step leaves: nq * nlist scores, or candidate lists of up to
+ * 1024 entries of 8 bytes, some 300 per query of a small batch.  The bytes also serve searches with the same nq and smaller
+ * nprobe or k; a smaller nq may need more (its candidate lists are cut finer). */
 rago_status rago_search_workspace_bytes(const rago_index* index, int32_t nq, int32_t nprobe, int32_t k,
                                         size_t* out_bytes);
 

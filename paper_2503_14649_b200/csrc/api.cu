@@ -126,6 +126,17 @@ static Layout make_layout(const IndexImpl* ix, int nq, int nprobe, int k) {
     return L;
 }
 
+// Workspace of a call, enough for the same batch with fewer probes too: a smaller nprobe may take candidate lists or a
+// pilot pass where a larger one takes the (smaller) score matrix.  Between the values of nprobe at which the plan
+// changes the layout only grows with it.
+static size_t workspace_bytes_for(const IndexImpl* ix, int nq, int nprobe, int k) {
+    size_t most = make_layout(ix, nq, nprobe, k).total;
+    const int pilot_end = ix->pilot_stride ? ix->nlist / ix->pilot_stride / 4 - PROBE_GUARD : 0;
+    for (const int p : {pilot_end, GEMM_NSEL_SMALL - PROBE_GUARD, GEMM_NSEL_LARGE - PROBE_GUARD})
+        if (p >= 1 && p < nprobe) most = std::max(most, make_layout(ix, nq, p, k).total);
+    return most;
+}
+
 // Every pointer an index holds, and everything derived at load, belongs to one device.
 static rago_status check_device(const IndexImpl* ix) {
     int dev = -1;
@@ -362,7 +373,7 @@ rago_status rago_search_workspace_bytes(const rago_index* index, int32_t nq, int
     if (!out_bytes) return fail(RAGO_EINVAL, "out_bytes is null");
     rago_status st = check_search_args(ix, nq, nprobe, k);
     if (st != RAGO_OK) return st;
-    *out_bytes = make_layout(ix, nq, nprobe, k).total;
+    *out_bytes = workspace_bytes_for(ix, nq, nprobe, k);
     return RAGO_OK;
 }
 

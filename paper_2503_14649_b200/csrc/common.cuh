@@ -238,6 +238,7 @@ inline int coarse_pilot_cols(const IndexImpl* ix, int nprobe) {
 }
 // gemm_select.cu
 constexpr int GEMM_CAP_SMALL = 512, GEMM_CAP_LARGE = 1024;  // candidate-list capacities (keys per list)
+constexpr int GEMM_NSEL_SMALL = GEMM_CAP_SMALL - 128, GEMM_NSEL_LARGE = GEMM_CAP_LARGE - 64;  // wanted keys they serve
 constexpr int GEMM_COL_HALVES = 2;  // a row has one candidate list per share of the grid AND per half of a 256-column tile
 struct GemmLaunch {
     const void* tmap_a;          // CUtensorMap of A: bf16 [a parts * a_part_rows][d]

@@ -643,7 +643,7 @@ cudaError_t make_tmap_bf16(void* out_map, const void* ptr, uint64_t rows, uint64
     return cudaSuccess;
 }
 
-int gemm_cand_cap(int nsel) { return nsel <= GEMM_CAP_SMALL - 128 ? GEMM_CAP_SMALL : (nsel <= GEMM_CAP_LARGE - 64 ? GEMM_CAP_LARGE : 0); }
+int gemm_cand_cap(int nsel) { return nsel <= GEMM_NSEL_SMALL ? GEMM_CAP_SMALL : (nsel <= GEMM_NSEL_LARGE ? GEMM_CAP_LARGE : 0); }
 
 // Grid shape and main loop.  *mg: 1 = one row tile per CTA (LOOP_SINGLE), 2 = two row tiles per CTA sharing each B
 // tile (LOOP_PAIR), 3 = two row tiles per CTA PAIR (LOOP_TWO_CTA: a cluster of two CTAs shares each B tile).

@@ -67,3 +67,22 @@ def test_scan_prefetches_what_comes_from_dram(N, nlist, M, nq, nprobe, prefetch)
     ix = _index(nlist, d=2 * M, M=M, N=N, metric="ip")
     assert ix.rago_debug_search_plan(nq, nprobe, 10)["prefetch"] == prefetch
     ix.close()
+
+
+# With 8192 lists the pilot pass ends behind nprobe = 120, with 65 536 candidate lists grow at 377 and end at 953.
+@pytest.mark.parametrize("nlist,nq,nprobes", [(8192, 17, (8, 120, 121, 128, 400)), (8192, 300, (1, 64, 120, 121, 1024)),
+                                              (65_536, 100, (16, 376, 377, 952, 953, 1016)), (255, 64, (1, 8, 255)),
+                                              (20_001, 1500, (20, 376, 377, 953))])
+def test_a_workspace_also_serves_fewer_probes(nlist, nq, nprobes):
+    ix = _index(nlist)
+    sizes = [ix.search_workspace_bytes(nq, p, 100) for p in nprobes]
+    assert sizes == sorted(sizes)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(nq)
+    q = torch.randn(nq, 64, generator=g, device="cuda")
+    ws = torch.zeros(sizes[-1], dtype=torch.uint8, device="cuda")
+    for p in nprobes:
+        ids, _ = ix.rago_search(q, p, 10, workspace=ws)  # refused if it asked for more than the largest nprobe did
+        ix.rago_check(ws)
+        assert int((ids >= 0).sum()) > 0
+    ix.close()
