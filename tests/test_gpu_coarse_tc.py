@@ -80,8 +80,30 @@ def test_long_rows_exercise_list_compaction(metric, bf16, pairing):
 
 def test_large_nprobe_uses_the_wide_lists_and_the_score_matrix(pairing):
     data = synth.make_ivfpq(3000, 64, 8192, 16, 150, metric="l2", seed=78)
-    _probe_parity(data, 300, mode=2)    # nsel = 308: 1024-key lists
+    _probe_parity(data, 300, mode=2)    # 128 columns per list: everything would be kept, so the score matrix
     _probe_parity(data, 1000, mode=2)   # nsel = 1008: score-matrix epilogue
+    data = synth.make_ivfpq(3000, 64, 65_536, 16, 150, metric="l2", seed=78)
+    _assert_lists(data, 400, cap=1024, pilot=True)
+    _probe_parity(data, 400, mode=2)    # nsel = 408 behind pilot thresholds: 1024-key lists
+
+
+def _assert_lists(data, nprobe, cap, pilot):
+    ix = binding.load_index_from(data, "cuda")
+    ix.rago_set_coarse_mode(2)
+    plan = ix.rago_debug_search_plan(data.queries.shape[0], nprobe, 1)
+    ix.close()
+    assert (plan["route"], plan["cap"], plan["pilot_cols"] > 0) == ("lists", cap, pilot), plan
+
+
+# No starting thresholds (the number of lists is not a multiple of 16) and more columns per list than it holds, so that lists
+# fill up and are cut; a ragged last tile; the plain compare (inner product) and the one with column terms (L2).
+@pytest.mark.parametrize("nlist,nq,nprobe,metric,bf16,cap", [
+    (30_001, 1100, 32, "l2", False, 512), (30_011, 1100, 32, "l2", True, 512), (30_001, 1100, 24, "ip", False, 512),
+    (60_001, 1100, 400, "l2", True, 1024), (60_101, 1100, 390, "ip", True, 1024)])
+def test_lists_without_starting_thresholds_are_cut(nlist, nq, nprobe, metric, bf16, cap, pairing):
+    data = synth.make_ivfpq(3000, 64, nlist, 16, nq, metric=metric, seed=nlist, coarse_bf16=bf16)
+    _assert_lists(data, nprobe, cap, pilot=False)
+    _probe_parity(data, nprobe, mode=2)
 
 
 def test_search_results_do_not_depend_on_the_coarse_kernel():
