@@ -93,7 +93,9 @@ static Layout make_layout(const IndexImpl* ix, int nq, int nprobe, int k) {
         L.qparts = take((size_t)ix->cparts_n * nq * ix->d * 2);
         const int pilot = coarse_pilot_cols(ix, nprobe);
         // Lists that would keep every score (no starting thresholds, no more columns per list than it holds) only spread
-        // them: the score matrix is half the bytes in 16-byte stores, and the selection reads it in order.
+        // them: the score matrix is half the bytes in 16-byte stores, and the selection reads it in order.  A list of
+        // exactly its capacity is still cut once, at its end, and the matrix wins all the same: 100 queries over 151 001
+        // lists 425 us against 430, 64 queries 211 against 260, 200 queries over 60 001 246 against 777.
         const int tiles = (ix->nlist + 255) / 256, per_list = (tiles + L.tc_nsplit - 1) / L.tc_nsplit * (256 / GEMM_COL_HALVES);
         L.tc_mode = L.tc_cap && (pilot || per_list > L.tc_cap) ? 0 : 1;
         if (L.tc_mode == 0) {

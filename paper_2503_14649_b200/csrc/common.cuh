@@ -200,9 +200,13 @@ void count_launch(int n = 1);
 // ---- back-to-back kernels of one search -------------------------------------------------------------
 // A kernel launched with launch_overlapped may be scheduled while the kernel before it on the stream is still
 // draining; it must not touch global memory before grid_dependency_wait(), which returns once that kernel has
-// completed and its writes are visible.  Every kernel of the chain waits first thing and then lets its own
-// successor be scheduled, so the order of all memory accesses is the stream order; what overlaps is launch
-// latency.  In a kernel launched the ordinary way both calls do nothing.
+// completed and its writes are visible.  The one exception: the tiny-batch coarse kernel asks for centroids before it
+// waits.  They are the caller's borrowed array, unchanged from index load to free, and no kernel launched this way may write
+// them; workspace, queries and results may never be touched early.  Every kernel of the chain waits and then lets its own
+// successor be scheduled (a tensor-core launch that fills the GPU does not, see gemm_early_successor), so the order of all
+// other memory accesses is the stream order; what overlaps is launch latency.  No kernel takes tensor memory before it
+// waits.  In a kernel launched the ordinary way (fp32 coarse scores of larger batches, flat search beyond the fused selection,
+// index set-up) both calls do nothing.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependents_may_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <class... P, class... A>

@@ -976,6 +976,9 @@ cudaError_t scan_plan(const IndexImpl* ix, ScanPlan* plan) {
 // about 5.5 us; more with a 4 096-key buffer 7 us, with a 2 048-key buffer (more cuts) 17; per tile 1 us for 36 KB, no
 // less than 0.8 us.  Where a share is shorter than the start of a query the tiles are short or few, no CTA waits long
 // for another, and leads only leave CTAs without work (64 queries over 100 000 vectors 64.8 -> 67.1 us per call): none.
+// The three starts were measured with 32, 64 and 48 bytes; the other sizes take them by table size and k (a small k on a 128 KB
+// table that of a 64 KB one), and the tile count is that of average lists.  Both only move work between CTAs: no result
+// depends on them.
 int scan_query_lead(const IndexImpl* ix, int nq, int nprobe, int k) {
     if (nq < 2 || ix->nlist < 1) return 0;
     const float start_us = k <= 32 ? 5.5f : (ix->plan.lut_bytes <= 65536 ? 7.f : 17.f);
