@@ -46,8 +46,8 @@ SECONDARY = ("mid", "flat", "coarse_hyper", "iter")
 # of codes; the capture-size rule) and carries over to the full size because the lists are uniform and no list is
 # shared through L2 at either size; "mid" was captured at full size and is not scaled to other sizes.
 SCAN_TRAFFIC = {
-    "hyper": {"scan_sha": "d571bdbd02bf662d", "dram_per_logical": (15953797376 + 10658560) / 16004289600},   # 0.9975
-    "mid": {"scan_sha": "d571bdbd02bf662d", "dram_per_logical": (31611325184 + 7421696) / 42427363200},      # 0.7452
+    "hyper": {"scan_sha": "73cf608dd7623529", "dram_per_logical": (15954677248 + 11764480) / 16004289600},   # 0.9976
+    "mid": {"scan_sha": "73cf608dd7623529", "dram_per_logical": (30972259072 + 7904512) / 42427363200},      # 0.7302
 }
 
 
