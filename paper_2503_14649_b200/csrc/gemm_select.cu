@@ -676,7 +676,7 @@ void gemm_grid(int nrows, int64_t ncols, int d, int num_sms, int* mg, int* nspli
 // A launch of at most half as many CTAs as there are SMs lets the kernel behind start early: its CTAs wait on idle SMs.  Behind
 // a launch that fills the GPU they would be packed onto the SMs whose CTA ends first, and a selection of about one CTA per
 // SM then runs two or three to an SM.  us per call, early / not: 100 queries, 200 of 65 536 lists (bf16, d = 256)
-// 124 / 105, flat 33 queries over 100 000 rows, k = 100 331 / 249, 1 query 35 / 31; for 17 queries over 300 to 18 000 lists (2 to
+// 124 / 105, the coarse step and what follows it for 1 024 queries over 4096 lists (fp32, d = 768) 522 / 382, flat 33 queries over 100 000 rows, k = 100 331 / 249, 1 query 35 / 31; for 17 queries over 300 to 18 000 lists (2 to
 // 71 CTAs), where it stays, 38 / 42 to 37.4 / 38.7.
 bool gemm_early_successor(int nrows, int mg, int nsplit) {
     const int mtiles = (nrows + GBM - 1) / GBM;
