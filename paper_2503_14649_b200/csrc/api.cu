@@ -7,6 +7,7 @@
 #include <new>
 #include <vector>
 
+#include "pair.cuh"
 #include "plan.cuh"
 
 namespace rago {
@@ -45,6 +46,8 @@ struct Layout {
     size_t pilot_scores, row_tau;   // pilot pass: scores of the sampled lists, per-query starting thresholds
     size_t lut_img, lut_inv, lut_scale;        // small batches: lookup tables built ahead of the scan, and their scales
     int prebuilt;
+    size_t pair;                    // pairs of queries: their part of the workspace (pair_layout)
+    int pairs;                      // the batch is looked through for pairs
     int pilot_cols;                 // 0: no pilot pass
     size_t nslots;
     int tc, tc_mode, tc_cap, tc_mg, tc_nsplit;  // coarse plan for this (nq, nprobe)
@@ -68,7 +71,11 @@ static Layout make_layout(const IndexImpl* ix, int nq, int nprobe, int k) {
         return at;
     };
     const size_t npairs = (size_t)nq * nprobe;
-    L.nslots = (size_t)nq + (size_t)ix->plan.ctas;  // one slot per (CTA, query) incidence
+    L.pairs = pair_applies(ix, nq, nprobe, k) ? 1 : 0;
+    const int pair_nq = std::min(nq, PAIR_MAX_NQ);  // reserved for larger batches too, as below
+    const bool pair_room = L.pairs || pair_reserves(ix, pair_nq, nprobe, k);
+    // one slot per (CTA, query) incidence; pairs and single queries are scanned, and numbered, apart
+    L.nslots = pair_room ? pair_slots(nq, ix->plan.ctas) : (size_t)nq + (size_t)ix->plan.ctas;
     L.err = take(256);
     L.probe_list = take(npairs * 4);
     L.probe_term = take(npairs * 4);
@@ -124,6 +131,7 @@ static Layout make_layout(const IndexImpl* ix, int nq, int nprobe, int k) {
     L.lut_img = take(nlut * ix->plan.lut_bytes);
     L.lut_inv = take(nlut * 4);
     L.lut_scale = take(nlut * 4);
+    L.pair = take(pair_room ? pair_layout(pair_nq, nprobe, ix->plan.lut_bytes).total : 0);
     L.total = o;
     return L;
 }
@@ -316,6 +324,7 @@ rago_status rago_index_load(rago_index** out, const void* coarse_centroids, rago
     }
     for (int i = 0; i <= RAGO_NUM_STAGES && e == cudaSuccess; ++i) e = cudaEventCreate(&ix->ev[i]);
     if (e == cudaSuccess) { ix->ev_valid = 1; e = scan_plan(ix, &ix->plan); }
+    pair_list_stats(ix, off.data());
     if (e == cudaSuccess) e = launch_centroid_norms(coarse_centroids, ix->coarse_bf16, nlist, d, ix->cnorm, s);
     if (e == cudaSuccess) e = launch_transpose_codebook(pq_codebooks, M, ix->dsub, ix->cbT, s);
     if (e == cudaSuccess) e = launch_codeword_norms(pq_codebooks, M, ix->dsub, ix->cwmax, s);
@@ -456,19 +465,35 @@ rago_status rago_search(const rago_index* index, const float* queries, int32_t n
                                        (int)L.nslots, lead, reinterpret_cast<uint32_t*>(ws + L.err) + ERR_TICKET_WORD, &fp);
     st = run_coarse(ix, queries, nq, nprobe, ws, L, fused ? &fp : nullptr, kernel_clears, s);
     if (st != RAGO_OK) return st;
+    // Queries that share long lists are scanned two at a time: from here on the scan goes by the entries of that order.
+    PairView view;
+    const PairView* pv = nullptr;
+    const int32_t* scan_list = probe_list;
+    const float* scan_term = probe_term;
+    if (L.pairs) {
+        const PairLayout PL = pair_layout(nq, nprobe, ix->plan.lut_bytes);
+        uint8_t* pw = ws + L.pair;
+        e = launch_build_tables(ix, queries, nq, lut_img, lut_inv, reinterpret_cast<float*>(ws + L.lut_scale),
+                                reinterpret_cast<int32_t*>(pw + PL.ok), s);
+        if (e == cudaSuccess) e = launch_pair_queries(ix, probe_list, probe_term, nq, nprobe, lut_img, lut_inv, pw, PL, &view, s);
+        if (e != cudaSuccess) return cuda_fail(e, "pairing of queries");
+        pv = &view;
+        scan_list = reinterpret_cast<const int32_t*>(pw + PL.entry_list);
+        scan_term = reinterpret_cast<const float*>(pw + PL.entry_term);
+    }
     if (!fused) {
-        e = launch_plan_work(ix, probe_list, npairs, ix->plan.tile_vecs, lead, reinterpret_cast<int32_t*>(ws + L.pair_tiles),
+        e = launch_plan_work(ix, scan_list, npairs, ix->plan.tile_vecs, lead, pv, reinterpret_cast<int32_t*>(ws + L.pair_tiles),
                              work_prefix, qthresh, nq, slot_cnt, (int)L.nslots, queries, lut_img, lut_inv,
                              L.prebuilt ? reinterpret_cast<float*>(ws + L.lut_scale) : nullptr, s);
         if (e != cudaSuccess) return cuda_fail(e, "work planning");
     }
     record(mix, 3, s);
-    e = launch_scan(ix, ix->plan, queries, probe_list, probe_term, work_prefix, nq, nprobe, k, qthresh, slot_cnt,
-                    slot_keys, reinterpret_cast<uint32_t*>(ws + L.err), lut_img, lut_inv, s);
+    e = launch_scan(ix, ix->plan, queries, scan_list, scan_term, work_prefix, nq, nprobe, k, qthresh, slot_cnt,
+                    slot_keys, reinterpret_cast<uint32_t*>(ws + L.err), lut_img, lut_inv, pv, s);
     if (e != cudaSuccess) return cuda_fail(e, "scan kernel");
     record(mix, 4, s);
     e = launch_merge(ix, work_prefix, nq, nprobe, k, ix->plan.ctas, slot_cnt, slot_keys, qthresh, queries, probe_list, probe_term,
-                     out_ids, out_dists, s);
+                     pv, out_ids, out_dists, s);
     if (e != cudaSuccess) return cuda_fail(e, "merge kernel");
     record(mix, 5, s);
     return RAGO_OK;

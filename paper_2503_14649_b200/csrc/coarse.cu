@@ -855,7 +855,7 @@ __global__ void __launch_bounds__(SEL_THREADS) select_probes_kernel(
                 }
                 __syncthreads();
                 if (s_last) {
-                    plan_pairs_cta(probe_list, fp.offsets, fp.nq * nprobe, nprobe, fp.tile_vecs, fp.lead, fp.prefix, fp.qthresh, fp.nq,
+                    plan_pairs_cta(probe_list, fp.offsets, fp.nq * nprobe, nprobe, fp.tile_vecs, fp.lead, PairTiles{nullptr, 0, 0}, fp.prefix, fp.qthresh, fp.nq,
                                    fp.slot_cnt, fp.nslots, plan_sums);
                     if (tid == 0) *fp.ticket = 0u;
                 }

@@ -27,6 +27,7 @@ struct ScanPlan {
     size_t smem_bytes;
     // shared-memory image of a query's lookup table, as the scan variant of this index lays it out
     int lut_bytes, lut_banked, lut_copies, lut_copy_off, lut_stride;
+    int pair_tile_vecs;  // vectors per tile where two queries are scanned together, 0: not with this index
 };
 
 // Batches of at most this many queries get their lookup tables from kernels of their own, spread over the whole
@@ -64,6 +65,7 @@ struct IndexImpl {
     int tree_min_cand;                  // fewest (sum of the b1 smallest): nprobe must not exceed it
     int device, num_sms;
     ScanPlan plan;
+    float list_weight[33], list_square[33];  // by the bits of their length: the lists' share of the vectors, and sum of squared shares
     int profile;
     cudaEvent_t ev[RAGO_NUM_STAGES + 1];
     float last_ms[RAGO_NUM_STAGES];
@@ -154,6 +156,21 @@ __device__ __forceinline__ void fence_barrier_init() {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// shared::cluster address of the same shared-memory location in CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync_all() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t lds_cluster_u32(uint32_t cluster_addr) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_addr) : "memory");
+    return v;
+}
 
 // 1-D bulk copy global -> shared, completion counted in bytes on an mbarrier.
 // dst/src 16-byte aligned, bytes a positive multiple of 16.
@@ -288,24 +305,26 @@ cudaError_t launch_vector_terms(const IndexImpl* ix, float* vterm, cudaStream_t 
 cudaError_t launch_transpose_codebook(const float* cb, int M, int dsub, float* cbT, cudaStream_t s);
 int scan_query_lead(const IndexImpl* ix, int nq, int nprobe, int k);  // work units that stand for the start of a query
 bool scan_prefetches(const IndexImpl* ix, int64_t npairs);  // tiles are pulled into L2 ahead of their copies
-cudaError_t launch_plan_work(const IndexImpl* ix, const int32_t* probe_list, int npairs, int tile_vecs, int lead,
+struct PairView;
+int scan_pair_lead(const IndexImpl* ix);  // the same for a pair of queries
+cudaError_t launch_plan_work(const IndexImpl* ix, const int32_t* probe_list, int npairs, int tile_vecs, int lead, const PairView* view,
                              int32_t* pair_tiles, int64_t* work_prefix, unsigned long long* qthresh, int nq,
                              int32_t* slot_cnt, int nslots, const float* queries, uint8_t* lut_img, float* lut_inv,
                              float* lut_scale, cudaStream_t s);
 cudaError_t launch_scan(const IndexImpl* ix, const ScanPlan& plan, const float* queries, const int32_t* probe_list,
                         const float* probe_term, const int64_t* work_prefix, int nq, int nprobe, int k,
                         unsigned long long* qthresh, int32_t* slot_cnt, unsigned long long* slot_keys,
-                        uint32_t* err_word, const uint8_t* lut_img, const float* lut_inv, cudaStream_t s);
+                        uint32_t* err_word, const uint8_t* lut_img, const float* lut_inv, const PairView* view, cudaStream_t s);
 cudaError_t launch_codeword_norms(const float* codebooks, int M, int dsub, float* cwmax, cudaStream_t s);
 cudaError_t launch_build_tables(const IndexImpl* ix, const float* queries, int nq, uint8_t* lut_img, float* lut_inv,
-                                float* lut_scale, cudaStream_t s);
+                                float* lut_scale, int32_t* ok, cudaStream_t s);  // ok (may be null): the table's bound holds
 // no_alloc.cu
 cudaError_t noalloc_prepare();  // with the index's device current: look up (and make resident) the built-in scratch array
 // merge.cu
 cudaError_t launch_merge(const IndexImpl* ix, const int64_t* work_prefix, int nq, int nprobe, int k, int ctas,
                          const int32_t* slot_cnt, const unsigned long long* slot_keys, const unsigned long long* qthresh,
-                         const float* queries, const int32_t* probe_list, const float* probe_bias, int64_t* out_ids,
-                         float* out_dists, cudaStream_t s);
+                         const float* queries, const int32_t* probe_list, const float* probe_bias, const PairView* view,
+                         int64_t* out_ids, float* out_dists, cudaStream_t s);
 // flat.cu
 size_t flat_workspace_bytes(int64_t N, int d, int nq, int k);
 cudaError_t launch_selftest_final_selection(int32_t* counts, unsigned long long* entries, int nlists, int stride, int nq, int k,

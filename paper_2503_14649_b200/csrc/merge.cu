@@ -10,6 +10,7 @@
 // in the direct form  sum_j ((q_j - c_j) - cw_j)^2  (all terms non-negative: relative error about sqrt(d) ulps),
 // and the winners are re-ordered if any value changed.  On ordinary data no winner qualifies and the check costs
 // one 4-byte load per winner.
+#include "pair.cuh"
 #include "topk.cuh"
 
 namespace rago {
@@ -81,18 +82,23 @@ template <int THREADS>
 __global__ void __launch_bounds__(THREADS) merge_kernel(
     const int64_t* __restrict__ work_prefix, const int64_t* __restrict__ ids, int npairs, int nprobe, int k, int ctas,
     int metric, const int32_t* __restrict__ slot_cnt, const unsigned long long* __restrict__ slot_keys,
-    const unsigned long long* __restrict__ qthresh, const RescoreArgs rs,
-    int64_t* __restrict__ out_ids, float* __restrict__ out_dists) {
+    const unsigned long long* __restrict__ qthresh, const RescoreArgs rs, const int32_t* __restrict__ pair_head,
+    const int32_t* __restrict__ pair_order, int64_t* __restrict__ out_ids, float* __restrict__ out_dists) {
     __shared__ unsigned long long keys[TOPK_CAP];
     __shared__ int cnt;
     __shared__ int p_list[MAX_K];          // re-scoring: the query's probed lists and their storage ranges
     __shared__ uint32_t p_lo[MAX_K], p_hi[MAX_K];
     __shared__ int redo[MAX_K], redo_list[MAX_K];  // winners to score again (index into keys) and their lists
     __shared__ int nredo;
-    const int q = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     auto sync = [] { __syncthreads(); };
     grid_dependency_wait();
     grid_dependents_may_launch();
+    // a batch with pairs of queries: CTA i takes the query at position i of the scans' order
+    const int q = pair_head != nullptr ? pair_order[blockIdx.x] : blockIdx.x;
+    PairPlace pl;
+    if (pair_head != nullptr) pl = pair_place(blockIdx.x, pair_head[0], gridDim.x, nprobe, ctas);
+    else { pl.unit = q; pl.e0 = q * nprobe; pl.per_unit = nprobe; pl.e_base = 0; pl.e_end = npairs; pl.slot_base = 0; pl.slot_stride = 1; }
     if (tid == 0) { cnt = 0; nredo = 0; }
     if (rs.enabled) {
         for (int i = tid; i < nprobe; i += THREADS) {
@@ -103,14 +109,16 @@ __global__ void __launch_bounds__(THREADS) merge_kernel(
         }
     }
     __syncthreads();
-    const long long W = work_prefix[npairs];
-    const long long u0 = work_prefix[(size_t)q * nprobe], u1 = work_prefix[(size_t)(q + 1) * nprobe];
+    const long long W0 = pl.e_base ? work_prefix[pl.e_base] : 0, W = work_prefix[pl.e_end] - W0;
+    const long long u0 = work_prefix[pl.e0] - W0, u1 = work_prefix[pl.e0 + pl.per_unit] - W0;
     // a key above the threshold the scan CTAs agreed on is not among the k best (it is some CTA's k-th key)
     unsigned long long tau = qthresh[q];
     if (tau != KEY_MAX) ++tau;  // the threshold key itself is a result
     if (u1 > u0) {
-        const long long s0 = (long long)q + cta_of_unit(u0, W, ctas);
-        const int nslots = (int)((long long)q + cta_of_unit(u1 - 1, W, ctas) - s0) + 1;
+        const long long b0 = cta_of_unit(u0, W, ctas);
+        const int nslots = (int)(cta_of_unit(u1 - 1, W, ctas) - b0) + 1;
+        const long long s0 = pl.slot_base + (pl.unit + b0) * pl.slot_stride;
+        const int ss = pl.slot_stride;
         // Slot s holds slot_cnt[s] keys in ascending order.  First the leading m keys of every slot, about 2k keys
         // in all: the k-th smallest of them bounds the k-th smallest overall, and because every slot is a random
         // part of the query's work the bound is nearly tight.  Then the rest of the slots against that bound.
@@ -122,7 +130,7 @@ __global__ void __launch_bounds__(THREADS) merge_kernel(
             const int e = e0 + tid;
             unsigned long long key = KEY_MAX;
             if (e < total_a) {
-                const long long s = s0 + e / m;
+                const long long s = s0 + (long long)(e / m) * ss;
                 const int i = e % m;
                 if (i < slot_cnt[s]) key = slot_keys[(size_t)s * k + i];
             }
@@ -141,7 +149,7 @@ __global__ void __launch_bounds__(THREADS) merge_kernel(
             const int cnt_a = cnt;
             __syncthreads();
             for (int sl = warp; sl < nslots; sl += THREADS / 32) {
-                const long long s = s0 + sl;
+                const long long s = s0 + (long long)sl * ss;
                 const int c = slot_cnt[s];
                 for (int i0 = m; i0 < c; i0 += 32) {
                     const int i = i0 + lane;
@@ -164,7 +172,7 @@ __global__ void __launch_bounds__(THREADS) merge_kernel(
                         const int e = e0 + j * THREADS + tid;
                         mine[j] = KEY_MAX;
                         if (e < total_b) {
-                            const long long s = s0 + e / rem;
+                            const long long s = s0 + (long long)(e / rem) * ss;
                             const int i = m + e % rem;
                             if (i < slot_cnt[s]) mine[j] = slot_keys[(size_t)s * k + i];
                         }
@@ -396,8 +404,8 @@ __global__ void __launch_bounds__(1024) merge_small_kernel(
 
 cudaError_t launch_merge(const IndexImpl* ix, const int64_t* work_prefix, int nq, int nprobe, int k, int ctas,
                          const int32_t* slot_cnt, const unsigned long long* slot_keys, const unsigned long long* qthresh,
-                         const float* queries, const int32_t* probe_list, const float* probe_bias, int64_t* out_ids,
-                         float* out_dists, cudaStream_t s) {
+                         const float* queries, const int32_t* probe_list, const float* probe_bias, const PairView* view,
+                         int64_t* out_ids, float* out_dists, cudaStream_t s) {
     RescoreArgs rs;
     rs.enabled = ix->metric == RAGO_L2 && ix->vterm != nullptr && ix->d % 4 == 0 ? 1 : 0;
     rs.queries = queries; rs.centroids = ix->centroids; rs.coarse_bf16 = ix->coarse_bf16; rs.cbT = ix->cbT;
@@ -413,10 +421,11 @@ cudaError_t launch_merge(const IndexImpl* ix, const int64_t* work_prefix, int nq
                           ix->metric, slot_cnt, slot_keys, qthresh, rs, out_ids, out_dists);
     else if (nq <= 64)
         launch_overlapped(merge_kernel<1024>, dim3(nq), dim3(1024), 0, s, work_prefix, ix->ids, nq * nprobe, nprobe, k, ctas,
-                          ix->metric, slot_cnt, slot_keys, qthresh, rs, out_ids, out_dists);
+                          ix->metric, slot_cnt, slot_keys, qthresh, rs, nullptr, nullptr, out_ids, out_dists);
     else
         launch_overlapped(merge_kernel<256>, dim3(nq), dim3(256), 0, s, work_prefix, ix->ids, nq * nprobe, nprobe, k, ctas,
-                          ix->metric, slot_cnt, slot_keys, qthresh, rs, out_ids, out_dists);
+                          ix->metric, slot_cnt, slot_keys, qthresh, rs, view ? view->head : nullptr, view ? view->order : nullptr,
+                          out_ids, out_dists);
     count_launch();
     return cudaGetLastError();
 }

@@ -17,6 +17,13 @@ struct TableArgs {
     uint8_t* lut_img; float* lut_inv;
 };
 
+// Planning of a batch with pairs of queries (pair.cuh): head[0] pairs own the first 2 * nprobe * head[0] entries, whose tiles
+// and leads are those of the pairs' launch.  head null: a batch without.
+struct PairTiles {
+    const int32_t* head;
+    int tile_vecs, lead;
+};
+
 // What the probe-selection kernel needs to plan the scan of a small batch itself (enabled = 0: it does not).
 // The CTAs after the first nq build the lookup tables; the CTA that finishes its query last plans.
 struct FusedPlan {
@@ -55,6 +62,15 @@ __device__ __forceinline__ int tiles_of(long long len, int tile_vecs) {
 // Units in front of pair p's first tile on the line of work units (see scan_query_lead): those of a query's start, except
 // for the first query, whose start costs no CTA more than any other's first one.
 __device__ __forceinline__ int pair_lead(int p, int nprobe, int lead) { return lead != 0 && p > 0 && p % nprobe == 0 ? lead : 0; }
+
+// The same for entry p of a batch with pairs: each launch's units start at its own first entry.
+__device__ __forceinline__ int entry_lead(int p, int nprobe, int lead, const PairTiles& pt) {
+    const int e1 = 2 * nprobe * pt.head[0];
+    return p < e1 ? pair_lead(p, 2 * nprobe, pt.lead) : pair_lead(p - e1, nprobe, lead);
+}
+__device__ __forceinline__ int entry_tile_vecs(int p, int nprobe, int tile_vecs, const PairTiles& pt) {
+    return p < 2 * nprobe * pt.head[0] ? pt.tile_vecs : tile_vecs;
+}
 
 // Part `part` of `parts` of query q's table, by all threads of the CTA.  sm: d + M floats of shared memory.
 __device__ __forceinline__ void build_table_part(const TableArgs& t, int q, int part, int parts, float* sm) {
@@ -118,7 +134,7 @@ __device__ __forceinline__ void build_table_part(const TableArgs& t, int q, int 
 // of shared memory.  The probe lists may have been written by other CTAs of the same launch (the caller has ordered
 // those writes before this call): they are read past the L1 cache.
 __device__ __forceinline__ void plan_pairs_cta(const int32_t* probe_list, const int64_t* __restrict__ offsets, int npairs,
-                                               int nprobe, int tile_vecs, int lead, int64_t* __restrict__ prefix,
+                                               int nprobe, int tile_vecs, int lead, const PairTiles& pt, int64_t* __restrict__ prefix,
                                                unsigned long long* __restrict__ qthresh, int nq,
                                                int32_t* __restrict__ slot_cnt, int nslots, long long* warp_sums) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -133,14 +149,15 @@ __device__ __forceinline__ void plan_pairs_cta(const int32_t* probe_list, const 
         list[j] = __ldcg(probe_list + (p < npairs ? p : npairs - 1));
     }
 #pragma unroll
-    for (int j = 0; j < PLAN_PER_THREAD; ++j) {
-        first[j] = offsets[list[j]];
-        mine[j] = offsets[list[j] + 1];
+    for (int j = 0; j < PLAN_PER_THREAD; ++j) {  // (an unused entry of a pair: list -1, no vectors)
+        first[j] = offsets[list[j] < 0 ? 0 : list[j]];
+        mine[j] = list[j] < 0 ? first[j] : offsets[list[j] + 1];
     }
 #pragma unroll
     for (int j = 0; j < PLAN_PER_THREAD; ++j) {
         const int p = tid * PLAN_PER_THREAD + j;
-        mine[j] = p < npairs ? tiles_of(mine[j] - first[j], tile_vecs) + pair_lead(p, nprobe, lead) : 0;
+        if (pt.head == nullptr) mine[j] = p < npairs ? tiles_of(mine[j] - first[j], tile_vecs) + pair_lead(p, nprobe, lead) : 0;
+        else mine[j] = p < npairs ? tiles_of(mine[j] - first[j], entry_tile_vecs(p, nprobe, tile_vecs, pt)) + entry_lead(p, nprobe, lead, pt) : 0;
         v += mine[j];
     }
     long long incl = v;

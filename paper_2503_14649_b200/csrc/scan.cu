@@ -45,17 +45,22 @@
 // threshold of a query is shared between CTAs through global memory, which only ever removes keys that
 // cannot be among the k best, so the result does not depend on timing.
 //
+// Batches whose queries share long lists are scanned two queries at a time (DUAL; pair.cuh says how the answers stay the same
+// bits): one look-up then serves both, and the kernel below is the same but for what happens to the sums.
+//
 // A warp works on RGW row groups of 32 (virtual) rows per tile, unrolled, so that several independent
 // chains code word -> address -> table entry are in flight per warp; with R lanes per vector one
 // epilogue (term, bias, key, push) serves R row groups.
+#include <cstring>
 #include <type_traits>
 
 #include "topk.cuh"
 #include "plan.cuh"
+#include "pair.cuh"
 
 namespace rago {
 
-constexpr int MAX_STAGES = 4;
+constexpr int MAX_STAGES = 5;
 constexpr int SCAN_PF = 2;                  // tiles ahead of the one being copied that are prefetched into L2 (measured: 1-2 best)
 // Prefetch of a contiguous global range into L2 (16-byte aligned start, size a multiple of 16 bytes).
 __device__ __forceinline__ void l2_prefetch(const void* g, uint32_t bytes) {
@@ -65,15 +70,17 @@ constexpr int SMEM_OPTIN = 227 * 1024;          // dynamic shared memory asked f
 constexpr uint32_t SMEM_BASE_EXPECTED = 1024;   // shared-window address of dynamic shared memory when the kernel has no static part
 constexpr int CTRL_BYTES = 1024;
 
-struct TileDesc {
-    int32_t pair;      // index into probe_list (query * nprobe + rank), -1: the CTA has no tile
-    float term;        // the pair's (query, list) term of the score
-    uint32_t pos0;     // storage position of the tile's first vector
-    int32_t nvec;      // vectors in this tile
-    int32_t newpair;   // bit 0: first tile of this pair inside this CTA; bit 1: cut the candidate buffer before this tile; bit 2: last tile of the CTA
-    int32_t vrem;      // index of the first vector's term inside the staged term block (0..3)
+struct alignas(16) TileDesc {
+    int32_t flags;       // bit 0: first tile of this pair inside this CTA; bit 1: cut the candidate buffer before this tile; bit 2: last tile of the CTA;
+                         // two queries at a time: bit 3: cut the second query's buffer; bits 4, 5: the first, the second query probes this list
+                         // from bit 8: vectors in this tile; negative: the CTA has no tile
+    uint32_t pos0;       // storage position of the tile's first vector
     uint32_t tile_addr;  // shared address of the stage's code tile
-    uint32_t vt_addr;    // shared address of the stage's per-vector terms
+    uint32_t tile_hi;    // split tiles: what takes its place for the warps whose rows lie in the upper part
+    uint32_t vt_addr;    // shared address of the first vector's term
+    int32_t pair;        // index into probe_list (query * nprobe + rank)
+    float term;          // the pair's (query, list) term of the score
+    float term_b;        // two queries at a time: the second query's term
 };
 
 struct ScanArgs {
@@ -97,6 +104,7 @@ struct ScanArgs {
                              // table the next search's coarse step reads stays in L2
     int32_t prefetch;        // pull tiles into L2 ahead of their copies
     uint32_t dyn_bytes;
+    PairView pv;             // batches in which queries are scanned two at a time (pair.cuh); pv.head null: not this one
 };
 
 template <int WV, int G, int R, int NCW_, int RGW_>
@@ -118,11 +126,17 @@ struct Cfg {
     static constexpr int TILE_VROWS = NCW * 32 * RGW;
     static constexpr int TV = TILE_VROWS / R;           // vectors per tile
     static constexpr int TILE_BYTES = TILE_VROWS * MV;
+    // A 128 KB table leaves 63 KB below it and 36 KB above.  Two tiles of 15 x 32 rows of 96 bytes fit that space in two parts
+    // each: the rows of the first ten warps below, those of the others above (the candidate buffers then lie in unused
+    // columns of the table, see StripKeys).
+    static constexpr bool SPLIT = M == 96 && NCW == 15;
+    static constexpr int LOW_WARPS = SPLIT ? 10 : NCW;
+    static constexpr int LOW_BYTES = LOW_WARPS * 32 * RGW * MV, HIGH_BYTES = TILE_BYTES - LOW_BYTES;
     static constexpr int VT_BYTES = (TV + 4) * 4;       // staged per-vector terms (start rounded down to 16 bytes)
     static constexpr int KCAP = LUT_BYTES <= 65536 ? 2 * TOPK_CAP : TOPK_CAP;  // keys of the CTA's candidate buffer
     // Banked tables start at this absolute shared address (a multiple of 64 KB).  Two tiles of more than 48 KB do not
     // fit above a table at 64 KB, so configurations with such tiles keep their tiles below a table at 128 KB.
-    static constexpr uint32_t LUT_WINDOW = (NBANK == 1 && TILE_BYTES > 48 * 1024) ? 0x20000u : 0x10000u;
+    static constexpr uint32_t LUT_WINDOW = (NBANK == 1 && LOW_BYTES > 48 * 1024) ? 0x20000u : 0x10000u;
     static_assert(WV % G == 0, "virtual rows are whole blocks");
     static_assert(TILE_VROWS % R == 0, "tile must hold whole vectors");
     static_assert(RGW % (R < RGW ? R : RGW) == 0, "row groups are taken min(R, RGW) at a time");
@@ -133,7 +147,7 @@ struct Cfg {
     static_assert(MAX_K + SMAX * TV <= KCAP, "k kept keys plus the pushes of all tiles in flight must fit");
     static_assert(COPY_OFF % 32 == (COPIES == 2 ? 16 : 0), "second copy must sit 16 banks away");
     static_assert(LSTRIDE % 32 == 0 || BANKED, "table rows must keep bank = column mod 32");
-    static_assert(VT_BYTES % 16 == 0 && TILE_BYTES % 16 == 0, "bulk-copy destinations are 16-byte granular");
+    static_assert(VT_BYTES % 16 == 0 && LOW_BYTES % 16 == 0 && HIGH_BYTES % 16 == 0, "bulk-copy destinations are 16-byte granular");
     // banked addressing: the columns one lane touches in one block stay inside one 64-column bank
     __host__ __device__ static constexpr bool banked_ok() {
         for (int copy = 0; copy < COPIES; ++copy)
@@ -156,15 +170,36 @@ struct Cfg {
     }
 };
 
+// The candidate buffer of one of two queries that are scanned together, or of the one query where tiles are split.  Tables of
+// two banks leave no room for two buffers (or for one, beside larger tiles), but do not use all of their columns (96 of 128, or
+// two copies of 48): key i lies in the unused columns of a table row, ROW_KEYS keys to a row.  The copy of the next
+// table overwrites them, when the buffers are empty.
+template <class C>
+struct StripKeys {
+    static constexpr bool STRIP = C::NBANK == 2;
+    static constexpr int ROW_KEYS = C::M == 96 ? 16 : 8;
+    // the strips lie outside every copy of the table and hold KCAP keys
+    static constexpr bool FITS = C::BANKED && (!STRIP || (C::KCAP <= 2048 && ((C::M == 96 && C::NCOLS == 96) || (C::M == 48 && C::COPY_OFF == 80))));
+    uint8_t* p;
+    // lut: the table, lin: the linear buffers
+    __device__ __forceinline__ StripKeys(uint8_t* lut, uint8_t* lin, int side) {
+        if (!STRIP) p = lin + (size_t)side * C::KCAP * 8;
+        else if (C::M == 96) p = lut + 65536 + 128 + side * 32768;  // columns 32-63 of the second bank, half of its rows each
+        else p = side ? lut + 65536 : lut + 192;                    // columns 48-63 of the first bank, 0-15 of the second
+    }
+    __device__ __forceinline__ unsigned long long& operator[](int i) const {
+        return *reinterpret_cast<unsigned long long*>(STRIP ? p + (size_t)(i / ROW_KEYS) * 256 + (i % ROW_KEYS) * 8 : p + (size_t)i * 8);
+    }
+};
 // Absolute shared-memory addresses of everything the kernel keeps there.  The same function runs on
 // the host (to choose the number of stages, with the expected window base) and in the kernel (with
 // the real base); a plan that does not fit makes the kernel report an error and return.
 struct SmemPlan {
-    uint32_t lut, ctrl, keys, rT, vt[MAX_STAGES], tile[MAX_STAGES];
+    uint32_t lut, ctrl, keys, rT, vt[MAX_STAGES], tile[MAX_STAGES], high[MAX_STAGES];
     int ok;
 };
 
-template <class C>
+template <class C, bool DUAL>
 __host__ __device__ inline SmemPlan plan_smem(uint32_t base, uint32_t dyn_bytes, int d, int stages, bool need_vt) {
     SmemPlan p;
     p.ok = 1;
@@ -188,12 +223,15 @@ __host__ __device__ inline SmemPlan plan_smem(uint32_t base, uint32_t dyn_bytes,
         return base;
     };
     // largest pieces first, each below the table if it fits there, else above it
-    for (int s = 0; s < MAX_STAGES; ++s) p.tile[s] = s < stages ? take(C::TILE_BYTES, 128) : base;
-    p.keys = take(C::KCAP * 8, 16);
+    for (int s = 0; s < MAX_STAGES; ++s) p.tile[s] = s < stages ? take(C::LOW_BYTES, 128) : base;
+    for (int s = 0; s < MAX_STAGES; ++s) p.high[s] = C::SPLIT && s < stages ? take(C::HIGH_BYTES, 128) : base;
+    // two queries at a time: two buffers, side by side or in the columns of the table that nothing uses
+    constexpr bool strips = C::SPLIT || (DUAL && StripKeys<C>::STRIP);
+    p.keys = strips ? base : take(C::KCAP * (DUAL ? 16 : 8), 16);
     for (int s = 0; s < MAX_STAGES; ++s) p.vt[s] = (s < stages && need_vt) ? take(C::VT_BYTES, 16) : base;
     // The scaled, transposed query is only alive while a table is built, when the candidate buffer is empty: it
     // shares the buffer's space when it fits there.
-    p.rT = (uint32_t)d * 4 <= (uint32_t)C::KCAP * 8 ? p.keys : take((uint32_t)d * 4, 16);
+    p.rT = DUAL ? base : !strips && (uint32_t)d * 4 <= (uint32_t)C::KCAP * 8 ? p.keys : take((uint32_t)d * 4, 16);
     p.ctrl = take(CTRL_BYTES, 16);
     return p;
 }
@@ -206,8 +244,10 @@ struct Ctrl {
     unsigned long long empty[MAX_STAGES];
     unsigned long long cbar;  // consumer barrier
     unsigned long long lutbar;  // a prebuilt table has landed
+    uint32_t tile[MAX_STAGES], high[MAX_STAGES], vt[MAX_STAGES];  // the stages' places (SmemPlan's, which would go to local memory to be indexed)
     TileDesc desc[MAX_STAGES];
     int cnt;
+    int cnt_b;  // two queries at a time: keys in the second query's buffer
     uint32_t abort_flag;
     float red[32];  // per-warp maxima of the table build
     uint32_t redu[2][32];  // per-warp minima / maxima / counts of the buffer cut
@@ -344,25 +384,104 @@ struct ScanBlocks {
     }
 };
 
-template <int WV, int G, int R, int NCW_, int RGW_>
+// ---- making a buffer of bounds exact (pairs of queries) ----
+// Both steps are written for few registers: what they hold beside the tile loop's values goes to local memory, which, with
+// nearly all of the SM's cache being shared memory, means trips to L2 (with 100 to 200 bytes of it the loop took twice as long).
+
+// A table image in the place of the one in use, around the key buffers that lie in its unused columns; 16-byte asynchronous
+// copies, which take no registers (bulk copies of the rows' pieces took 8 to 16 us).  Called by all consumer threads after a barrier, followed by one.
+template <class C>
+__device__ __forceinline__ void dual_table(uint32_t lut, const uint8_t* src, int ctid) {
+    constexpr int PER_ROW = C::LUT_BYTES / 4096 - (StripKeys<C>::STRIP ? 8 : 0), TOTAL = KSUB * PER_ROW;
+    for (int i = ctid; i < TOTAL; i += C::NCT) {
+        uint32_t at = (uint32_t)i * 16u;
+        if (StripKeys<C>::STRIP) {  // 24 pieces to a row: 16 and 8, or 12 and 12
+            const uint32_t row = (uint32_t)i / PER_ROW, c = (uint32_t)i % PER_ROW;
+            if (C::M == 96) at = c < 16u ? row * 256u + c * 16u : 65536u + row * 256u + (c - 16u) * 16u;
+            else at = c < 12u ? row * 256u + c * 16u : 65536u + row * 256u + 64u + (c - 12u) * 16u;
+        }
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(lut + at), "l"(src + at) : "memory");
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+// First step, a thread per key: the bound in the upper word of a key is replaced by the sum of the terms of its list (found among
+// the unit's entries by the vector's position) and of the vector.
+template <class C>
+__device__ __forceinline__ void dual_terms(const StripKeys<C> kb, int kept, const float* terms, const uint2* ranges, int per_unit,
+                                           const float* vterm, bool ip, int ctid) {
+#pragma unroll 1
+    for (int i = ctid; i < kept; i += C::NCT) {
+        const uint32_t pos = (uint32_t)kb[i];
+        int at = 0;
+#pragma unroll 8
+        for (int e = 0; e < per_unit; ++e) {
+            const uint2 r = __ldg(ranges + e);
+            if (pos >= r.x && pos < r.y) at = e;
+        }
+        const float t = __ldg(terms + at), vt = vterm != nullptr ? __ldg(vterm + pos) : 0.f;
+        kb[i] = ((unsigned long long)__float_as_uint((ip ? -t : t) + vt) << 32) | pos;
+    }
+}
+// Second step, a warp to a few keys, lanes over sub-spaces: the entries of the query's own 32-bit table at `lut`, summed and scored as
+// the scan of one query does.
+template <class C>
+__device__ __forceinline__ void dual_exact(const StripKeys<C> kb, int kept, const uint8_t* codes, uint32_t lut, float inv, int ctid) {
+    constexpr int MP = (C::M + 31) / 32, UN = C::THREADS > 512 ? 4 : 8;
+    const int lane = ctid & 31;
+#pragma unroll 1
+    for (int i0 = ctid >> 5; i0 < kept; i0 += C::NCW * UN) {  // keys i0, i0 + NCW, ...
+        uint32_t code[UN];  // a lane's codes, one byte each
+#pragma unroll
+        for (int u = 0; u < UN; ++u) {
+            const uint32_t pos = (uint32_t)kb[i0 + u * C::NCW < kept ? i0 + u * C::NCW : i0];
+            code[u] = 0u;
+#pragma unroll
+            for (int j = 0; j < MP; ++j)
+                if (lane + 32 * j < C::M) code[u] |= (uint32_t)__ldg(codes + (size_t)pos * C::M + lane + 32 * j) << (8 * j);
+        }
+#pragma unroll
+        for (int u = 0; u < UN; ++u) {
+            int sum = 0;
+#pragma unroll
+            for (int j = 0; j < MP; ++j)  // bank = column mod 32 = lane
+                if (lane + 32 * j < C::M) sum += (int)lds_u32(lut + C::lut_off((int)((code[u] >> (8 * j)) & 0xFFu), lane + 32 * j));
+            sum = __reduce_add_sync(0xffffffffu, sum);
+            if (lane == 0 && i0 + u * C::NCW < kept) {
+                const unsigned long long key = kb[i0 + u * C::NCW];
+                kb[i0 + u * C::NCW] = make_key(__uint_as_float((uint32_t)(key >> 32)) + (float)sum * inv, (uint32_t)key);
+            }
+        }
+    }
+}
+
+// DUAL: every unit of work is a pair of queries (pair.cuh).
+template <int WV, int G, int R, int NCW_, int RGW_, bool DUAL>
 __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_kernel(const ScanArgs a) {
     using C = Cfg<WV, G, R, NCW_, RGW_>;
     constexpr int NCW = C::NCW, NCT = C::NCT;
+    static_assert(!DUAL || StripKeys<C>::FITS, "two candidate buffers");
     extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int S = a.stages;
     const uint32_t base = smem_u32(smem);
-    const SmemPlan P = plan_smem<C>(base, a.dyn_bytes, a.d, S, a.vterm != nullptr);
+    const SmemPlan P = plan_smem<C, DUAL>(base, a.dyn_bytes, a.d, S, a.vterm != nullptr);
     if (!P.ok) {  // uniform: every thread sees the same plan
         if (tid == 0) atomicExch(a.err, (uint32_t)ERR_SMEM_LAYOUT);
         return;
     }
     Ctrl* ctrl = reinterpret_cast<Ctrl*>(smem + (P.ctrl - base));
-    unsigned long long* keys = reinterpret_cast<unsigned long long*>(smem + (P.keys - base));
+    uint8_t* const lut_gen = smem + (P.lut - base);
+    auto make_keys = [&]() {
+        if constexpr (C::SPLIT) return StripKeys<C>(lut_gen, nullptr, 0);
+        else return reinterpret_cast<unsigned long long*>(smem + (P.keys - base));
+    };
+    const auto keys = make_keys();
     float* rT = reinterpret_cast<float*>(smem + (P.rT - base));
     volatile uint32_t* abort_flag = &ctrl->abort_flag;
 
     if (tid == 0) {
+#pragma unroll
+        for (int s = 0; s < MAX_STAGES; ++s) { ctrl->tile[s] = P.tile[s]; ctrl->high[s] = P.high[s]; ctrl->vt[s] = P.vt[s]; }
         for (int s = 0; s < S; ++s) {
             mbar_init(smem_u32(&ctrl->full[s]), 1);
             mbar_init(smem_u32(&ctrl->empty[s]), NCW);
@@ -370,6 +489,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
         mbar_init(smem_u32(&ctrl->cbar), NCW);
         mbar_init(smem_u32(&ctrl->lutbar), 1);
         ctrl->cnt = 0;
+        ctrl->cnt_b = 0;
         ctrl->abort_flag = 0;
         fence_barrier_init();
         fence_proxy_async();
@@ -385,7 +505,12 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
     // asked for.  With at most 32 pairs lane i of every warp reads pair i's first unit beside the total, so the
     // first pair follows from one vote; the producer warp reads the rest of every pair's description in the same
     // round trip (the offsets in a second one), and the consumers know their first query without the producer.
-    const bool few_pairs = a.npairs <= 32;
+    // (Not where the entries of the batch are divided between pairs and single queries.)
+    const bool few_pairs = !DUAL && a.npairs <= 32 && a.pv.head == nullptr;
+    // the entries this launch scans, and how many of them make a unit: a query, or a pair of queries
+    const int npairs_q = DUAL || a.pv.head != nullptr ? a.pv.head[0] : 0;
+    const int per_unit = DUAL ? 2 * a.nprobe : a.nprobe;
+    const int e_base = DUAL ? 0 : 2 * a.nprobe * npairs_q, e_end = DUAL ? 2 * a.nprobe * npairs_q : a.npairs;
     const long long pw = few_pairs ? a.work_prefix[lane < a.npairs ? lane : a.npairs] : 0;  // >= npairs: the total
     int c_list = 0; long long c_off = 0, c_len = 0, c_ws = 0, c_we = 0; float c_term = 0.f; int c_tv = C::TV;  // producer: lane i's cached pair
     if (few_pairs && warp == NCW && lane < a.npairs) {
@@ -396,9 +521,9 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
         c_len = a.list_offsets[c_list + 1] - c_off;
     }
     // This CTA's share of the work units: the tiles whose place on the line of units lies in [u_begin, u_end).
-    const long long W = a.work_prefix[a.npairs];
-    const long long u_begin = (long long)blockIdx.x * W / gridDim.x;
-    const long long u_end = (long long)(blockIdx.x + 1) * W / gridDim.x;
+    const long long W0 = e_base ? a.work_prefix[e_base] : 0, W = a.work_prefix[e_end];
+    const long long u_begin = W0 + (long long)blockIdx.x * (W - W0) / gridDim.x;
+    const long long u_end = W0 + (long long)(blockIdx.x + 1) * (W - W0) / gridDim.x;
     if (u_end <= u_begin) return;
     // few pairs: the pair whose range contains u_begin = the largest p with work_prefix[p] <= u_begin
     const int first_pair = few_pairs ? __popc(__ballot_sync(0xffffffffu, pw <= u_begin)) - 1 : -1;
@@ -406,7 +531,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
     if (warp == NCW) {
         // ================= producer warp =================
         // first pair whose range contains u_begin: largest p with work_prefix[p] <= u_begin
-        int lo = 0, hi = a.npairs;  // invariant: work_prefix[lo] <= u_begin < work_prefix[hi]
+        int lo = e_base, hi = e_end;  // invariant: work_prefix[lo] <= u_begin < work_prefix[hi]
         while (!few_pairs && hi - lo > 1) {  // 32 probes per step, evenly spaced: lane i looks at lo + (i + 1) * step
             const int step = (hi - lo + 31) / 32;
             const int pp = lo + (lane + 1) * step;
@@ -433,15 +558,18 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
             }
         };
         static_assert(C::TV % 32 == 0, "a rounded-up tile must not exceed the tile it was cut from");
+        float c_term_b = 0.f; int c_mask = 0;
         auto fill = [&]() {
             const int p = cache_base + lane;
-            if (p < a.npairs) {
+            if (p < e_end) {
                 c_list = a.probe_list[p];
+                if (DUAL && c_list < 0) c_list = 0;  // an unused entry: no tiles
                 c_off = a.list_offsets[c_list];
                 c_len = a.list_offsets[c_list + 1] - c_off;
-                c_ws = a.work_prefix[p] + pair_lead(p, a.nprobe, a.lead);  // place of its first tile
+                c_ws = a.work_prefix[p] + pair_lead(p - e_base, per_unit, a.lead);  // place of its first tile
                 c_we = a.work_prefix[p + 1];
                 c_term = a.probe_term[p];
+                if (DUAL) { c_term_b = a.pv.term_b[p]; c_mask = a.pv.mask[p]; }
             } else {
                 c_list = 0; c_off = 0; c_len = 0; c_ws = c_we = W; c_term = 0.f;
             }
@@ -467,7 +595,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
         };
         bool more = advance();
         if (!more && lane == 0) {  // a share without a tile: a descriptor with no copy says so
-            ctrl->desc[0].pair = -1;
+            ctrl->desc[0].flags = -1;
             mbar_arrive(smem_u32(&ctrl->full[0]));
         }
         for (int n = 0; more; ++n) {
@@ -478,6 +606,8 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
             const long long off = __shfl_sync(0xffffffffu, c_off, cur);
             const long long len = __shfl_sync(0xffffffffu, c_len, cur);
             const float term = __shfl_sync(0xffffffffu, c_term, cur);
+            const float term_b = DUAL ? __shfl_sync(0xffffffffu, c_term_b, cur) : 0.f;
+            const int mask = DUAL ? __shfl_sync(0xffffffffu, c_mask, cur) : 0;
             const int tv = __shfl_sync(0xffffffffu, c_tv, cur);
             const int pair = cache_base + cur;
             const long long t_in_pair = u - ws;
@@ -496,24 +626,39 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
             if (dead) break;
             if (lane == 0) {
                 TileDesc& D = ctrl->desc[st];
-                D.pair = pair;
-                D.term = term;
-                D.pos0 = pos0;
-                D.nvec = nvec;
                 // everything tiles n-S+1 .. n can still push must fit behind what is in the buffer now
                 const int cnt_seen = *reinterpret_cast<volatile int*>(&ctrl->cnt);
-                const int cut = cnt_seen + (S + 1) * C::TV > C::KCAP ? 2 : 0;
-                D.newpair = ((n == 0 || t_in_pair == 0) ? 1 : 0) | cut | (more ? 0 : 4);
-                D.vrem = (int32_t)(pos0 & 3u);
-                D.tile_addr = P.tile[st];
-                D.vt_addr = P.vt[st];
+                int flags = ((n == 0 || t_in_pair == 0) ? 1 : 0) | (cnt_seen + (S + 1) * C::TV > C::KCAP ? 2 : 0) | (more ? 0 : 4) | (nvec << 8);
+                if (DUAL) {
+                    const int seen_b = *reinterpret_cast<volatile int*>(&ctrl->cnt_b);
+                    flags |= (seen_b + (S + 1) * C::TV > C::KCAP ? 8 : 0) | (mask << 4);
+                    D.term_b = term_b;
+                }
+                const uint32_t tile_at = ctrl->tile[st], vt_at = ctrl->vt[st];
+                D.flags = flags;
+                D.pos0 = pos0;
+                D.tile_addr = tile_at;
+                D.vt_addr = vt_at + (pos0 & 3u) * 4u;
+                D.pair = pair;
+                D.term = term;
+                const uint8_t* src = a.codes + (size_t)pos0 * C::M;
+                uint32_t low = bytes;
                 mbar_arrive_expect_tx(bar, bytes + vbytes);
+                if constexpr (C::SPLIT) {
+                    const uint32_t high_at = ctrl->high[st];
+                    D.tile_hi = high_at - (uint32_t)C::LOW_BYTES;
+                    if (bytes > (uint32_t)C::LOW_BYTES) {
+                        low = (uint32_t)C::LOW_BYTES;
+                        if (a.stream_once) bulk_g2s_hint(high_at, src + low, bytes - low, bar, once_policy);
+                        else bulk_g2s(high_at, src + low, bytes - low, bar);
+                    }
+                }
                 if (a.stream_once) {  // small batch: the codes are read once and should leave L2 first
-                    bulk_g2s_hint(P.tile[st], a.codes + (size_t)pos0 * C::M, bytes, bar, once_policy);
-                    if (vbytes) bulk_g2s_hint(P.vt[st], a.vterm + (pos0 & ~3u), vbytes, bar, once_policy);
+                    bulk_g2s_hint(tile_at, src, low, bar, once_policy);
+                    if (vbytes) bulk_g2s_hint(vt_at, a.vterm + (pos0 & ~3u), vbytes, bar, once_policy);
                 } else {
-                    bulk_g2s(P.tile[st], a.codes + (size_t)pos0 * C::M, bytes, bar);
-                    if (vbytes) bulk_g2s(P.vt[st], a.vterm + (pos0 & ~3u), vbytes, bar);
+                    bulk_g2s(tile_at, src, low, bar);
+                    if (vbytes) bulk_g2s(vt_at, a.vterm + (pos0 & ~3u), vbytes, bar);
                 }
                 // pull the tiles a few steps ahead in this list into L2, with their terms, so that their copies find them there
                 if (a.prefetch) {
@@ -578,7 +723,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
         sel[t] = C::BANKED ? ((uint32_t)(4 + (t & 1)) | ((uint32_t)(t ^ xb) << 4) | 0x7600u)
                            : (0x4440u | (uint32_t)(t ^ xb));
 
-    int cur_q = -1;
+    int cur_u = -1, cur_q = -1;  // the unit the CTA is working on, and its query
     unsigned long long tau = KEY_MAX;
     float bias = 0.f;
     const int k = a.k;
@@ -601,11 +746,11 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
             // particular order.  Otherwise (or if ties leave too many) it is bisected, the score words re-read from
             // shared memory in every round.
             if (warp == 0) {
-                const uint32_t* kw = reinterpret_cast<const uint32_t*>(keys);  // score word of key i: kw[2 i + 1]
+                auto kw = [&](int i) { return reinterpret_cast<const uint32_t*>(&keys[i])[1]; };  // score word of key i
                 uint32_t lmn = 0xFFFFFFFFu, wmx = 0u;  // this lane's smallest score word, the largest of all
 #pragma unroll 4
                 for (int i = lane; i < n; i += 32) {
-                    const uint32_t o = kw[2 * i + 1];
+                    const uint32_t o = kw(i);
                     lmn = o < lmn ? o : lmn;
                     wmx = o > wmx ? o : wmx;
                 }
@@ -627,7 +772,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
                         const uint32_t mid = (uint32_t)(lo + (hi - lo) / 2);
                         uint32_t c = 0;
 #pragma unroll 4
-                        for (int i = lane; i < nn; i += 32) c += kw[2 * i + 1] <= mid ? 1u : 0u;
+                        for (int i = lane; i < nn; i += 32) c += kw(i) <= mid ? 1u : 0u;
                         c = __reduce_add_sync(0xffffffffu, c);
                         if (c < (uint32_t)k) lo = mid; else { hi = mid; c_hi = c; }
                     }
@@ -740,9 +885,10 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
             if (dead) return;
         }
         if (kept == k && ctid == 0) atomicMin(&a.qthresh[cur_q], keys[k - 1]);
-        const size_t slot = (size_t)cur_q + blockIdx.x;
+        const size_t slot = (a.pv.head != nullptr ? 2 * ((size_t)npairs_q + gridDim.x) : 0) + cur_u + blockIdx.x;
         for (int i = ctid; i < kept; i += NCT) a.slot_keys[slot * k + i] = keys[i];
         if (ctid == 0) a.slot_cnt[slot] = kept;
+        if (C::SPLIT) fence_proxy_async();  // the next table's copy writes where keys were written and read
         csync();
     };
 
@@ -750,7 +896,9 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
     // Small k: once the first tiles of a query have put a hundred-odd keys into the buffer it is cut at once (cheap at
     // that length), so that the tiles that follow are pushed against a threshold instead of in full.
     bool early = false;
-    auto begin_query = [&](int q) {
+    auto begin_query = [&](int unit) {
+        const int q = a.pv.head != nullptr ? a.pv.order[2 * npairs_q + unit] : unit;
+        cur_u = unit;
         cur_q = q;
         early = k <= 32;
         if (a.lut_img != nullptr) {  // the table was built ahead of the scan: fetch its shared-memory image
@@ -803,34 +951,218 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
         csync();
     };
 
+    // ---- two queries at a time (pair.cuh): their buffers hold keys of lower bounds until a query is closed ----
+    int dq[2] = {0, 0}, dbase[2] = {0, 0}, dshift[2] = {0, 0};
+    float dinv[2] = {1.f, 1.f}, dunit[2] = {1.f, 1.f}, dbias[2] = {0.f, 0.f}, dlimit[2];
+    unsigned long long dtau[2] = {KEY_MAX, KEY_MAX};
+    bool duse[2] = {false, false};
+    dlimit[0] = dlimit[1] = 0.f;
+    auto dual_keys = [&](int side) { return StripKeys<C>(lut_gen, smem + (P.keys - base), side); };
+    // Limits of the scan's first test.  A bound is  bias + vt + (base + half * 2^s) * inv  up to its roundings, the test's left side
+    // is  x = (2^23 + half) * unit + vt  with unit = 2^s * inv, so a bound at or below the threshold's score t has
+    // x <= t - bias - base * inv + 2^23 * unit, up to roundings of both that lie below 2^-20 of the sum of all magnitudes (that
+    // of vt is at most that of the others together where the two sides are close).  No threshold yet: t is NaN, and so is the
+    // limit, which nothing is above.  A list that the query does not probe: nothing passes.
+    auto dual_limits = [&]() {
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {
+            const double t = (double)orderable_f32((uint32_t)(dtau[side] >> 32)), b = (double)dbias[side];
+            const double base = (double)dbase[side] * (double)dinv[side], top = 8388608.0 * (double)dunit[side];
+            const double lim = t - b - base + top;
+            dlimit[side] = duse[side] ? __double2float_ru(lim + (fabs(t) + fabs(b) + fabs(base) + 2.0 * top) * 0x1p-20) : -__int_as_float(0x7f800000);
+        }
+    };
+    // Cuts the buffers of the sides in `sides` (bits), or closes both.  One body for both, called from one place: its size counts.
+    //
+    // A cut is that of cut_buffer on the bounds.  The k-th smallest bound T does not bound the k-th best score, but the score
+    // of a vector whose bound is at most T is at most T + M (2^s - 1) units and the roundings of the three operations, all of
+    // which lie below 2^-22 of the value and 128 units: everything up to that is kept, and it is the new threshold.  If
+    // that is more than the buffer can hold beside the tiles in flight (coarse shifts, equal codes), or the query is closed,
+    // the keys are replaced by those of the exact scores - entries of the query's own 32-bit table, which takes the place of
+    // the pair's, summed and scored as the scan of one query does, a few keys to a warp at a time, lanes over sub-spaces - and
+    // cut to k.  (Gathered from the table in global memory, which the codes have pushed out of L2 by then, the entries
+    // of about 250 keys took 75 us a query.)
+    auto dual_settle = [&](int sides, bool close) {
+        constexpr int KPT = (C::KCAP + NCT - 1) / NCT;
+        csync();
+        if (dead) return;
+#pragma unroll 1
+        for (int side = 0; side < 2; ++side) {
+            if (!((sides >> side) & 1)) continue;
+            const StripKeys<C> kb = dual_keys(side);
+            int* cn = side ? &ctrl->cnt_b : &ctrl->cnt;
+            const int q = side ? dq[1] : dq[0];
+            const float inv = side ? dinv[1] : dinv[0];
+            const int n = *cn < C::KCAP ? *cn : C::KCAP;
+            // closing: cutting first costs less than the exact scores it saves
+            const bool cut = n > (close ? k + (k >> 2) + WARP_SORT_MAX : k);
+            unsigned long long bound = KEY_MAX;
+            if (cut) {  // uniform
+                unsigned long long mine[KPT];
+                uint32_t mn = 0xFFFFFFFFu, mx = 0u;
+#pragma unroll
+                for (int j = 0; j < KPT; ++j) {
+                    const int i = ctid + j * NCT;
+                    mine[j] = i < n ? kb[i] : KEY_MAX;
+                    if (i < n) {
+                        const uint32_t o = (uint32_t)(mine[j] >> 32);
+                        mn = o < mn ? o : mn;
+                        mx = o > mx ? o : mx;
+                    }
+                }
+                mn = __reduce_min_sync(0xffffffffu, mn);
+                mx = __reduce_max_sync(0xffffffffu, mx);
+                if (lane == 0) { ctrl->redu[0][warp] = mn; ctrl->redu[1][warp] = mx; }
+                csync();
+                if (dead) return;
+                for (int w = 0; w < NCW; ++w) {
+                    mn = ctrl->redu[0][w] < mn ? ctrl->redu[0][w] : mn;
+                    mx = ctrl->redu[1][w] > mx ? ctrl->redu[1][w] : mx;
+                }
+                if (ctid == 0) *cn = 0;  // every thread holds its keys in registers
+                csync();
+                if (dead) return;
+                long long lo = (long long)mn - 1, hi = mx;  // #(score <= lo) < k <= #(score <= hi)
+                uint32_t c_hi = (uint32_t)n;
+                const uint32_t want_max = (uint32_t)(k + (close ? k >> 3 : k >> 1) + 8);
+                int round = 0;
+                while (hi - lo > 1 && c_hi > want_max) {  // uniform across the CTA
+                    const uint32_t mid = bisect_mid(lo, hi, round);
+                    uint32_t c = 0;
+#pragma unroll
+                    for (int j = 0; j < KPT; ++j) c += (mine[j] != KEY_MAX && (uint32_t)(mine[j] >> 32) <= mid) ? 1u : 0u;
+                    c = __reduce_add_sync(0xffffffffu, c);
+                    if (lane == 0) ctrl->redu[round & 1][warp] = c;
+                    csync();
+                    if (dead) return;
+                    c = 0;
+                    for (int w = 0; w < NCW; ++w) c += ctrl->redu[round & 1][w];
+                    if (c < (uint32_t)k) lo = mid; else { hi = mid; c_hi = c; }
+                    ++round;
+                }
+                const double t = (double)orderable_f32((uint32_t)hi);
+                const double slack = ((double)C::M * (double)((1u << (side ? dshift[1] : dshift[0])) - 1u) + 128.0) * (double)inv;
+                const uint32_t T = f32_orderable(__double2float_ru(t + slack + (fabs(t) + slack) * 0x1p-22));
+#pragma unroll
+                for (int j = 0; j < KPT; ++j)
+                    warp_push(kb, cn, mine[j] != KEY_MAX && (uint32_t)(mine[j] >> 32) <= T, mine[j], C::KCAP);
+                bound = ((unsigned long long)T << 32) | 0xFFFFFFFFull;  // >= the k-th best key
+                csync();
+                if (dead) return;
+            }
+            int kept = *cn;
+            if (close || kept > C::KCAP - (S + 1) * C::TV) {  // uniform
+                const size_t eb = (size_t)e_base + (size_t)cur_u * per_unit;
+                dual_terms<C>(kb, kept, (side ? a.pv.term_b : a.probe_term) + eb, a.pv.range + (side ? (size_t)a.npairs : 0) + eb, per_unit, a.vterm, ip, ctid);
+                dual_table<C>(P.lut, a.lut_img + (size_t)q * C::LUT_BYTES, ctid);  // in the place of the pair's
+                csync();
+                if (dead) return;
+                dual_exact<C>(kb, kept, a.codes, P.lut, inv, ctid);
+                csync();
+                if (dead) return;
+                if (kept > 1) {
+                    kept = block_select_short<2 * RANK_MAX>(kb, cn, k, ctid, NCT, csync, C::KCAP);
+                    if (dead) return;
+                }
+                if (kept == k) bound = kb[k - 1];
+                if (!close) {
+                    dual_table<C>(P.lut, a.pv.img + (size_t)cur_u * C::LUT_BYTES, ctid);
+                }
+                if (close) {
+                    const size_t slot = 2 * ((size_t)cur_u + blockIdx.x) + side;
+                    for (int i = ctid; i < kept; i += NCT) a.slot_keys[slot * k + i] = kb[i];
+                    if (ctid == 0) a.slot_cnt[slot] = kept;
+                }
+            }
+            if (ctid == 0 && bound != KEY_MAX) atomicMin(&a.qthresh[q], bound);
+            if (side) { if (bound < dtau[1]) dtau[1] = bound; } else { if (bound < dtau[0]) dtau[0] = bound; }
+        }
+        if (!close) {
+#pragma unroll
+            for (int side = 0; side < 2; ++side) {
+                const unsigned long long g = *reinterpret_cast<volatile unsigned long long*>(&a.qthresh[dq[side]]);
+                if (g < dtau[side]) dtau[side] = g;
+            }
+        }
+        fence_proxy_async();  // strips: the next table's copy writes where keys were written and read
+        csync();
+    };
+    auto dual_begin = [&](int unit) {
+        cur_u = unit;
+        if (ctid == 0) {
+            ctrl->cnt = 0;
+            ctrl->cnt_b = 0;
+            fence_proxy_async();
+            const uint8_t* src = a.pv.img + (size_t)unit * C::LUT_BYTES;
+            const uint32_t bar = smem_u32(&ctrl->lutbar);
+            mbar_arrive_expect_tx(bar, (uint32_t)C::LUT_BYTES);
+            constexpr uint32_t PIECE = 32768;
+            for (uint32_t o = 0; o < (uint32_t)C::LUT_BYTES; o += PIECE)
+                bulk_g2s(P.lut + o, src + o, (uint32_t)C::LUT_BYTES - o < PIECE ? (uint32_t)C::LUT_BYTES - o : PIECE, bar);
+        }
+        const PairParams* pp = a.pv.params + unit;
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {
+            dq[side] = pp->q[side]; dbase[side] = pp->base[side]; dshift[side] = pp->shift[side]; dinv[side] = pp->inv[side];
+            dunit[side] = dinv[side] * (float)(1u << dshift[side]);
+        }
+#pragma unroll
+        for (int side = 0; side < 2; ++side) dtau[side] = *reinterpret_cast<volatile unsigned long long*>(&a.qthresh[dq[side]]);
+        dead = dead || !mbar_wait(smem_u32(&ctrl->lutbar), lphase, abort_flag, a.err);
+        lphase ^= 1u;
+        csync();
+    };
+
     // few pairs: the first query is known without the producer, so its table is fetched while the first tile is
     // still on its way (the tile loop finds cur_q set and goes straight to the scan)
     if (few_pairs) begin_query(first_pair / a.nprobe);
     int cst = 0;            // n % S and the parity of n / S, kept by counting
     uint32_t cparity = 0;
-    for (bool last = false; !last && !dead;) {
+    for (bool last = false; (DUAL || !last) && !dead;) {
         const int st = cst;
-        const uint32_t parity = cparity;
-        if (++cst == S) { cst = 0; cparity ^= 1u; }
-        dead = dead || !mbar_wait(smem_u32(&ctrl->full[st]), parity, abort_flag, a.err);
-        if (dead) break;
-        const TileDesc D = ctrl->desc[st];
-        if (D.pair < 0) break;
-        last = (D.newpair & 4) != 0;
-        if (D.newpair & 1) {
-            const int q = D.pair / a.nprobe;
-            if (q != cur_q) {
-                if (cur_q >= 0) finalize();
+        const bool end = DUAL && last;  // pairs: one more round closes the last one
+        TileDesc D;
+        if (!end) {
+            const uint32_t parity = cparity;
+            if (++cst == S) { cst = 0; cparity ^= 1u; }
+            dead = dead || !mbar_wait(smem_u32(&ctrl->full[st]), parity, abort_flag, a.err);
+            if (dead) break;
+            D = ctrl->desc[st];
+            if (D.flags < 0) break;
+            last = (D.flags & 4) != 0;
+        }
+        if constexpr (DUAL) {
+            int unit = cur_u;
+            if (!end && (D.flags & 1)) {
+                unit = (D.pair - e_base) / per_unit;
+                dbias[0] = ip ? -D.term : D.term;
+                dbias[1] = ip ? -D.term_b : D.term_b;
+                duse[0] = (D.flags & 16) != 0;
+                duse[1] = (D.flags & 32) != 0;
+            }
+            const bool close = cur_u >= 0 && (end || unit != cur_u);
+            const int sides = close ? 3 : (end || unit != cur_u ? 0 : ((D.flags >> 1) & 1) | ((D.flags >> 2) & 2));
+            if (sides) dual_settle(sides, close);
+            if (dead || end) break;
+            if (unit != cur_u) {
+                dual_begin(unit);
                 if (dead) break;
-                begin_query(q);
+            }
+            if (sides || (D.flags & 1)) dual_limits();
+        } else if (D.flags & 1) {
+            const int unit = (D.pair - e_base) / per_unit;
+            if (unit != cur_u) {
+                if (cur_u >= 0) finalize();
+                if (dead) break;
+                begin_query(unit);
                 if (dead) break;
             }
             bias = ip ? -D.term : D.term;
         }
         // the producer saw the buffer filling up, or (small k) this is the query's second tile in this CTA: keep the
         // best k (or a few more), lower the threshold.  One site for both, so that the cut is in the loop once.
-        const bool full_cut = (D.newpair & 2) != 0;
-        if (full_cut || (early && !(D.newpair & 1))) {
+        const bool full_cut = (D.flags & 2) != 0;
+        if (!DUAL && (full_cut || (early && !(D.flags & 1)))) {
             csync();
             if (dead) break;
             if (ctrl->cnt > (full_cut ? k : 2 * WARP_SORT_MAX)) {  // uniform: nothing is pushed between the two barriers
@@ -845,9 +1177,9 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
         }
 
         // ---- scan this tile: warp w owns row groups w*RGW .. w*RGW+RGW-1 ----
-        const int nvr = D.nvec * R;
-        const uint32_t tile_base = D.tile_addr;
-        const uint32_t vt_base = D.vt_addr + (uint32_t)D.vrem * 4u;
+        const int nvr = (D.flags >> 8) * R;
+        const uint32_t tile_base = C::SPLIT && warp >= C::LOW_WARPS ? D.tile_hi : D.tile_addr;
+        const uint32_t vt_base = D.vt_addr;
         // Row groups are taken MERGE at a time: with R lanes per vector every lane of an R-group ends up with
         // the vector's sum, so lane slice g finishes row group g and one epilogue serves MERGE row groups.
         constexpr int MERGE = R < C::RGW ? R : C::RGW;
@@ -878,7 +1210,6 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
             if constexpr (MERGE >= 3) group(std::integral_constant<int, 2>{});
             if constexpr (MERGE >= 4) group(std::integral_constant<int, 3>{});
             const int vr = vr0 + (MERGE == 1 ? 0 : sr * 32) + lane;  // the virtual row whose vector this lane finishes
-            const float s = (float)mine * inv_scale;
             // per-vector term of the L2 expansion (0 for inner product); rows past the tile's end read
             // stale but in-bounds shared memory and are never pushed
             const float vt = a.vterm != nullptr ? lds_f32(vt_base + (uint32_t)(vr / R) * 4u) : 0.f;
@@ -889,10 +1220,29 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
                 if (lane == 0) mbar_arrive(smem_u32(&ctrl->empty[st]));
                 released = true;
             }
-            const float score = (bias + vt) + s;  // smaller is better for both metrics
-            const unsigned long long key = make_key(score, D.pos0 + (uint32_t)(vr / R));
             const bool owner = MERGE == 1 ? sr == 0 : sr < MERGE;
-            warp_push(keys, &ctrl->cnt, vr < nvr && owner && key < tau, key, C::KCAP);
+            const uint32_t pos = D.pos0 + (uint32_t)(vr / R);
+            if constexpr (DUAL) {
+                // The two halves of the sum are lower bounds.  Most are above the threshold's score, which this shows in three
+                // instructions a side: 2^23 + half as a float (its bits are 0x4B00 and the half), times the unit, plus the
+                // vector's term, against the limit that dual_limits has made of all the rest.
+                const float xa = fmaf(__uint_as_float(__byte_perm((uint32_t)mine, 0x4B00u, 0x5410u)), dunit[0], vt);
+                const float xb = fmaf(__uint_as_float(__byte_perm((uint32_t)mine, 0x4B00u, 0x5432u)), dunit[1], vt);
+                const bool live = vr < nvr && owner;
+                const bool pa = live && !(xa > dlimit[0]), pb = live && !(xb > dlimit[1]);
+                if (__any_sync(0xffffffffu, pa || pb)) {
+                    const float sa = (float)(dbase[0] + (int)(((uint32_t)mine & 0xFFFFu) << dshift[0])) * dinv[0];
+                    const float sb = (float)(dbase[1] + (int)(((uint32_t)mine >> 16) << dshift[1])) * dinv[1];
+                    const unsigned long long key_a = make_key((dbias[0] + vt) + sa, pos), key_b = make_key((dbias[1] + vt) + sb, pos);
+                    warp_push(dual_keys(0), &ctrl->cnt, pa && duse[0] && key_a < dtau[0], key_a, C::KCAP);
+                    warp_push(dual_keys(1), &ctrl->cnt_b, pb && duse[1] && key_b < dtau[1], key_b, C::KCAP);
+                }
+            } else {
+                const float s = (float)mine * inv_scale;
+                const float score = (bias + vt) + s;  // smaller is better for both metrics
+                const unsigned long long key = make_key(score, pos);
+                warp_push(keys, &ctrl->cnt, vr < nvr && owner && key < tau, key, C::KCAP);
+            }
             return true;
         };
         static_assert(C::RGW / MERGE <= 4, "passes are written out below");
@@ -905,7 +1255,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
             if (lane == 0) mbar_arrive(smem_u32(&ctrl->empty[st]));
         }
     }
-    if (!dead && cur_q >= 0) finalize();
+    if constexpr (!DUAL) { if (!dead && cur_u >= 0) finalize(); }
 }
 
 // ---- host side ----------------------------------------------------------------------------------
@@ -916,15 +1266,15 @@ struct Variant {
     int (*stages_for)(int d, bool need_vt);
     int lut_bytes, lut_banked, lut_copies, lut_copy_off, lut_stride;
 };
-template <class C>
+template <class C, bool DUAL>
 static int stages_for(int d, bool need_vt) {
     for (int s = C::SMAX; s >= 2; --s)
-        if (plan_smem<C>(SMEM_BASE_EXPECTED, SMEM_OPTIN, d, s, need_vt).ok) return s;
+        if (plan_smem<C, DUAL>(SMEM_BASE_EXPECTED, SMEM_OPTIN, d, s, need_vt).ok) return s;
     return 0;
 }
-#define RAGO_VARIANT(WV, G, R, NCW, RGW) \
-    { Cfg<WV, G, R, NCW, RGW>::M, scan_kernel<WV, G, R, NCW, RGW>, Cfg<WV, G, R, NCW, RGW>::THREADS, \
-      Cfg<WV, G, R, NCW, RGW>::TV, stages_for<Cfg<WV, G, R, NCW, RGW>>, Cfg<WV, G, R, NCW, RGW>::LUT_BYTES, \
+#define RAGO_VARIANT(WV, G, R, NCW, RGW, DUAL) \
+    { Cfg<WV, G, R, NCW, RGW>::M, scan_kernel<WV, G, R, NCW, RGW, DUAL>, Cfg<WV, G, R, NCW, RGW>::THREADS, \
+      Cfg<WV, G, R, NCW, RGW>::TV, stages_for<Cfg<WV, G, R, NCW, RGW>, DUAL>, Cfg<WV, G, R, NCW, RGW>::LUT_BYTES, \
       Cfg<WV, G, R, NCW, RGW>::BANKED ? 1 : 0, Cfg<WV, G, R, NCW, RGW>::COPIES, Cfg<WV, G, R, NCW, RGW>::COPY_OFF, \
       Cfg<WV, G, R, NCW, RGW>::LSTRIDE }
 // Warps x unrolled row groups per warp were chosen by measurement: independent row groups in flight inside a warp
@@ -933,18 +1283,32 @@ static int stages_for(int d, bool need_vt) {
 // M = 48: +6%, M = 64: +4.5%).  Where a code size has two entries the first one whose shared-memory plan fits the
 // index (dimension, metric) is taken.
 static const Variant kVariants[] = {
-    RAGO_VARIANT(4, 4, 1, 16, 2),   // M = 16
-    RAGO_VARIANT(8, 8, 1, 15, 2),   // M = 32
-    RAGO_VARIANT(12, 4, 1, 15, 1),  // M = 48 (two table copies: 128 KB, a 2 048-key buffer, tiles of at most 512 vectors)
-    RAGO_VARIANT(8, 8, 2, 15, 4),   // M = 64: 15 + 1 warps fill the four schedulers evenly; two 60 KB tiles below the table
-    RAGO_VARIANT(8, 8, 2, 12, 4),   // M = 64 where those do not fit
-    RAGO_VARIANT(20, 4, 1, 8, 1),   // M = 80
-    RAGO_VARIANT(24, 8, 1, 12, 1),  // M = 96
-    RAGO_VARIANT(8, 8, 4, 12, 3),   // M = 128
+    RAGO_VARIANT(4, 4, 1, 16, 2, false),   // M = 16
+    RAGO_VARIANT(8, 8, 1, 15, 2, false),   // M = 32
+    RAGO_VARIANT(12, 4, 1, 15, 1, false),  // M = 48 (two table copies: 128 KB, a 2 048-key buffer, tiles of at most 512 vectors)
+    RAGO_VARIANT(8, 8, 2, 15, 4, false),   // M = 64: 15 + 1 warps fill the four schedulers evenly; two 60 KB tiles below the table
+    RAGO_VARIANT(8, 8, 2, 12, 4, false),   // M = 64 where those do not fit
+    RAGO_VARIANT(20, 4, 1, 8, 1, false),   // M = 80
+    RAGO_VARIANT(24, 8, 1, 15, 1, false),  // M = 96: split tiles
+    RAGO_VARIANT(24, 8, 1, 12, 1, false),  // M = 96 where those do not fit
+    RAGO_VARIANT(8, 8, 4, 12, 3, false),   // M = 128
+};
+// The same table layouts for pairs of queries (the tables of 80 and 128 bytes leave no room for two buffers).
+static const Variant kPairVariants[] = {
+    RAGO_VARIANT(4, 4, 1, 15, 2, true),    // M = 16: 16 warps and the producer would leave 96 registers a thread, too few
+    RAGO_VARIANT(8, 8, 1, 15, 2, true),
+    RAGO_VARIANT(12, 4, 1, 15, 1, true),
+    RAGO_VARIANT(8, 8, 2, 15, 2, true),    // M = 64: the tiles in flight have to fit each buffer twice over
+    RAGO_VARIANT(24, 8, 1, 15, 1, true),
 };
 
 static const Variant* find_variant(int M, int d, bool need_vt) {
     for (const Variant& v : kVariants)
+        if (v.M == M && v.stages_for(d, need_vt) >= 2) return &v;
+    return nullptr;
+}
+static const Variant* find_pair_variant(int M, int d, bool need_vt) {
+    for (const Variant& v : kPairVariants)
         if (v.M == M && v.stages_for(d, need_vt) >= 2) return &v;
     return nullptr;
 }
@@ -965,6 +1329,12 @@ cudaError_t scan_plan(const IndexImpl* ix, ScanPlan* plan) {
     plan->smem_bytes = SMEM_OPTIN;
     plan->lut_bytes = v->lut_bytes; plan->lut_banked = v->lut_banked; plan->lut_copies = v->lut_copies;
     plan->lut_copy_off = v->lut_copy_off; plan->lut_stride = v->lut_stride;
+    const Variant* pv = find_pair_variant(ix->M, ix->d, ix->metric != RAGO_IP);
+    plan->pair_tile_vecs = pv ? pv->tile_vecs : 0;
+    if (pv) {
+        const cudaError_t e = cudaFuncSetAttribute(pv->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_OPTIN);
+        if (e != cudaSuccess) return e;
+    }
     return cudaFuncSetAttribute(v->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_OPTIN);
 }
 
@@ -988,6 +1358,13 @@ int scan_query_lead(const IndexImpl* ix, int nq, int nprobe, int k) {
     return (int64_t)nq * nprobe * tiles_per_list >= (int64_t)lead * ix->plan.ctas ? lead : 0;
 }
 
+// The start of a pair of queries: two buffers are closed (cut, made exact, ranked: about 90 000 cycles in all) and filled again.
+// (1 024 queries, 96 bytes: with 30 us the CTAs of the short lists, 18 closes each, ended 12% after the others.)
+int scan_pair_lead(const IndexImpl* ix) {
+    const float tile_us = (float)(ix->plan.pair_tile_vecs * ix->M) / 36000.f;
+    return (int)(60.f / tile_us + 0.5f);
+}
+
 // Prefetching into L2 pays where the tiles in flight are small (a copy from DRAM takes longer than the tile in front
 // of it is scanned) and the batch does not meet each list several times, which brings most tiles from L2 anyway and
 // makes the prefetches only extra traffic.  Without / with, us per call: 48-byte codes, 2.3 probes per list
@@ -1003,11 +1380,13 @@ bool scan_prefetches(const IndexImpl* ix, int64_t npairs) {
     return (tile_bytes <= 40 * 1024 && npairs <= 4ll * ix->nlist) || (ix->M >= 48 && tile_bytes <= 24 * 1024 && long_lists);
 }
 
+// view (may be null): the batch's pairs of queries, scanned by a launch of their own in front of that of the single ones.
 cudaError_t launch_scan(const IndexImpl* ix, const ScanPlan& plan, const float* queries, const int32_t* probe_list,
                         const float* probe_term, const int64_t* work_prefix, int nq, int nprobe, int k,
                         unsigned long long* qthresh, int32_t* slot_cnt, unsigned long long* slot_keys,
-                        uint32_t* err_word, const uint8_t* lut_img, const float* lut_inv, cudaStream_t s) {
-    const Variant* v = find_variant(ix->M, ix->d, ix->metric != RAGO_IP);
+                        uint32_t* err_word, const uint8_t* lut_img, const float* lut_inv, const PairView* view, cudaStream_t s) {
+    const bool need_vt = ix->metric != RAGO_IP;
+    const Variant* v = find_variant(ix->M, ix->d, need_vt);
     if (!v) return cudaErrorInvalidValue;
     ScanArgs a;
     a.codes = ix->codes; a.list_offsets = ix->list_offsets; a.probe_list = probe_list; a.probe_term = probe_term;
@@ -1020,6 +1399,18 @@ cudaError_t launch_scan(const IndexImpl* ix, const ScanPlan& plan, const float* 
     a.metric = ix->metric; a.k = k; a.stages = plan.stages; a.dyn_bytes = (uint32_t)plan.smem_bytes;
     a.stream_once = nq <= 64 ? 1 : 0;
     a.prefetch = scan_prefetches(ix, a.npairs) ? 1 : 0;
+    std::memset(&a.pv, 0, sizeof(a.pv));
+    if (view) {
+        const Variant* p = find_pair_variant(ix->M, ix->d, need_vt);
+        if (!p) return cudaErrorInvalidValue;
+        ScanArgs b = a;
+        b.pv = a.pv = *view;
+        b.lead = a.lead ? scan_pair_lead(ix) : 0;
+        b.stages = p->stages_for(ix->d, need_vt);
+        const cudaError_t e = launch_overlapped(p->kernel, dim3(plan.ctas), dim3(p->threads), plan.smem_bytes, s, b);
+        if (e != cudaSuccess) return e;
+        count_launch();
+    }
     const cudaError_t e = launch_overlapped(v->kernel, dim3(plan.ctas), dim3(v->threads), plan.smem_bytes, s, a);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
@@ -1079,25 +1470,29 @@ static int table_parts(const IndexImpl* ix, int nq) {
 // its own, because a CTA sees only a slice of the sub-spaces.
 __global__ void __launch_bounds__(128) table_scales_kernel(const float* __restrict__ queries,
                                                             const float* __restrict__ cwmax, int d, int dsub, int M,
-                                                            float* __restrict__ lut_scale, float* __restrict__ lut_inv) {
+                                                            float* __restrict__ lut_scale, float* __restrict__ lut_inv,
+                                                            int32_t* __restrict__ ok) {
     __shared__ float red[4];
     grid_dependency_wait();
     grid_dependents_may_launch();
     const int q = blockIdx.x, tid = threadIdx.x;
     const float* qrow = queries + (size_t)q * d;
     float mx = 0.f;
+    bool finite = true;
     for (int m = tid; m < M; m += 128) {
         float n2 = 0.f;
         for (int u = 0; u < dsub; ++u) { const float v = qrow[m * dsub + u]; n2 = fmaf(v, v, n2); }
+        finite = finite && n2 < 3.0e38f;  // not so for NaN
         mx = fmaxf(mx, 2.0002f * sqrtf(n2) * cwmax[m]);
     }
     for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if ((tid & 31) == 0) red[tid >> 5] = mx;
-    __syncthreads();
+    finite = __syncthreads_and(finite);
     if (tid == 0) {
         mx = fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3]));
         int ex = 0;
         if (mx > 0.f && mx < 3.0e38f) frexpf(mx * (float)M, &ex);
+        if (ok != nullptr) ok[q] = finite && mx * (float)M < 1e36f ? 1 : 0;  // no sum of M entries reaches 2^30 + M / 2 (1e36 < 2^120)
         ex = ex < -90 ? -90 : (ex > 120 ? 120 : ex);
         lut_scale[q] = ldexpf(1.f, 30 - ex);
         lut_inv[q] = ldexpf(1.f, ex - 30);
@@ -1179,11 +1574,11 @@ __global__ void __launch_bounds__(256) build_tables_batch_kernel(const TableArgs
 }
 
 cudaError_t launch_build_tables(const IndexImpl* ix, const float* queries, int nq, uint8_t* lut_img, float* lut_inv,
-                                float* lut_scale, cudaStream_t s) {
+                                float* lut_scale, int32_t* ok, cudaStream_t s) {
     const int dsub = ix->dsub;
     const TableArgs t = table_args(ix, queries, lut_img, lut_inv);
     if (nq > 64 && lut_scale && (dsub == 4 || dsub == 8 || dsub == 12 || dsub == 16)) {
-        launch_overlapped(table_scales_kernel, dim3(nq), dim3(128), 0, s, queries, ix->cwmax, ix->d, dsub, ix->M, lut_scale, lut_inv);
+        launch_overlapped(table_scales_kernel, dim3(nq), dim3(128), 0, s, queries, ix->cwmax, ix->d, dsub, ix->M, lut_scale, lut_inv, ok);
         const int ept = BTB_CW_FLOATS / dsub;
         const int G = 256 / ix->M;  // >= 2: the scan supports M <= 128
         const int threads = ix->M * G;
@@ -1272,7 +1667,7 @@ cudaError_t launch_vector_terms(const IndexImpl* ix, float* vterm, cudaStream_t 
 constexpr int PT_THREADS = 256;
 __global__ void __launch_bounds__(PT_THREADS) pair_tiles_kernel(const int32_t* __restrict__ probe_list,
                                                                 const int64_t* __restrict__ offsets, int npairs, int nprobe,
-                                                                int tile_vecs, int lead, int64_t* __restrict__ prefix,
+                                                                int tile_vecs, int lead, const PairTiles pt, int64_t* __restrict__ prefix,
                                                                 long long* __restrict__ block_sums) {
     __shared__ long long warp_sums[PT_THREADS / 32];
     grid_dependency_wait();
@@ -1281,7 +1676,8 @@ __global__ void __launch_bounds__(PT_THREADS) pair_tiles_kernel(const int32_t* _
     long long v = 0;
     if (p < npairs) {
         const int l = probe_list[p];
-        v = tiles_of(offsets[l + 1] - offsets[l], tile_vecs) + pair_lead(p, nprobe, lead);
+        if (pt.head == nullptr) v = tiles_of(offsets[l + 1] - offsets[l], tile_vecs) + pair_lead(p, nprobe, lead);
+        else v = (l < 0 ? 0 : tiles_of(offsets[l + 1] - offsets[l], entry_tile_vecs(p, nprobe, tile_vecs, pt))) + entry_lead(p, nprobe, lead, pt);
     }
     long long incl = v;
     for (int o = 1; o < 32; o <<= 1) {
@@ -1352,7 +1748,7 @@ __global__ void __launch_bounds__(PT_THREADS) add_offsets_kernel(int64_t* __rest
 // queries only, so nothing orders them against the planning).
 __global__ void __launch_bounds__(PFX_THREADS) plan_small_kernel(const int32_t* __restrict__ probe_list,
                                                                  const int64_t* __restrict__ offsets, int npairs, int nprobe,
-                                                                 int tile_vecs, int lead, int64_t* __restrict__ prefix,
+                                                                 int tile_vecs, int lead, const PairTiles pt, int64_t* __restrict__ prefix,
                                                                  unsigned long long* __restrict__ qthresh, int nq,
                                                                  int32_t* __restrict__ slot_cnt, int nslots,
                                                                  const TableArgs tables, int table_parts) {
@@ -1365,7 +1761,7 @@ __global__ void __launch_bounds__(PFX_THREADS) plan_small_kernel(const int32_t* 
         return;
     }
     __shared__ long long warp_sums[32];
-    plan_pairs_cta(probe_list, offsets, npairs, nprobe, tile_vecs, lead, prefix, qthresh, nq, slot_cnt, nslots, warp_sums);
+    plan_pairs_cta(probe_list, offsets, npairs, nprobe, tile_vecs, lead, pt, prefix, qthresh, nq, slot_cnt, nslots, warp_sums);
 }
 
 // Small batches whose probe selection plans the scan itself (see FusedPlan): what that kernel needs, or false when
@@ -1390,20 +1786,23 @@ bool fused_plan_args(const IndexImpl* ix, int nq, int npairs, const float* queri
     return true;
 }
 
-cudaError_t launch_plan_work(const IndexImpl* ix, const int32_t* probe_list, int npairs, int tile_vecs, int lead,
+// view (may be null): probe_list holds the entries of a batch with pairs of queries (the tables are built by then).
+cudaError_t launch_plan_work(const IndexImpl* ix, const int32_t* probe_list, int npairs, int tile_vecs, int lead, const PairView* view,
                              int32_t* pair_tiles, int64_t* work_prefix, unsigned long long* qthresh, int nq,
                              int32_t* slot_cnt, int nslots, const float* queries, uint8_t* lut_img, float* lut_inv,
                              float* lut_scale, cudaStream_t s) {
     const bool fused_tables = lut_img && npairs <= PLAN_SMALL_MAX && nq <= 64;
-    if (lut_img && !fused_tables) {
-        const cudaError_t et = launch_build_tables(ix, queries, nq, lut_img, lut_inv, lut_scale, s);
+    if (lut_img && !fused_tables && !view) {
+        const cudaError_t et = launch_build_tables(ix, queries, nq, lut_img, lut_inv, lut_scale, nullptr, s);
         if (et != cudaSuccess) return et;
     }
+    PairTiles pt = {nullptr, 0, 0};
+    if (view) { pt.head = view->head; pt.tile_vecs = ix->plan.pair_tile_vecs; pt.lead = lead ? scan_pair_lead(ix) : 0; }
     if (npairs <= PLAN_SMALL_MAX) {
         const int parts = fused_tables ? table_parts(ix, nq) : 0;
         launch_overlapped(plan_small_kernel, dim3(1 + parts * nq), dim3(PFX_THREADS),
                           parts ? (size_t)(ix->d + ix->M) * 4 : 0, s,
-            probe_list, ix->list_offsets, npairs, npairs / nq, tile_vecs, lead, work_prefix, qthresh, nq, slot_cnt, nslots,
+            probe_list, ix->list_offsets, npairs, npairs / nq, tile_vecs, lead, pt, work_prefix, qthresh, nq, slot_cnt, nslots,
             table_args(ix, queries, lut_img, lut_inv), parts);
         count_launch();
         return cudaGetLastError();
@@ -1412,7 +1811,7 @@ cudaError_t launch_plan_work(const IndexImpl* ix, const int32_t* probe_list, int
     const int nblocks = (npairs + PT_THREADS - 1) / PT_THREADS;
     long long* block_sums = reinterpret_cast<long long*>(pair_tiles);
     launch_overlapped(pair_tiles_kernel, dim3(nblocks), dim3(PT_THREADS), 0, s, probe_list, ix->list_offsets, npairs, npairs / nq,
-                      tile_vecs, lead, work_prefix, block_sums);
+                      tile_vecs, lead, pt, work_prefix, block_sums);
     launch_overlapped(scan_totals_kernel, dim3(1), dim3(PFX_THREADS), 0, s, block_sums, nblocks, work_prefix + npairs);
     launch_overlapped(add_offsets_kernel, dim3(nblocks), dim3(PT_THREADS), 0, s, work_prefix, npairs, block_sums, qthresh, nq,
                       slot_cnt, nslots);

@@ -25,8 +25,8 @@ __device__ __forceinline__ uint32_t bisect_mid(long long lo, long long hi, int r
 
 // Ascending bitonic sort of n keys (n a power of two) by `nthreads` threads; sync() is the barrier
 // those threads share.  Ends with a barrier.
-template <class Sync>
-__device__ __forceinline__ void block_bitonic_sort(unsigned long long* keys, int n, int tid, int nthreads,
+template <class Keys, class Sync>
+__device__ __forceinline__ void block_bitonic_sort(Keys keys, int n, int tid, int nthreads,
                                                    Sync sync) {
     for (int size = 2; size <= n; size <<= 1) {
         for (int stride = size >> 1; stride > 0; stride >>= 1) {
@@ -48,8 +48,8 @@ __device__ __forceinline__ void block_bitonic_sort(unsigned long long* keys, int
 // Sort the *cnt buffered keys ascending and cut the buffer to at most k entries.
 // Must be called by all cooperating threads, after a barrier that made *cnt and the keys visible.
 // Returns the new count; ends with a barrier.
-template <class Sync>
-__device__ __forceinline__ int block_select(unsigned long long* keys, int* cnt, int k, int tid, int nthreads,
+template <class Keys, class Sync>
+__device__ __forceinline__ int block_select(Keys keys, int* cnt, int k, int tid, int nthreads,
                                             Sync sync, int cap = TOPK_CAP) {
     int n = *cnt;
     if (n > cap) n = cap;
@@ -71,7 +71,8 @@ __device__ __forceinline__ unsigned long long shfl_xor_u64(unsigned long long v,
     const uint32_t hi = __shfl_xor_sync(0xffffffffu, (uint32_t)(v >> 32), m);
     return ((unsigned long long)hi << 32) | lo;
 }
-__device__ __forceinline__ void warp_bitonic_sort(unsigned long long* keys, int n2, int lane) {
+template <class Keys>
+__device__ __forceinline__ void warp_bitonic_sort(Keys keys, int n2, int lane) {
     unsigned long long k0 = lane < n2 ? keys[lane] : KEY_MAX;
     unsigned long long k1 = lane + 32 < n2 ? keys[lane + 32] : KEY_MAX;
     const int top = n2 > 32 ? 64 : 32;  // padding keys are maximal, so sorting more slots than n2 is harmless
@@ -118,31 +119,31 @@ __device__ __forceinline__ uint32_t warp_sort_u32(uint32_t v, int lane) {
 // key and rank in registers across one barrier and then stores the key at its rank: two barriers and a few dozen
 // instructions per warp, where a bitonic network on shuffles is several hundred dependent ones in a single warp.
 // Same contract as block_select.
-template <class Sync>
-__device__ __forceinline__ int block_select_short(unsigned long long* keys, int* cnt, int k, int tid, int nthreads,
+template <int RMAX = RANK_MAX, class Keys, class Sync>
+__device__ __forceinline__ int block_select_short(Keys keys, int* cnt, int k, int tid, int nthreads,
                                                   Sync sync, int cap = TOPK_CAP) {
     int n = *cnt;
     if (n > cap) n = cap;
     const int kept = n < k ? n : k;
     if (n > WARP_SORT_MAX) {
-        if (n > RANK_MAX || cap < 2 * RANK_MAX || nthreads < 256) return block_select(keys, cnt, k, tid, nthreads, sync, cap);
-        // Up to RANK_MAX keys are ranked too: a lane holds every 32nd key in registers, a warp takes the keys one
+        if (n > RMAX || cap < 2 * RMAX || nthreads < 256) return block_select(keys, cnt, k, tid, nthreads, sync, cap);
+        // Up to RMAX keys are ranked too: a lane holds every 32nd key in registers, a warp takes the keys one
         // after the other, counts the smaller ones with one compare per register and a warp-wide sum, and stores
         // the key at its rank in the free part of the buffer; three barriers where the bitonic network has dozens.
         const int warp = tid >> 5, lane = tid & 31, nwarps = nthreads >> 5;
-        unsigned long long a[RANK_MAX / 32];
+        unsigned long long a[RMAX / 32];
 #pragma unroll
-        for (int j = 0; j < RANK_MAX / 32; ++j) a[j] = lane + 32 * j < n ? keys[lane + 32 * j] : KEY_MAX;
+        for (int j = 0; j < RMAX / 32; ++j) a[j] = lane + 32 * j < n ? keys[lane + 32 * j] : KEY_MAX;
         for (int i = warp; i < n; i += nwarps) {  // uniform within the warp
             const unsigned long long x = keys[i];
             uint32_t c = 0;
 #pragma unroll
-            for (int j = 0; j < RANK_MAX / 32; ++j) c += a[j] < x ? 1u : 0u;
+            for (int j = 0; j < RMAX / 32; ++j) c += a[j] < x ? 1u : 0u;
             c = __reduce_add_sync(0xffffffffu, c);
-            if (lane == 0 && (int)c < kept) keys[RANK_MAX + c] = x;  // keys [0, n) are only read here
+            if (lane == 0 && (int)c < kept) keys[RMAX + c] = x;  // keys [0, n) are only read here
         }
         sync();
-        for (int i = tid; i < kept; i += nthreads) keys[i] = keys[RANK_MAX + i];
+        for (int i = tid; i < kept; i += nthreads) keys[i] = keys[RMAX + i];
         if (tid == 0) *cnt = kept;
         sync();
         return kept;
@@ -188,7 +189,8 @@ __device__ __forceinline__ int block_select_short(unsigned long long* keys, int*
 }
 
 // Append `key` for the lanes with pred set; one shared atomic per warp.  Whole warp must call.
-__device__ __forceinline__ void warp_push(unsigned long long* keys, int* cnt, bool pred, unsigned long long key,
+template <class Keys>
+__device__ __forceinline__ void warp_push(Keys keys, int* cnt, bool pred, unsigned long long key,
                                           int cap = TOPK_CAP) {
     const unsigned mask = __ballot_sync(0xffffffffu, pred);
     if (mask == 0) return;
