@@ -26,9 +26,25 @@ struct ScanPlan {
     int ctas;          // persistent CTAs (one per SM)
     size_t smem_bytes;
     // shared-memory image of a query's lookup table, as the scan variant of this index lays it out
-    int lut_bytes, lut_banked, lut_copies, lut_copy_off, lut_stride;
+    int lut_bytes, lut_kind;
     int pair_tile_vecs;  // vectors per tile where two queries are scanned together, 0: not with this index
 };
+
+// Layouts of a query's lookup table, in shared memory and in the images that are built ahead (scan.cu says which code size takes
+// which).  LUT_DOT: parts of 32 columns, 256 rows (code values) of 128 bytes each, 32 sub-spaces to a part.  LUT_DOT2: the
+// same parts with 16 sub-spaces and the same 16 again, so that lanes whose columns agree mod 16 can read different banks.
+// LUT_PERM: rows of 256 bytes, up to 64 sub-spaces.
+enum : int { LUT_PERM = 0, LUT_DOT = 1, LUT_DOT2 = 2 };
+constexpr uint32_t LUT_ROW = 128, LUT_PART = KSUB * LUT_ROW, LUT_COPY = 64;
+__host__ __device__ constexpr uint32_t lut_row(int kind) { return kind == LUT_PERM ? 256u : LUT_ROW; }
+__host__ __device__ constexpr uint32_t lut_offset(int kind, int j, int m) {
+    return kind == LUT_PERM ? (uint32_t)j * 256u + (uint32_t)m * 4u
+         : kind == LUT_DOT2 ? (uint32_t)(m / 16) * LUT_PART + (uint32_t)j * LUT_ROW + (uint32_t)(m % 16) * 4u
+                            : (uint32_t)(m / 32) * LUT_PART + (uint32_t)j * LUT_ROW + (uint32_t)(m % 32) * 4u;
+}
+__host__ __device__ constexpr int lut_image_bytes(int M, int kind) {
+    return kind == LUT_PERM ? 65536 : M / (kind == LUT_DOT2 ? 16 : 32) * (int)LUT_PART;
+}
 
 // Batches of at most this many queries get their lookup tables from kernels of their own, spread over the whole
 // GPU, instead of every scan CTA building the table of each query it meets.

@@ -181,7 +181,7 @@ constexpr int PI_CTAS = 4, PI_THREADS = 256, PI_SHIFTS = 17;
 template <int M>
 __global__ void __cluster_dims__(PI_CTAS, 1, 1) __launch_bounds__(PI_THREADS) pair_tables_kernel(
     const int32_t* __restrict__ head, const int32_t* __restrict__ order, const uint8_t* __restrict__ lut_img,
-    const float* __restrict__ lut_inv, int lut_bytes, int copies, int copy_off, PairParams* __restrict__ params, uint8_t* __restrict__ img) {
+    const float* __restrict__ lut_inv, int lut_bytes, int kind, PairParams* __restrict__ params, uint8_t* __restrict__ img) {
     constexpr int COLS = M / PI_CTAS, C4 = COLS / 4, G = PI_THREADS / C4, ROWS = (KSUB + G - 1) / G;
     static_assert(M % (4 * PI_CTAS) == 0, "whole groups of four columns");
     __shared__ int s_mn[2][G][COLS], s_mx[2][G][COLS];
@@ -194,14 +194,14 @@ __global__ void __cluster_dims__(PI_CTAS, 1, 1) __launch_bounds__(PI_THREADS) pa
     if (u >= head[0]) return;  // uniform over the cluster
     const int c = tid % C4, g = tid / C4, col = rank * COLS + c * 4;
     const int q[2] = {order[2 * u], order[2 * u + 1]};
-    auto off = [](int j, int column) -> uint32_t { return (uint32_t)(column / 64) * 65536u + (uint32_t)j * 256u + (uint32_t)(column % 64) * 4u; };
+    const uint32_t off0 = lut_offset(kind, 0, col);  // four neighbouring columns lie in one row
     int4 v[2][ROWS];
 #pragma unroll
     for (int side = 0; side < 2; ++side)
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) {
             const int j = g + r * G;
-            if (g < G && j < KSUB) v[side][r] = __ldg(reinterpret_cast<const int4*>(lut_img + (size_t)q[side] * lut_bytes + off(j, col)));
+            if (g < G && j < KSUB) v[side][r] = __ldg(reinterpret_cast<const int4*>(lut_img + (size_t)q[side] * lut_bytes + off0 + (uint32_t)j * lut_row(kind)));
         }
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
@@ -260,8 +260,8 @@ __global__ void __cluster_dims__(PI_CTAS, 1, 1) __launch_bounds__(PI_THREADS) pa
             if (j >= KSUB) continue;
             const int4 x = v[0][r], y = v[1][r];
             const uint4 e = make_uint4(half2(x.x, la.x, y.x, lb.x), half2(x.y, la.y, y.y, lb.y), half2(x.z, la.z, y.z, lb.z), half2(x.w, la.w, y.w, lb.w));
-            *reinterpret_cast<uint4*>(out + off(j, col)) = e;
-            if (copies == 2) *reinterpret_cast<uint4*>(out + off(j, copy_off + col)) = e;
+            *reinterpret_cast<uint4*>(out + off0 + (uint32_t)j * lut_row(kind)) = e;
+            if (kind == LUT_DOT2) *reinterpret_cast<uint4*>(out + off0 + (uint32_t)j * lut_row(kind) + LUT_COPY) = e;
         }
     }
     if (rank == 0 && tid < 2) {
@@ -380,7 +380,7 @@ cudaError_t launch_pair_queries(const IndexImpl* ix, const int32_t* probe_list, 
     if (e != cudaSuccess) return e;
     auto tables = [&](auto kernel) {
         return launch_overlapped(kernel, dim3(PI_CTAS * (nq / 2)), dim3(PI_THREADS), 0, s, head, order, lut_img, lut_inv, pl.lut_bytes,
-                                 pl.lut_copies, pl.lut_copy_off, params, img);
+                                 pl.lut_kind, params, img);
     };
     switch (ix->M) {
         case 16: e = tables(pair_tables_kernel<16>); break;

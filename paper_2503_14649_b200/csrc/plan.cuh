@@ -13,7 +13,7 @@ constexpr int PLAN_SMALL_MAX = PFX_THREADS * PLAN_PER_THREAD;
 
 struct TableArgs {
     const float* queries; const float* cbT; const float* cwmax;
-    int d, dsub, M, metric, lut_bytes, banked, copies, copy_off, lstride;
+    int d, dsub, M, metric, lut_bytes, kind;
     uint8_t* lut_img; float* lut_inv;
 };
 
@@ -94,10 +94,6 @@ __device__ __forceinline__ void build_table_part(const TableArgs& t, int q, int 
     const float scale = ldexpf(1.f, 30 - ex);
     if (part == 0 && tid == 0) t.lut_inv[q] = ldexpf(1.f, ex - 30);
     uint8_t* img = t.lut_img + (size_t)q * t.lut_bytes;
-    auto off = [&](int j, int col) -> uint32_t {
-        return t.banked ? (uint32_t)(col / 64) * 65536u + (uint32_t)j * 256u + (uint32_t)(col % 64) * 4u
-                        : ((uint32_t)j * t.lstride + (uint32_t)col) * 4u;
-    };
     const int total = KSUB * M;
     const int per = (total + parts - 1) / parts;
     const int e1 = (part + 1) * per < total ? (part + 1) * per : total;
@@ -121,8 +117,8 @@ __device__ __forceinline__ void build_table_part(const TableArgs& t, int q, int 
             for (int u = 0; u < dsub; ++u) acc = fmaf(rT[u * M + m], __ldg(cw + u), acc);
         }
         const int v = __float2int_rn(acc * scale);
-        *reinterpret_cast<int*>(img + off(j, m)) = v;
-        if (t.copies == 2) *reinterpret_cast<int*>(img + off(j, t.copy_off + m)) = v;
+        *reinterpret_cast<int*>(img + lut_offset(t.kind, j, m)) = v;
+        if (t.kind == LUT_DOT2) *reinterpret_cast<int*>(img + lut_offset(LUT_DOT2, j, m) + LUT_COPY) = v;
         j += step_j;
         m += step_m;
         if (m >= M) { m -= M; ++j; }

@@ -25,11 +25,14 @@
 // into R "virtual rows" handled by adjacent lanes and summed with a shuffle; sub-space counts that
 // are 16 mod 32 keep two table copies so lanes L and L^4 never collide.
 //
-// Table addressing.  Per code byte the inner loop spends one byte-permute, one shared load and one
-// add: the table is stored as 64-column banks of 256 rows x 256 bytes that start at a shared-memory
-// address which is a multiple of 64 KB, so the load address  (bank << 16) | (code << 8) | column*4
-// is assembled by a single PRMT from the code word and a per-lane constant.  Tables wider than two
-// banks (M = 80 with its two copies) fall back to a multiply-add address.
+// Table addressing.  Per code byte the inner loop spends one instruction on the address, one shared load and half an add.
+// LUT_DOT (16, 48, 80, 96, 128 bytes): rows of 128 bytes; a byte dot product of the code word with 128 in the byte's place,
+// plus the lane's address of the column in row 0, is the address.  It runs on the multiplier pipe, while byte permutations
+// share theirs with everything else of the loop (58% busy beside 50% of the load pipe for 96 bytes), the rows need no padding and
+// the table may lie anywhere.  LUT_PERM (32 and 64 bytes): rows of 256 bytes from a multiple of 64 KB on, the address
+// (place << 16) | (code << 8) | column*4  is one PRMT of the code word and a lane constant for every two bytes, half as many
+// registers.  us per call, permutation / dot product: 96 bytes (400 queries, lists of 2 200) 710 / 667, 80 bytes 358 / 335, 16 bytes
+// 569 / 548, 128 bytes 437 / 432; 64 bytes 483 / 494, 32 bytes 592 / 621, 48 bytes 499 / 512 (pairs 1 188 / 1 174).
 //
 // Fixed-point table.  Entries are stored as 32-bit integers scaled by a per-query power of two chosen
 // so that a sum of M entries cannot overflow (|sum| < 2^30): the scan then adds two entries per
@@ -60,7 +63,7 @@
 
 namespace rago {
 
-constexpr int MAX_STAGES = 5;
+constexpr int MAX_STAGES = 4;
 constexpr int SCAN_PF = 2;                  // tiles ahead of the one being copied that are prefetched into L2 (measured: 1-2 best)
 // Prefetch of a contiguous global range into L2 (16-byte aligned start, size a multiple of 16 bytes).
 __device__ __forceinline__ void l2_prefetch(const void* g, uint32_t bytes) {
@@ -76,11 +79,11 @@ struct alignas(16) TileDesc {
                          // from bit 8: vectors in this tile; negative: the CTA has no tile
     uint32_t pos0;       // storage position of the tile's first vector
     uint32_t tile_addr;  // shared address of the stage's code tile
-    uint32_t tile_hi;    // split tiles: what takes its place for the warps whose rows lie in the upper part
+    float term_b;        // two queries at a time: the second query's term
     uint32_t vt_addr;    // shared address of the first vector's term
     int32_t pair;        // index into probe_list (query * nprobe + rank)
     float term;          // the pair's (query, list) term of the score
-    float term_b;        // two queries at a time: the second query's term
+    int32_t unused;
 };
 
 struct ScanArgs {
@@ -115,28 +118,17 @@ struct Cfg {
     static constexpr int MV = WV * 4;                   // bytes per virtual row
     static constexpr int M = MV * R;                    // code bytes per vector
     static constexpr int NBLK = WV / G;                 // blocks of G words per virtual row
-    static constexpr int COPIES = G == 4 ? 2 : 1;
-    static constexpr int COPY_OFF = COPIES == 1 ? 0 : (M == 16 ? 16 : (M == 48 ? 80 : M));  // 16 mod 32
-    static constexpr int NCOLS = COPIES == 1 ? M : COPY_OFF + M;
-    static constexpr bool BANKED = NCOLS <= 128;        // PRMT addressing
-    static constexpr int NBANK = (NCOLS + 63) / 64;
-    static constexpr int LSTRIDE = NCOLS;               // words per table row (multiply-add addressing)
-    static constexpr int LUT_BYTES = BANKED ? NBANK * 65536 : KSUB * LSTRIDE * 4;
+    static constexpr int KIND = G == 4 ? LUT_DOT2 : (M == 32 || M == 64 ? LUT_PERM : LUT_DOT);
+    static constexpr int LUT_BYTES = lut_image_bytes(M, KIND);
     static constexpr int RGW = RGW_;                    // 32-row groups per warp per tile (unrolled: independent work in flight)
     static constexpr int TILE_VROWS = NCW * 32 * RGW;
     static constexpr int TV = TILE_VROWS / R;           // vectors per tile
     static constexpr int TILE_BYTES = TILE_VROWS * MV;
-    // A 128 KB table leaves 63 KB below it and 36 KB above.  Two tiles of 15 x 32 rows of 96 bytes fit that space in two parts
-    // each: the rows of the first ten warps below, those of the others above (the candidate buffers then lie in unused
-    // columns of the table, see StripKeys).
-    static constexpr bool SPLIT = M == 96 && NCW == 15;
-    static constexpr int LOW_WARPS = SPLIT ? 10 : NCW;
-    static constexpr int LOW_BYTES = LOW_WARPS * 32 * RGW * MV, HIGH_BYTES = TILE_BYTES - LOW_BYTES;
     static constexpr int VT_BYTES = (TV + 4) * 4;       // staged per-vector terms (start rounded down to 16 bytes)
-    static constexpr int KCAP = LUT_BYTES <= 65536 ? 2 * TOPK_CAP : TOPK_CAP;  // keys of the CTA's candidate buffer
-    // Banked tables start at this absolute shared address (a multiple of 64 KB).  Two tiles of more than 48 KB do not
+    static constexpr int KCAP = LUT_BYTES <= 65536 || M == 48 ? 2 * TOPK_CAP : TOPK_CAP;  // keys of the CTA's candidate buffer
+    // Tables of the kind LUT_PERM start at this absolute shared address (a multiple of 64 KB).  Two tiles of more than 48 KB do not
     // fit above a table at 64 KB, so configurations with such tiles keep their tiles below a table at 128 KB.
-    static constexpr uint32_t LUT_WINDOW = (NBANK == 1 && LOW_BYTES > 48 * 1024) ? 0x20000u : 0x10000u;
+    static constexpr uint32_t LUT_WINDOW = TILE_BYTES > 48 * 1024 ? 0x20000u : 0x10000u;
     static_assert(WV % G == 0, "virtual rows are whole blocks");
     static_assert(TILE_VROWS % R == 0, "tile must hold whole vectors");
     static_assert(RGW % (R < RGW ? R : RGW) == 0, "row groups are taken min(R, RGW) at a time");
@@ -145,57 +137,16 @@ struct Cfg {
     static constexpr int SMAX = KCAP / TV / 2 < MAX_STAGES ? KCAP / TV / 2 : MAX_STAGES;
     static_assert(SMAX >= 2, "two tiles in flight must fit the candidate buffer twice over");
     static_assert(MAX_K + SMAX * TV <= KCAP, "k kept keys plus the pushes of all tiles in flight must fit");
-    static_assert(COPY_OFF % 32 == (COPIES == 2 ? 16 : 0), "second copy must sit 16 banks away");
-    static_assert(LSTRIDE % 32 == 0 || BANKED, "table rows must keep bank = column mod 32");
-    static_assert(VT_BYTES % 16 == 0 && LOW_BYTES % 16 == 0 && HIGH_BYTES % 16 == 0, "bulk-copy destinations are 16-byte granular");
-    // banked addressing: the columns one lane touches in one block stay inside one 64-column bank
-    __host__ __device__ static constexpr bool banked_ok() {
-        for (int copy = 0; copy < COPIES; ++copy)
-            for (int sr = 0; sr < R; ++sr)
-                for (int blk = 0; blk < NBLK; ++blk) {
-                    const int cb = copy * COPY_OFF + sr * MV;
-                    if ((cb % 64) + ((blk * 4 * G) % 64) + 4 * G > 64) return false;
-                }
-        return true;
-    }
-    static_assert(!BANKED || banked_ok(), "a lane's columns of one block straddle two banks");
-    // address of table entry (code j, column col) relative to the table's start
-    __host__ __device__ static constexpr uint32_t lut_off(int j, int col) {
-        return BANKED ? (uint32_t)(col / 64) * 65536u + (uint32_t)j * 256u + (uint32_t)(col % 64) * 4u
-                      : ((uint32_t)j * LSTRIDE + (uint32_t)col) * 4u;
-    }
-    // immediate added for block blk (banked addressing)
-    __host__ __device__ static constexpr uint32_t blk_imm(int blk) {
-        return (uint32_t)((blk * 4 * G) / 64) * 65536u + (uint32_t)((blk * 4 * G) % 64) * 4u;
-    }
+    static_assert(VT_BYTES % 16 == 0 && TILE_BYTES % 16 == 0, "bulk-copy destinations are 16-byte granular");
+    static_assert(KIND == LUT_DOT2 ? G == 4 && R == 1 : MV % 32 == 0, "a lane's columns of a block of words lie in one 32-column part of the table");
+    static_assert(KIND != LUT_PERM || NBLK == 1, "one block of words to a (virtual) row");
 };
 
-// The candidate buffer of one of two queries that are scanned together, or of the one query where tiles are split.  Tables of
-// two banks leave no room for two buffers (or for one, beside larger tiles), but do not use all of their columns (96 of 128, or
-// two copies of 48): key i lies in the unused columns of a table row, ROW_KEYS keys to a row.  The copy of the next
-// table overwrites them, when the buffers are empty.
-template <class C>
-struct StripKeys {
-    static constexpr bool STRIP = C::NBANK == 2;
-    static constexpr int ROW_KEYS = C::M == 96 ? 16 : 8;
-    // the strips lie outside every copy of the table and hold KCAP keys
-    static constexpr bool FITS = C::BANKED && (!STRIP || (C::KCAP <= 2048 && ((C::M == 96 && C::NCOLS == 96) || (C::M == 48 && C::COPY_OFF == 80))));
-    uint8_t* p;
-    // lut: the table, lin: the linear buffers
-    __device__ __forceinline__ StripKeys(uint8_t* lut, uint8_t* lin, int side) {
-        if (!STRIP) p = lin + (size_t)side * C::KCAP * 8;
-        else if (C::M == 96) p = lut + 65536 + 128 + side * 32768;  // columns 32-63 of the second bank, half of its rows each
-        else p = side ? lut + 65536 : lut + 192;                    // columns 48-63 of the first bank, 0-15 of the second
-    }
-    __device__ __forceinline__ unsigned long long& operator[](int i) const {
-        return *reinterpret_cast<unsigned long long*>(STRIP ? p + (size_t)(i / ROW_KEYS) * 256 + (i % ROW_KEYS) * 8 : p + (size_t)i * 8);
-    }
-};
 // Absolute shared-memory addresses of everything the kernel keeps there.  The same function runs on
 // the host (to choose the number of stages, with the expected window base) and in the kernel (with
 // the real base); a plan that does not fit makes the kernel report an error and return.
 struct SmemPlan {
-    uint32_t lut, ctrl, keys, rT, vt[MAX_STAGES], tile[MAX_STAGES], high[MAX_STAGES];
+    uint32_t lut, ctrl, keys, rT, vt[MAX_STAGES], tile[MAX_STAGES];
     int ok;
 };
 
@@ -204,17 +155,16 @@ __host__ __device__ inline SmemPlan plan_smem(uint32_t base, uint32_t dyn_bytes,
     SmemPlan p;
     p.ok = 1;
     const uint32_t end = base + dyn_bytes;
-    uint32_t lo_cur, lo_end, hi_cur;
-    if (C::BANKED) {
-        p.lut = C::LUT_WINDOW;
+    uint32_t lo_cur = base, lo_end = base, hi_cur;
+    if (C::KIND == LUT_PERM) {
+        p.lut = lo_end = C::LUT_WINDOW;
         if (base > C::LUT_WINDOW) p.ok = 0;
-        lo_cur = base; lo_end = C::LUT_WINDOW; hi_cur = C::LUT_WINDOW + C::LUT_BYTES;
     } else {
-        p.lut = (base + 127u) & ~127u;
-        lo_cur = lo_end = 0; hi_cur = p.lut + C::LUT_BYTES;
+        p.lut = (base + 127u) & ~127u;  // rows of 128 bytes: bank = column
     }
+    hi_cur = p.lut + C::LUT_BYTES;
     if (hi_cur > end) p.ok = 0;
-    auto take = [&](uint32_t bytes, uint32_t align) -> uint32_t {
+    auto take = [&](uint32_t bytes, uint32_t align) -> uint32_t {  // below the table if it fits there, else above
         uint32_t a = (lo_cur + align - 1) & ~(align - 1);
         if (a + bytes <= lo_end) { lo_cur = a + bytes; return a; }
         a = (hi_cur + align - 1) & ~(align - 1);
@@ -222,16 +172,13 @@ __host__ __device__ inline SmemPlan plan_smem(uint32_t base, uint32_t dyn_bytes,
         p.ok = 0;
         return base;
     };
-    // largest pieces first, each below the table if it fits there, else above it
-    for (int s = 0; s < MAX_STAGES; ++s) p.tile[s] = s < stages ? take(C::LOW_BYTES, 128) : base;
-    for (int s = 0; s < MAX_STAGES; ++s) p.high[s] = C::SPLIT && s < stages ? take(C::HIGH_BYTES, 128) : base;
-    // two queries at a time: two buffers, side by side or in the columns of the table that nothing uses
-    constexpr bool strips = C::SPLIT || (DUAL && StripKeys<C>::STRIP);
-    p.keys = strips ? base : take(C::KCAP * (DUAL ? 16 : 8), 16);
+    // largest pieces first
+    for (int s = 0; s < MAX_STAGES; ++s) p.tile[s] = s < stages ? take(C::TILE_BYTES, 128) : base;
+    p.keys = take(C::KCAP * (DUAL ? 16 : 8), 16);  // two queries at a time: two buffers
     for (int s = 0; s < MAX_STAGES; ++s) p.vt[s] = (s < stages && need_vt) ? take(C::VT_BYTES, 16) : base;
     // The scaled, transposed query is only alive while a table is built, when the candidate buffer is empty: it
     // shares the buffer's space when it fits there.
-    p.rT = DUAL ? base : !strips && (uint32_t)d * 4 <= (uint32_t)C::KCAP * 8 ? p.keys : take((uint32_t)d * 4, 16);
+    p.rT = DUAL ? base : (uint32_t)d * 4 <= (uint32_t)C::KCAP * 8 ? p.keys : take((uint32_t)d * 4, 16);
     p.ctrl = take(CTRL_BYTES, 16);
     return p;
 }
@@ -244,7 +191,7 @@ struct Ctrl {
     unsigned long long empty[MAX_STAGES];
     unsigned long long cbar;  // consumer barrier
     unsigned long long lutbar;  // a prebuilt table has landed
-    uint32_t tile[MAX_STAGES], high[MAX_STAGES], vt[MAX_STAGES];  // the stages' places (SmemPlan's, which would go to local memory to be indexed)
+    uint32_t tile[MAX_STAGES], vt[MAX_STAGES];  // the stages' places (SmemPlan's, which would go to local memory to be indexed)
     TileDesc desc[MAX_STAGES];
     int cnt;
     int cnt_b;  // two queries at a time: keys in the second query's buffer
@@ -302,7 +249,7 @@ __device__ __forceinline__ float build_table(const float* __restrict__ cbT, cons
                 acc = fmaf(rT[(4 * i + 2) * C::M + m], cv[u][i].z, acc);
                 acc = fmaf(rT[(4 * i + 3) * C::M + m], cv[u][i].w, acc);
             }
-            sts_f32(lut + C::lut_off(j, m), acc);
+            sts_f32(lut + lut_offset(C::KIND, j, m), acc);
             mx = fmaxf(mx, fabsf(acc));
         }
     }
@@ -316,7 +263,7 @@ __device__ __forceinline__ float build_table_any(const float* __restrict__ cbT, 
         const int j = e / C::M, m = e - j * C::M;
         float acc = 0.f;
         for (int t = 0; t < dsub; ++t) acc = fmaf(rT[t * C::M + m], __ldg(cbT + (size_t)e * dsub + t), acc);
-        sts_f32(lut + C::lut_off(j, m), acc);
+        sts_f32(lut + lut_offset(C::KIND, j, m), acc);
         mx = fmaxf(mx, fabsf(acc));
     }
     return mx;
@@ -327,10 +274,10 @@ template <class C>
 __device__ __forceinline__ void quantise_table(uint32_t lut, int ctid, float scale) {
     for (int e = ctid; e < KSUB * C::M; e += C::NCT) {
         const int j = e / C::M, m = e - j * C::M;
-        const uint32_t addr = lut + C::lut_off(j, m);
+        const uint32_t addr = lut + lut_offset(C::KIND, j, m);
         const int q = __float2int_rn(lds_f32(addr) * scale);
         sts_f32(addr, __int_as_float(q));
-        if (C::COPIES == 2) sts_f32(lut + C::lut_off(j, C::COPY_OFF + m), __int_as_float(q));
+        if (C::KIND == LUT_DOT2) sts_f32(addr + LUT_COPY, __int_as_float(q));
     }
 }
 
@@ -350,8 +297,7 @@ struct LoadWords {
 // One block (G code words = 4G sub-spaces) of one virtual row: 4G look-ups, written as three passes over
 // half a block (all addresses, all loads, all adds).
 template <class C, int G, int BLK>
-__device__ __forceinline__ void scan_block(const uint32_t (&x)[G], const uint32_t (&cc)[G][2], const uint32_t (&sel)[4],
-                                           const uint32_t (&lo)[G][4], uint32_t lut, int (&acc)[4]) {
+__device__ __forceinline__ void scan_block(const uint32_t (&x)[G], const uint32_t (&at)[G][4], const uint32_t (&pick)[4], int (&acc)[4]) {
     constexpr int H = G / 2;
 #pragma unroll
     for (int h0 = 0; h0 < G; h0 += H) {
@@ -361,13 +307,11 @@ __device__ __forceinline__ void scan_block(const uint32_t (&x)[G], const uint32_
         for (int i = 0; i < H; ++i)
 #pragma unroll
             for (int t = 0; t < 4; ++t)
-                ad[i][t] = C::BANKED ? __byte_perm(x[h0 + i], cc[h0 + i][t >> 1], sel[t])
-                                     : lut + __byte_perm(x[h0 + i], 0u, sel[t]) * (uint32_t)(C::LSTRIDE * 4) + lo[h0 + i][t];
+                ad[i][t] = C::KIND == LUT_PERM ? __byte_perm(x[h0 + i], at[h0 + i][t >> 1], pick[t]) : __dp4a(x[h0 + i], pick[t], at[h0 + i][t]);
 #pragma unroll
         for (int i = 0; i < H; ++i)
 #pragma unroll
-            for (int t = 0; t < 4; ++t)
-                vv[i][t] = C::BANKED ? lds_u32_imm<(int)C::blk_imm(BLK)>(ad[i][t]) : lds_u32_imm<BLK * G * 16>(ad[i][t]);
+            for (int t = 0; t < 4; ++t) vv[i][t] = lds_u32_imm<BLK * (int)LUT_PART>(ad[i][t]);
 #pragma unroll
         for (int i = 0; i < H; i += 2)  // two entries per add
 #pragma unroll
@@ -376,38 +320,20 @@ __device__ __forceinline__ void scan_block(const uint32_t (&x)[G], const uint32_
 }
 template <class C, int G, int BLK>
 struct ScanBlocks {
-    __device__ __forceinline__ static void run(const uint32_t (&x)[C::NBLK][G], const uint32_t (&cc)[G][2],
-                                               const uint32_t (&sel)[4], const uint32_t (&lo)[G][4], uint32_t lut,
+    __device__ __forceinline__ static void run(const uint32_t (&x)[C::NBLK][G], const uint32_t (&at)[G][4], const uint32_t (&pick)[4],
                                                int (&acc)[4]) {
-        scan_block<C, G, BLK>(x[BLK], cc, sel, lo, lut, acc);
-        if constexpr (BLK + 1 < C::NBLK) ScanBlocks<C, G, BLK + 1>::run(x, cc, sel, lo, lut, acc);
+        scan_block<C, G, BLK>(x[BLK], at, pick, acc);
+        if constexpr (BLK + 1 < C::NBLK) ScanBlocks<C, G, BLK + 1>::run(x, at, pick, acc);
     }
 };
 
 // ---- making a buffer of bounds exact (pairs of queries) ----
 // Both steps are written for few registers: what they hold beside the tile loop's values goes to local memory, which, with
 // nearly all of the SM's cache being shared memory, means trips to L2 (with 100 to 200 bytes of it the loop took twice as long).
-
-// A table image in the place of the one in use, around the key buffers that lie in its unused columns; 16-byte asynchronous
-// copies, which take no registers (bulk copies of the rows' pieces took 8 to 16 us).  Called by all consumer threads after a barrier, followed by one.
-template <class C>
-__device__ __forceinline__ void dual_table(uint32_t lut, const uint8_t* src, int ctid) {
-    constexpr int PER_ROW = C::LUT_BYTES / 4096 - (StripKeys<C>::STRIP ? 8 : 0), TOTAL = KSUB * PER_ROW;
-    for (int i = ctid; i < TOTAL; i += C::NCT) {
-        uint32_t at = (uint32_t)i * 16u;
-        if (StripKeys<C>::STRIP) {  // 24 pieces to a row: 16 and 8, or 12 and 12
-            const uint32_t row = (uint32_t)i / PER_ROW, c = (uint32_t)i % PER_ROW;
-            if (C::M == 96) at = c < 16u ? row * 256u + c * 16u : 65536u + row * 256u + (c - 16u) * 16u;
-            else at = c < 12u ? row * 256u + c * 16u : 65536u + row * 256u + 64u + (c - 12u) * 16u;
-        }
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(lut + at), "l"(src + at) : "memory");
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-}
 // First step, a thread per key: the bound in the upper word of a key is replaced by the sum of the terms of its list (found among
 // the unit's entries by the vector's position) and of the vector.
 template <class C>
-__device__ __forceinline__ void dual_terms(const StripKeys<C> kb, int kept, const float* terms, const uint2* ranges, int per_unit,
+__device__ __forceinline__ void dual_terms(unsigned long long* kb, int kept, const float* terms, const uint2* ranges, int per_unit,
                                            const float* vterm, bool ip, int ctid) {
 #pragma unroll 1
     for (int i = ctid; i < kept; i += C::NCT) {
@@ -425,7 +351,7 @@ __device__ __forceinline__ void dual_terms(const StripKeys<C> kb, int kept, cons
 // Second step, a warp to a few keys, lanes over sub-spaces: the entries of the query's own 32-bit table at `lut`, summed and scored as
 // the scan of one query does.
 template <class C>
-__device__ __forceinline__ void dual_exact(const StripKeys<C> kb, int kept, const uint8_t* codes, uint32_t lut, float inv, int ctid) {
+__device__ __forceinline__ void dual_exact(unsigned long long* kb, int kept, const uint8_t* codes, uint32_t lut, float inv, int ctid) {
     constexpr int MP = (C::M + 31) / 32, UN = C::THREADS > 512 ? 4 : 8;
     const int lane = ctid & 31;
 #pragma unroll 1
@@ -443,8 +369,9 @@ __device__ __forceinline__ void dual_exact(const StripKeys<C> kb, int kept, cons
         for (int u = 0; u < UN; ++u) {
             int sum = 0;
 #pragma unroll
-            for (int j = 0; j < MP; ++j)  // bank = column mod 32 = lane
-                if (lane + 32 * j < C::M) sum += (int)lds_u32(lut + C::lut_off((int)((code[u] >> (8 * j)) & 0xFFu), lane + 32 * j));
+            for (int j = 0; j < MP; ++j)  // bank = lane (of two copies the upper half of the lanes read the second)
+                if (lane + 32 * j < C::M)
+                    sum += (int)lds_u32(lut + lut_offset(C::KIND, (int)((code[u] >> (8 * j)) & 0xFFu), lane + 32 * j) + (C::KIND == LUT_DOT2 && lane >= 16 ? LUT_COPY : 0u));
             sum = __reduce_add_sync(0xffffffffu, sum);
             if (lane == 0 && i0 + u * C::NCW < kept) {
                 const unsigned long long key = kb[i0 + u * C::NCW];
@@ -459,7 +386,6 @@ template <int WV, int G, int R, int NCW_, int RGW_, bool DUAL>
 __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_kernel(const ScanArgs a) {
     using C = Cfg<WV, G, R, NCW_, RGW_>;
     constexpr int NCW = C::NCW, NCT = C::NCT;
-    static_assert(!DUAL || StripKeys<C>::FITS, "two candidate buffers");
     extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int S = a.stages;
@@ -470,18 +396,13 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
         return;
     }
     Ctrl* ctrl = reinterpret_cast<Ctrl*>(smem + (P.ctrl - base));
-    uint8_t* const lut_gen = smem + (P.lut - base);
-    auto make_keys = [&]() {
-        if constexpr (C::SPLIT) return StripKeys<C>(lut_gen, nullptr, 0);
-        else return reinterpret_cast<unsigned long long*>(smem + (P.keys - base));
-    };
-    const auto keys = make_keys();
+    unsigned long long* keys = reinterpret_cast<unsigned long long*>(smem + (P.keys - base));
     float* rT = reinterpret_cast<float*>(smem + (P.rT - base));
     volatile uint32_t* abort_flag = &ctrl->abort_flag;
 
     if (tid == 0) {
 #pragma unroll
-        for (int s = 0; s < MAX_STAGES; ++s) { ctrl->tile[s] = P.tile[s]; ctrl->high[s] = P.high[s]; ctrl->vt[s] = P.vt[s]; }
+        for (int s = 0; s < MAX_STAGES; ++s) { ctrl->tile[s] = P.tile[s]; ctrl->vt[s] = P.vt[s]; }
         for (int s = 0; s < S; ++s) {
             mbar_init(smem_u32(&ctrl->full[s]), 1);
             mbar_init(smem_u32(&ctrl->empty[s]), NCW);
@@ -642,22 +563,12 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
                 D.pair = pair;
                 D.term = term;
                 const uint8_t* src = a.codes + (size_t)pos0 * C::M;
-                uint32_t low = bytes;
                 mbar_arrive_expect_tx(bar, bytes + vbytes);
-                if constexpr (C::SPLIT) {
-                    const uint32_t high_at = ctrl->high[st];
-                    D.tile_hi = high_at - (uint32_t)C::LOW_BYTES;
-                    if (bytes > (uint32_t)C::LOW_BYTES) {
-                        low = (uint32_t)C::LOW_BYTES;
-                        if (a.stream_once) bulk_g2s_hint(high_at, src + low, bytes - low, bar, once_policy);
-                        else bulk_g2s(high_at, src + low, bytes - low, bar);
-                    }
-                }
                 if (a.stream_once) {  // small batch: the codes are read once and should leave L2 first
-                    bulk_g2s_hint(tile_at, src, low, bar, once_policy);
+                    bulk_g2s_hint(tile_at, src, bytes, bar, once_policy);
                     if (vbytes) bulk_g2s_hint(vt_at, a.vterm + (pos0 & ~3u), vbytes, bar, once_policy);
                 } else {
-                    bulk_g2s(tile_at, src, low, bar);
+                    bulk_g2s(tile_at, src, bytes, bar);
                     if (vbytes) bulk_g2s(vt_at, a.vterm + (pos0 & ~3u), vbytes, bar);
                 }
                 // pull the tiles a few steps ahead in this list into L2, with their terms, so that their copies find them there
@@ -702,26 +613,28 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
     const int xb = lane & 3;                            // byte xor
     const int copy = G == 4 ? ((lane >> 2) & 1) : 0;
     const int sr = lane % R;                            // which slice of the vector this lane sums
-    const int colbase = copy * C::COPY_OFF + sr * C::MV;
-    uint32_t xo[G], cc[G][2], lo[G][4], sel[4];
+    // xo: offset in a tile of the lane's word il of the warp's first row group.  An address of the table from a word's byte t:
+    // LUT_DOT   at: the column in row 0 of the first part; pick: the rows' distance in the byte's place, so that the dot product of
+    //           word and pick, plus at, is the address
+    // LUT_PERM  at[0, 1]: bytes  column * 4 of t = 2h, of t = 2h + 1, the table's place / 64 KB; pick: selects the column's
+    //           byte, the word's byte and the place into (place << 16) | (byte << 8) | column * 4
+    uint32_t xo[G], at[G][4], pick[4];
 #pragma unroll
     for (int il = 0; il < G; ++il) {
-        xo[il] = (uint32_t)(warp * C::RGW * 32 + lane) * C::MV + 4u * (uint32_t)(il ^ xa);  // offset in a tile of the lane's word il of the warp's first row group
+        xo[il] = (uint32_t)(warp * C::RGW * 32 + lane) * C::MV + 4u * (uint32_t)(il ^ xa);
 #pragma unroll
-        for (int t = 0; t < 4; ++t)
-            lo[il][t] = C::BANKED ? 0u : 4u * (uint32_t)(colbase + 4 * (il ^ xa) + (t ^ xb));
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            // bytes: column*4 for t = 2h, column*4 for t = 2h+1, table bank, 0
-            const uint32_t c0 = 4u * (uint32_t)((colbase % 64) + 4 * (il ^ xa) + ((2 * h) ^ xb));
-            const uint32_t c1 = 4u * (uint32_t)((colbase % 64) + 4 * (il ^ xa) + ((2 * h + 1) ^ xb));
-            cc[il][h] = c0 | (c1 << 8) | (((P.lut >> 16) + (uint32_t)(colbase / 64)) << 16);
+        for (int t = 0; t < 4; ++t) {
+            const uint32_t col = 16u * (uint32_t)(il ^ xa);
+            if (C::KIND == LUT_PERM)
+                at[il][t] = (uint32_t)sr * C::MV * 4u + col + 4u * (uint32_t)((2 * (t & 1)) ^ xb)
+                          | ((uint32_t)sr * C::MV * 4u + col + 4u * (uint32_t)((2 * (t & 1) + 1) ^ xb)) << 8 | P.lut;
+            else
+                at[il][t] = P.lut + (uint32_t)(sr * (C::MV / 32)) * LUT_PART + (copy ? LUT_COPY : 0u) + col + 4u * (uint32_t)(t ^ xb);
         }
     }
 #pragma unroll
     for (int t = 0; t < 4; ++t)
-        sel[t] = C::BANKED ? ((uint32_t)(4 + (t & 1)) | ((uint32_t)(t ^ xb) << 4) | 0x7600u)
-                           : (0x4440u | (uint32_t)(t ^ xb));
+        pick[t] = C::KIND == LUT_PERM ? (uint32_t)(4 + (t & 1)) | ((uint32_t)(t ^ xb) << 4) | 0x7600u : LUT_ROW << (8 * (t ^ xb));
 
     int cur_u = -1, cur_q = -1;  // the unit the CTA is working on, and its query
     unsigned long long tau = KEY_MAX;
@@ -746,11 +659,11 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
             // particular order.  Otherwise (or if ties leave too many) it is bisected, the score words re-read from
             // shared memory in every round.
             if (warp == 0) {
-                auto kw = [&](int i) { return reinterpret_cast<const uint32_t*>(&keys[i])[1]; };  // score word of key i
+                const uint32_t* kw = reinterpret_cast<const uint32_t*>(keys);  // score word of key i: kw[2 i + 1]
                 uint32_t lmn = 0xFFFFFFFFu, wmx = 0u;  // this lane's smallest score word, the largest of all
 #pragma unroll 4
                 for (int i = lane; i < n; i += 32) {
-                    const uint32_t o = kw(i);
+                    const uint32_t o = kw[2 * i + 1];
                     lmn = o < lmn ? o : lmn;
                     wmx = o > wmx ? o : wmx;
                 }
@@ -772,7 +685,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
                         const uint32_t mid = (uint32_t)(lo + (hi - lo) / 2);
                         uint32_t c = 0;
 #pragma unroll 4
-                        for (int i = lane; i < nn; i += 32) c += kw(i) <= mid ? 1u : 0u;
+                        for (int i = lane; i < nn; i += 32) c += kw[2 * i + 1] <= mid ? 1u : 0u;
                         c = __reduce_add_sync(0xffffffffu, c);
                         if (c < (uint32_t)k) lo = mid; else { hi = mid; c_hi = c; }
                     }
@@ -888,7 +801,6 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
         const size_t slot = (a.pv.head != nullptr ? 2 * ((size_t)npairs_q + gridDim.x) : 0) + cur_u + blockIdx.x;
         for (int i = ctid; i < kept; i += NCT) a.slot_keys[slot * k + i] = keys[i];
         if (ctid == 0) a.slot_cnt[slot] = kept;
-        if (C::SPLIT) fence_proxy_async();  // the next table's copy writes where keys were written and read
         csync();
     };
 
@@ -902,8 +814,8 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
         cur_q = q;
         early = k <= 32;
         if (a.lut_img != nullptr) {  // the table was built ahead of the scan: fetch its shared-memory image
-            // One thread asks the copy engine for the image (bulk copies, completion counted on a barrier): the 64 or
-            // 128 KB arrive at the rate of the L2 -> shared-memory path instead of a few 16-byte loads per thread
+            // One thread asks the copy engine for the image (bulk copies, completion counted on a barrier): the 32
+            // to 160 KB arrive at the rate of the L2 -> shared-memory path instead of a few 16-byte loads per thread
             // and round trip.  Every consumer is past its last look-up in the old table (the barrier that ended the
             // previous query); the fence orders those reads before the copies' writes.
             if (ctid == 0) {
@@ -957,7 +869,20 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
     unsigned long long dtau[2] = {KEY_MAX, KEY_MAX};
     bool duse[2] = {false, false};
     dlimit[0] = dlimit[1] = 0.f;
-    auto dual_keys = [&](int side) { return StripKeys<C>(lut_gen, smem + (P.keys - base), side); };
+    auto dual_keys = [&](int side) { return keys + (side ? C::KCAP : 0); };
+    // A table image takes the place of the one in use (every consumer is past its last look-up); ends with it there for this thread.
+    auto fetch_table = [&](const uint8_t* src) {
+        if (ctid == 0) {
+            fence_proxy_async();
+            const uint32_t bar = smem_u32(&ctrl->lutbar);
+            mbar_arrive_expect_tx(bar, (uint32_t)C::LUT_BYTES);
+            constexpr uint32_t PIECE = 32768;
+            for (uint32_t o = 0; o < (uint32_t)C::LUT_BYTES; o += PIECE)
+                bulk_g2s(P.lut + o, src + o, (uint32_t)C::LUT_BYTES - o < PIECE ? (uint32_t)C::LUT_BYTES - o : PIECE, bar);
+        }
+        dead = dead || !mbar_wait(smem_u32(&ctrl->lutbar), lphase, abort_flag, a.err);
+        lphase ^= 1u;
+    };
     // Limits of the scan's first test.  A bound is  bias + vt + (base + half * 2^s) * inv  up to its roundings, the test's left side
     // is  x = (2^23 + half) * unit + vt  with unit = 2^s * inv, so a bound at or below the threshold's score t has
     // x <= t - bias - base * inv + 2^23 * unit, up to roundings of both that lie below 2^-20 of the sum of all magnitudes (that
@@ -989,7 +914,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
 #pragma unroll 1
         for (int side = 0; side < 2; ++side) {
             if (!((sides >> side) & 1)) continue;
-            const StripKeys<C> kb = dual_keys(side);
+            unsigned long long* kb = dual_keys(side);
             int* cn = side ? &ctrl->cnt_b : &ctrl->cnt;
             const int q = side ? dq[1] : dq[0];
             const float inv = side ? dinv[1] : dinv[0];
@@ -1054,7 +979,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
             if (close || kept > C::KCAP - (S + 1) * C::TV) {  // uniform
                 const size_t eb = (size_t)e_base + (size_t)cur_u * per_unit;
                 dual_terms<C>(kb, kept, (side ? a.pv.term_b : a.probe_term) + eb, a.pv.range + (side ? (size_t)a.npairs : 0) + eb, per_unit, a.vterm, ip, ctid);
-                dual_table<C>(P.lut, a.lut_img + (size_t)q * C::LUT_BYTES, ctid);  // in the place of the pair's
+                fetch_table(a.lut_img + (size_t)q * C::LUT_BYTES);  // in the place of the pair's
                 csync();
                 if (dead) return;
                 dual_exact<C>(kb, kept, a.codes, P.lut, inv, ctid);
@@ -1066,7 +991,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
                 }
                 if (kept == k) bound = kb[k - 1];
                 if (!close) {
-                    dual_table<C>(P.lut, a.pv.img + (size_t)cur_u * C::LUT_BYTES, ctid);
+                    fetch_table(a.pv.img + (size_t)cur_u * C::LUT_BYTES);
                 }
                 if (close) {
                     const size_t slot = 2 * ((size_t)cur_u + blockIdx.x) + side;
@@ -1084,22 +1009,11 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
                 if (g < dtau[side]) dtau[side] = g;
             }
         }
-        fence_proxy_async();  // strips: the next table's copy writes where keys were written and read
         csync();
     };
     auto dual_begin = [&](int unit) {
         cur_u = unit;
-        if (ctid == 0) {
-            ctrl->cnt = 0;
-            ctrl->cnt_b = 0;
-            fence_proxy_async();
-            const uint8_t* src = a.pv.img + (size_t)unit * C::LUT_BYTES;
-            const uint32_t bar = smem_u32(&ctrl->lutbar);
-            mbar_arrive_expect_tx(bar, (uint32_t)C::LUT_BYTES);
-            constexpr uint32_t PIECE = 32768;
-            for (uint32_t o = 0; o < (uint32_t)C::LUT_BYTES; o += PIECE)
-                bulk_g2s(P.lut + o, src + o, (uint32_t)C::LUT_BYTES - o < PIECE ? (uint32_t)C::LUT_BYTES - o : PIECE, bar);
-        }
+        if (ctid == 0) { ctrl->cnt = 0; ctrl->cnt_b = 0; }
         const PairParams* pp = a.pv.params + unit;
 #pragma unroll
         for (int side = 0; side < 2; ++side) {
@@ -1108,8 +1022,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
         }
 #pragma unroll
         for (int side = 0; side < 2; ++side) dtau[side] = *reinterpret_cast<volatile unsigned long long*>(&a.qthresh[dq[side]]);
-        dead = dead || !mbar_wait(smem_u32(&ctrl->lutbar), lphase, abort_flag, a.err);
-        lphase ^= 1u;
+        fetch_table(a.pv.img + (size_t)unit * C::LUT_BYTES);
         csync();
     };
 
@@ -1178,7 +1091,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
 
         // ---- scan this tile: warp w owns row groups w*RGW .. w*RGW+RGW-1 ----
         const int nvr = (D.flags >> 8) * R;
-        const uint32_t tile_base = C::SPLIT && warp >= C::LOW_WARPS ? D.tile_hi : D.tile_addr;
+        const uint32_t tile_base = D.tile_addr;
         const uint32_t vt_base = D.vt_addr;
         // Row groups are taken MERGE at a time: with R lanes per vector every lane of an R-group ends up with
         // the vector's sum, so lane slice g finishes row group g and one epilogue serves MERGE row groups.
@@ -1199,7 +1112,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
                 int acc[4] = {0, 0, 0, 0};
                 uint32_t x[C::NBLK][G];
                 LoadWords<C, G, 0, (rg + g) * 32 * C::MV>::run(wa, x);
-                ScanBlocks<C, G, 0>::run(x, cc, sel, lo, P.lut, acc);
+                ScanBlocks<C, G, 0>::run(x, at, pick, acc);
                 int si = (acc[0] + acc[1]) + (acc[2] + acc[3]);
                 if (R >= 2) si += __shfl_xor_sync(0xffffffffu, si, 1);
                 if (R >= 4) si += __shfl_xor_sync(0xffffffffu, si, 2);
@@ -1264,7 +1177,7 @@ struct Variant {
     void (*kernel)(const ScanArgs);
     int threads, tile_vecs;
     int (*stages_for)(int d, bool need_vt);
-    int lut_bytes, lut_banked, lut_copies, lut_copy_off, lut_stride;
+    int lut_bytes, lut_kind;
 };
 template <class C, bool DUAL>
 static int stages_for(int d, bool need_vt) {
@@ -1275,8 +1188,7 @@ static int stages_for(int d, bool need_vt) {
 #define RAGO_VARIANT(WV, G, R, NCW, RGW, DUAL) \
     { Cfg<WV, G, R, NCW, RGW>::M, scan_kernel<WV, G, R, NCW, RGW, DUAL>, Cfg<WV, G, R, NCW, RGW>::THREADS, \
       Cfg<WV, G, R, NCW, RGW>::TV, stages_for<Cfg<WV, G, R, NCW, RGW>, DUAL>, Cfg<WV, G, R, NCW, RGW>::LUT_BYTES, \
-      Cfg<WV, G, R, NCW, RGW>::BANKED ? 1 : 0, Cfg<WV, G, R, NCW, RGW>::COPIES, Cfg<WV, G, R, NCW, RGW>::COPY_OFF, \
-      Cfg<WV, G, R, NCW, RGW>::LSTRIDE }
+      Cfg<WV, G, R, NCW, RGW>::KIND }
 // Warps x unrolled row groups per warp were chosen by measurement: independent row groups in flight inside a warp
 // hide the look-up latency better than more warps do (M = 64: 16 x 2 -> 12 x 4 gave +30%), and 15 consumer warps
 // (four warps on every scheduler, the producer included) beat 12, 14 and 16 wherever their tiles fit (M = 32: +3%,
@@ -1285,12 +1197,11 @@ static int stages_for(int d, bool need_vt) {
 static const Variant kVariants[] = {
     RAGO_VARIANT(4, 4, 1, 16, 2, false),   // M = 16
     RAGO_VARIANT(8, 8, 1, 15, 2, false),   // M = 32
-    RAGO_VARIANT(12, 4, 1, 15, 1, false),  // M = 48 (two table copies: 128 KB, a 2 048-key buffer, tiles of at most 512 vectors)
-    RAGO_VARIANT(8, 8, 2, 15, 4, false),   // M = 64: 15 + 1 warps fill the four schedulers evenly; two 60 KB tiles below the table
+    RAGO_VARIANT(12, 4, 1, 15, 1, false),  // M = 48
+    RAGO_VARIANT(8, 8, 2, 15, 4, false),   // M = 64: two 60 KB tiles below the table
     RAGO_VARIANT(8, 8, 2, 12, 4, false),   // M = 64 where those do not fit
     RAGO_VARIANT(20, 4, 1, 8, 1, false),   // M = 80
-    RAGO_VARIANT(24, 8, 1, 15, 1, false),  // M = 96: split tiles
-    RAGO_VARIANT(24, 8, 1, 12, 1, false),  // M = 96 where those do not fit
+    RAGO_VARIANT(24, 8, 1, 15, 1, false),  // M = 96
     RAGO_VARIANT(8, 8, 4, 12, 3, false),   // M = 128
 };
 // The same table layouts for pairs of queries (the tables of 80 and 128 bytes leave no room for two buffers).
@@ -1327,8 +1238,7 @@ cudaError_t scan_plan(const IndexImpl* ix, ScanPlan* plan) {
     plan->stages = stages;
     plan->ctas = ix->num_sms;
     plan->smem_bytes = SMEM_OPTIN;
-    plan->lut_bytes = v->lut_bytes; plan->lut_banked = v->lut_banked; plan->lut_copies = v->lut_copies;
-    plan->lut_copy_off = v->lut_copy_off; plan->lut_stride = v->lut_stride;
+    plan->lut_bytes = v->lut_bytes; plan->lut_kind = v->lut_kind;
     const Variant* pv = find_pair_variant(ix->M, ix->d, ix->metric != RAGO_IP);
     plan->pair_tile_vecs = pv ? pv->tile_vecs : 0;
     if (pv) {
@@ -1456,8 +1366,8 @@ static TableArgs table_args(const IndexImpl* ix, const float* queries, uint8_t* 
     TableArgs t;
     t.queries = queries; t.cbT = ix->cbT; t.cwmax = ix->cwmax;
     t.d = ix->d; t.dsub = ix->dsub; t.M = ix->M; t.metric = ix->metric;
-    t.lut_bytes = pl.lut_bytes; t.banked = pl.lut_banked; t.copies = pl.lut_copies; t.copy_off = pl.lut_copy_off;
-    t.lstride = pl.lut_stride; t.lut_img = lut_img; t.lut_inv = lut_inv;
+    t.lut_bytes = pl.lut_bytes; t.kind = pl.lut_kind;
+    t.lut_img = lut_img; t.lut_inv = lut_inv;
     return t;
 }
 static int table_parts(const IndexImpl* ix, int nq) {
@@ -1523,8 +1433,7 @@ __global__ void __launch_bounds__(256) build_tables_batch_kernel(const TableArgs
 #pragma unroll
         for (int u = 0; u < DSUB; ++u) cw[i][u] = 0.f;
         if (j < KSUB) {
-            off[i] = t.banked ? (uint32_t)(m / 64) * 65536u + (uint32_t)j * 256u + (uint32_t)(m % 64) * 4u
-                              : ((uint32_t)j * t.lstride + (uint32_t)m) * 4u;
+            off[i] = lut_offset(t.kind, j, m);
             const float* src = t.cbT + ((size_t)j * M + m) * DSUB;
 #pragma unroll
             for (int u = 0; u < DSUB; u += 4) {
@@ -1534,8 +1443,7 @@ __global__ void __launch_bounds__(256) build_tables_batch_kernel(const TableArgs
         }
     }
     // second copy of a column (layouts that keep one), as a byte distance inside the image
-    const uint32_t copy_delta = t.copies == 2
-        ? (t.banked ? (uint32_t)((t.copy_off / 64) * 65536 + (t.copy_off % 64) * 4) : (uint32_t)t.copy_off * 4u) : 0u;
+    const uint32_t copy_delta = t.kind == LUT_DOT2 ? LUT_COPY : 0u;
     const float lut_s = t.metric == RAGO_IP ? -1.f : -2.f;
     const int q0 = blockIdx.y * qchunk;
     const int q1 = q0 + qchunk < nq ? q0 + qchunk : nq;
