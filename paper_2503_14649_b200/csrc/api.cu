@@ -73,7 +73,7 @@ static Layout make_layout(const IndexImpl* ix, int nq, int nprobe, int k) {
     const size_t npairs = (size_t)nq * nprobe;
     L.pairs = pair_applies(ix, nq, nprobe, k) ? 1 : 0;
     const int pair_nq = std::min(nq, PAIR_MAX_NQ);  // reserved for larger batches too, as below
-    const bool pair_room = L.pairs || pair_reserves(ix, pair_nq, nprobe, k);
+    const bool pair_room = L.pairs || pair_reserves(ix, pair_nq, nprobe);
     // one slot per (CTA, query) incidence; pairs and single queries are scanned, and numbered, apart
     L.nslots = pair_room ? pair_slots(nq, ix->plan.ctas) : (size_t)nq + (size_t)ix->plan.ctas;
     L.err = take(256);

@@ -321,10 +321,10 @@ static bool pair_worth(const IndexImpl* ix, int nq, int nprobe) {
     return shared >= PAIR_MIN_SHARE * scanned && 0.5 * shared * nq * ix->M >= PAIR_MIN_US * PAIR_BYTES_PER_US;
 }
 bool pair_applies(const IndexImpl* ix, int nq, int nprobe, int k) { return pair_possible(ix, nq, k) && pair_worth(ix, nq, nprobe); }
-// Workspace is set aside where any number of probes up to nprobe takes pairs: the shared part is a ratio of two linear
-// functions of it, so largest at one end, and the amount grows with it.
-bool pair_reserves(const IndexImpl* ix, int nq, int nprobe, int k) {
-    if (!pair_possible(ix, nq, k)) return false;
+// Workspace is set aside where any k, and any number of probes up to nprobe, takes pairs: the shared part is a ratio of two
+// linear functions of it, so largest at one end, and the amount grows with it.
+bool pair_reserves(const IndexImpl* ix, int nq, int nprobe) {
+    if (!pair_possible(ix, nq, 1)) return false;
     double s1, h1, s2, h2;
     pair_expect(ix, nq, 1, &s1, &h1);
     pair_expect(ix, nq, nprobe, &s2, &h2);

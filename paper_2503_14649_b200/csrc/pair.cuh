@@ -68,7 +68,7 @@ struct PairLayout {
 PairLayout pair_layout(int nq, int nprobe, int lut_bytes);
 // Whether a batch of these sizes is looked through for pairs.
 bool pair_applies(const IndexImpl* ix, int nq, int nprobe, int k);
-bool pair_reserves(const IndexImpl* ix, int nq, int nprobe, int k);
+bool pair_reserves(const IndexImpl* ix, int nq, int nprobe);
 void pair_list_stats(IndexImpl* ix, const int64_t* offsets);
 cudaError_t launch_pair_queries(const IndexImpl* ix, const int32_t* probe_list, const float* probe_term, int nq, int nprobe,
                                 const uint8_t* lut_img, const float* lut_inv, uint8_t* ws, const PairLayout& L, PairView* view,

@@ -91,6 +91,22 @@ def test_pairs_with_more_equal_scores_than_a_buffer_holds(M, k):
     ix.close()
 
 
+# A workspace sized for a larger k, more probes or more queries than pairs go with serves fewer of them, with pairs.
+@pytest.mark.parametrize("nq,nprobe,k", [(128, 3, 1024), (128, 4, 100), (300, 3, 100), (5000, 4, 1024)])
+def test_a_larger_workspace_serves_a_call_with_pairs(nq, nprobe, k):
+    ix, c, _ = _index(64, 4, [900_000, 5000, 4000, 300], seed=6)
+    q = _queries(c, [0] * 90 + [1] * 38)
+    ws = torch.empty(ix.search_workspace_bytes(nq, nprobe, k), dtype=torch.uint8, device="cuda")
+    n = binding.rago_kernel_launches()
+    ids, dists = ix.rago_search(q, 3, 100, workspace=ws)
+    n = binding.rago_kernel_launches() - n
+    torch.cuda.synchronize()
+    assert n == _launches(ix, q, 3, 1024)[0] + 5
+    i, s = ix.rago_search(q[:64].contiguous(), 3, 100)
+    assert torch.equal(ids[:64], i) and torch.equal(dists[:64], s)
+    ix.close()
+
+
 # Queries whose tables are not bounded have no partner; the others' answers do not change.
 def test_queries_with_infinite_and_huge_values_have_no_partner():
     ix, c, _ = _index(64, 4, [900_000, 5000, 4000, 300], seed=5)
