@@ -419,7 +419,11 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
 
     // Everything above touched shared memory and kernel arguments only; from here on the kernel reads what the
     // kernels before it wrote.
-    grid_dependency_wait();
+    // The launch for the single queries of a batch with pairs needs nothing of the pairs' launch in front of it, and that one
+    // lets it start only when all of its own CTAs have seen the kernels before complete: it waits at its end instead (so that
+    // what waits for it has waited for both), and takes the SMs that the pairs leave one after the other.
+    const bool late_wait = !DUAL && a.pv.head != nullptr;
+    if (!late_wait) grid_dependency_wait();
     grid_dependents_may_launch();
     // A batch of a few queries is latency-bound, and most of a CTA's start-up would be a chain of dependent reads
     // (total, binary search for the first pair, the pair's list, the list's offset) before its first tile can be
@@ -445,7 +449,10 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
     const long long W0 = e_base ? a.work_prefix[e_base] : 0, W = a.work_prefix[e_end];
     const long long u_begin = W0 + (long long)blockIdx.x * (W - W0) / gridDim.x;
     const long long u_end = W0 + (long long)(blockIdx.x + 1) * (W - W0) / gridDim.x;
-    if (u_end <= u_begin) return;
+    if (u_end <= u_begin) {
+        if (late_wait) grid_dependency_wait();
+        return;
+    }
     // few pairs: the pair whose range contains u_begin = the largest p with work_prefix[p] <= u_begin
     const int first_pair = few_pairs ? __popc(__ballot_sync(0xffffffffu, pw <= u_begin)) - 1 : -1;
 
@@ -543,9 +550,20 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
             more = advance();
             // All of the above stands before the wait for the stage, so that as little as possible lies between its coming
             // free and its refill (looking for the next tile after the wait: 48-byte codes, 300 queries 1 588 us, before it 1 500).
+            const uint32_t tile_at = ctrl->tile[st], vt_at = ctrl->vt[st];
+            const uint8_t* src = a.codes + (size_t)pos0 * C::M;
             if (round > 0) dead = !mbar_wait(smem_u32(&ctrl->empty[st]), (round - 1) & 1, abort_flag, a.err);
             if (dead) break;
             if (lane == 0) {
+                // The copies first, then the descriptor, then the arrival: the barrier's count of bytes may run ahead of what it is
+                // told to expect, and its phase cannot end without the arrival, which also makes the descriptor visible.
+                if (a.stream_once) {  // small batch: the codes are read once and should leave L2 first
+                    bulk_g2s_hint(tile_at, src, bytes, bar, once_policy);
+                    if (vbytes) bulk_g2s_hint(vt_at, a.vterm + (pos0 & ~3u), vbytes, bar, once_policy);
+                } else {
+                    bulk_g2s(tile_at, src, bytes, bar);
+                    if (vbytes) bulk_g2s(vt_at, a.vterm + (pos0 & ~3u), vbytes, bar);
+                }
                 TileDesc& D = ctrl->desc[st];
                 // everything tiles n-S+1 .. n can still push must fit behind what is in the buffer now
                 const int cnt_seen = *reinterpret_cast<volatile int*>(&ctrl->cnt);
@@ -555,22 +573,13 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
                     flags |= (seen_b + (S + 1) * C::TV > C::KCAP ? 8 : 0) | (mask << 4);
                     D.term_b = term_b;
                 }
-                const uint32_t tile_at = ctrl->tile[st], vt_at = ctrl->vt[st];
                 D.flags = flags;
                 D.pos0 = pos0;
                 D.tile_addr = tile_at;
                 D.vt_addr = vt_at + (pos0 & 3u) * 4u;
                 D.pair = pair;
                 D.term = term;
-                const uint8_t* src = a.codes + (size_t)pos0 * C::M;
                 mbar_arrive_expect_tx(bar, bytes + vbytes);
-                if (a.stream_once) {  // small batch: the codes are read once and should leave L2 first
-                    bulk_g2s_hint(tile_at, src, bytes, bar, once_policy);
-                    if (vbytes) bulk_g2s_hint(vt_at, a.vterm + (pos0 & ~3u), vbytes, bar, once_policy);
-                } else {
-                    bulk_g2s(tile_at, src, bytes, bar);
-                    if (vbytes) bulk_g2s(vt_at, a.vterm + (pos0 & ~3u), vbytes, bar);
-                }
                 // pull the tiles a few steps ahead in this list into L2, with their terms, so that their copies find them there
                 if (a.prefetch) {
                     for (int ahead = (t_in_pair == 0 ? 1 : SCAN_PF); ahead <= SCAN_PF && u_this + ahead < u_end; ++ahead) {
@@ -593,6 +602,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
                 for (int it = 0; it < (1 << 16) && !mbar_try_wait(bar, (n / S) & 1); ++it) __nanosleep(64);
             }
         }
+        if (late_wait) grid_dependency_wait();
         return;
     }
 
@@ -1169,6 +1179,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
         }
     }
     if constexpr (!DUAL) { if (!dead && cur_u >= 0) finalize(); }
+    if (late_wait) grid_dependency_wait();
 }
 
 // ---- host side ----------------------------------------------------------------------------------
@@ -1190,14 +1201,15 @@ static int stages_for(int d, bool need_vt) {
       Cfg<WV, G, R, NCW, RGW>::TV, stages_for<Cfg<WV, G, R, NCW, RGW>, DUAL>, Cfg<WV, G, R, NCW, RGW>::LUT_BYTES, \
       Cfg<WV, G, R, NCW, RGW>::KIND }
 // Warps x unrolled row groups per warp were chosen by measurement: independent row groups in flight inside a warp
-// hide the look-up latency better than more warps do (M = 64: 16 x 2 -> 12 x 4 gave +30%), and 15 consumer warps
+// hide the look-up latency better than more warps do (M = 64: 16 x 2 -> 12 x 4 gave +30%; M = 48: 15 x 1 -> 15 x 2 +13 to 17%, for
+// pairs 15 x 1 -> 10 x 2 +6%, 8 x 2 -6%; M = 96: 15 x 1 -> 8 x 2 -4%, for pairs 15 x 1 -> 7 x 2 -11%), and 15 consumer warps
 // (four warps on every scheduler, the producer included) beat 12, 14 and 16 wherever their tiles fit (M = 32: +3%,
-// M = 48: +6%, M = 64: +4.5%).  Where a code size has two entries the first one whose shared-memory plan fits the
+// M = 64: +4.5%).  Where a code size has two entries the first one whose shared-memory plan fits the
 // index (dimension, metric) is taken.
 static const Variant kVariants[] = {
     RAGO_VARIANT(4, 4, 1, 16, 2, false),   // M = 16
     RAGO_VARIANT(8, 8, 1, 15, 2, false),   // M = 32
-    RAGO_VARIANT(12, 4, 1, 15, 1, false),  // M = 48
+    RAGO_VARIANT(12, 4, 1, 15, 2, false),  // M = 48: two 46 KB tiles beside the 96 KB table
     RAGO_VARIANT(8, 8, 2, 15, 4, false),   // M = 64: two 60 KB tiles below the table
     RAGO_VARIANT(8, 8, 2, 12, 4, false),   // M = 64 where those do not fit
     RAGO_VARIANT(20, 4, 1, 8, 1, false),   // M = 80
@@ -1208,7 +1220,7 @@ static const Variant kVariants[] = {
 static const Variant kPairVariants[] = {
     RAGO_VARIANT(4, 4, 1, 15, 2, true),    // M = 16: 16 warps and the producer would leave 96 registers a thread, too few
     RAGO_VARIANT(8, 8, 1, 15, 2, true),
-    RAGO_VARIANT(12, 4, 1, 15, 1, true),
+    RAGO_VARIANT(12, 4, 1, 10, 2, true),   // M = 48: two row groups for as many warps as the two buffers leave room for
     RAGO_VARIANT(8, 8, 2, 15, 2, true),    // M = 64: the tiles in flight have to fit each buffer twice over
     RAGO_VARIANT(24, 8, 1, 15, 1, true),
 };
@@ -1285,7 +1297,7 @@ int scan_pair_lead(const IndexImpl* ix) {
 // 9 520 / 8 940, 80 bytes 19 490 / 18 950.  With lists below 32 tiles, inside L2, and for the other sizes (6 M vectors in 64
 // lists, 16 bytes 3%, 64 bytes 3%, 96 bytes 1% more) it is the other way round or equal.
 bool scan_prefetches(const IndexImpl* ix, int64_t npairs) {
-    const int tile_bytes = ix->plan.tile_vecs * ix->M;
+    const int tile_bytes = ix->plan.tile_vecs * ix->M / (ix->M == 48 ? 2 : 1);  // 48 bytes: measured with tiles of half the size
     const bool long_lists = ix->N / ix->nlist >= 32ll * ix->plan.tile_vecs && ix->N * ix->M > (128ll << 20);
     return (tile_bytes <= 40 * 1024 && npairs <= 4ll * ix->nlist) || (ix->M >= 48 && tile_bytes <= 24 * 1024 && long_lists);
 }
