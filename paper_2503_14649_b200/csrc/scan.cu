@@ -1299,7 +1299,7 @@ int scan_pair_lead(const IndexImpl* ix) {
 bool scan_prefetches(const IndexImpl* ix, int64_t npairs) {
     const int tile_bytes = ix->plan.tile_vecs * ix->M / (ix->M == 48 ? 2 : 1);  // 48 bytes: measured with tiles of half the size
     const bool long_lists = ix->N / ix->nlist >= 32ll * ix->plan.tile_vecs && ix->N * ix->M > (128ll << 20);
-    return (tile_bytes <= 40 * 1024 && npairs <= 4ll * ix->nlist) || (ix->M >= 48 && tile_bytes <= 24 * 1024 && long_lists);
+    return (tile_bytes <= 48 * 1024 && npairs <= 4ll * ix->nlist) || (ix->M >= 48 && tile_bytes <= 24 * 1024 && long_lists);
 }
 
 // view (may be null): the batch's pairs of queries, scanned by a launch of their own in front of that of the single ones.
