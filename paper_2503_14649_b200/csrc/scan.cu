@@ -759,15 +759,17 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
         }
         csync();  // the minima / maxima have been read; redu is free for the counts
         if (dead) return;
-        long long lo = (long long)mn - 1, hi = mx;  // #(score <= lo) < k <= #(score <= hi)
+        // Whole keys are bisected, not scores: of a group of equal scores larger than the buffer (duplicates among the vectors) the
+        // first by position are kept, and room remains for what is better than all of them.  #(key <= lo) < k <= #(key <= hi)
+        unsigned long long lo = mn ? ((unsigned long long)mn << 32) - 1 : 0ull, hi = ((unsigned long long)mx << 32) | 0xFFFFFFFFull;
         uint32_t c_hi = (uint32_t)n;
         const uint32_t want_max = (uint32_t)(k + (k >> 2) + 8);
         int round = 0;
         while (hi - lo > 1 && c_hi > want_max) {  // uniform across the CTA
-            const uint32_t mid = (uint32_t)(lo + (hi - lo) / 2);
+            const unsigned long long mid = lo + (hi - lo) / 2;
             uint32_t c = 0;
 #pragma unroll
-            for (int j = 0; j < KPT; ++j) c += (mine[j] != KEY_MAX && (uint32_t)(mine[j] >> 32) <= mid) ? 1u : 0u;
+            for (int j = 0; j < KPT; ++j) c += mine[j] <= mid ? 1u : 0u;  // (mid < KEY_MAX, the value of a slot without a key)
             c = __reduce_add_sync(0xffffffffu, c);
             if (lane == 0) ctrl->redu[round & 1][warp] = c;
             csync();
@@ -777,16 +779,14 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
             if (c < (uint32_t)k) lo = mid; else { hi = mid; c_hi = c; }
             ++round;
         }
-        const uint32_t T = (uint32_t)hi;
         if (ctid == 0) ctrl->cnt = 0;  // every thread holds its keys in registers since the first barrier above
         csync();
         if (dead) return;
 #pragma unroll
         for (int j = 0; j < KPT; ++j)
-            warp_push(keys, &ctrl->cnt, mine[j] != KEY_MAX && (uint32_t)(mine[j] >> 32) <= T, mine[j], C::KCAP);
-        const unsigned long long bound = ((unsigned long long)T << 32) | 0xFFFFFFFFull;  // >= the k-th best key
-        if (bound < tau) tau = bound;
-        if (ctid == 0) atomicMin(&a.qthresh[cur_q], bound);
+            warp_push(keys, &ctrl->cnt, mine[j] != KEY_MAX && mine[j] <= hi, mine[j], C::KCAP);
+        if (hi < tau) tau = hi;  // >= the k-th best key
+        if (ctid == 0) atomicMin(&a.qthresh[cur_q], hi);
     };
 
     // Close the current query's candidate buffer: keep at most k keys and park them in this CTA's slot.

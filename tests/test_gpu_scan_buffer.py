@@ -1,0 +1,48 @@
+"""Candidate buffers of the scan: groups of equal scores larger than a buffer, and values of k near its capacity."""
+
+import pytest
+import torch
+
+from paper_2503_14649_b200 import binding
+
+pytestmark = pytest.mark.gpu
+
+
+def _scores(q, c, books, codes, metric):
+    """Exact scores (smaller is better) of codes under one list with centroid c, in fp64."""
+    M, _, dsub = books.shape
+    out = torch.empty(q.shape[0], codes.shape[0], dtype=torch.float64, device=q.device)
+    for i in range(q.shape[0]):
+        r = (q[i] - c).double().view(M, 1, dsub)
+        t = ((r - books.double()) ** 2).sum(2) if metric == "l2" else -(q[i].double().view(M, 1, dsub) * (books.double() + c.double().view(M, 1, dsub))).sum(2)
+        out[i] = t[torch.arange(M, device=q.device)[None, :], codes.long()].sum(1)
+    return out
+
+
+# One list of mostly identical vectors, farther from the query than the few others among them: more equal scores than a buffer holds
+# reach every CTA before the better ones do.  Sums of M fp32 terms: 1e-5 of the largest score covers their rounding.
+@pytest.mark.parametrize("M,metric,nq,k", [(16, "l2", 1, 100), (32, "ip", 1, 33), (48, "l2", 1, 100), (64, "ip", 1, 100), (64, "l2", 1, 300), (80, "l2", 1, 40),
+                                           (96, "l2", 1, 100), (96, "ip", 2, 500), (128, "ip", 1, 100), (64, "l2", 1, 10), (96, "l2", 70, 100)])
+def test_better_vectors_behind_more_equal_ones_than_a_buffer_holds(M, metric, nq, k):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + k)
+    N, d = 1_400_000, 4 * M
+    c = torch.randn(1, d, generator=g, device="cuda")
+    books = 0.3 * torch.randn(M, 256, 4, generator=g, device="cuda")
+    q = (c + 0.3 * torch.randn(1, d, generator=g, device="cuda")).repeat(nq, 1).contiguous()
+    every = torch.arange(256, device="cuda")[:, None].expand(256, M).to(torch.uint8)
+    per_code = torch.stack([_scores(q[:1], c[0], books * (torch.arange(M, device="cuda") == m).view(M, 1, 1), every, metric)[0] for m in range(M)], 1)
+    codes = per_code.argmax(0).to(torch.uint8).expand(N, M).contiguous()  # the worst code of every sub-space
+    few = torch.randperm(N, generator=g, device="cuda")[:N // 1000]
+    codes[few] = torch.randint(0, 256, (few.numel(), M), generator=g, device="cuda", dtype=torch.uint8)
+    ix = binding.rago_index_load(c, books, codes, torch.tensor([0, N], device="cuda"), torch.arange(N, device="cuda"), metric)
+    ids, dists = ix.rago_search(q, 1, k)
+    torch.cuda.synchronize()
+    ix.rago_check()
+    exact = _scores(q[:1], c[0], books, codes[few], metric)[0]
+    want, at = exact.sort()
+    sign = 1.0 if metric == "l2" else -1.0
+    for i in (0, nq - 1):
+        assert torch.allclose(sign * dists[i].double(), want[:k], rtol=0, atol=1e-5 * float(want.abs().max()))
+        assert set(ids[i].tolist()) <= set(few[at[:k + 5]].tolist())
+    ix.close()
