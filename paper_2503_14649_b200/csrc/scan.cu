@@ -392,6 +392,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
     const uint32_t base = smem_u32(smem);
     const SmemPlan P = plan_smem<C, DUAL>(base, a.dyn_bytes, a.d, S, a.vterm != nullptr);
     if (!P.ok) {  // uniform: every thread sees the same plan
+        grid_dependency_wait();  // a CTA that exits lets the next kernel go on as one that has waited does
         if (tid == 0) atomicExch(a.err, (uint32_t)ERR_SMEM_LAYOUT);
         return;
     }
@@ -418,12 +419,9 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
     __syncthreads();
 
     // Everything above touched shared memory and kernel arguments only; from here on the kernel reads what the
-    // kernels before it wrote.
-    // The launch for the single queries of a batch with pairs needs nothing of the pairs' launch in front of it, and that one
-    // lets it start only when all of its own CTAs have seen the kernels before complete: it waits at its end instead (so that
-    // what waits for it has waited for both), and takes the SMs that the pairs leave one after the other.
-    const bool late_wait = !DUAL && a.pv.head != nullptr;
-    if (!late_wait) grid_dependency_wait();
+    // kernels before it wrote.  That holds for the launch for the single queries of a batch with pairs too, although it reads nothing
+    // of the pairs' launch in front of it: that one's wait says nothing about what this one sees.
+    grid_dependency_wait();
     grid_dependents_may_launch();
     // A batch of a few queries is latency-bound, and most of a CTA's start-up would be a chain of dependent reads
     // (total, binary search for the first pair, the pair's list, the list's offset) before its first tile can be
@@ -449,10 +447,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
     const long long W0 = e_base ? a.work_prefix[e_base] : 0, W = a.work_prefix[e_end];
     const long long u_begin = W0 + (long long)blockIdx.x * (W - W0) / gridDim.x;
     const long long u_end = W0 + (long long)(blockIdx.x + 1) * (W - W0) / gridDim.x;
-    if (u_end <= u_begin) {
-        if (late_wait) grid_dependency_wait();
-        return;
-    }
+    if (u_end <= u_begin) return;
     // few pairs: the pair whose range contains u_begin = the largest p with work_prefix[p] <= u_begin
     const int first_pair = few_pairs ? __popc(__ballot_sync(0xffffffffu, pw <= u_begin)) - 1 : -1;
 
@@ -602,7 +597,6 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
                 for (int it = 0; it < (1 << 16) && !mbar_try_wait(bar, (n / S) & 1); ++it) __nanosleep(64);
             }
         }
-        if (late_wait) grid_dependency_wait();
         return;
     }
 
@@ -1179,7 +1173,6 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_ke
         }
     }
     if constexpr (!DUAL) { if (!dead && cur_u >= 0) finalize(); }
-    if (late_wait) grid_dependency_wait();
 }
 
 // ---- host side ----------------------------------------------------------------------------------
