@@ -110,8 +110,9 @@ struct ScanArgs {
     PairView pv;             // batches in which queries are scanned two at a time (pair.cuh); pv.head null: not this one
 };
 
-template <int WV, int G, int R, int NCW_, int RGW_>
+template <int WV, int G, int R, int NCW_, int RGW_, bool DUAL_>
 struct Cfg {
+    static constexpr bool DUAL = DUAL_;                 // two queries at a time
     static constexpr int NCW = NCW_;                    // consumer warps
     static constexpr int NCT = NCW * 32;                // consumer threads
     static constexpr int THREADS = NCT + 32;            // + one producer warp
@@ -125,7 +126,9 @@ struct Cfg {
     static constexpr int TV = TILE_VROWS / R;           // vectors per tile
     static constexpr int TILE_BYTES = TILE_VROWS * MV;
     static constexpr int VT_BYTES = (TV + 4) * 4;       // staged per-vector terms (start rounded down to 16 bytes)
-    static constexpr int KCAP = LUT_BYTES <= 65536 || M == 48 ? 2 * TOPK_CAP : TOPK_CAP;  // keys of the CTA's candidate buffer
+    // Keys of a candidate buffer (two queries at a time: two buffers): as many as fit beside two tiles.  Few keys mean a cut
+    // before every tile: 96 bytes, 400 queries over lists of 2 200, k = 500, 2 048 / 4 096 keys 1 305 / 726 us, k = 1 024 1 590 / 800.
+    static constexpr int KCAP = LUT_BYTES + 2 * (TILE_BYTES + VT_BYTES) + (DUAL ? 2 : 1) * 2 * TOPK_CAP * 8 + CTRL_BYTES <= SMEM_OPTIN ? 2 * TOPK_CAP : TOPK_CAP;
     // Tables of the kind LUT_PERM start at this absolute shared address (a multiple of 64 KB).  Two tiles of more than 48 KB do not
     // fit above a table at 64 KB, so configurations with such tiles keep their tiles below a table at 128 KB.
     static constexpr uint32_t LUT_WINDOW = TILE_BYTES > 48 * 1024 ? 0x20000u : 0x10000u;
@@ -133,10 +136,13 @@ struct Cfg {
     static_assert(TILE_VROWS % R == 0, "tile must hold whole vectors");
     static_assert(RGW % (R < RGW ? R : RGW) == 0, "row groups are taken min(R, RGW) at a time");
     // The producer asks for a cut of the candidate buffer when the count it sees plus everything the tiles in
-    // flight can still push would not fit; SMAX bounds the ring depth so that this leaves room to work in.
-    static constexpr int SMAX = KCAP / TV / 2 < MAX_STAGES ? KCAP / TV / 2 : MAX_STAGES;
-    static_assert(SMAX >= 2, "two tiles in flight must fit the candidate buffer twice over");
-    static_assert(MAX_K + SMAX * TV <= KCAP, "k kept keys plus the pushes of all tiles in flight must fit");
+    // flight can still push would not fit.  It reads the count while a cut may be rewriting it, and may see less than the cut
+    // keeps: the tiles in flight are then pushed behind that without another cut, so both must fit.  SMAX bounds the ring depth
+    // accordingly, and so that half the buffer is left to work in.
+    static constexpr int CUT_KEEPS = DUAL ? PAIR_MAX_K + TV : MAX_K + MAX_K / 4 + 8;  // of pairs at most KCAP - (S + 1) * TV
+    static constexpr int SFIT = (KCAP - CUT_KEEPS) / TV, SHALF = KCAP / TV / 2;
+    static constexpr int SMAX = SFIT < SHALF ? (SFIT < MAX_STAGES ? SFIT : MAX_STAGES) : (SHALF < MAX_STAGES ? SHALF : MAX_STAGES);
+    static_assert(SMAX >= 2, "two tiles in flight must fit the candidate buffer twice over, and behind what a cut keeps");
     static_assert(VT_BYTES % 16 == 0 && TILE_BYTES % 16 == 0, "bulk-copy destinations are 16-byte granular");
     static_assert(KIND == LUT_DOT2 ? G == 4 && R == 1 : MV % 32 == 0, "a lane's columns of a block of words lie in one 32-column part of the table");
     static_assert(KIND != LUT_PERM || NBLK == 1, "one block of words to a (virtual) row");
@@ -150,7 +156,7 @@ struct SmemPlan {
     int ok;
 };
 
-template <class C, bool DUAL>
+template <class C>
 __host__ __device__ inline SmemPlan plan_smem(uint32_t base, uint32_t dyn_bytes, int d, int stages, bool need_vt) {
     SmemPlan p;
     p.ok = 1;
@@ -174,11 +180,11 @@ __host__ __device__ inline SmemPlan plan_smem(uint32_t base, uint32_t dyn_bytes,
     };
     // largest pieces first
     for (int s = 0; s < MAX_STAGES; ++s) p.tile[s] = s < stages ? take(C::TILE_BYTES, 128) : base;
-    p.keys = take(C::KCAP * (DUAL ? 16 : 8), 16);  // two queries at a time: two buffers
+    p.keys = take(C::KCAP * (C::DUAL ? 16 : 8), 16);  // two queries at a time: two buffers
     for (int s = 0; s < MAX_STAGES; ++s) p.vt[s] = (s < stages && need_vt) ? take(C::VT_BYTES, 16) : base;
     // The scaled, transposed query is only alive while a table is built, when the candidate buffer is empty: it
     // shares the buffer's space when it fits there.
-    p.rT = DUAL ? base : (uint32_t)d * 4 <= (uint32_t)C::KCAP * 8 ? p.keys : take((uint32_t)d * 4, 16);
+    p.rT = C::DUAL ? base : (uint32_t)d * 4 <= (uint32_t)C::KCAP * 8 ? p.keys : take((uint32_t)d * 4, 16);
     p.ctrl = take(CTRL_BYTES, 16);
     return p;
 }
@@ -383,14 +389,14 @@ __device__ __forceinline__ void dual_exact(unsigned long long* kb, int kept, con
 
 // DUAL: every unit of work is a pair of queries (pair.cuh).
 template <int WV, int G, int R, int NCW_, int RGW_, bool DUAL>
-__global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_>::THREADS, 1) scan_kernel(const ScanArgs a) {
-    using C = Cfg<WV, G, R, NCW_, RGW_>;
+__global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_, DUAL>::THREADS, 1) scan_kernel(const ScanArgs a) {
+    using C = Cfg<WV, G, R, NCW_, RGW_, DUAL>;
     constexpr int NCW = C::NCW, NCT = C::NCT;
     extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int S = a.stages;
     const uint32_t base = smem_u32(smem);
-    const SmemPlan P = plan_smem<C, DUAL>(base, a.dyn_bytes, a.d, S, a.vterm != nullptr);
+    const SmemPlan P = plan_smem<C>(base, a.dyn_bytes, a.d, S, a.vterm != nullptr);
     if (!P.ok) {  // uniform: every thread sees the same plan
         grid_dependency_wait();  // a CTA that exits lets the next kernel go on as one that has waited does
         if (tid == 0) atomicExch(a.err, (uint32_t)ERR_SMEM_LAYOUT);
@@ -1183,16 +1189,16 @@ struct Variant {
     int (*stages_for)(int d, bool need_vt);
     int lut_bytes, lut_kind;
 };
-template <class C, bool DUAL>
+template <class C>
 static int stages_for(int d, bool need_vt) {
     for (int s = C::SMAX; s >= 2; --s)
-        if (plan_smem<C, DUAL>(SMEM_BASE_EXPECTED, SMEM_OPTIN, d, s, need_vt).ok) return s;
+        if (plan_smem<C>(SMEM_BASE_EXPECTED, SMEM_OPTIN, d, s, need_vt).ok) return s;
     return 0;
 }
 #define RAGO_VARIANT(WV, G, R, NCW, RGW, DUAL) \
-    { Cfg<WV, G, R, NCW, RGW>::M, scan_kernel<WV, G, R, NCW, RGW, DUAL>, Cfg<WV, G, R, NCW, RGW>::THREADS, \
-      Cfg<WV, G, R, NCW, RGW>::TV, stages_for<Cfg<WV, G, R, NCW, RGW>, DUAL>, Cfg<WV, G, R, NCW, RGW>::LUT_BYTES, \
-      Cfg<WV, G, R, NCW, RGW>::KIND }
+    { Cfg<WV, G, R, NCW, RGW, DUAL>::M, scan_kernel<WV, G, R, NCW, RGW, DUAL>, Cfg<WV, G, R, NCW, RGW, DUAL>::THREADS, \
+      Cfg<WV, G, R, NCW, RGW, DUAL>::TV, stages_for<Cfg<WV, G, R, NCW, RGW, DUAL>>, Cfg<WV, G, R, NCW, RGW, DUAL>::LUT_BYTES, \
+      Cfg<WV, G, R, NCW, RGW, DUAL>::KIND }
 // Warps x unrolled row groups per warp were chosen by measurement: independent row groups in flight inside a warp
 // hide the look-up latency better than more warps do (M = 64: 16 x 2 -> 12 x 4 gave +30%; M = 48: 15 x 1 -> 15 x 2 +13 to 17%, for
 // pairs 15 x 1 -> 10 x 2 +6%, 8 x 2 -6%; M = 96: 15 x 1 -> 8 x 2 -4%, for pairs 15 x 1 -> 7 x 2 -11%), and 15 consumer warps

@@ -46,3 +46,31 @@ def test_better_vectors_behind_more_equal_ones_than_a_buffer_holds(M, metric, nq
         assert torch.allclose(sign * dists[i].double(), want[:k], rtol=0, atol=1e-5 * float(want.abs().max()))
         assert set(ids[i].tolist()) <= set(few[at[:k + 5]].tolist())
     ix.close()
+
+
+# Vectors from the farthest to the closest, over and over: nearly every one passes the threshold, the buffer is cut every few tiles, and what a
+# cut keeps (up to k * 5 / 4 keys) has the tiles in flight pushed behind it.  Long enough that some cut meets the producer's look at the count.
+@pytest.mark.parametrize("M,metric,k", [(16, "l2", 1024), (32, "ip", 1024), (48, "l2", 1000), (64, "ip", 1024), (80, "l2", 1024), (96, "l2", 1024),
+                                        (96, "ip", 980), (96, "l2", 600), (128, "ip", 1024)])
+def test_large_k_over_vectors_in_descending_order_of_score(M, metric, k):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + k)
+    N, d, block = 2_000_000, 4 * M, 13_000
+    c = torch.randn(1, d, generator=g, device="cuda")
+    books = 0.3 * torch.randn(M, 256, 4, generator=g, device="cuda")
+    q = (c + 0.3 * torch.randn(1, d, generator=g, device="cuda")).contiguous()
+    codes = torch.randint(0, 256, (N, M), generator=g, device="cuda", dtype=torch.uint8)
+    score = torch.cat([_scores(q, c[0], books, part, metric)[0] for part in codes.split(100_000)])
+    order = torch.cat([b + score[b:b + block].argsort(descending=True) for b in range(0, N, block)])
+    codes, score = codes[order].contiguous(), score[order]
+    ix = binding.rago_index_load(c, books, codes, torch.tensor([0, N], device="cuda"), torch.arange(N, device="cuda"), metric)
+    want, at = score.sort()
+    allowed = set(at[:k + 8].tolist())
+    sign = 1.0 if metric == "l2" else -1.0
+    for _ in range(10):
+        ids, dists = ix.rago_search(q, 1, k)
+        torch.cuda.synchronize()
+        ix.rago_check()
+        assert torch.allclose(sign * dists[0].double(), want[:k], rtol=0, atol=1e-5 * float(want.abs().max()))
+        assert set(ids[0].tolist()) <= allowed
+    ix.close()
