@@ -24,6 +24,7 @@ struct ScanPlan {
     int tile_vecs;     // vectors per code tile
     int stages;        // tiles in flight per CTA
     int ctas;          // persistent CTAs (one per SM)
+    int buffer_keys;   // keys of a CTA's candidate buffer
     size_t smem_bytes;
     // shared-memory image of a query's lookup table, as the scan variant of this index lays it out
     int lut_bytes, lut_kind;

@@ -1187,7 +1187,7 @@ struct Variant {
     void (*kernel)(const ScanArgs);
     int threads, tile_vecs;
     int (*stages_for)(int d, bool need_vt);
-    int lut_bytes, lut_kind;
+    int lut_bytes, lut_kind, buffer_keys;
 };
 template <class C>
 static int stages_for(int d, bool need_vt) {
@@ -1198,7 +1198,7 @@ static int stages_for(int d, bool need_vt) {
 #define RAGO_VARIANT(WV, G, R, NCW, RGW, DUAL) \
     { Cfg<WV, G, R, NCW, RGW, DUAL>::M, scan_kernel<WV, G, R, NCW, RGW, DUAL>, Cfg<WV, G, R, NCW, RGW, DUAL>::THREADS, \
       Cfg<WV, G, R, NCW, RGW, DUAL>::TV, stages_for<Cfg<WV, G, R, NCW, RGW, DUAL>>, Cfg<WV, G, R, NCW, RGW, DUAL>::LUT_BYTES, \
-      Cfg<WV, G, R, NCW, RGW, DUAL>::KIND }
+      Cfg<WV, G, R, NCW, RGW, DUAL>::KIND, Cfg<WV, G, R, NCW, RGW, DUAL>::KCAP }
 // Warps x unrolled row groups per warp were chosen by measurement: independent row groups in flight inside a warp
 // hide the look-up latency better than more warps do (M = 64: 16 x 2 -> 12 x 4 gave +30%; M = 48: 15 x 1 -> 15 x 2 +13 to 17%, for
 // pairs 15 x 1 -> 10 x 2 +6%, 8 x 2 -6%; M = 96: 15 x 1 -> 8 x 2 -4%, for pairs 15 x 1 -> 7 x 2 -11%), and 15 consumer warps
@@ -1247,6 +1247,7 @@ cudaError_t scan_plan(const IndexImpl* ix, ScanPlan* plan) {
     const int stages = v->stages_for(ix->d, ix->metric != RAGO_IP);
     plan->tile_vecs = v->tile_vecs;
     plan->stages = stages;
+    plan->buffer_keys = v->buffer_keys;
     plan->ctas = ix->num_sms;
     plan->smem_bytes = SMEM_OPTIN;
     plan->lut_bytes = v->lut_bytes; plan->lut_kind = v->lut_kind;
@@ -1267,12 +1268,13 @@ cudaError_t scan_plan(const IndexImpl* ix, ScanPlan* plan) {
 // about 5.5 us; more with a 4 096-key buffer 7 us, with a 2 048-key buffer (more cuts) 17; per tile 1 us for 36 KB, no
 // less than 0.8 us.  Where a share is shorter than the start of a query the tiles are short or few, no CTA waits long
 // for another, and leads only leave CTAs without work (64 queries over 100 000 vectors 64.8 -> 67.1 us per call): none.
-// The three starts were measured with 32, 64 and 48 bytes; the other sizes take them by table size and k (a small k on a 128 KB
-// table that of a 64 KB one), and the tile count is that of average lists.  Both only move work between CTAs: no result
-// depends on them.
+// 7 and 17 were measured with 64 bytes and with 48 in their former buffer of 2 048 keys; the other sizes take them by their
+// buffer, and the tile count is that of average lists.  With 7 / 17 for the buffers of 4 096 keys beside 96 KB tables, us per call: 48 bytes,
+// lists of 2 200, 40 queries 95.0 / 98.8, 100 queries 170.2 / 169.1, 200 over lists of 10 000 686 / 682; 96 bytes the same 126.6 / 127.8,
+// 230.4 / 234.2, 1 158 / 1 156.  All of them only move work between CTAs: no result depends on them.
 int scan_query_lead(const IndexImpl* ix, int nq, int nprobe, int k) {
     if (nq < 2 || ix->nlist < 1) return 0;
-    const float start_us = k <= 32 ? 5.5f : (ix->plan.lut_bytes <= 65536 ? 7.f : 17.f);
+    const float start_us = k <= 32 ? 5.5f : (ix->plan.buffer_keys > TOPK_CAP ? 7.f : 17.f);
     const float tile_us = (float)(ix->plan.tile_vecs * ix->M) / 36000.f;
     const int lead = (int)(start_us / (tile_us > 0.8f ? tile_us : 0.8f) + 0.5f);
     const int64_t tiles_per_list = (ix->N / ix->nlist + ix->plan.tile_vecs) / ix->plan.tile_vecs;  // of a list of average length

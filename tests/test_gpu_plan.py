@@ -86,3 +86,12 @@ def test_a_workspace_also_serves_fewer_probes(nlist, nq, nprobes):
         ix.rago_check(ws)
         assert int((ids >= 0).sum()) > 0
     ix.close()
+
+
+# The start of a query weighs 7 us where the candidate buffer holds 4 096 keys, 17 where it holds 2 048, 5.5 for a small k, in tiles of 36 000
+# bytes a us (at least 0.8 us each): buffers of 2 048 are those of 80 and 128 bytes.
+@pytest.mark.parametrize("M,k,lead", [(48, 100, 5), (96, 100, 5), (64, 100, 4), (32, 100, 8), (80, 100, 21), (128, 100, 17), (48, 20, 4), (96, 20, 4)])
+def test_the_weight_of_a_query_start_goes_by_the_candidate_buffer(M, k, lead):
+    ix = _index(64, d=4 * M, M=M, N=200_000)
+    assert ix.rago_debug_search_plan(400, 32, k)["lead"] == lead
+    ix.close()
