@@ -107,7 +107,7 @@ struct ScanArgs {
                              // table the next search's coarse step reads stays in L2
     int32_t prefetch;        // pull tiles into L2 ahead of their copies
     uint32_t dyn_bytes;
-    PairView pv;             // batches in which queries are scanned two at a time (pair.cuh); pv.head null: not this one
+    PairView pv;             // batches in which queries are scanned two at a time (pair.cuh)
 };
 
 template <int WV, int G, int R, int NCW_, int RGW_, bool DUAL_>
@@ -387,9 +387,13 @@ __device__ __forceinline__ void dual_exact(unsigned long long* kb, int kept, con
     }
 }
 
-// DUAL: every unit of work is a pair of queries (pair.cuh).
-template <int WV, int G, int R, int NCW_, int RGW_, bool DUAL>
-__global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_, DUAL>::THREADS, 1) scan_kernel(const ScanArgs a) {
+// SCAN_PAIRS: every unit of work is a pair of queries (pair.cuh).  SCAN_BESIDE: the single queries of a batch with pairs.  SCAN_ALONE: every
+// query of a batch without.  (One kernel for the latter two, which found the entries of its launch at run time, was 1 to 6% slower on
+// batches without pairs: us per call, 200 queries, 512 of 1 024 lists of 980 vectors, 32 bytes 1 250 / 1 226, 128 bytes 3 240 / 3 047.)
+enum ScanMode { SCAN_ALONE, SCAN_BESIDE, SCAN_PAIRS };
+template <int WV, int G, int R, int NCW_, int RGW_, ScanMode MODE>
+__global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_, MODE == SCAN_PAIRS>::THREADS, 1) scan_kernel(const ScanArgs a) {
+    constexpr bool DUAL = MODE == SCAN_PAIRS;
     using C = Cfg<WV, G, R, NCW_, RGW_, DUAL>;
     constexpr int NCW = C::NCW, NCT = C::NCT;
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -435,9 +439,9 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_, DUAL>::THREADS, 1) s
     // first pair follows from one vote; the producer warp reads the rest of every pair's description in the same
     // round trip (the offsets in a second one), and the consumers know their first query without the producer.
     // (Not where the entries of the batch are divided between pairs and single queries.)
-    const bool few_pairs = !DUAL && a.npairs <= 32 && a.pv.head == nullptr;
+    const bool few_pairs = MODE == SCAN_ALONE && a.npairs <= 32;
     // the entries this launch scans, and how many of them make a unit: a query, or a pair of queries
-    const int npairs_q = DUAL || a.pv.head != nullptr ? a.pv.head[0] : 0;
+    const int npairs_q = MODE == SCAN_ALONE ? 0 : a.pv.head[0];
     const int per_unit = DUAL ? 2 * a.nprobe : a.nprobe;
     const int e_base = DUAL ? 0 : 2 * a.nprobe * npairs_q, e_end = DUAL ? 2 * a.nprobe * npairs_q : a.npairs;
     const long long pw = few_pairs ? a.work_prefix[lane < a.npairs ? lane : a.npairs] : 0;  // >= npairs: the total
@@ -808,7 +812,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_, DUAL>::THREADS, 1) s
             if (dead) return;
         }
         if (kept == k && ctid == 0) atomicMin(&a.qthresh[cur_q], keys[k - 1]);
-        const size_t slot = (a.pv.head != nullptr ? 2 * ((size_t)npairs_q + gridDim.x) : 0) + cur_u + blockIdx.x;
+        const size_t slot = (MODE == SCAN_BESIDE ? 2 * ((size_t)npairs_q + gridDim.x) : 0) + cur_u + blockIdx.x;
         for (int i = ctid; i < kept; i += NCT) a.slot_keys[slot * k + i] = keys[i];
         if (ctid == 0) a.slot_cnt[slot] = kept;
         csync();
@@ -819,7 +823,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_, DUAL>::THREADS, 1) s
     // that length), so that the tiles that follow are pushed against a threshold instead of in full.
     bool early = false;
     auto begin_query = [&](int unit) {
-        const int q = a.pv.head != nullptr ? a.pv.order[2 * npairs_q + unit] : unit;
+        const int q = MODE == SCAN_BESIDE ? a.pv.order[2 * npairs_q + unit] : unit;
         cur_u = unit;
         cur_q = q;
         early = k <= 32;
@@ -1185,6 +1189,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_, DUAL>::THREADS, 1) s
 struct Variant {
     int M;
     void (*kernel)(const ScanArgs);
+    void (*beside)(const ScanArgs);  // the same for the single queries of a batch with pairs, null where there are none
     int threads, tile_vecs;
     int (*stages_for)(int d, bool need_vt);
     int lut_bytes, lut_kind, buffer_keys;
@@ -1195,10 +1200,14 @@ static int stages_for(int d, bool need_vt) {
         if (plan_smem<C>(SMEM_BASE_EXPECTED, SMEM_OPTIN, d, s, need_vt).ok) return s;
     return 0;
 }
-#define RAGO_VARIANT(WV, G, R, NCW, RGW, DUAL) \
-    { Cfg<WV, G, R, NCW, RGW, DUAL>::M, scan_kernel<WV, G, R, NCW, RGW, DUAL>, Cfg<WV, G, R, NCW, RGW, DUAL>::THREADS, \
-      Cfg<WV, G, R, NCW, RGW, DUAL>::TV, stages_for<Cfg<WV, G, R, NCW, RGW, DUAL>>, Cfg<WV, G, R, NCW, RGW, DUAL>::LUT_BYTES, \
-      Cfg<WV, G, R, NCW, RGW, DUAL>::KIND, Cfg<WV, G, R, NCW, RGW, DUAL>::KCAP }
+#define RAGO_VARIANT(WV, G, R, NCW, RGW, MODE, BESIDE) \
+    { Cfg<WV, G, R, NCW, RGW, MODE == SCAN_PAIRS>::M, scan_kernel<WV, G, R, NCW, RGW, MODE>, BESIDE, \
+      Cfg<WV, G, R, NCW, RGW, MODE == SCAN_PAIRS>::THREADS, Cfg<WV, G, R, NCW, RGW, MODE == SCAN_PAIRS>::TV, \
+      stages_for<Cfg<WV, G, R, NCW, RGW, MODE == SCAN_PAIRS>>, Cfg<WV, G, R, NCW, RGW, MODE == SCAN_PAIRS>::LUT_BYTES, \
+      Cfg<WV, G, R, NCW, RGW, MODE == SCAN_PAIRS>::KIND, Cfg<WV, G, R, NCW, RGW, MODE == SCAN_PAIRS>::KCAP }
+#define RAGO_SINGLE(WV, G, R, NCW, RGW) RAGO_VARIANT(WV, G, R, NCW, RGW, SCAN_ALONE, (scan_kernel<WV, G, R, NCW, RGW, SCAN_BESIDE>))
+#define RAGO_ALONE(WV, G, R, NCW, RGW) RAGO_VARIANT(WV, G, R, NCW, RGW, SCAN_ALONE, nullptr)
+#define RAGO_PAIR(WV, G, R, NCW, RGW) RAGO_VARIANT(WV, G, R, NCW, RGW, SCAN_PAIRS, nullptr)
 // Warps x unrolled row groups per warp were chosen by measurement: independent row groups in flight inside a warp
 // hide the look-up latency better than more warps do (M = 64: 16 x 2 -> 12 x 4 gave +30%; M = 48: 15 x 1 -> 15 x 2 +13 to 17%, for
 // pairs 15 x 1 -> 10 x 2 +6%, 8 x 2 -6%; M = 96: 15 x 1 -> 8 x 2 -4%, for pairs 15 x 1 -> 7 x 2 -11%), and 15 consumer warps
@@ -1206,22 +1215,22 @@ static int stages_for(int d, bool need_vt) {
 // M = 64: +4.5%).  Where a code size has two entries the first one whose shared-memory plan fits the
 // index (dimension, metric) is taken.
 static const Variant kVariants[] = {
-    RAGO_VARIANT(4, 4, 1, 16, 2, false),   // M = 16
-    RAGO_VARIANT(8, 8, 1, 15, 2, false),   // M = 32
-    RAGO_VARIANT(12, 4, 1, 15, 2, false),  // M = 48: two 46 KB tiles beside the 96 KB table
-    RAGO_VARIANT(8, 8, 2, 15, 4, false),   // M = 64: two 60 KB tiles below the table
-    RAGO_VARIANT(8, 8, 2, 12, 4, false),   // M = 64 where those do not fit
-    RAGO_VARIANT(20, 4, 1, 8, 1, false),   // M = 80
-    RAGO_VARIANT(24, 8, 1, 15, 1, false),  // M = 96
-    RAGO_VARIANT(8, 8, 4, 12, 3, false),   // M = 128
+    RAGO_SINGLE(4, 4, 1, 16, 2),   // M = 16
+    RAGO_SINGLE(8, 8, 1, 15, 2),   // M = 32
+    RAGO_SINGLE(12, 4, 1, 15, 2),  // M = 48: two 46 KB tiles beside the 96 KB table
+    RAGO_SINGLE(8, 8, 2, 15, 4),   // M = 64: two 60 KB tiles below the table
+    RAGO_SINGLE(8, 8, 2, 12, 4),   // M = 64 where those do not fit
+    RAGO_ALONE(20, 4, 1, 8, 1),   // M = 80
+    RAGO_SINGLE(24, 8, 1, 15, 1),  // M = 96
+    RAGO_ALONE(8, 8, 4, 12, 3),   // M = 128
 };
 // The same table layouts for pairs of queries (the tables of 80 and 128 bytes leave no room for two buffers).
 static const Variant kPairVariants[] = {
-    RAGO_VARIANT(4, 4, 1, 15, 2, true),    // M = 16: 16 warps and the producer would leave 96 registers a thread, too few
-    RAGO_VARIANT(8, 8, 1, 15, 2, true),
-    RAGO_VARIANT(12, 4, 1, 10, 2, true),   // M = 48: two row groups for as many warps as the two buffers leave room for
-    RAGO_VARIANT(8, 8, 2, 15, 2, true),    // M = 64: the tiles in flight have to fit each buffer twice over
-    RAGO_VARIANT(24, 8, 1, 15, 1, true),
+    RAGO_PAIR(4, 4, 1, 15, 2),    // M = 16: 16 warps and the producer would leave 96 registers a thread, too few
+    RAGO_PAIR(8, 8, 1, 15, 2),
+    RAGO_PAIR(12, 4, 1, 10, 2),   // M = 48: two row groups for as many warps as the two buffers leave room for
+    RAGO_PAIR(8, 8, 2, 15, 2),    // M = 64: the tiles in flight have to fit each buffer twice over
+    RAGO_PAIR(24, 8, 1, 15, 1),
 };
 
 static const Variant* find_variant(int M, int d, bool need_vt) {
@@ -1254,8 +1263,10 @@ cudaError_t scan_plan(const IndexImpl* ix, ScanPlan* plan) {
     const Variant* pv = find_pair_variant(ix->M, ix->d, ix->metric != RAGO_IP);
     plan->pair_tile_vecs = pv ? pv->tile_vecs : 0;
     if (pv) {
-        const cudaError_t e = cudaFuncSetAttribute(pv->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_OPTIN);
-        if (e != cudaSuccess) return e;
+        for (auto kernel : {pv->kernel, v->beside}) {
+            const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_OPTIN);
+            if (e != cudaSuccess) return e;
+        }
     }
     return cudaFuncSetAttribute(v->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_OPTIN);
 }
@@ -1334,7 +1345,7 @@ cudaError_t launch_scan(const IndexImpl* ix, const ScanPlan& plan, const float* 
         if (e != cudaSuccess) return e;
         count_launch();
     }
-    const cudaError_t e = launch_overlapped(v->kernel, dim3(plan.ctas), dim3(v->threads), plan.smem_bytes, s, a);
+    const cudaError_t e = launch_overlapped(view ? v->beside : v->kernel, dim3(plan.ctas), dim3(v->threads), plan.smem_bytes, s, a);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }
