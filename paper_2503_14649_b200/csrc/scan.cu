@@ -122,6 +122,10 @@ struct Cfg {
     static constexpr int KIND = G == 4 ? LUT_DOT2 : (M == 32 || M == 64 ? LUT_PERM : LUT_DOT);
     static constexpr int LUT_BYTES = lut_image_bytes(M, KIND);
     static constexpr int RGW = RGW_;                    // 32-row groups per warp per tile (unrolled: independent work in flight)
+    // Row group g of warp w is g * NCW + w where a tile is longer than lists often are (48 bytes, 960 vectors), so that short lists occupy
+    // all warps, and w * RGW + g elsewhere.  us per call side by side / dealt (with one row group per warp and a 128 KB table): 200 queries,
+    // 512 of 1 024 lists of 390 vectors 827 / 731 (694), of 980 1 420 / 1 322 (1 413); 400 queries, lists of 2 200 404 / 407 (461).
+    static constexpr bool DEALT = M == 48 && !DUAL;
     static constexpr int TILE_VROWS = NCW * 32 * RGW;
     static constexpr int TV = TILE_VROWS / R;           // vectors per tile
     static constexpr int TILE_BYTES = TILE_VROWS * MV;
@@ -135,6 +139,7 @@ struct Cfg {
     static_assert(WV % G == 0, "virtual rows are whole blocks");
     static_assert(TILE_VROWS % R == 0, "tile must hold whole vectors");
     static_assert(RGW % (R < RGW ? R : RGW) == 0, "row groups are taken min(R, RGW) at a time");
+    static_assert(!DEALT || R == 1, "row groups taken together lie side by side");
     // The producer asks for a cut of the candidate buffer when the count it sees plus everything the tiles in
     // flight can still push would not fit.  It reads the count while a cut may be rewriting it, and may see less than the cut
     // keeps: the tiles in flight are then pushed behind that without another cut, so both must fit.  SMAX bounds the ring depth
@@ -635,7 +640,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_, MODE == SCAN_PAIRS>:
     uint32_t xo[G], at[G][4], pick[4];
 #pragma unroll
     for (int il = 0; il < G; ++il) {
-        xo[il] = (uint32_t)(warp * C::RGW * 32 + lane) * C::MV + 4u * (uint32_t)(il ^ xa);
+        xo[il] = (uint32_t)(warp * (C::DEALT ? 1 : C::RGW) * 32 + lane) * C::MV + 4u * (uint32_t)(il ^ xa);
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
             const uint32_t col = 16u * (uint32_t)(il ^ xa);
@@ -1103,7 +1108,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_, MODE == SCAN_PAIRS>:
             if (dead) break;
         }
 
-        // ---- scan this tile: warp w owns row groups w*RGW .. w*RGW+RGW-1 ----
+        // ---- scan this tile: a warp owns RGW row groups (Cfg::DEALT says which) ----
         const int nvr = (D.flags >> 8) * R;
         const uint32_t tile_base = D.tile_addr;
         const uint32_t vt_base = D.vt_addr;
@@ -1118,14 +1123,14 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_, MODE == SCAN_PAIRS>:
         // so that every shared-memory offset below is a compile-time constant.  Returns false when the tile ended.
         auto pass = [&](auto RG) -> bool {
             constexpr int rg = decltype(RG)::value;
-            const int vr0 = (warp * C::RGW + rg) * 32;
+            const int vr0 = C::DEALT ? (rg * NCW + warp) * 32 : (warp * C::RGW + rg) * 32;
             if (vr0 >= nvr) return false;
             int mine = 0;
             auto group = [&](auto GI) {
                 constexpr int g = decltype(GI)::value;
                 int acc[4] = {0, 0, 0, 0};
                 uint32_t x[C::NBLK][G];
-                LoadWords<C, G, 0, (rg + g) * 32 * C::MV>::run(wa, x);
+                LoadWords<C, G, 0, (rg + g) * (C::DEALT ? NCW : 1) * 32 * C::MV>::run(wa, x);
                 ScanBlocks<C, G, 0>::run(x, at, pick, acc);
                 int si = (acc[0] + acc[1]) + (acc[2] + acc[3]);
                 if (R >= 2) si += __shfl_xor_sync(0xffffffffu, si, 1);
@@ -1142,7 +1147,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_, MODE == SCAN_PAIRS>:
             const float vt = a.vterm != nullptr ? lds_f32(vt_base + (uint32_t)(vr / R) * 4u) : 0.f;
             // In the last pass over the tile that was this warp's last read of the stage: hand the stage back
             // before the rest of the epilogue, so that the refill starts that much earlier (M = 96: -1%).
-            if constexpr (rg + MERGE >= C::RGW) {
+            if (rg + MERGE >= C::RGW || (C::DEALT && vr0 + NCW * 32 >= nvr)) {
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&ctrl->empty[st]));
                 released = true;

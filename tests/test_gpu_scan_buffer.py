@@ -74,3 +74,35 @@ def test_large_k_over_vectors_in_descending_order_of_score(M, metric, k):
         assert torch.allclose(sign * dists[0].double(), want[:k], rtol=0, atol=1e-5 * float(want.abs().max()))
         assert set(ids[0].tolist()) <= allowed
     ix.close()
+
+
+# Row groups of 48-byte tiles are dealt over the warps: lists that end on, before and behind a group, a round of 15 groups and a tile of 960.
+@pytest.mark.parametrize("metric,k", [("l2", 100), ("ip", 10), ("l2", 1)])
+def test_lists_around_the_row_groups_of_a_48_byte_tile(metric, k):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(48 + k)
+    sizes = [1, 31, 32, 33, 64, 65, 479, 480, 481, 511, 513, 928, 959, 960, 961, 1439, 1440, 1441, 1920, 1953]
+    nlist, N, M = len(sizes), sum(sizes), 48
+    c = torch.randn(nlist, 4 * M, generator=g, device="cuda")
+    books = 0.3 * torch.randn(M, 256, 4, generator=g, device="cuda")
+    codes = torch.randint(0, 256, (N, M), generator=g, device="cuda", dtype=torch.uint8)
+    offsets = torch.tensor([0] + sizes, device="cuda").cumsum(0)
+    ix = binding.rago_index_load(c, books, codes, offsets, torch.arange(N, device="cuda"), metric)
+    q = torch.randn(20, 4 * M, generator=g, device="cuda")
+    sign = 1.0 if metric == "l2" else -1.0
+    for nprobe in (1, nlist):  # a query's own list alone (its last vectors among the results), and all of them
+        near = (c + 0.1 * q).contiguous()
+        ids, dists = ix.rago_search(near, nprobe, k)
+        torch.cuda.synchronize()
+        ix.rago_check()
+        lists, _ = ix.rago_search_probes(near, nprobe)
+        for i in range(nlist):
+            score = torch.full((N,), float("inf"), dtype=torch.float64, device="cuda")
+            for l in lists[i].tolist():
+                a, b = int(offsets[l]), int(offsets[l + 1])
+                score[a:b] = _scores(near[i:i + 1], c[l], books, codes[a:b], metric)[0]
+            want, at = score.sort()
+            n = min(k, int(torch.isfinite(score).sum()))
+            assert torch.allclose(sign * dists[i, :n].double(), want[:n], rtol=0, atol=1e-5 * float(want[:n].abs().max()))
+            assert set(ids[i, :n].tolist()) <= set(at[:n + 5].tolist())
+    ix.close()
