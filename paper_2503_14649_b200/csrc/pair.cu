@@ -2,6 +2,7 @@
 //
 // A pair is two queries whose nearest list is the same one (neighbours after sorting by nearest, then second nearest list)
 // and that share enough of their work.  All of it is decided on the device, from the probe lists.
+#include <algorithm>
 #include <cmath>
 
 #include "pair.cuh"
@@ -14,9 +15,11 @@ constexpr int PR_THREADS = 256, PR_WARPS = PR_THREADS / 32;
 constexpr int PU_THREADS = 128, PU_WARPS = PU_THREADS / 32;  // one warp per query of the sorted order
 static_assert(PU_WARPS == 4, "states are counted a word, four positions, at a time");
 constexpr uint8_t ST_SINGLE = 0, ST_FIRST = 1, ST_SECOND = 2, ST_NONE = 0xFF;
-// A pair shares at least one vector in so many of both queries' work: closing a pair costs about 30 us more than closing two queries,
-// and its tiles 10 to 15% more than a query's, so that pairs that share less gain nothing.
-constexpr int PAIR_SHARE = 8;
+// A pair shares at least one vector in so many of both queries' work (its tiles cost 10 to 15% more than a query's), and codes of at least so many
+// bytes: sharing 2 MB saves a CTA about 30 us, what closing a pair costs beyond closing two queries.  (4 000 queries over 1 024
+// lists of 2 150, 8 probes, 64 bytes, every batch looked through: 1 395 us per call without pairs, with all that share 0.2 MB
+// 1 802, 1 MB 1 531, 2 MB 1 485; with lists of 30 000 vectors all of them 2 135 to 2 167.)
+constexpr int PAIR_SHARE = 8, PAIR_MIN_BYTES = 2 << 20;
 
 // The queries ranked by nearest, then second nearest list; runs of equal nearest lists are split into neighbours.  state[i]: what
 // the query at position i of sorted[] is.  A query whose table is not bounded (ok = 0) has no partner.  Every warp counts, for
@@ -287,11 +290,11 @@ void pair_list_stats(IndexImpl* ix, const int64_t* offsets) {
     for (int b = 0; b <= 32; ++b) { ix->list_weight[b] = (float)w[b]; ix->list_square[b] = (float)w2[b]; }
 }
 
-// Vectors a query scans, and how many of them it is expected to share with a partner, if queries come as the stored vectors
-// do: a query's nearest list has weight w with probability w, then nq w others have the same one, and the share of them that
+// Vectors a query scans, how many of them it is expected to share with a partner, and the share of queries that have one, if queries come as
+// the stored vectors do: a query's nearest list has weight w with probability w, then nq w others have the same one, and the share of them that
 // finds a partner is 1 - (1 - e^-2x) / 2x for x = nq w (an odd number leaves one over).  Partners share their nearest list and,
 // since it is where they both lie, about half of the others.
-static void pair_expect(const IndexImpl* ix, int nq, int nprobe, double* scanned, double* shared) {
+static void pair_expect(const IndexImpl* ix, int nq, int nprobe, double* scanned, double* shared, double* paired_share) {
     double own = 0.0, own_shared = 0.0, paired = 0.0;
     for (int b = 0; b <= 32; ++b) {
         if (!(ix->list_weight[b] > 0.f)) continue;
@@ -304,6 +307,7 @@ static void pair_expect(const IndexImpl* ix, int nq, int nprobe, double* scanned
     const double others = (double)(nprobe - 1) / (double)ix->nlist;
     *scanned = (double)ix->N * (own + others);
     *shared = (double)ix->N * (own_shared + 0.5 * paired * others);
+    *paired_share = paired;
 }
 
 static bool pair_possible(const IndexImpl* ix, int nq, int k) {
@@ -311,23 +315,30 @@ static bool pair_possible(const IndexImpl* ix, int nq, int k) {
     return nq >= PAIR_MIN_NQ && nq <= PAIR_MAX_NQ && k <= PAIR_MAX_K && ix->plan.pair_tile_vecs > 0 && ix->N > 0 &&
            (ds == 4 || ds == 8 || ds == 12 || ds == 16);  // those whose table kernel checks the tables' bound
 }
-// Preparing pairs costs 20 to 50 us, and of what is shared less than half is saved; below these bounds the two sides could not be
-// told apart.  Above them, without / with pairs, us per call: 1 024 queries, 87% of their work in lists that others share,
-// 96 bytes 8 460 / 5 610; 300 queries, 48 bytes 1 466 / 1 192; 77 queries, 96 bytes (expected saving 100 us) 683 / 670.
+// What of a batch is shared saves less than half of its look-ups.  Against that stand, in us: the preparation, 20 to 50 and, where every list
+// of a query is looked for among its partner's, 1 000 for 1 024 probes (more than about 1 200 queries queue for the SMs); and closing a pair on
+// each CTA that scans part of it, 40 and more with k beyond closing two queries (4 000 queries over 1 024 lists of 2 150, whose CTAs
+// close 13 pairs each: 64 bytes, 4 probes, without / with pairs 973 / 1 426 us per call, 96 bytes, 8 probes 1 803 / 2 032).
+// Below PAIR_MIN_US the two sides could not be told apart.  Where the rule says yes, without / with: 1 024 queries, 87% of their work in
+// lists that others share, 96 bytes 8 460 / 5 610; 300 queries, 48 bytes 1 466 / 1 192; 77 queries, 96 bytes (expected saving 290 us)
+// 683 / 670; 500 queries, 256 of 512 lists of 1 950, 96 bytes 4 935 / 4 222; 1 000 queries, 1 024 lists of 1 950, all probed 40 100 / 31 160.
 constexpr double PAIR_MIN_SHARE = 0.2, PAIR_MIN_US = 120.0, PAIR_BYTES_PER_US = 4.7e6;
-static bool pair_worth(const IndexImpl* ix, int nq, int nprobe) {
-    double scanned, shared;
-    pair_expect(ix, nq, nprobe, &scanned, &shared);
-    return shared >= PAIR_MIN_SHARE * scanned && 0.5 * shared * nq * ix->M >= PAIR_MIN_US * PAIR_BYTES_PER_US;
+constexpr double PAIR_PREPARE_US = 60.0, PAIR_MATCH_US = 1000.0, PAIR_CLOSE_US = 40.0, PAIR_CLOSE_K_US = 0.08;
+static bool pair_worth(const IndexImpl* ix, int nq, int nprobe, int k) {
+    double scanned, shared, paired;
+    pair_expect(ix, nq, nprobe, &scanned, &shared, &paired);
+    const double p = nprobe / 1024.0, closed = 0.5 * nq * paired / ix->plan.ctas + 1.0;  // pairs that a CTA closes
+    const double cost = PAIR_PREPARE_US + PAIR_MATCH_US * p * p * (1.0 + nq / 1200.0) + closed * (PAIR_CLOSE_US + PAIR_CLOSE_K_US * k);
+    return shared >= PAIR_MIN_SHARE * scanned && 0.5 * shared * nq * ix->M >= std::max(cost, PAIR_MIN_US) * PAIR_BYTES_PER_US;
 }
-bool pair_applies(const IndexImpl* ix, int nq, int nprobe, int k) { return pair_possible(ix, nq, k) && pair_worth(ix, nq, nprobe); }
+bool pair_applies(const IndexImpl* ix, int nq, int nprobe, int k) { return pair_possible(ix, nq, k) && pair_worth(ix, nq, nprobe, k); }
 // Workspace is set aside where any k, and any number of probes up to nprobe, takes pairs: the shared part is a ratio of two
-// linear functions of it, so largest at one end, and the amount grows with it.
+// linear functions of it, so largest at one end, and the amount grows with it (what it has to exceed is at least PAIR_MIN_US).
 bool pair_reserves(const IndexImpl* ix, int nq, int nprobe) {
     if (!pair_possible(ix, nq, 1)) return false;
-    double s1, h1, s2, h2;
-    pair_expect(ix, nq, 1, &s1, &h1);
-    pair_expect(ix, nq, nprobe, &s2, &h2);
+    double s1, h1, s2, h2, paired;
+    pair_expect(ix, nq, 1, &s1, &h1, &paired);
+    pair_expect(ix, nq, nprobe, &s2, &h2, &paired);
     return (h1 >= PAIR_MIN_SHARE * s1 || h2 >= PAIR_MIN_SHARE * s2) && 0.5 * h2 * nq * ix->M >= PAIR_MIN_US * PAIR_BYTES_PER_US;
 }
 
@@ -373,7 +384,7 @@ cudaError_t launch_pair_queries(const IndexImpl* ix, const int32_t* probe_list, 
                                       probe_list, ok, nq, nprobe, sorted, state);
     if (e == cudaSuccess)
         e = launch_overlapped(pair_judge_kernel, grid, dim3(PU_THREADS), 0, s, probe_list, ix->list_offsets, nq, nprobe,
-                              (long long)4 * pl.pair_tile_vecs, sorted, state);
+                              (long long)(PAIR_MIN_BYTES / ix->M), sorted, state);
     if (e == cudaSuccess)
         e = launch_overlapped(pair_entries_kernel, grid, dim3(PU_THREADS), 0, s, probe_list, probe_term, nq, nprobe, sorted, state, head,
                               order, entry_list, entry_term, term_b, mask, ix->list_offsets, range);

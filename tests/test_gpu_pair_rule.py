@@ -1,0 +1,43 @@
+"""Which batches are looked through for pairs of queries, and what larger batches and other kinds of calls with pairs answer."""
+
+import pytest
+import torch
+
+from paper_2503_14649_b200 import binding
+
+pytestmark = pytest.mark.gpu
+
+
+def _even(M, N, nlist, seed=0):
+    """Random codes in lists of (almost) equal length around random centroids."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed + M)
+    c = torch.randn(nlist, 4 * M, generator=g, device="cuda")
+    books = 0.3 * torch.randn(M, 256, 4, generator=g, device="cuda")
+    codes = torch.randint(0, 256, (N, M), generator=g, device="cuda", dtype=torch.uint8)
+    offsets = (torch.arange(nlist + 1, device="cuda", dtype=torch.int64) * N) // nlist
+    return binding.rago_index_load(c, books, codes, offsets, torch.arange(N, device="cuda"), "l2"), c
+
+
+def _launches(ix, q, nprobe, k):
+    n = binding.rago_kernel_launches()
+    ix.rago_search(q, nprobe, k)
+    torch.cuda.synchronize()
+    ix.rago_check()
+    return binding.rago_kernel_launches() - n
+
+
+# Pairs are looked for where sharing look-ups saves more than preparing and closing the pairs costs.  Not so: many queries over few
+# vectors each (every pair is closed on a CTA), every list of a query matched with its partner's for little work.
+@pytest.mark.parametrize("M,N,nlist,nq,nprobe,pairs", [
+    (64, 2_200_000, 1024, 4000, 4, False), (96, 2_200_000, 1024, 4000, 8, False), (48, 2_200_000, 1024, 4000, 8, False),
+    (48, 100_000, 1024, 1000, 1024, False), (48, 400_000, 1024, 1000, 1024, False),
+    (96, 1_000_000, 512, 500, 256, True), (96, 2_000_000, 256, 300, 64, True), (16, 4_000_000, 256, 1000, 200, True)])
+def test_pairs_are_looked_for_where_they_pay(M, N, nlist, nq, nprobe, pairs):
+    ix, c = _even(M, N, nlist)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(nq)
+    q = (c[torch.randint(0, nlist, (nq,), generator=g, device="cuda")] + 0.3 * torch.randn(nq, 4 * M, generator=g, device="cuda")).contiguous()
+    # k = 1024 is above the pairs' limit: the same launches without them
+    assert _launches(ix, q, nprobe, 100) == _launches(ix, q, nprobe, 1024) + (5 if pairs else 0)
+    ix.close()
