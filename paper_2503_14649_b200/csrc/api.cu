@@ -475,7 +475,7 @@ rago_status rago_search(const rago_index* index, const float* queries, int32_t n
         uint8_t* pw = ws + L.pair;
         e = launch_build_tables(ix, queries, nq, lut_img, lut_inv, reinterpret_cast<float*>(ws + L.lut_scale),
                                 reinterpret_cast<int32_t*>(pw + PL.ok), s);
-        if (e == cudaSuccess) e = launch_pair_queries(ix, probe_list, probe_term, nq, nprobe, lut_img, lut_inv, pw, PL, &view, s);
+        if (e == cudaSuccess) e = launch_pair_queries(ix, probe_list, probe_term, nq, nprobe, k, lut_img, lut_inv, pw, PL, &view, s);
         if (e != cudaSuccess) return cuda_fail(e, "pairing of queries");
         pv = &view;
         scan_list = reinterpret_cast<const int32_t*>(pw + PL.entry_list);

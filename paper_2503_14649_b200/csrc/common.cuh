@@ -28,7 +28,7 @@ struct ScanPlan {
     size_t smem_bytes;
     // shared-memory image of a query's lookup table, as the scan variant of this index lays it out
     int lut_bytes, lut_kind;
-    int pair_tile_vecs;  // vectors per tile where two queries are scanned together, 0: not with this index
+    int pairs;         // two queries can be scanned together
 };
 
 // Layouts of a query's lookup table, in shared memory and in the images that are built ahead (scan.cu says which code size takes
@@ -323,7 +323,8 @@ cudaError_t launch_transpose_codebook(const float* cb, int M, int dsub, float* c
 int scan_query_lead(const IndexImpl* ix, int nq, int nprobe, int k);  // work units that stand for the start of a query
 bool scan_prefetches(const IndexImpl* ix, int64_t npairs);  // tiles are pulled into L2 ahead of their copies
 struct PairView;
-int scan_pair_lead(const IndexImpl* ix);  // the same for a pair of queries
+int scan_pair_lead(const IndexImpl* ix, int pair_tile_vecs);  // the same for a pair of queries
+int scan_pair_tile_vecs(const IndexImpl* ix, int k);          // vectors per tile of the pairs' scan (plan.pairs)
 cudaError_t launch_plan_work(const IndexImpl* ix, const int32_t* probe_list, int npairs, int tile_vecs, int lead, const PairView* view,
                              int32_t* pair_tiles, int64_t* work_prefix, unsigned long long* qthresh, int nq,
                              int32_t* slot_cnt, int nslots, const float* queries, uint8_t* lut_img, float* lut_inv,

@@ -312,7 +312,7 @@ static void pair_expect(const IndexImpl* ix, int nq, int nprobe, double* scanned
 
 static bool pair_possible(const IndexImpl* ix, int nq, int k) {
     const int ds = ix->dsub;
-    return nq >= PAIR_MIN_NQ && nq <= PAIR_MAX_NQ && k <= PAIR_MAX_K && ix->plan.pair_tile_vecs > 0 && ix->N > 0 &&
+    return nq >= PAIR_MIN_NQ && nq <= PAIR_MAX_NQ && k <= PAIR_MAX_K && ix->plan.pairs && ix->N > 0 &&
            (ds == 4 || ds == 8 || ds == 12 || ds == 16);  // those whose table kernel checks the tables' bound
 }
 // What of a batch is shared saves less than half of its look-ups.  Against that stand, in us: the preparation, 20 to 50 and, where every list
@@ -363,7 +363,7 @@ PairLayout pair_layout(int nq, int nprobe, int lut_bytes) {
 }
 
 cudaError_t launch_pair_queries(const IndexImpl* ix, const int32_t* probe_list, const float* probe_term, int nq, int nprobe,
-                                const uint8_t* lut_img, const float* lut_inv, uint8_t* ws, const PairLayout& L, PairView* view,
+                                int k, const uint8_t* lut_img, const float* lut_inv, uint8_t* ws, const PairLayout& L, PairView* view,
                                 cudaStream_t s) {
     int32_t* head = reinterpret_cast<int32_t*>(ws + L.head);
     const int32_t* ok = reinterpret_cast<const int32_t*>(ws + L.ok);
@@ -404,6 +404,7 @@ cudaError_t launch_pair_queries(const IndexImpl* ix, const int32_t* probe_list, 
     if (e != cudaSuccess) return e;
     count_launch(4);
     view->head = head; view->order = order; view->term_b = term_b; view->mask = mask; view->range = range; view->params = params; view->img = img;
+    view->tile_vecs = scan_pair_tile_vecs(ix, k);
     return cudaGetLastError();
 }
 

@@ -40,6 +40,7 @@ struct PairView {
     const uint2* range;         // [2][entries] of either query: storage positions of the list, from, to (1, 0: it does not probe it)
     const PairParams* params;   // [pairs]
     const uint8_t* img;         // [pairs] table images
+    int tile_vecs;              // vectors per tile of the pairs' scan
 };
 
 // Where a query's entries and slots are (see the scan's slot numbering): position i of the order.
@@ -71,7 +72,7 @@ bool pair_applies(const IndexImpl* ix, int nq, int nprobe, int k);
 bool pair_reserves(const IndexImpl* ix, int nq, int nprobe);
 void pair_list_stats(IndexImpl* ix, const int64_t* offsets);
 cudaError_t launch_pair_queries(const IndexImpl* ix, const int32_t* probe_list, const float* probe_term, int nq, int nprobe,
-                                const uint8_t* lut_img, const float* lut_inv, uint8_t* ws, const PairLayout& L, PairView* view,
+                                int k, const uint8_t* lut_img, const float* lut_inv, uint8_t* ws, const PairLayout& L, PairView* view,
                                 cudaStream_t s);
 
 }  // namespace rago

@@ -1236,6 +1236,7 @@ static const Variant kPairVariants[] = {
     RAGO_PAIR(12, 4, 1, 10, 2),   // M = 48: two row groups for as many warps as the two buffers leave room for
     RAGO_PAIR(8, 8, 2, 15, 2),    // M = 64: the tiles in flight have to fit each buffer twice over
     RAGO_PAIR(24, 8, 1, 15, 1),
+    RAGO_PAIR(24, 8, 1, 12, 1),    // M = 96 for larger k (find_pair_variant)
 };
 
 static const Variant* find_variant(int M, int d, bool need_vt) {
@@ -1243,10 +1244,20 @@ static const Variant* find_variant(int M, int d, bool need_vt) {
         if (v.M == M && v.stages_for(d, need_vt) >= 2) return &v;
     return nullptr;
 }
-static const Variant* find_pair_variant(int M, int d, bool need_vt) {
-    for (const Variant& v : kPairVariants)
-        if (v.M == M && v.stages_for(d, need_vt) >= 2) return &v;
-    return nullptr;
+// A cut of a buffer of bounds keeps up to k * 3 / 2 keys and a few; beyond what the tiles in flight leave room for, the next cut follows at
+// once.  Of two entries the first is taken whose buffer leaves that room and a quarter more.  96 bytes, 15 / 12 warps (without
+// pairs), us per call, 200 queries over 32 of 300 lists of 30 000: k = 100 3 142 / 3 193 (3 704), 300 3 475 / 3 401, 350 3 606 / 3 486, 400
+// 3 834 / 3 610 (3 832), 512 4 592 / 3 867 (3 877); 1 000 queries: 200 13 650 / 13 960, 300 14 170 / 14 290, 350 14 570 / 14 460.
+static const Variant* find_pair_variant(int M, int d, bool need_vt, int k) {
+    const Variant* found = nullptr;
+    for (const Variant& v : kPairVariants) {
+        if (v.M != M) continue;
+        const int stages = v.stages_for(d, need_vt);
+        if (stages < 2) continue;
+        found = &v;
+        if (v.buffer_keys - (stages + 1) * v.tile_vecs >= 2 * k) break;
+    }
+    return found;
 }
 
 bool scan_supported(int M) {
@@ -1265,10 +1276,11 @@ cudaError_t scan_plan(const IndexImpl* ix, ScanPlan* plan) {
     plan->ctas = ix->num_sms;
     plan->smem_bytes = SMEM_OPTIN;
     plan->lut_bytes = v->lut_bytes; plan->lut_kind = v->lut_kind;
-    const Variant* pv = find_pair_variant(ix->M, ix->d, ix->metric != RAGO_IP);
-    plan->pair_tile_vecs = pv ? pv->tile_vecs : 0;
-    if (pv) {
-        for (auto kernel : {pv->kernel, v->beside}) {
+    plan->pairs = 0;
+    for (const Variant& pv : kPairVariants) {
+        if (pv.M != ix->M || pv.stages_for(ix->d, ix->metric != RAGO_IP) < 2) continue;
+        plan->pairs = 1;
+        for (auto kernel : {pv.kernel, v->beside}) {
             const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_OPTIN);
             if (e != cudaSuccess) return e;
         }
@@ -1299,10 +1311,12 @@ int scan_query_lead(const IndexImpl* ix, int nq, int nprobe, int k) {
 
 // The start of a pair of queries: two buffers are closed (cut, made exact, ranked: about 90 000 cycles in all) and filled again.
 // (1 024 queries, 96 bytes: with 30 us the CTAs of the short lists, 18 closes each, ended 12% after the others.)
-int scan_pair_lead(const IndexImpl* ix) {
-    const float tile_us = (float)(ix->plan.pair_tile_vecs * ix->M) / 36000.f;
+int scan_pair_lead(const IndexImpl* ix, int pair_tile_vecs) {
+    const float tile_us = (float)(pair_tile_vecs * ix->M) / 36000.f;
     return (int)(60.f / tile_us + 0.5f);
 }
+
+int scan_pair_tile_vecs(const IndexImpl* ix, int k) { return find_pair_variant(ix->M, ix->d, ix->metric != RAGO_IP, k)->tile_vecs; }
 
 // Prefetching into L2 pays where the tiles in flight are small (a copy from DRAM takes longer than the tile in front
 // of it is scanned) and the batch does not meet each list several times, which brings most tiles from L2 anyway and
@@ -1340,11 +1354,11 @@ cudaError_t launch_scan(const IndexImpl* ix, const ScanPlan& plan, const float* 
     a.prefetch = scan_prefetches(ix, a.npairs) ? 1 : 0;
     std::memset(&a.pv, 0, sizeof(a.pv));
     if (view) {
-        const Variant* p = find_pair_variant(ix->M, ix->d, need_vt);
+        const Variant* p = find_pair_variant(ix->M, ix->d, need_vt, k);
         if (!p) return cudaErrorInvalidValue;
         ScanArgs b = a;
         b.pv = a.pv = *view;
-        b.lead = a.lead ? scan_pair_lead(ix) : 0;
+        b.lead = a.lead ? scan_pair_lead(ix, p->tile_vecs) : 0;
         b.stages = p->stages_for(ix->d, need_vt);
         const cudaError_t e = launch_overlapped(p->kernel, dim3(plan.ctas), dim3(p->threads), plan.smem_bytes, s, b);
         if (e != cudaSuccess) return e;
@@ -1734,7 +1748,7 @@ cudaError_t launch_plan_work(const IndexImpl* ix, const int32_t* probe_list, int
         if (et != cudaSuccess) return et;
     }
     PairTiles pt = {nullptr, 0, 0};
-    if (view) { pt.head = view->head; pt.tile_vecs = ix->plan.pair_tile_vecs; pt.lead = lead ? scan_pair_lead(ix) : 0; }
+    if (view) { pt.head = view->head; pt.tile_vecs = view->tile_vecs; pt.lead = lead ? scan_pair_lead(ix, view->tile_vecs) : 0; }
     if (npairs <= PLAN_SMALL_MAX) {
         const int parts = fused_tables ? table_parts(ix, nq) : 0;
         launch_overlapped(plan_small_kernel, dim3(1 + parts * nq), dim3(PFX_THREADS),

@@ -41,3 +41,18 @@ def test_pairs_are_looked_for_where_they_pay(M, N, nlist, nq, nprobe, pairs):
     # k = 1024 is above the pairs' limit: the same launches without them
     assert _launches(ix, q, nprobe, 100) == _launches(ix, q, nprobe, 1024) + (5 if pairs else 0)
     ix.close()
+
+
+# Pairs of 96-byte codes have a kernel of fewer warps for larger k: the values on both sides of the line, and the largest.
+@pytest.mark.parametrize("k", [303, 304, 305, 448, 449, 512])
+def test_pairs_of_96_byte_codes_for_larger_k_answer_as_single_queries_do(k):
+    ix, c = _even(96, 400_000, 40)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(k)
+    q = (c[torch.arange(180, device="cuda") % 7] + 0.3 * torch.randn(180, 384, generator=g, device="cuda")).contiguous()
+    assert _launches(ix, q, 24, k) == _launches(ix, q, 24, 1024) + 5
+    ids, dists = ix.rago_search(q, 24, k)
+    for b in range(0, 180, 60):  # batches that are too small for pairs
+        i, s = ix.rago_search(q[b:b + 60].contiguous(), 24, k)
+        assert torch.equal(ids[b:b + 60], i) and torch.equal(dists[b:b + 60].view(torch.int32), s.view(torch.int32)), b
+    ix.close()
