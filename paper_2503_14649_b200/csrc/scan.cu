@@ -1320,17 +1320,21 @@ int scan_pair_tile_vecs(const IndexImpl* ix, int k) { return find_pair_variant(i
 
 // Prefetching into L2 pays where the tiles in flight are small (a copy from DRAM takes longer than the tile in front
 // of it is scanned) and the batch does not meet each list several times, which brings most tiles from L2 anyway and
-// makes the prefetches only extra traffic.  Without / with, us per call: 48-byte codes, 2.3 probes per list
-// 1672 / 1618; 96 bytes, 0.6 probes 753 / 741; 96 bytes, 8 probes 8890 / 9100 (with terms 9190); 64 bytes (60 KB
-// tiles), 4 096 queries 14 560 / 14 730, 33 queries 226.9 / 233.8.
+// makes the prefetches only extra traffic.  Without / with, us per call: 64 bytes (60 KB tiles), 4 096 queries 14 560 / 14 730, 33
+// queries 226.9 / 233.8.  Tiles of 46 KB (48 and 96 bytes) lose by it where a batch meets few of the lists: lists of 2 200, 0.47 probes per
+// list 96 bytes 157.5 / 162.8 (inner product 154.7 / 164.4), 48 bytes 114.5 / 115.7, 0.23 probes 106.1 / 110.3; lists of 15 000, 0.53 probes
+// 143.0 / 155.2, 0.96 220.9 / 230.4; from one probe on they gain a little: 2.1 412.5 / 411.7, 1.0 272.6 / 271.6, 1.6 374.8 / 372.6, 2.3
+// 516 / 513 (inner product 530 / 518).
 // Long lists of a database beyond L2 come from DRAM however often they are met, which shows where a tile is scanned in a
-// short time (48 and 80 bytes: 23 and 20 KB).  64 lists of 47 000 vectors, 600 queries with 32 probes, without / with: 48 bytes
-// 9 520 / 8 940, 80 bytes 19 490 / 18 950.  With lists below 32 tiles, inside L2, and for the other sizes (6 M vectors in 64
-// lists, 16 bytes 3%, 64 bytes 3%, 96 bytes 1% more) it is the other way round or equal.
+// short time: 80 bytes (20 KB tiles), 64 lists of 47 000 vectors, 600 queries with 32 probes, without / with 19 490 / 18 950, and 48 bytes,
+// whose tiles took as long while they were as small (9 520 / 8 940) and gain less now: lists of 30 000 1 794 / 1 767, 20 000 1 246 /
+// 1 239, 9 000 638 / 633, 47 000 1 274 / 1 267.  Lists below 640 KB, inside L2, and the other sizes (16 bytes 3%, 64 bytes 3%
+// more): the other way round or equal.
 bool scan_prefetches(const IndexImpl* ix, int64_t npairs) {
-    const int tile_bytes = ix->plan.tile_vecs * ix->M / (ix->M == 48 ? 2 : 1);  // 48 bytes: measured with tiles of half the size
-    const bool long_lists = ix->N / ix->nlist >= 32ll * ix->plan.tile_vecs && ix->N * ix->M > (128ll << 20);
-    return (tile_bytes <= 48 * 1024 && npairs <= 4ll * ix->nlist) || (ix->M >= 48 && tile_bytes <= 24 * 1024 && long_lists);
+    const int tile_bytes = ix->plan.tile_vecs * ix->M;
+    const bool few = npairs <= 4ll * ix->nlist && (tile_bytes <= 40 * 1024 || (tile_bytes <= 48 * 1024 && npairs >= ix->nlist));
+    const bool long_lists = ix->N / ix->nlist * ix->M >= 640 * 1024 && ix->N * ix->M > (128ll << 20);
+    return few || (ix->M >= 48 && ix->plan.lut_kind == LUT_DOT2 && long_lists);
 }
 
 // view (may be null): the batch's pairs of queries, scanned by a launch of their own in front of that of the single ones.

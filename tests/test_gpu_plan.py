@@ -95,3 +95,14 @@ def test_the_weight_of_a_query_start_goes_by_the_candidate_buffer(M, k, lead):
     ix = _index(64, d=4 * M, M=M, N=200_000)
     assert ix.rago_debug_search_plan(400, 32, k)["lead"] == lead
     ix.close()
+
+
+# Tiles of 46 KB (48 and 96 bytes) from one probe per list on; lists of 640 KB of 48-byte codes (13 654 vectors) however often they are probed.
+@pytest.mark.parametrize("N,nlist,M,nq,nprobe,prefetch", [
+    (400_000, 512, 96, 15, 32, 0), (400_000, 512, 96, 16, 32, 1), (400_000, 512, 96, 64, 32, 1), (400_000, 512, 96, 65, 32, 0),
+    (400_000, 512, 48, 15, 32, 0), (400_000, 512, 48, 16, 32, 1), (400_000, 512, 128, 1, 32, 1), (400_000, 512, 32, 1, 32, 1),
+    (3_004_000, 220, 48, 600, 32, 1), (3_003_000, 220, 48, 600, 32, 0), (2_800_000, 187, 48, 600, 32, 1), (2_700_000, 187, 48, 600, 32, 0)])
+def test_scan_prefetches_by_the_bytes_of_tiles_and_lists(N, nlist, M, nq, nprobe, prefetch):
+    ix = _index(nlist, d=2 * M, M=M, N=N, metric="ip")
+    assert ix.rago_debug_search_plan(nq, nprobe, 10)["prefetch"] == prefetch
+    ix.close()
