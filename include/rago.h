@@ -138,10 +138,14 @@ rago_status rago_index_free(rago_index* index);
 
 /* Bytes of device scratch rago_search / rago_search_probes / rago_search_host need for a batch
  * of nq queries with these nprobe and k (1 <= nprobe <= nlist, 1 <= k <= 1024).  Its largest parts are
- * the per-query lookup tables (64 to 160 KB each, for at most 4096 queries of a batch: 128 KB per
+ * the per-query lookup tables (32 to 160 KB each, for at most 4096 queries of a batch: 96 KB per
  * query at M = 96) and what the coarse step leaves: nq * nlist scores, or candidate lists of up to
  * 1024 entries of 8 bytes, some 300 per query of a small batch.  The bytes also serve searches with the same nq and smaller
- * nprobe or k; a smaller nq may need more (its candidate lists are cut finer). */
+ * nprobe or k; a smaller nq may need more (its candidate lists are cut finer).
+ * Where the lists of the index are so long that queries of a batch can be expected to share them, room for scanning two queries
+ * at a time is added: half the lookup tables again, for at most 4096 queries, also set aside for larger batches and larger k that do not
+ * use it, so that their workspace serves smaller ones.  A search whose workspace holds everything but this part
+ * scans one query at a time, more slowly and with the same results. */
 rago_status rago_search_workspace_bytes(const rago_index* index, int32_t nq, int32_t nprobe, int32_t k,
                                         size_t* out_bytes);
 
@@ -152,7 +156,7 @@ rago_status rago_search_workspace_bytes(const rago_index* index, int32_t nq, int
  *   queries    dev [nq][d] fp32, 16-byte aligned
  *   out_ids    dev [nq][k] int64, best first
  *   out_dists  dev [nq][k] fp32: squared L2 distance, or inner-product score
- *   workspace  dev, 256-byte aligned, at least rago_search_workspace_bytes(...) bytes; contents
+ *   workspace  dev, 256-byte aligned, at least rago_search_workspace_bytes(...) bytes (fewer: see there); contents
  *              are scratch.  Two searches that overlap on the GPU need distinct workspaces.
  *
  * With a RAGO_BF16 coarse quantiser the query is rounded to bf16 (nearest-even) for the coarse

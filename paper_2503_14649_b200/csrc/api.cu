@@ -62,7 +62,8 @@ static bool use_tensor_cores(const IndexImpl* ix, int nq) {
     return ix->coarse_mode == 2 || nq >= TC_MIN_NQ;
 }
 
-static Layout make_layout(const IndexImpl* ix, int nq, int nprobe, int k) {
+// pairs_too = false: the layout of a search that does not look for pairs of queries, whatever its sizes.
+static Layout make_layout(const IndexImpl* ix, int nq, int nprobe, int k, bool pairs_too = true) {
     Layout L;
     size_t o = 0;
     auto take = [&](size_t bytes) {
@@ -71,9 +72,9 @@ static Layout make_layout(const IndexImpl* ix, int nq, int nprobe, int k) {
         return at;
     };
     const size_t npairs = (size_t)nq * nprobe;
-    L.pairs = pair_applies(ix, nq, nprobe, k) ? 1 : 0;
+    L.pairs = pairs_too && pair_applies(ix, nq, nprobe, k) ? 1 : 0;
     const int pair_nq = std::min(nq, PAIR_MAX_NQ);  // reserved for larger batches too, as below
-    const bool pair_room = L.pairs || pair_reserves(ix, pair_nq, nprobe);
+    const bool pair_room = pairs_too && (L.pairs || pair_reserves(ix, pair_nq, nprobe));
     // one slot per (CTA, query) incidence; pairs and single queries are scanned, and numbered, apart
     L.nslots = pair_room ? pair_slots(nq, ix->plan.ctas) : (size_t)nq + (size_t)ix->plan.ctas;
     L.err = take(256);
@@ -134,6 +135,13 @@ static Layout make_layout(const IndexImpl* ix, int nq, int nprobe, int k) {
     L.pair = take(pair_room ? pair_layout(pair_nq, nprobe, ix->plan.lut_bytes).total : 0);
     L.total = o;
     return L;
+}
+
+// The layout of a search in a workspace of so many bytes.  Pairs of queries only make a search faster: where the workspace holds
+// everything but their part, it goes without them (total > bytes: it does not hold that either).
+static Layout layout_within(const IndexImpl* ix, int nq, int nprobe, int k, size_t bytes) {
+    const Layout L = make_layout(ix, nq, nprobe, k);
+    return L.total <= bytes ? L : make_layout(ix, nq, nprobe, k, false);
 }
 
 // Workspace of a call, enough for the same batch with fewer probes too: a smaller nprobe may take candidate lists or a
@@ -407,7 +415,7 @@ rago_status rago_search_probes(const rago_index* index, const float* queries, in
     if (!aligned(queries, 16) || !aligned(workspace, 256)) return fail(RAGO_EALIGN, "queries need 16-byte, workspace 256-byte alignment");
     st = check_device(ix);
     if (st != RAGO_OK) return st;
-    const Layout L = make_layout(ix, nq, nprobe, 1);
+    const Layout L = make_layout(ix, nq, nprobe, 1, false);
     if (workspace_bytes < L.total) return fail(RAGO_ENOMEM, "workspace holds %zu bytes, %zu needed", workspace_bytes, L.total);
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
@@ -434,7 +442,7 @@ rago_status rago_search(const rago_index* index, const float* queries, int32_t n
         return fail(RAGO_EALIGN, "queries need 16-byte, workspace 256-byte alignment");
     st = check_device(ix);
     if (st != RAGO_OK) return st;
-    const Layout L = make_layout(ix, nq, nprobe, k);
+    const Layout L = layout_within(ix, nq, nprobe, k, workspace_bytes);
     if (workspace_bytes < L.total) return fail(RAGO_ENOMEM, "workspace holds %zu bytes, %zu needed", workspace_bytes, L.total);
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
@@ -510,9 +518,9 @@ rago_status rago_search_host(const rago_index* index, const float* host_queries,
     if (!aligned(workspace, 256)) return fail(RAGO_EALIGN, "workspace needs 256-byte alignment");
     st = check_device(ix);
     if (st != RAGO_OK) return st;
-    const Layout L = make_layout(ix, nq, nprobe, k);
     size_t staging = 0;
     rago_host_staging_bytes(index, nq, k, &staging);
+    const Layout L = layout_within(ix, nq, nprobe, k, workspace_bytes > staging ? workspace_bytes - staging : 0);
     if (workspace_bytes < L.total + staging)
         return fail(RAGO_ENOMEM, "workspace holds %zu bytes, %zu needed", workspace_bytes, L.total + staging);
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);

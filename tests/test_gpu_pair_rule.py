@@ -56,3 +56,37 @@ def test_pairs_of_96_byte_codes_for_larger_k_answer_as_single_queries_do(k):
         i, s = ix.rago_search(q[b:b + 60].contiguous(), 24, k)
         assert torch.equal(ids[b:b + 60], i) and torch.equal(dists[b:b + 60].view(torch.int32), s.view(torch.int32)), b
     ix.close()
+
+
+# Room for pairs is not a condition of a search: a workspace that lacks a little of it, or all of the pairs' tables, is searched one
+# query at a time.
+@pytest.mark.parametrize("M,k", [(64, 100), (96, 1), (16, 512)])
+def test_a_workspace_without_room_for_pairs_is_searched_one_query_at_a_time(M, k):
+    N, nlist, nq, nprobe = 64_000_000 // M, 4, 140, 3
+    ix, c = _even(M, N, nlist)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(k)
+    q = (c[torch.arange(nq, device="cuda") % nlist] + 0.3 * torch.randn(nq, 4 * M, generator=g, device="cuda")).contiguous()
+    need, staging = ix.search_workspace_bytes(nq, nprobe, k), ix.host_staging_bytes(nq, k)
+    ids, dists = ix.rago_search(q, nprobe, k)
+    alone = _launches(ix, q, nprobe, 1024)
+    assert _launches(ix, q, nprobe, k) == alone + 5
+    per_pair = {16: 32768, 64: 65536, 96: 98304}[M]  # the pair's table, in the part that may be missing
+    for size, launches in ((need, alone + 5), (need - 256, alone), (need - nq // 2 * per_pair, alone)):
+        ws = torch.empty(size + staging, dtype=torch.uint8, device="cuda")
+        n = binding.rago_kernel_launches()
+        i, s = ix.rago_search(q, nprobe, k, workspace=ws[:size])
+        assert binding.rago_kernel_launches() - n == launches
+        torch.cuda.synchronize()
+        ix.rago_check(ws)
+        assert torch.equal(i, ids) and torch.equal(s.view(torch.int32), dists.view(torch.int32))
+        hi, hs = torch.empty((nq, k), dtype=torch.int64), torch.empty((nq, k))
+        n = binding.rago_kernel_launches()
+        ix.rago_search_host(q.cpu(), nprobe, k, hi, hs, ws)
+        assert binding.rago_kernel_launches() - n == launches
+        assert torch.equal(hi, ids.cpu()) and torch.equal(hs, dists.cpu())
+        lists, _ = ix.rago_search_probes(q, nprobe, workspace=ws[:size])
+        assert torch.equal(lists, ix.rago_search_probes(q, nprobe)[0])
+    with pytest.raises(RuntimeError):
+        ix.rago_search(q, nprobe, k, workspace=torch.empty(nq * per_pair, dtype=torch.uint8, device="cuda"))  # the tables of the queries alone
+    ix.close()
