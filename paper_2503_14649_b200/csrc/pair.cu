@@ -187,8 +187,7 @@ __global__ void __cluster_dims__(PI_CTAS, 1, 1) __launch_bounds__(PI_THREADS) pa
     const float* __restrict__ lut_inv, int lut_bytes, int kind, PairParams* __restrict__ params, uint8_t* __restrict__ img) {
     constexpr int COLS = M / PI_CTAS, C4 = COLS / 4, G = PI_THREADS / C4, ROWS = (KSUB + G - 1) / G;
     static_assert(M % (4 * PI_CTAS) == 0, "whole groups of four columns");
-    __shared__ int s_mn[2][G][COLS], s_mx[2][G][COLS];
-    __shared__ int low[2][COLS];
+    __shared__ alignas(16) int s_mn[2][G][COLS], s_mx[2][G][COLS], low[2][COLS];  // read and written as int4 too
     __shared__ uint32_t range[2][COLS];
     __shared__ int part[2][PI_SHIFTS + 1];  // sums of the ranges >> s over this CTA's columns, and of the lows
     grid_dependency_wait();
