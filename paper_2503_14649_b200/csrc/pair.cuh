@@ -19,7 +19,10 @@
 namespace rago {
 
 constexpr int PAIR_MIN_NQ = 65;    // smaller batches are planned by the selection kernel and merged by a kernel of their own
-constexpr int PAIR_MAX_NQ = 4096;  // queries that one CTA sorts; also PREBUILT_MAX_NQ
+// Queries of a batch: their keys fit a CTA's static shared memory (every CTA of pair_rank_kernel holds all of them) and carry the query's
+// number in 12 bits, and their tables are built ahead.
+constexpr int PAIR_MAX_NQ = 4096;
+static_assert(PAIR_MAX_NQ * 8 <= 48 * 1024 && PAIR_MAX_NQ <= 1 << 12 && PAIR_MAX_NQ <= PREBUILT_MAX_NQ, "limits of a batch with pairs");
 constexpr int PAIR_MAX_K = 512;
 
 struct PairParams {   // of a pair of queries

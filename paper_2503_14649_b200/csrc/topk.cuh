@@ -25,8 +25,8 @@ __device__ __forceinline__ uint32_t bisect_mid(long long lo, long long hi, int r
 
 // Ascending bitonic sort of n keys (n a power of two) by `nthreads` threads; sync() is the barrier
 // those threads share.  Ends with a barrier.
-template <class Keys, class Sync>
-__device__ __forceinline__ void block_bitonic_sort(Keys keys, int n, int tid, int nthreads,
+template <class Sync>
+__device__ __forceinline__ void block_bitonic_sort(unsigned long long* keys, int n, int tid, int nthreads,
                                                    Sync sync) {
     for (int size = 2; size <= n; size <<= 1) {
         for (int stride = size >> 1; stride > 0; stride >>= 1) {
@@ -48,8 +48,8 @@ __device__ __forceinline__ void block_bitonic_sort(Keys keys, int n, int tid, in
 // Sort the *cnt buffered keys ascending and cut the buffer to at most k entries.
 // Must be called by all cooperating threads, after a barrier that made *cnt and the keys visible.
 // Returns the new count; ends with a barrier.
-template <class Keys, class Sync>
-__device__ __forceinline__ int block_select(Keys keys, int* cnt, int k, int tid, int nthreads,
+template <class Sync>
+__device__ __forceinline__ int block_select(unsigned long long* keys, int* cnt, int k, int tid, int nthreads,
                                             Sync sync, int cap = TOPK_CAP) {
     int n = *cnt;
     if (n > cap) n = cap;
@@ -71,8 +71,7 @@ __device__ __forceinline__ unsigned long long shfl_xor_u64(unsigned long long v,
     const uint32_t hi = __shfl_xor_sync(0xffffffffu, (uint32_t)(v >> 32), m);
     return ((unsigned long long)hi << 32) | lo;
 }
-template <class Keys>
-__device__ __forceinline__ void warp_bitonic_sort(Keys keys, int n2, int lane) {
+__device__ __forceinline__ void warp_bitonic_sort(unsigned long long* keys, int n2, int lane) {
     unsigned long long k0 = lane < n2 ? keys[lane] : KEY_MAX;
     unsigned long long k1 = lane + 32 < n2 ? keys[lane + 32] : KEY_MAX;
     const int top = n2 > 32 ? 64 : 32;  // padding keys are maximal, so sorting more slots than n2 is harmless
@@ -119,8 +118,8 @@ __device__ __forceinline__ uint32_t warp_sort_u32(uint32_t v, int lane) {
 // key and rank in registers across one barrier and then stores the key at its rank: two barriers and a few dozen
 // instructions per warp, where a bitonic network on shuffles is several hundred dependent ones in a single warp.
 // Same contract as block_select.
-template <int RMAX = RANK_MAX, class Keys, class Sync>
-__device__ __forceinline__ int block_select_short(Keys keys, int* cnt, int k, int tid, int nthreads,
+template <int RMAX = RANK_MAX, class Sync>
+__device__ __forceinline__ int block_select_short(unsigned long long* keys, int* cnt, int k, int tid, int nthreads,
                                                   Sync sync, int cap = TOPK_CAP) {
     int n = *cnt;
     if (n > cap) n = cap;
@@ -189,8 +188,7 @@ __device__ __forceinline__ int block_select_short(Keys keys, int* cnt, int k, in
 }
 
 // Append `key` for the lanes with pred set; one shared atomic per warp.  Whole warp must call.
-template <class Keys>
-__device__ __forceinline__ void warp_push(Keys keys, int* cnt, bool pred, unsigned long long key,
+__device__ __forceinline__ void warp_push(unsigned long long* keys, int* cnt, bool pred, unsigned long long key,
                                           int cap = TOPK_CAP) {
     const unsigned mask = __ballot_sync(0xffffffffu, pred);
     if (mask == 0) return;
