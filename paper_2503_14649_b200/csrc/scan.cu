@@ -28,8 +28,7 @@
 // Table addressing.  Per code byte the inner loop spends one instruction on the address, one shared load and half an add.
 // LUT_DOT (16, 48, 80, 96, 128 bytes): rows of 128 bytes; a byte dot product of the code word with 128 in the byte's place,
 // plus the lane's address of the column in row 0, is the address.  It runs on the multiplier pipe, while byte permutations
-// share theirs with everything else of the loop (58% busy beside 50% of the load pipe for 96 bytes), the rows need no padding and
-// the table may lie anywhere.  LUT_PERM (32 and 64 bytes): rows of 256 bytes from a multiple of 64 KB on, the address
+// share theirs with everything else of the loop, the rows need no padding and the table may lie anywhere.  LUT_PERM (32 and 64 bytes): rows of 256 bytes from a multiple of 64 KB on, the address
 // (place << 16) | (code << 8) | column*4  is one PRMT of the code word and a lane constant for every two bytes, half as many
 // registers.  us per call, permutation / dot product: 96 bytes (400 queries, lists of 2 200) 710 / 667, 80 bytes 358 / 335, 16 bytes
 // 569 / 548, 128 bytes 437 / 432; 64 bytes 483 / 494, 32 bytes 592 / 621, 48 bytes 499 / 512 (pairs 1 188 / 1 174).
@@ -43,12 +42,12 @@
 //
 // Candidates better than the running threshold go to a shared buffer (topk.cuh).  The producer warp
 // watches the buffer count and marks a tile "cut first" when the tiles in flight could overflow it; a
-// cut is a CTA-wide bisection on the ordered score bits that keeps the k best keys and a few more (one
-// barrier per step), and the exact k best are sorted once, when the CTA leaves the query.  The
+// cut is a CTA-wide bisection on the keys (ordered score bits, then position) that keeps the k best and a few
+// more (one barrier per step), and the exact k best are sorted once, when the CTA leaves the query.  The
 // threshold of a query is shared between CTAs through global memory, which only ever removes keys that
 // cannot be among the k best, so the result does not depend on timing.
 //
-// Batches whose queries share long lists are scanned two queries at a time (DUAL; pair.cuh says how the answers stay the same
+// Batches whose queries share long lists are scanned two queries at a time (SCAN_PAIRS; pair.cuh says how the answers stay the same
 // bits): one look-up then serves both, and the kernel below is the same but for what happens to the sums.
 //
 // A warp works on RGW row groups of 32 (virtual) rows per tile, unrolled, so that several independent
@@ -665,9 +664,9 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_, MODE == SCAN_PAIRS>:
 
     // Cut the candidate buffer (more than k keys, count stable, called by all consumer threads after a csync and
     // followed by another before the buffer or its count is used again):
-    // every thread takes its share of the keys into registers, the CTA bisects on the ordered score bits for a
-    // value T with between k and k + k/4 keys at or below it (one barrier per step instead of the ~66 of a full
-    // sort), and the keys up to T are pushed back.  All keys of the k best are kept; T bounds the k-th best.
+    // every thread takes its share of the keys into registers, the CTA bisects for a key with between k and
+    // k + k/4 keys at or below it (one barrier per step instead of the ~66 of a full sort), and the keys up to
+    // it are pushed back.  All keys of the k best are kept; that key bounds the k-th best.
     auto cut_buffer = [&]() {
         constexpr int KPT = (C::KCAP + NCT - 1) / NCT;
         const int n = ctrl->cnt < C::KCAP ? ctrl->cnt : C::KCAP;
@@ -1218,7 +1217,7 @@ static int stages_for(int d, bool need_vt) {
 // pairs 15 x 1 -> 10 x 2 +6%, 8 x 2 -6%; M = 96: 15 x 1 -> 8 x 2 -4%, for pairs 15 x 1 -> 7 x 2 -11%), and 15 consumer warps
 // (four warps on every scheduler, the producer included) beat 12, 14 and 16 wherever their tiles fit (M = 32: +3%,
 // M = 64: +4.5%).  Where a code size has two entries the first one whose shared-memory plan fits the
-// index (dimension, metric) is taken.
+// index (dimension, metric) is taken (of the pairs': find_pair_variant).
 static const Variant kVariants[] = {
     RAGO_SINGLE(4, 4, 1, 16, 2),   // M = 16
     RAGO_SINGLE(8, 8, 1, 15, 2),   // M = 32
