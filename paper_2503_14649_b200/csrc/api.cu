@@ -490,7 +490,7 @@ rago_status rago_search(const rago_index* index, const float* queries, int32_t n
         scan_term = reinterpret_cast<const float*>(pw + PL.entry_term);
     }
     if (!fused) {
-        e = launch_plan_work(ix, scan_list, npairs, ix->plan.tile_vecs, lead, pv, reinterpret_cast<int32_t*>(ws + L.pair_tiles),
+        e = launch_plan_work(ix, scan_list, npairs, scan_tile_vecs(ix, nq, nprobe), lead, pv, reinterpret_cast<int32_t*>(ws + L.pair_tiles),
                              work_prefix, qthresh, nq, slot_cnt, (int)L.nslots, queries, lut_img, lut_inv,
                              L.prebuilt ? reinterpret_cast<float*>(ws + L.lut_scale) : nullptr, s);
         if (e != cudaSuccess) return cuda_fail(e, "work planning");

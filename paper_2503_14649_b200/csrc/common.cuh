@@ -320,6 +320,7 @@ bool scan_supported(int M);
 cudaError_t scan_plan(const IndexImpl* ix, ScanPlan* plan);
 cudaError_t launch_vector_terms(const IndexImpl* ix, float* vterm, cudaStream_t s);
 cudaError_t launch_transpose_codebook(const float* cb, int M, int dsub, float* cbT, cudaStream_t s);
+int scan_tile_vecs(const IndexImpl* ix, int nq, int nprobe);  // vectors per tile of a batch's scan
 int scan_query_lead(const IndexImpl* ix, int nq, int nprobe, int k);  // work units that stand for the start of a query
 bool scan_prefetches(const IndexImpl* ix, int64_t npairs);  // tiles are pulled into L2 ahead of their copies
 struct PairView;

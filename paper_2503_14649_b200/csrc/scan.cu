@@ -105,6 +105,7 @@ struct ScanArgs {
     int32_t stream_once;     // the batch is small: code tiles are fetched with an evict-first hint, so that the centroid
                              // table the next search's coarse step reads stays in L2
     int32_t prefetch;        // pull tiles into L2 ahead of their copies
+    int32_t tile_vecs;       // vectors per tile of this launch (scan_tile_vecs)
     uint32_t dyn_bytes;
     PairView pv;             // batches in which queries are scanned two at a time (pair.cuh)
 };
@@ -128,6 +129,7 @@ struct Cfg {
     static constexpr int TILE_VROWS = NCW * 32 * RGW;
     static constexpr int TV = TILE_VROWS / R;           // vectors per tile
     static constexpr int TILE_BYTES = TILE_VROWS * MV;
+    static constexpr bool CUT_SMALLER = !DUAL && TILE_BYTES > 40 * 1024 && TILE_BYTES <= 48 * 1024;  // scan_tile_vecs
     static constexpr int VT_BYTES = (TV + 4) * 4;       // staged per-vector terms (start rounded down to 16 bytes)
     // Keys of a candidate buffer (two queries at a time: two buffers): as many as fit beside two tiles.  Few keys mean a cut
     // before every tile: 96 bytes, 400 queries over lists of 2 200, k = 500, 2 048 / 4 096 keys 1 305 / 726 us, k = 1 024 1 590 / 800.
@@ -449,7 +451,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_, MODE == SCAN_PAIRS>:
     const int per_unit = DUAL ? 2 * a.nprobe : a.nprobe;
     const int e_base = DUAL ? 0 : 2 * a.nprobe * npairs_q, e_end = DUAL ? 2 * a.nprobe * npairs_q : a.npairs;
     const long long pw = few_pairs ? a.work_prefix[lane < a.npairs ? lane : a.npairs] : 0;  // >= npairs: the total
-    int c_list = 0; long long c_off = 0, c_len = 0, c_ws = 0, c_we = 0; float c_term = 0.f; int c_tv = C::TV;  // producer: lane i's cached pair
+    int c_list = 0; long long c_off = 0, c_len = 0, c_ws = 0, c_we = 0; float c_term = 0.f; int c_tv = C::CUT_SMALLER ? a.tile_vecs : C::TV;  // producer: lane i's cached pair
     if (few_pairs && warp == NCW && lane < a.npairs) {
         c_list = a.probe_list[lane];
         c_term = a.probe_term[lane];
@@ -488,7 +490,7 @@ __global__ void __launch_bounds__(Cfg<WV, G, R, NCW_, RGW_, MODE == SCAN_PAIRS>:
         // (Not for a few pairs, where a CTA has a tile or two and the division would stand before its first copy.)
         auto tile_size = [&]() {
             const uint32_t nt = (uint32_t)(c_we - c_ws), n = (uint32_t)c_len;  // positions are 32-bit
-            c_tv = C::TV;
+            c_tv = C::CUT_SMALLER ? a.tile_vecs : C::TV;
             if (nt > 1u) {
                 const uint32_t share = n / nt;
                 c_tv = (int)((share + (share * nt != n ? 32u : 31u)) & ~31u);
@@ -1287,6 +1289,16 @@ cudaError_t scan_plan(const IndexImpl* ix, ScanPlan* plan) {
     return cudaFuncSetAttribute(v->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_OPTIN);
 }
 
+// Vectors per tile of a batch's scan.  Tiles of 46 KB (48 and 96 bytes) are smaller where whole ones would leave half of the CTAs without one: the
+// lists are then spread over more CTAs, each of which waits for less.  Lists of 1 216 vectors, us per call with 480 / 256 vectors (384 before the
+// tiles grew), 96 bytes: one query, 16 probes 43.0 / 36.3 (38.4), 4 probes 40.0 / 36.6 (38.6); 48 bytes with 960 / 256: 39.6 / 35.1, 36.8 /
+// 34.2; but 8 queries, 8 probes (192 tiles) 43.3 / 48.0, 16 queries, 32 probes 67.3 / 69.6.
+int scan_tile_vecs(const IndexImpl* ix, int nq, int nprobe) {
+    const int whole = ix->plan.tile_vecs, tile_bytes = whole * ix->M;  // bounds: Cfg::CUT_SMALLER, a constant of the kernels (32 bytes 1% slower with a run-time size)
+    const int64_t tiles = (int64_t)nq * nprobe * ((ix->N / ix->nlist + whole) / whole);
+    return tile_bytes > 40 * 1024 && tile_bytes <= 48 * 1024 && 2 * tiles <= ix->plan.ctas ? 256 : whole;
+}
+
 // Work units (tiles) that stand for the start of a query on the line that is cut into one share per CTA.  Every CTA opens
 // the query its share begins with; one that meets the start of another query closes the first (cut, rank), fetches
 // the second's table and fills its candidate buffer without a threshold, which takes as long as scanning several tiles: in
@@ -1302,9 +1314,10 @@ cudaError_t scan_plan(const IndexImpl* ix, ScanPlan* plan) {
 int scan_query_lead(const IndexImpl* ix, int nq, int nprobe, int k) {
     if (nq < 2 || ix->nlist < 1) return 0;
     const float start_us = k <= 32 ? 5.5f : (ix->plan.buffer_keys > TOPK_CAP ? 7.f : 17.f);
-    const float tile_us = (float)(ix->plan.tile_vecs * ix->M) / 36000.f;
+    const int tile_vecs = scan_tile_vecs(ix, nq, nprobe);
+    const float tile_us = (float)(tile_vecs * ix->M) / 36000.f;
     const int lead = (int)(start_us / (tile_us > 0.8f ? tile_us : 0.8f) + 0.5f);
-    const int64_t tiles_per_list = (ix->N / ix->nlist + ix->plan.tile_vecs) / ix->plan.tile_vecs;  // of a list of average length
+    const int64_t tiles_per_list = (ix->N / ix->nlist + tile_vecs) / tile_vecs;  // of a list of average length
     return (int64_t)nq * nprobe * tiles_per_list >= (int64_t)lead * ix->plan.ctas ? lead : 0;
 }
 
@@ -1355,6 +1368,7 @@ cudaError_t launch_scan(const IndexImpl* ix, const ScanPlan& plan, const float* 
     a.metric = ix->metric; a.k = k; a.stages = plan.stages; a.dyn_bytes = (uint32_t)plan.smem_bytes;
     a.stream_once = nq <= 64 ? 1 : 0;
     a.prefetch = scan_prefetches(ix, a.npairs) ? 1 : 0;
+    a.tile_vecs = scan_tile_vecs(ix, nq, nprobe);
     std::memset(&a.pv, 0, sizeof(a.pv));
     if (view) {
         const Variant* p = find_pair_variant(ix->M, ix->d, need_vt, k);
@@ -1729,7 +1743,7 @@ bool fused_plan_args(const IndexImpl* ix, int nq, int npairs, const float* queri
     fp->nq = nq;
     fp->ticket = ticket;
     fp->offsets = ix->list_offsets;
-    fp->tile_vecs = ix->plan.tile_vecs;
+    fp->tile_vecs = scan_tile_vecs(ix, nq, npairs / nq);
     fp->lead = lead;
     fp->prefix = work_prefix;
     fp->qthresh = qthresh;

@@ -106,3 +106,32 @@ def test_lists_around_the_row_groups_of_a_48_byte_tile(metric, k):
             assert torch.allclose(sign * dists[i, :n].double(), want[:n], rtol=0, atol=1e-5 * float(want[:n].abs().max()))
             assert set(ids[i, :n].tolist()) <= set(at[:n + 5].tolist())
     ix.close()
+
+
+# Few 46 KB tiles are cut into tiles of 256 vectors: lists around that size, and as many probes as leave whole tiles (of 74 CTAs' worth) on either side.
+@pytest.mark.parametrize("M,nq,nprobe,k", [(96, 1, 20, 100), (48, 1, 20, 100), (96, 3, 20, 10), (48, 2, 11, 300), (96, 3, 5, 1), (48, 4, 20, 7), (96, 10, 10, 50)])
+def test_few_tiles_are_smaller(M, nq, nprobe, k):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + nq)
+    sizes = [1, 31, 255, 256, 257, 479, 480, 481, 511, 512, 513, 767, 768, 769, 959, 960, 961, 1023, 1024, 1025]
+    N, nlist = sum(sizes), len(sizes)
+    c = torch.randn(nlist, 4 * M, generator=g, device="cuda")
+    books = 0.3 * torch.randn(M, 256, 4, generator=g, device="cuda")
+    codes = torch.randint(0, 256, (N, M), generator=g, device="cuda", dtype=torch.uint8)
+    offsets = torch.tensor([0] + sizes, device="cuda").cumsum(0)
+    ix = binding.rago_index_load(c, books, codes, offsets, torch.arange(N, device="cuda"), "l2")
+    q = torch.randn(nq, 4 * M, generator=g, device="cuda")
+    ids, dists = ix.rago_search(q, nprobe, k)
+    torch.cuda.synchronize()
+    ix.rago_check()
+    lists, _ = ix.rago_search_probes(q, nprobe)
+    for i in range(nq):
+        score = torch.full((N,), float("inf"), dtype=torch.float64, device="cuda")
+        for l in lists[i].tolist():
+            a, b = int(offsets[l]), int(offsets[l + 1])
+            score[a:b] = _scores(q[i:i + 1], c[l], books, codes[a:b], "l2")[0]
+        want, at = score.sort()
+        n = min(k, int(torch.isfinite(score).sum()))
+        assert torch.allclose(dists[i, :n].double(), want[:n], rtol=0, atol=1e-5 * float(want[:n].abs().max()))
+        assert set(ids[i, :n].tolist()) <= set(at[:n + 5].tolist())
+    ix.close()
